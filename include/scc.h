@@ -5,11 +5,15 @@
  * Gu, Sun, "Parallel Strong Connectivity Based on Faster Reachability"
  * (SIGMOD 2023): trimming (Sec. 4.1), a first SCC from one pivot by forward and
  * backward single-reachability (Sec. 4.2), then forward and backward
- * multi-reachability searches over prefix-doubling batches of random pivots
- * (Alg. 1; Sec. 4.3), labelling/partitioning by reachability signature
- * (Alg. 1; Sec. 4.4). Every reachability search uses vertical granularity control
- * (bounded multi-hop local searches, Sec. 3.1-3.2) and a hash-bag frontier
- * (Sec. 3.3). All of it runs in hand-written CUDA kernels on one GPU.
+ * reachability over batches of random pivots (Alg. 1), labelling/partitioning
+ * by reachability signature (Alg. 1; Sec. 4.4). A batch after the first takes
+ * every active vertex as a source and keeps, per vertex, the largest source
+ * reaching it and the largest it reaches: all that Alg. 1's labels use. A graph
+ * of fewer than 8 arcs a vertex without hubs (no row of more than 64 arcs and
+ * 16 times the mean) runs such batches from the start. The single- and
+ * multi-source searches use vertical granularity control (bounded multi-hop
+ * local searches, Sec. 3.1-3.2) and a hash-bag frontier (Sec. 3.3). All of it
+ * runs in hand-written CUDA kernels on one GPU.
  *
  * Conventions shared by every entry point:
  *  - Graphs are int32 CSR: row v of targets is targets[offsets[v] .. offsets[v+1]),
@@ -74,9 +78,8 @@ SCC_API const char* scc_error_string(int code);
  *               which on a graph of high degree grows faster with tau than the
  *               rounds it saves, and on a lattice or k-NN graph more slowly.
  *   beta        prefix-doubling multiplier in (1, 64] (Alg. 1 doubles the batches, the
- *               experiments use 1.5). Default 2: a batch costs rounds whose
- *               time on the GPU is set by memory latency more than by the pairs
- *               they visit, so fewer and larger batches are faster here.
+ *               experiments use 1.5), default 2. Validated and kept; scc_run's
+ *               batches after the first take every active vertex at once.
  *   lambda      first hash-bag chunk size in slots, a power of two in [1024, 2^24]
  *               (Sec. 3.3; chunks grow lambda, 2*lambda, ...). Default 16384.
  *   sigma       hash-bag samples per chunk before it is declared full (Sec. 3.3),
@@ -90,7 +93,8 @@ SCC_API const char* scc_error_string(int code);
  *               (bottom-up) mode of Sec. 4.2; 1: it does once a round's frontier
  *               holds 1/20 of the searched class (the default); k in [2, 1024]:
  *               once it holds 1/k of it.
- *   seed        seed of the pivot permutation (default 0x5CC00).
+ *   seed        seed of the pivot permutation, and of the order of the sources in
+ *               a batch (default 0x5CC00).
  *   ldd_beta    growth factor of the centre batches of cc_run's low-diameter
  *               decomposition, in (1, 64] (Sec. 5.1 uses 1.2). Default 2: each
  *               batch adds a round whose time on the GPU is mostly barrier and
@@ -148,8 +152,7 @@ SCC_API int scc_set_config(scc_handle h, const scc_config* cfg);
  * labels_out[v] = the smallest vertex id u with u ~> v and v ~> u. The result is
  * deterministic and independent of the configuration and seed.
  *   labels_out  host or device int32[n], written.
- * Host-driven rounds: the call synchronises `stream` a few times per round and
- * before returning.
+ * The call synchronises `stream` between its steps and before returning.
  */
 SCC_API int scc_run(scc_handle h, int32_t* labels_out, void* stream);
 
@@ -203,17 +206,17 @@ SCC_API int reach_multi_noalloc(scc_handle h, const int32_t* sources, int32_t k,
  */
 typedef struct scc_stats {
     int32_t n_trimmed;         /* vertices removed by trimming */
-    int32_t first_scc_size;    /* size of the SCC found from the first pivot */
-    int32_t batches;           /* prefix-doubling batches run (including the first) */
-    int32_t search_rounds;     /* reachability rounds (frontier swaps), all searches */
-    int64_t pairs;             /* reachability pairs inserted by multi-reachability */
-    int32_t table_resizes;     /* pair-table regrowths */
+    int32_t first_scc_size;    /* size of the SCC of the first pivot */
+    int32_t batches;           /* batches run (including the first pivot's) */
+    int32_t search_rounds;     /* rounds of the first SCC's searches, and searches of the later batches */
+    int64_t pairs;             /* times the later batches raised a vertex's largest source */
+    int32_t table_resizes;     /* 0 (no pair table is kept) */
     int32_t engine_launches;   /* launches of the reachability engine kernel */
     double ms_trim, ms_first_scc, ms_multi_search, ms_resize, ms_label;
     double ms_engine;          /* summed duration of the first-SCC engine launches */
     int64_t engine_arcs;       /* arcs examined by the first-SCC engine launches */
     int64_t engine_items;      /* items they expanded (adjacency rows read) */
-    int64_t engine_inserted;   /* reachability pairs inserted by multi-reachability */
+    int64_t engine_inserted;   /* the same count as pairs */
     /* graph construction (scc_graph_create of this handle), CUDA events on the
        creating stream: total; the intake pass (copy and range check of the
        targets with the sub-bucket histogram of the transpose); the passes that
@@ -225,13 +228,13 @@ typedef struct scc_stats {
     int32_t n_class_trimmed;   /* vertices finished this way */
     int32_t class_trim_passes; /* passes run */
     double ms_class_trim;
-    /* the launches of the device-side batch loop (multi-reachability) */
+    /* the launch of the later batches */
     int32_t multi_launches;
-    int64_t multi_arcs;        /* arcs examined */
-    int64_t multi_items;       /* items expanded */
+    int64_t multi_arcs;        /* arcs followed from raised vertices */
+    int64_t multi_items;       /* the same count as pairs */
     int32_t tau;               /* the VGC edge budget used (config tau, or the automatic one) */
     double ms_transpose_split; /* transpose: buckets cut into sub-buckets (ms_transpose_rows: their rows) */
-    int64_t multi_active_sum;  /* active vertices summed over the multi-reachability batches */
+    int64_t multi_active_sum;  /* 0 */
 } scc_stats;
 
 SCC_API int scc_get_stats(scc_handle h, scc_stats* out);

@@ -22,6 +22,7 @@ struct scc_graph {
     int32_t n = 0;
     int64_t m_in = 0;      // arcs of the input
     int64_t mt = 0;        // arcs without self-loops (= arcs of G^T)
+    int32_t max_out = 0;   // the longest row of the input
     int32_t* off = nullptr;
     int32_t* adj = nullptr;
     int32_t* toff = nullptr;
@@ -38,15 +39,11 @@ struct scc_graph {
     int32_t* sources = nullptr;
     unsigned long long* fmax = nullptr;
     unsigned long long* bmax = nullptr;
-    unsigned long long* hit = nullptr;
     uint32_t* bits_f = nullptr;
     uint32_t* bits_b = nullptr;
     uint32_t* fbits = nullptr;               // dense-round frontier bitmap (kept zero)
-    long long* bounds_d = nullptr;           // batch bounds on the device
-    int32_t* rem_pos = nullptr;              // remaining active pivot positions / vertices
-    int32_t* rem_v = nullptr;
-    int bounds_cap = 0;
-    void* bgss_ctl = nullptr;
+    uint32_t* act_bits = nullptr;            // active vertices (signature propagation)
+    void* prop_dev = nullptr;                // its control block
     unsigned long long* counters = nullptr;  // [0] nact [1] ndone [2] scratch
     int* flags = nullptr;                    // [0] k [1] bad [2] overflow
     unsigned long long* tab[2] = {nullptr, nullptr};
@@ -210,16 +207,14 @@ int reserve_run_state(scc_graph* h, cudaStream_t s) {
     SCC_TRY(dalloc_t(&h->sources, std::max<int64_t>(n, 64), s));
     SCC_TRY(dalloc_t(&h->fmax, n, s));
     SCC_TRY(dalloc_t(&h->bmax, n, s));
-    SCC_TRY(dalloc_t(&h->hit, n, s));
     SCC_TRY(dalloc_t(&h->bits_f, nw, s));
     SCC_TRY(dalloc_t(&h->bits_b, nw, s));
     SCC_TRY(dalloc_t(&h->counters, 4, s));
     SCC_TRY(dalloc_t(&h->flags, 4, s));
     SCC_TRY(dalloc_t(&h->fbits, 2 * nw, s));
     SCC_CUDA(cudaMemsetAsync(h->fbits, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(2 * nw, 1), s));
-    SCC_TRY(dalloc(&h->bgss_ctl, bgss_ctl_bytes(), s));
-    SCC_TRY(dalloc_t(&h->rem_pos, n, s));
-    SCC_TRY(dalloc_t(&h->rem_v, n, s));
+    SCC_TRY(dalloc(&h->prop_dev, prop_dev_bytes(), s));
+    SCC_TRY(dalloc_t(&h->act_bits, nw, s));
     return SCC_OK;
 }
 
@@ -404,14 +399,14 @@ static int graph_create_impl(scc_graph* h, int32_t n, int64_t m, const int32_t* 
     int32_t* selfrow = nullptr;
     unsigned long long *bcnt = nullptr, *btmp = nullptr;
     unsigned char* stmp = nullptr;
-    SCC_TRY(tmp.alloc(&bad, 1));
+    SCC_TRY(tmp.alloc(&bad, 2));
     SCC_TRY(tmp.alloc(&selfrow, (size_t)n + 1));
     const size_t hist_words = transpose_hist_words(n, shift, K);  // [hist_words - 1]: self-loops found
     SCC_TRY(tmp.alloc(&bcnt, hist_words));
     SCC_TRY(tmp.alloc(&btmp, transpose_tmp_words(n, shift, K)));
     SCC_TRY(tmp.alloc(&stmp, scan_tmp_bytes(n)));
     unsigned long long* self_cnt = bcnt + hist_words - 1;
-    SCC_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
+    SCC_CUDA(cudaMemsetAsync(bad, 0, 2 * sizeof(int), s));
     SCC_CUDA(cudaMemsetAsync(selfrow, 0, sizeof(int32_t) * ((size_t)n + 1), s));
     SCC_CUDA(cudaMemsetAsync(bcnt, 0, sizeof(unsigned long long) * hist_words, s));
     // validation before any kernel indexes with these arrays: the offsets, then
@@ -443,13 +438,14 @@ static int graph_create_impl(scc_graph* h, int32_t n, int64_t m, const int32_t* 
     }
     // the range check and (bucketed path) the partition's self-loop count in
     // one host round trip
-    int hbad = 0;
+    int hbad[2] = {0, 0};
     unsigned long long hself0 = 0;
-    SCC_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+    SCC_CUDA(cudaMemcpyAsync(hbad, bad, sizeof(hbad), cudaMemcpyDeviceToHost, s));
     if (bucketed) SCC_CUDA(cudaMemcpyAsync(&hself0, self_cnt, sizeof(hself0), cudaMemcpyDeviceToHost, s));
     SCC_CUDA(cudaStreamSynchronize(s));
     tmp.release(bad);
-    if (hbad) return SCC_ERR_INVALID_ARG;
+    if (hbad[0]) return SCC_ERR_INVALID_ARG;
+    h->max_out = hbad[1];
     h->mt = m;
     int64_t m_cur = m;
     // forward CSR without its self-loops (selfrow counts them per row)
@@ -546,7 +542,6 @@ static void graph_free(scc_graph* h, cudaStream_t s) {
     dfree(h->sources, s);
     dfree(h->fmax, s);
     dfree(h->bmax, s);
-    dfree(h->hit, s);
     dfree(h->bits_f, s);
     dfree(h->bits_b, s);
     dfree(h->counters, s);
@@ -554,10 +549,8 @@ static void graph_free(scc_graph* h, cudaStream_t s) {
     dfree(h->tab[0], s);
     dfree(h->tab[1], s);
     dfree(h->fbits, s);
-    dfree(h->bounds_d, s);
-    dfree(h->bgss_ctl, s);
-    dfree(h->rem_pos, s);
-    dfree(h->rem_v, s);
+    dfree(h->prop_dev, s);
+    dfree(h->act_bits, s);
     engine_release(&h->eb32, s);
     engine_release(&h->eb64, s);
     dfree(h->soff, s);
@@ -625,6 +618,37 @@ int scc_graph_info(scc_handle h, int32_t* n, int64_t* m, int64_t* m_t) {
     return SCC_OK;
 }
 
+static PropArgs prop_args(scc_graph* h) {
+    PropArgs a;
+    a.off = h->off;
+    a.adj = h->adj;
+    a.toff = h->toff;
+    a.tadj = h->tadj;
+    a.n = h->n;
+    a.m = h->mt;
+    a.seed = h->cfg.seed;
+    a.sf = h->fmax;
+    a.sb = h->bmax;
+    a.act = h->act_bits;
+    a.df = h->bits_f;
+    a.db = h->bits_b;
+    a.rep = h->rep;
+    a.minid = h->tmp_b;
+    a.dev = h->prop_dev;
+    a.num_sms = h->di.num_sms;
+    return a;
+}
+
+static void prop_stats(const PropResult& r, scc_stats* st) {
+    st->batches += r.batches;
+    st->search_rounds += r.searches;
+    st->pairs = (int64_t)r.items;
+    st->engine_inserted = (int64_t)r.items;
+    st->multi_launches = 1;
+    st->multi_arcs = (int64_t)r.arcs;
+    st->multi_items = (int64_t)r.items;
+}
+
 static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
     const int32_t n = h->n;
     scc_stats& st = h->stats;
@@ -633,6 +657,28 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
     if (n == 0) return SCC_OK;
     SCC_TRY(reserve_run_state(h, s));
     EngineOpts o = opts_of(h);
+    const bool host_out = !is_device_ptr(labels_out);
+    int32_t* const dst = host_out ? h->tmp_a : labels_out;
+
+    // ---- graphs of low degree without hubs: the whole run in one launch
+    if ((double)h->mt < kDenseDegree * (double)n &&
+        !prop_skewed((unsigned long long)h->max_out, (unsigned long long)n, (unsigned long long)h->mt)) {
+        EvTimer tp(s);
+        tp.start();
+        PropArgs a = prop_args(h);
+        a.out = dst;
+        PropResult r;
+        SCC_TRY(run_prop(a, &r, s));
+        if (r.status == 0) {
+            if (host_out) SCC_CUDA(cudaMemcpyAsync(labels_out, dst, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost, s));
+            st.n_trimmed = (int32_t)(n - r.active);
+            st.first_scc_size = r.first;
+            st.batches = 1;
+            st.ms_multi_search = tp.stop();
+            prop_stats(r, &st);
+            return SCC_OK;
+        }
+    }
 
     // ---- trimming (Sec. 4.1) and the active list
     EvTimer t(s);
@@ -647,26 +693,6 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
     st.n_trimmed = (int32_t)(n - N);
 
     if (N > 0) {
-        // ---- prefix-doubling batches over the seeded pivot order (Alg. 1)
-        std::vector<int64_t> bounds{0};
-        {
-            double x = 1.0;
-            int64_t pos = 0;
-            while (pos < N) {
-                int64_t sz;
-                if (x >= (double)N) sz = N;
-                else {
-                    sz = (int64_t)x;
-                    if ((double)sz < x) ++sz;
-                }
-                if (sz < 1) sz = 1;
-                pos = (N - pos < sz) ? N : pos + sz;
-                bounds.push_back(pos);
-                x *= h->cfg.beta;
-            }
-        }
-        const int nb = (int)bounds.size() - 1;
-
         // ---- first SCC: single-reachability both ways from the first pivot (Sec. 4.2)
         t.start();
         int64_t p0 = feistel_perm_host(0, N, h->cfg.seed);
@@ -721,125 +747,21 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
         }
         st.batches = 1;
 
-        // ---- multi-reachability batches (Alg. 1; Sec. 4.3-4.5): one device-side loop
-        if (nb > 1 && (int64_t)hc[1] < N) {
-            if (h->bounds_cap < nb + 1) {
-                dfree(h->bounds_d, s);
-                h->bounds_d = nullptr;
-                h->bounds_cap = 0;
-                SCC_TRY(dalloc_t(&h->bounds_d, (size_t)nb + 1, s));
-                h->bounds_cap = nb + 1;
-            }
-            SCC_CUDA(cudaMemcpyAsync(h->bounds_d, bounds.data(), sizeof(long long) * (size_t)(nb + 1),
-                                     cudaMemcpyHostToDevice, s));
-            long long tab_alloc = std::max<long long>(1 << 14, pow2ceil(4 * (int64_t)std::ceil(0.3 * (double)(N - (int64_t)hc[1]))));
-            // the labelling maxima start untagged (only the batches use them)
-            SCC_CUDA(cudaMemsetAsync(h->fmax, 0, (size_t)n * 8, s));
-            SCC_CUDA(cudaMemsetAsync(h->bmax, 0, (size_t)n * 8, s));
-            SCC_CUDA(cudaMemsetAsync(h->hit, 0, (size_t)n * 8, s));
-            BgssArgs a;
-            a.off = h->off;
-            a.adj = h->adj;
-            a.toff = h->toff;
-            a.tadj = h->tadj;
-            a.n = n;
+        // ---- the remaining pivots (Alg. 1): signature propagation
+        if ((int64_t)hc[1] < N) {
+            PropArgs a = prop_args(h);
             a.label = h->label;
-            a.rep = h->rep;
-            a.fmax = h->fmax;
-            a.bmax = h->bmax;
-            a.hit = h->hit;
-            // the pivot positions after the first batch whose vertex is still active
-            SCC_TRY(launch_remaining(h->act, N, h->cfg.seed, bounds[1], h->label, h->tmp_a, h->tmp_b, h->scan_tmp,
-                                     h->rem_pos, h->rem_v, s));
-            int32_t nrem = 0;
-            SCC_CUDA(cudaMemcpyAsync(&nrem, h->tmp_b + (N - bounds[1]), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-            SCC_CUDA(cudaStreamSynchronize(s));
-            a.rem_pos = h->rem_pos;
-            a.rem_v = h->rem_v;
-            a.nrem = nrem;
-            a.N = N;
-            a.bounds = h->bounds_d;
-            a.nb = nb;
-            a.first = 1;
-            a.sources = h->sources;
-            a.bgss_ctl = h->bgss_ctl;
-            a.ndone = hc[1];
-            a.a_prev[0] = a.a_prev[1] = 0;
-            a.ka_prev = 0;
-            a.o = o;
-            // Grid sized to the active vertices (about 2k per block, at least 16
-            // blocks): small remainders run on fewer blocks, whose barriers cost
-            // less; the launch stops for a smaller grid once it could shrink 4x.
-            const int full = bgss_full_grid(h->di.num_sms);
-            const int min_grid = std::min(16, full);
-            auto grid_for_active = [&](long long b) {
-                return (int)std::max<long long>(min_grid, std::min<long long>(full, (b + 2047) / 2048));
-            };
-            auto plan = [&](long long b) {
-                a.grid = grid_for_active(b);
-                a.shrink_below = a.grid >= 4 * min_grid ? (long long)(a.grid / 4) * 2048 : 0;
-            };
-            plan(N - (int64_t)hc[1]);
-            bool fresh = true;  // tables (and bag) must be emptied before the next launch
-            for (int attempt = 0;; ++attempt) {
-                if (attempt > 80) return SCC_ERR_CAPACITY;
-                SCC_TRY(reserve_table(h, 0, tab_alloc, s));
-                SCC_TRY(reserve_table(h, 1, tab_alloc, s));
-                // a search holds at most 3/4 of each of the two tables
-                SCC_TRY(engine_reserve(&h->eb64, 8, (long long)(1.5 * (double)tab_alloc) + (1 << 20), h->cfg.lambda,
-                                       h->mt, h->di.num_sms, s));
-                if (fresh) {  // the kernel keeps both tables empty between batches
-                    SCC_CUDA(cudaMemsetAsync(h->tab[0], 0xff, (size_t)tab_alloc * 8, s));
-                    SCC_CUDA(cudaMemsetAsync(h->tab[1], 0xff, (size_t)tab_alloc * 8, s));
-                    SCC_TRY(engine_reset_slots(&h->eb64, s));
-                    fresh = false;
-                }
-                a.tab[0] = h->tab[0];
-                a.tab[1] = h->tab[1];
-                a.tab_alloc = tab_alloc;
-                a.eb = &h->eb64;
-                BgssResult r;
-                SCC_TRY(run_bgss_device(a, &r, s));
-                st.ms_multi_search += r.ms;
-                st.batches += r.batches;
-                st.search_rounds += r.rounds;
-                st.pairs += (int64_t)r.pairs;
-                st.multi_active_sum += (int64_t)r.active_sum;
-                st.engine_inserted += (int64_t)r.pairs;
-                st.multi_launches++;
-                st.multi_arcs += (int64_t)r.edges;
-                st.multi_items += (int64_t)r.items;
-                hc[1] = r.ndone;
-                if (r.status == 0) break;
-                if (r.status == 2) {  // stopped between batches: tables and bag are empty
-                    a.first = r.batch;
-                    a.ndone = r.ndone;
-                    a.a_prev[0] = r.a_prev[0];
-                    a.a_prev[1] = r.a_prev[1];
-                    a.ka_prev = r.ka_prev;
-                    a.first_min_cap = 0;
-                    plan(N - (int64_t)r.ndone);
-                    continue;
-                }
-                fresh = true;  // stopped inside a batch
-                st.table_resizes++;
-                tab_alloc = std::max<long long>(tab_alloc, pow2ceil(r.need_cap));
-                a.first = r.batch;
-                a.first_min_cap = r.need_cap;
-                a.ndone = r.ndone;
-                a.a_prev[0] = r.a_prev[0];
-                a.a_prev[1] = r.a_prev[1];
-                a.ka_prev = r.ka_prev;
-            }
+            a.N = N - (int64_t)hc[1];
+            t.start();
+            PropResult r;
+            SCC_TRY(run_prop(a, &r, s));
+            st.ms_multi_search = t.stop();
+            prop_stats(r, &st);
         }
-        if ((int64_t)hc[1] != N) return SCC_ERR_INTERNAL;  // every active vertex must be finished
     }
 
     // ---- canonical minimum labels
     t.start();
-    int32_t* dst = labels_out;
-    bool host_out = !is_device_ptr(labels_out);
-    if (host_out) dst = h->tmp_a;
     SCC_CUDA(cudaMemsetAsync(h->flags + 1, 0, sizeof(int), s));
     SCC_TRY(launch_canonicalize(h->rep, n, h->tmp_b, dst, h->flags + 1, s));
     if (host_out) SCC_CUDA(cudaMemcpyAsync(labels_out, dst, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost, s));

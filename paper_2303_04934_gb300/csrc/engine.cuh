@@ -165,6 +165,7 @@ struct GridScope {
     __device__ __forceinline__ static int blocks() { return gridDim.x; }
     __device__ __forceinline__ static bool sync(GridBarrier* b, int* err) { return grid_sync(b, err); }
     __device__ __forceinline__ static int32_t ld(const int32_t* p) { return __ldg(p); }
+    __device__ __forceinline__ static void fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 };
 struct CtaScope {
     __device__ __forceinline__ static int block() { return 0; }
@@ -174,6 +175,7 @@ struct CtaScope {
         return true;
     }
     __device__ __forceinline__ static int32_t ld(const int32_t* p) { return *p; }
+    __device__ __forceinline__ static void fence() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 };
 
 // adjacency arrays of an item's graph

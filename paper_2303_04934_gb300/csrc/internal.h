@@ -97,7 +97,7 @@ int device_info(DeviceInfo* out);
 
 // --------------------------------------------------------- graph building --
 // Validate CSR offsets on the device (off[0] = 0, off[n] = m, non-decreasing);
-// *bad (device int) becomes nonzero if malformed.
+// bad[0] (device int[2]) becomes nonzero if malformed, bad[1] the longest row.
 int launch_validate_offsets(const int32_t* off, int32_t n, int64_t m, int* bad, cudaStream_t s);
 // Transposed CSR (transpose.cu). bucket_shift(n): vertices per coarse bucket
 // = 2^shift, at most 512 buckets.
@@ -185,12 +185,6 @@ int launch_init_labels(const int32_t* off, const int32_t* toff, int32_t n, int32
                        unsigned long long* nact, cudaStream_t s);
 // act = increasing list of v with label[v] >= 0 (scan-based, order preserving).
 int launch_compact_active(const int32_t* label, int32_t n, void* scan_tmp, int32_t* act, cudaStream_t s);
-// Pivot positions p in [p0, N) whose vertex act[pi(p)] is still active, in
-// increasing p: rem_pos[j] = p, rem_v[j] = the vertex; their number is
-// pos_tmp[N - p0] after the call (exclusive scan of the flags).
-int launch_remaining(const int32_t* act, int64_t N, uint64_t seed, int64_t p0, const int32_t* label,
-                     int32_t* flags_tmp, int32_t* pos_tmp, void* scan_tmp, int32_t* rem_pos, int32_t* rem_v,
-                     cudaStream_t s);
 // order[p] = act[pi(p)] for p < N (debug hook).
 int launch_pivot_order(const int32_t* act, int64_t N, uint64_t seed, int32_t* order, cudaStream_t s);
 
@@ -314,50 +308,43 @@ int run_mask2(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* 
 int run_mask(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* sources, int32_t k,
              unsigned long long* mask, EngineBuf* b, const EngineOpts& o, EngineRun* out, cudaStream_t st);
 
-// Device-side loop over the multi-reachability batches (bgss.cu).
-struct BgssArgs {
+// Signature propagation (prop.cu). With label == nullptr the whole SCC of the
+// graph: labels into out (device), unless a row is far longer than the mean
+// (prop_skewed; status 1: nothing was computed, the first SCC should be found by
+// a search of its own); otherwise the N vertices with label[v] >= 0 of a run whose first
+// SCC is done: rep[v] becomes a vertex of v's SCC, the same for all of it.
+struct PropArgs {
     const int32_t *off, *adj, *toff, *tadj;
     int32_t n;
-    int32_t* label;
-    int32_t* rep;
-    unsigned long long *fmax, *bmax, *hit;
-    const int32_t* rem_pos;   // remaining active pivot positions (increasing) and their vertices
-    const int32_t* rem_v;
-    long long nrem;
-    long long N;              // active vertices after trimming (pivot positions)
-    const long long* bounds;  // device, nb + 1 entries
-    int nb;
-    int first;
-    long long first_min_cap = 0;
-    long long shrink_below = 0;  // return with status 2 once fewer vertices are active
-    int grid = 0;                // blocks of the cooperative launch (0 = all co-resident)
-    int32_t* sources;
-    unsigned long long* tab[2];
-    long long tab_alloc;
-    EngineBuf* eb;
-    void* bgss_ctl;  // device, bgss_ctl_bytes()
-    unsigned long long ndone;
-    unsigned long long a_prev[2];
-    int ka_prev = 0;  // sources of the batch whose pairs a_prev holds (0: unknown)
-    EngineOpts o;
+    long long m;
+    uint64_t seed;
+    unsigned long long *sf, *sb;   // n words each
+    uint32_t *act, *df, *db;       // ceil(n / 32) words each
+    int32_t* rep;                  // n
+    const int32_t* label = nullptr;
+    long long N = 0;
+    int32_t* minid = nullptr;      // n (label == nullptr)
+    int32_t* out = nullptr;        // n (label == nullptr)
+    void* dev = nullptr;           // prop_dev_bytes()
+    int num_sms = 0;
 };
-struct BgssResult {
-    float ms = 0;
-    int status = 0;  // 0 finished; 1 grow to need_cap and resume at batch; 2 resume with a smaller grid
-    int batch = 0;
-    long long need_cap = 0;
-    unsigned long long ndone = 0;
-    unsigned long long a_prev[2] = {0, 0};
-    int ka_prev = 0;
-    unsigned long long pairs = 0;
-    int batches = 0;
-    int rounds = 0;
-    unsigned long long edges = 0, items = 0;
-    unsigned long long active_sum = 0;  // active vertices summed over the launch's batches
+struct PropResult {
+    int status = 0;
+    int64_t active = 0;   // untrimmed vertices
+    int32_t first = 0;    // vertices in the SCC of the first pivot
+    int batches = 0;      // batches that ran searches
+    int searches = 0;     // searches, those resumed after a check included
+    unsigned long long items = 0, arcs = 0;
 };
-size_t bgss_ctl_bytes();
-int bgss_full_grid(int num_sms);
-int run_bgss_device(const BgssArgs& a, BgssResult* res, cudaStream_t st);
+size_t prop_dev_bytes();
+// A graph with a row of more than 64 arcs and of more than 16 times the mean
+// degree: a hub's value grows several times, and each time costs its whole row,
+// while the first SCC's bitmap searches read it once (the batched kernel draws
+// its line between dense and shared rounds at the same factor).
+__host__ __device__ inline bool prop_skewed(unsigned long long max_deg, unsigned long long n, unsigned long long m) {
+    return max_deg > 64 && max_deg * n > 16 * m;
+}
+int run_prop(const PropArgs& a, PropResult* res, cudaStream_t st);
 
 // Batched SCC kernel on caller-owned packed device arrays (batch.cu), working
 // memory allocated once: for a serving loop. budget 0: half the free memory,

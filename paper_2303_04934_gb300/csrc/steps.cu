@@ -51,12 +51,19 @@ __device__ __forceinline__ void tile_rows(const int32_t* off, int32_t n, int64_t
 }
 
 // ---------------------------------------------------------------- validate --
+// bad[0]: the offsets are malformed; bad[1]: the longest row.
 __global__ void k_validate_offsets(const int32_t* __restrict__ off, int32_t n, int64_t m, int* bad) {
     int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     if (tid == 0 && (off[0] != 0 || (int64_t)off[n] != m)) atomicExch(bad, 1);
-    for (int64_t i = tid; i < n; i += stride)
-        if (off[i] > off[i + 1]) atomicExch(bad, 1);
+    int most = 0;
+    for (int64_t i = tid; i < n; i += stride) {
+        const int a = off[i], b = off[i + 1];
+        if (a > b) atomicExch(bad, 1);
+        else if (a >= 0) most = max(most, b - a);
+    }
+    most = __reduce_max_sync(kFull, most);
+    if (lane_id() == 0 && most > ld_volatile(&bad[1])) atomicMax(&bad[1], most);
 }
 
 // Forward CSR without self-loops. Rows without self-loops are copied arc-parallel;
@@ -222,24 +229,6 @@ __global__ void k_init_labels(const int32_t* __restrict__ off, const int32_t* __
 __global__ void k_pivot_order(const int32_t* __restrict__ act, int64_t N, Feistel f, int32_t* order) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
         order[p] = act[f.perm((uint64_t)p, (uint64_t)N)];
-}
-
-// Remaining pivot positions p >= p0 whose vertex is still active, in order.
-__global__ void k_rem_flags(const int32_t* __restrict__ act, int64_t N, Feistel f, int64_t p0,
-                            const int32_t* __restrict__ label, int32_t* flags) {
-    for (int64_t p = p0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
-        flags[p - p0] = label[act[f.perm((uint64_t)p, (uint64_t)N)]] >= 0;
-}
-// rem_pos/rem_v of the remaining pivots, at the places the scan of the flags gives.
-__global__ void k_rem_scatter(const int32_t* __restrict__ act, int64_t N, Feistel f, int64_t p0,
-                              const int32_t* __restrict__ flags, const int32_t* __restrict__ pos, int32_t* rem_pos,
-                              int32_t* rem_v) {
-    for (int64_t p = p0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (int64_t)gridDim.x * blockDim.x)
-        if (flags[p - p0]) {
-            const int32_t j = pos[p - p0];
-            rem_pos[j] = (int32_t)p;
-            rem_v[j] = act[f.perm((uint64_t)p, (uint64_t)N)];
-        }
 }
 
 // Active list (vertices with label >= 0, in increasing order) in two passes
@@ -615,21 +604,6 @@ int64_t feistel_perm_host(int64_t p, int64_t N, uint64_t seed) {
     Feistel f;
     f.init(seed, (uint64_t)N);
     return (int64_t)f.perm((uint64_t)p, (uint64_t)N);
-}
-
-int launch_remaining(const int32_t* act, int64_t N, uint64_t seed, int64_t p0, const int32_t* label,
-                     int32_t* flags_tmp, int32_t* pos_tmp, void* scan_tmp, int32_t* rem_pos, int32_t* rem_v,
-                     cudaStream_t s) {
-    const int64_t cnt = N - p0;
-    if (cnt <= 0) return SCC_OK;
-    Feistel f;
-    f.init(seed, (uint64_t)N);
-    k_rem_flags<<<grid_for(cnt, kBlk), kBlk, 0, s>>>(act, N, f, p0, label, flags_tmp);
-    SCC_LAUNCH();
-    SCC_TRY(launch_scan(flags_tmp, pos_tmp, cnt, scan_tmp, s));
-    k_rem_scatter<<<grid_for(cnt, kBlk), kBlk, 0, s>>>(act, N, f, p0, flags_tmp, pos_tmp, rem_pos, rem_v);
-    SCC_LAUNCH();
-    return SCC_OK;
 }
 
 int launch_pivot_order(const int32_t* act, int64_t N, uint64_t seed, int32_t* order, cudaStream_t s) {
