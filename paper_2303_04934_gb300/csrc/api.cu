@@ -23,6 +23,7 @@ struct scc_graph {
     int64_t m_in = 0;      // arcs of the input
     int64_t mt = 0;        // arcs without self-loops (= arcs of G^T)
     int32_t max_out = 0;   // the longest row of the input
+    int32_t hub = -1;      // a vertex of large degree both ways (found on first use)
     int32_t* off = nullptr;
     int32_t* adj = nullptr;
     int32_t* toff = nullptr;
@@ -42,7 +43,7 @@ struct scc_graph {
     uint32_t* bits_f = nullptr;
     uint32_t* bits_b = nullptr;
     uint32_t* fbits = nullptr;               // dense-round frontier bitmap (kept zero)
-    uint32_t* act_bits = nullptr;            // active vertices (signature propagation)
+    uint32_t* act_bits = nullptr;            // active vertices (signature propagation), dirty ones (reach_multi)
     void* prop_dev = nullptr;                // its control block
     unsigned long long* counters = nullptr;  // [0] nact [1] ndone [2] scratch
     int* flags = nullptr;                    // [0] k [1] bad [2] overflow
@@ -204,7 +205,7 @@ int reserve_run_state(scc_graph* h, cudaStream_t s) {
     SCC_TRY(dalloc_t(&h->tmp_a, n + 1, s));
     SCC_TRY(dalloc_t(&h->tmp_b, n + 1, s));
     SCC_TRY(dalloc(&h->scan_tmp, scan_tmp_bytes(n), s));
-    SCC_TRY(dalloc_t(&h->sources, std::max<int64_t>(n, 64), s));
+    SCC_TRY(dalloc_t(&h->sources, std::max<int64_t>(n, 128), s));
     SCC_TRY(dalloc_t(&h->fmax, n, s));
     SCC_TRY(dalloc_t(&h->bmax, n, s));
     SCC_TRY(dalloc_t(&h->bits_f, nw, s));
@@ -270,6 +271,52 @@ struct EvTimer {
 // ==================================================================== ABI ====
 namespace scc {
 
+// Arcs from which reach_multi on a graph of high degree with hubs starts with the
+// hub's own two sets: those cost 0.8-1.5 ms whatever the size (their rounds are
+// bound by latency), the masks alone about 0.04 ms a million arcs. Masks alone
+// against the hub first, R-MAT of edge factor 16, 64 sources: 1 M vertices 0.87 /
+// 0.84 ms, 2 M 1.51 / 1.01, 4 M 2.54 / 1.17, 8 M 4.35 / 1.53; without hubs or below 8
+// arcs a vertex the masks alone win (4 M x 16 uniform 1.50 / 1.64, R-MAT 4 M x 8
+// 1.52 / 1.72, k-NN 1 M x 8 0.82 / 2.09).
+constexpr int64_t kHubArcs = 1 << 24;
+
+// Masks of the sources dsrc (device) along direction dir: words = 1 or 2 mask
+// words per vertex.
+static int reach_masks(scc_graph* h, const int32_t* dsrc, int32_t k, int32_t dir, unsigned long long* mask, int words,
+                       cudaStream_t s) {
+    SCC_TRY(reserve_run_state(h, s));
+    const int32_t n = h->n;
+    ReachArgs a;
+    a.off = dir ? h->toff : h->off;
+    a.adj = dir ? h->tadj : h->adj;
+    a.toff = dir ? h->off : h->toff;
+    a.tadj = dir ? h->adj : h->tadj;
+    a.n = n;
+    a.m = h->mt;
+    a.src = dsrc;
+    a.k = k;
+    a.words = words;
+    a.mask = mask;
+    a.dirty = h->act_bits;
+    a.dev = h->prop_dev;
+    a.num_sms = h->di.num_sms;
+    EngineOpts o = opts_of(h);
+    const bool skewed = prop_skewed((unsigned long long)h->max_out, (unsigned long long)n, (unsigned long long)h->mt);
+    const bool hubs = o.high_degree && skewed && h->mt >= kHubArcs;
+    a.pull = !skewed && prop_pulls(h->mt, h->di.num_sms);
+    if (hubs) {
+        if (h->hub < 0) SCC_TRY(find_hub(h->off, h->toff, n, h->counters + 3, h->di.num_sms, &h->hub, s));
+        SCC_TRY(engine_reserve(&h->eb32, 4, (long long)n + 1024, h->cfg.lambda, h->mt, h->di.num_sms, s));
+        SCC_TRY(launch_prefill_bits(nullptr, 0, n, h->bits_f, h->bits_b, s));
+        EngineRun r;
+        SCC_TRY(run_single(h->off, h->adj, n, h->hub, h->bits_f, dense_opts(h, 0, n), &h->eb32, o, &r, s));
+        SCC_TRY(run_single(h->toff, h->tadj, n, h->hub, h->bits_b, dense_opts(h, 1, n), &h->eb32, o, &r, s));
+        a.from_hub = dir ? h->bits_b : h->bits_f;
+        a.to_hub = dir ? h->bits_f : h->bits_b;
+    }
+    return run_reach(a, s);
+}
+
 // reach_multi with 1..128 sources already on the device: mask2 (device, two
 // words per vertex) gets bit j of vertex v (word 2 v + j / 64, bit j % 64) iff
 // sources[j] reaches v (dir 0) or v reaches sources[j] (dir 1).
@@ -277,24 +324,7 @@ int reach_multi_wide(scc_graph* h, const int32_t* sources_d, int32_t k, int32_t 
                           unsigned long long* mask2, cudaStream_t s) {
     if (!h || !sources_d || !mask2 || k < 1 || k > 128 || (dir != 0 && dir != 1)) return SCC_ERR_INVALID_ARG;
     h->last = s;
-    const int32_t n = h->n;
-    SCC_TRY(reserve_run_state(h, s));
-    for (int attempt = 0;; ++attempt) {  // bag too small: restart with twice the buffers
-        if (attempt > 8) return SCC_ERR_CAPACITY;
-        SCC_CUDA(cudaMemsetAsync(mask2, 0, (size_t)n * 16, s));
-        SCC_CUDA(cudaMemsetAsync(h->flags + 1, 0, sizeof(int), s));
-        SCC_TRY(launch_mask_init(sources_d, k, n, 2, mask2, h->flags + 1, s));
-        int bad = 0;
-        SCC_CUDA(cudaMemcpyAsync(&bad, h->flags + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-        SCC_CUDA(cudaStreamSynchronize(s));
-        if (bad) return SCC_ERR_INVALID_ARG;
-        SCC_TRY(engine_reserve(&h->eb32, 4, ((long long)n + 1024) << attempt, h->cfg.lambda, h->mt, h->di.num_sms, s));
-        EngineRun r;
-        int rc = run_mask2(dir == 0 ? h->off : h->toff, dir == 0 ? h->adj : h->tadj, n, sources_d, k, mask2, &h->eb32,
-                           opts_of(h), &r, s);
-        if (rc == SCC_ERR_CAPACITY) continue;
-        return rc;
-    }
+    return reach_masks(h, sources_d, k, dir, mask2, 2, s);
 }
 
 }  // namespace scc
@@ -666,6 +696,7 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
         EvTimer tp(s);
         tp.start();
         PropArgs a = prop_args(h);
+        a.pull = prop_pulls(h->mt, h->di.num_sms);
         a.out = dst;
         PropResult r;
         SCC_TRY(run_prop(a, &r, s));
@@ -749,7 +780,7 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
 
         // ---- the remaining pivots (Alg. 1): signature propagation
         if ((int64_t)hc[1] < N) {
-            PropArgs a = prop_args(h);
+            PropArgs a = prop_args(h);  // marking, not pulling: a hub's row would be read in every pass
             a.label = h->label;
             a.N = N - (int64_t)hc[1];
             t.start();
@@ -793,26 +824,7 @@ int reach_multi(scc_handle h, const int32_t* sources, int32_t k, int32_t dir, ui
     SCC_TRY(to_device(dsrc, sources, sizeof(int32_t) * (size_t)k, s));
     bool dev_out = is_device_ptr(out);
     unsigned long long* mask = dev_out ? reinterpret_cast<unsigned long long*>(out) : h->fmax;
-    // A vertex re-enters the frontier each time it gains source bits, so a round
-    // can hold more than n items; if the bag runs out of room the search restarts
-    // from the sources with twice the buffers.
-    for (int attempt = 0;; ++attempt) {
-        if (attempt > 8) return SCC_ERR_CAPACITY;
-        SCC_CUDA(cudaMemsetAsync(mask, 0, (size_t)n * 8, s));
-        SCC_CUDA(cudaMemsetAsync(h->flags + 1, 0, sizeof(int), s));
-        SCC_TRY(launch_mask_init(dsrc, k, n, 1, mask, h->flags + 1, s));
-        int bad = 0;
-        SCC_CUDA(cudaMemcpyAsync(&bad, h->flags + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-        SCC_CUDA(cudaStreamSynchronize(s));
-        if (bad) return SCC_ERR_INVALID_ARG;
-        SCC_TRY(engine_reserve(&h->eb32, 4, ((long long)n + 1024) << attempt, h->cfg.lambda, h->mt, h->di.num_sms, s));
-        EngineRun r;
-        int rc = run_mask(dir == 0 ? h->off : h->toff, dir == 0 ? h->adj : h->tadj, n, dsrc, k, mask, &h->eb32,
-                          opts_of(h), &r, s);
-        if (rc == SCC_ERR_CAPACITY) continue;
-        SCC_TRY(rc);
-        break;
-    }
+    SCC_TRY(reach_masks(h, dsrc, k, dir, mask, 1, s));
     if (!dev_out) SCC_TRY(from_device(out, mask, (size_t)n * 8, s));
     SCC_CUDA(cudaStreamSynchronize(s));
     // mask mode uses fmax as scratch: the next scc_run clears it

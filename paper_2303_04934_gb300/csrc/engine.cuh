@@ -1105,42 +1105,6 @@ struct PolMask {
     }
 };
 
-// reach_multi with up to 128 sources: two 64-bit words per vertex, mask[2 v]
-// holding sources 0..63 and mask[2 v + 1] sources 64..127 (the same search as
-// PolMask, with the item's two words as its context).
-struct Mask128 {
-    unsigned long long lo, hi;
-};
-__device__ __forceinline__ Mask128 shfl_any(const Mask128& v, int src) {
-    return {__shfl_sync(kFull, v.lo, src), __shfl_sync(kFull, v.hi, src)};
-}
-struct PolMask2 {
-    using Item = uint32_t;
-    static constexpr int kQueue = 256;
-    static constexpr bool kCountInserts = false;
-    static constexpr bool kDense = false;
-    static constexpr bool kCtxInQueue = false;
-    using Ctx = Mask128;
-    static constexpr bool kTwoGraphs = false;
-    static constexpr bool kInject = false;
-    static constexpr const char* kName = "mask-reach-128";
-    unsigned long long* mask;
-    bool test_first;  // read the target's words before the atomics (high-degree graphs)
-    __device__ __forceinline__ int vertex(Item it) const { return (int)it; }
-    __device__ __forceinline__ Mask128 ctx(Item it) const {
-        return {ld_volatile(&mask[2 * (size_t)it]), ld_volatile(&mask[2 * (size_t)it + 1])};
-    }
-    __device__ __forceinline__ bool seed(Item) const { return true; }
-    __device__ __forceinline__ bool visit(Item, const Mask128& mu, int w, Item& child) const {
-        unsigned long long* tw = mask + 2 * (size_t)w;
-        if (test_first && ((mu.lo & ~ld_volatile(&tw[0])) | (mu.hi & ~ld_volatile(&tw[1]))) == 0) return false;
-        const unsigned long long o0 = mu.lo ? atomicOr(&tw[0], mu.lo) : 0ull;
-        const unsigned long long o1 = mu.hi ? atomicOr(&tw[1], mu.hi) : 0ull;
-        child = (Item)w;
-        return ((mu.lo & ~o0) | (mu.hi & ~o1)) != 0;
-    }
-};
-
 // Low-diameter decomposition (Sec. 5.1, Alg. 4 function LDD) on the symmetric
 // graph: vertex items; an arc (u, w) claims an unvisited w for u's centre
 // (center[w] = center[u] by CAS from -1: Alg. 4 "visit[u] <- true, L(u) <-

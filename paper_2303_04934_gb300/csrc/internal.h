@@ -301,13 +301,6 @@ int run_single(const int32_t* off, const int32_t* adj, int32_t n, int32_t s, uin
 int run_pairs(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* label, const int32_t* sources,
               int32_t k, unsigned long long* table, int64_t cap, long long max_inserted, EngineBuf* b,
               const EngineOpts& o, EngineRun* out, cudaStream_t st);
-// Mask reachability: mask already holds the source bits; init = sources.
-// mask2: two words per vertex, k <= 128
-int run_mask2(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* sources, int32_t k,
-              unsigned long long* mask2, EngineBuf* b, const EngineOpts& o, EngineRun* out, cudaStream_t st);
-int run_mask(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* sources, int32_t k,
-             unsigned long long* mask, EngineBuf* b, const EngineOpts& o, EngineRun* out, cudaStream_t st);
-
 // Signature propagation (prop.cu). With label == nullptr the whole SCC of the
 // graph: labels into out (device), unless a row is far longer than the mean
 // (prop_skewed; status 1: nothing was computed, the first SCC should be found by
@@ -320,6 +313,7 @@ struct PropArgs {
     uint64_t seed;
     unsigned long long *sf, *sb;   // n words each
     uint32_t *act, *df, *db;       // ceil(n / 32) words each
+    bool pull = false;             // the searches only pull (prop_pulls)
     int32_t* rep;                  // n
     const int32_t* label = nullptr;
     long long N = 0;
@@ -337,6 +331,7 @@ struct PropResult {
     unsigned long long items = 0, arcs = 0;
 };
 size_t prop_dev_bytes();
+bool prop_pulls(long long m, int num_sms);
 // A graph with a row of more than 64 arcs and of more than 16 times the mean
 // degree: a hub's value grows several times, and each time costs its whole row,
 // while the first SCC's bitmap searches read it once (the batched kernel draws
@@ -345,6 +340,31 @@ __host__ __device__ inline bool prop_skewed(unsigned long long max_deg, unsigned
     return max_deg > 64 && max_deg * n > 16 * m;
 }
 int run_prop(const PropArgs& a, PropResult* res, cudaStream_t st);
+
+// Multi-source reachability (reach.cu): mask word(s) of v get bit j iff src[j]
+// reaches v along (off, adj), whose transpose is (toff, tadj); words = 1 (k <=
+// 64) or 2 (k <= 128). SCC_ERR_INVALID_ARG when a source is out of range.
+// from_hub, to_hub: bitmaps of the vertices that one vertex reaches, and that
+// reach it, along (off, adj); both or neither (null).
+struct ReachArgs {
+    const int32_t *off, *adj, *toff, *tadj;
+    int32_t n;
+    long long m;
+    const int32_t* src;  // device
+    int k;
+    int words;
+    unsigned long long* mask;  // n * words
+    uint32_t* dirty;           // ceil(n / 32)
+    bool pull = false;         // the search only pulls (prop_pulls)
+    const uint32_t* from_hub = nullptr;
+    const uint32_t* to_hub = nullptr;
+    void* dev;  // prop_dev_bytes()
+    int num_sms;
+};
+int run_reach(const ReachArgs& a, cudaStream_t st);
+// A vertex whose smaller degree is the largest (n > 0); tmp: one device word.
+int find_hub(const int32_t* off, const int32_t* toff, int32_t n, unsigned long long* tmp, int num_sms, int32_t* hub,
+             cudaStream_t st);
 
 // Batched SCC kernel on caller-owned packed device arrays (batch.cu), working
 // memory allocated once: for a serving loop. budget 0: half the free memory,

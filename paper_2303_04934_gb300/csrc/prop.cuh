@@ -44,7 +44,6 @@ constexpr uint32_t kPropDone = 0xffffffffu;
 constexpr int kPropQueue = 256;    // vertices a warp gathers before it works on them
 constexpr int kPropMarks = 384;    // marks a warp gathers before it publishes them
 constexpr int kPropBigRow = 64;    // rows longer than this are relaxed by the whole warp
-constexpr int kPropPoll = 2;       // bitmap words of each direction a lane polls at a time
 constexpr int kPropUnroll = 4;     // arcs of a row in flight per lane
 constexpr unsigned kPropSweepMin = 1;  // a sweep follows while the last one raised n values or more
 constexpr int kPropTrimPasses = 3; // trimming passes at the start of a batch, at most
@@ -68,23 +67,11 @@ __host__ __device__ __forceinline__ uint32_t prop_unmix(uint32_t x) {
     return x;
 }
 
-struct PropGraph {
-    const int32_t *off, *adj, *toff, *tadj;
-    int32_t n;
-    uint32_t k0;  // key(v) = prop_mix(v ^ k0)
-    unsigned long long *sf, *sb;  // forward (from ancestors) and backward state
-    uint32_t *act;                // active vertices
-    uint32_t *df, *db;            // dirty vertices, per direction
-    int32_t* rep;                 // a vertex of v's SCC, the same for all of it
-    __device__ __forceinline__ uint32_t key(uint32_t v) const { return prop_mix(v ^ k0); }
-    __device__ __forceinline__ uint32_t vertex(uint32_t key) const { return prop_unmix(key) ^ k0; }
-};
-
 struct PropCtl {
     GridBarrier bar;
     int err;
     int idle;                 // idle blocks
-    unsigned int found;       // last check that found a dirty word
+    unsigned int found;       // last check that found work left
     unsigned long long count[4];  // vertices finished by a counting step, a ring over the steps
     unsigned long long items, arcs;
     unsigned long long active0;  // active vertices after the first trim
@@ -96,25 +83,135 @@ struct PropCtl {
     unsigned int first;  // vertices in the first pivot's SCC
 };
 
+struct PropShared {
+    int idle;  // idle warps of the block
+    int exit;  // the search is over (or failed)
+};
+
 __device__ __forceinline__ unsigned long long prop_pack(uint32_t lab, uint32_t key) {
     return ((unsigned long long)lab << 32) | key;
 }
 
-struct PropShared {
-    int idle;  // idle warps of the block
-    int exit;  // the search is over (or failed)
-    int ok;
+// ----------------------------------------------------------------- values --
+// What a search spreads along the arcs: a value per vertex and direction that
+// only grows. gains: whether a vertex holding t grows by mine; raise: the same
+// in memory. part: what a vertex holding a can take from t, folded over its
+// neighbours before it is compared with a (more) and put into it (with).
+
+// the largest source, inside a class (state class << 32 | key)
+struct PropMax {
+    using Val = unsigned long long;
+    static constexpr int kDirs = 2;  // from ancestors along G, from descendants along G^T
+    static constexpr bool kNamed = true;  // a value names a vertex, whose own value may be larger
+    uint32_t k0;  // key(v) = prop_mix(v ^ k0)
+    __device__ __forceinline__ uint32_t key(uint32_t v) const { return prop_mix(v ^ k0); }
+    __device__ __forceinline__ uint32_t vertex(uint32_t key) const { return prop_unmix(key) ^ k0; }
+    __device__ __forceinline__ uint32_t named(Val x) const { return vertex((uint32_t)x); }
+    __device__ __forceinline__ static Val load(const Val* p, size_t i) { return ld_volatile(&p[i]); }
+    __device__ __forceinline__ static void store(Val* p, size_t i, Val x) { *(volatile Val*)&p[i] = x; }
+    __device__ __forceinline__ static bool gains(Val mine, Val t) { return (t >> 32) == (mine >> 32) && t < mine; }
+    using Part = uint32_t;  // the key, 0 outside the class
+    __device__ __forceinline__ static Part part(Val a, Val t) { return (t >> 32) == (a >> 32) ? (uint32_t)t : 0u; }
+    __device__ __forceinline__ static Part fold(Part a, Part b) { return max(a, b); }
+    __device__ __forceinline__ static Val with(Val a, Part p) { return (a & ~0xffffffffull) | p; }
+    __device__ __forceinline__ static bool more(Part p, Val a) { return p > (uint32_t)a; }
+    __device__ __forceinline__ static void raise(Val* p, size_t i, Val mine) { atomicMax(&p[i], mine); }
+    __device__ __forceinline__ static Val none() { return prop_pack(kPropDone, 0); }  // takes and gives nothing
+};
+// the set of sources, 64 or 128 of them (mask words v, or 2 v and 2 v + 1)
+struct PropOr {
+    using Val = unsigned long long;
+    static constexpr int kDirs = 1;
+    static constexpr bool kNamed = false;
+    __device__ __forceinline__ uint32_t named(Val) const { return 0; }
+    __device__ __forceinline__ static Val load(const Val* p, size_t i) { return ld_volatile(&p[i]); }
+    __device__ __forceinline__ static void store(Val* p, size_t i, Val x) { *(volatile Val*)&p[i] = x; }
+    __device__ __forceinline__ static bool gains(Val mine, Val t) { return (mine & ~t) != 0; }
+    using Part = Val;
+    __device__ __forceinline__ static Part part(Val, Val t) { return t; }
+    __device__ __forceinline__ static Part fold(Part a, Part b) { return a | b; }
+    __device__ __forceinline__ static Val with(Val a, Part p) { return a | p; }
+    __device__ __forceinline__ static bool more(Part p, Val a) { return (p & ~a) != 0; }
+    __device__ __forceinline__ static void raise(Val* p, size_t i, Val mine) { atomicOr(&p[i], mine); }
+    __device__ __forceinline__ static Val none() { return 0; }
+};
+struct PropOr2 {
+    struct Val {
+        unsigned long long lo, hi;
+    };
+    static constexpr int kDirs = 1;
+    static constexpr bool kNamed = false;
+    __device__ __forceinline__ uint32_t named(Val) const { return 0; }
+    __device__ __forceinline__ static Val load(const Val* p, size_t i) {
+        return {ld_volatile(&p[i].lo), ld_volatile(&p[i].hi)};
+    }
+    __device__ __forceinline__ static void store(Val* p, size_t i, Val x) {
+        *(volatile unsigned long long*)&p[i].lo = x.lo;
+        *(volatile unsigned long long*)&p[i].hi = x.hi;
+    }
+    __device__ __forceinline__ static bool gains(Val mine, Val t) { return ((mine.lo & ~t.lo) | (mine.hi & ~t.hi)) != 0; }
+    using Part = Val;
+    __device__ __forceinline__ static Part part(const Val&, const Val& t) { return t; }
+    __device__ __forceinline__ static Part fold(Part a, Part b) { return {a.lo | b.lo, a.hi | b.hi}; }
+    __device__ __forceinline__ static Val with(Val a, Part p) { return {a.lo | p.lo, a.hi | p.hi}; }
+    __device__ __forceinline__ static bool more(Part p, Val a) { return ((p.lo & ~a.lo) | (p.hi & ~a.hi)) != 0; }
+    __device__ __forceinline__ static void raise(Val* p, size_t i, Val mine) {
+        if (mine.lo) atomicOr(&p[i].lo, mine.lo);
+        if (mine.hi) atomicOr(&p[i].hi, mine.hi);
+    }
+    __device__ __forceinline__ static Val none() { return {0, 0}; }
+};
+template <class V>
+__device__ __forceinline__ V prop_shfl(const V& x, int l) {
+    if constexpr (sizeof(V) == 8) return __shfl_sync(kFull, x, l);
+    else return {__shfl_sync(kFull, x.lo, l), __shfl_sync(kFull, x.hi, l)};
+}
+template <class V>
+__device__ __forceinline__ V prop_shfl_xor(const V& x, int d) {
+    if constexpr (sizeof(V) <= 8) return __shfl_xor_sync(kFull, x, d);
+    else return {__shfl_xor_sync(kFull, x.lo, d), __shfl_xor_sync(kFull, x.hi, d)};
+}
+
+template <class Op>
+struct PropGraph {
+    using Val = typename Op::Val;
+    const int32_t* off[2];  // the graph, its transpose
+    const int32_t* adj[2];
+    int32_t n;
+    Val* s[Op::kDirs];            // values; direction 1 travels along the transpose
+    uint32_t* d[Op::kDirs];       // dirty vertices
+    uint32_t* act;                // active vertices (null: all)
+    int32_t* rep;                 // a vertex of v's SCC, the same for all of it
+    __device__ __forceinline__ uint32_t active(long long w) const {
+        if (act) return act[w];
+        const long long left = (long long)n - w * 32;
+        return left >= 32 ? kFull : (1u << left) - 1u;
+    }
 };
 
-// the run of bitmap words of this warp
+// The bitmap words of a warp: runs of 2^l words dealt out to the warps in turn,
+// so that a busy part of the graph is shared by many warps (3D torus 256^3, the
+// head start and the searches of the first batch: runs of 32 words 4.98 ms, of 8
+// 5.62, one run a warp 7.37). Word i of the warp, i < cnt, may be past the end
+// (>= nw).
+struct PropSlice {
+    long long nw, wid, warps;
+    int l;
+    long long cnt;
+    __device__ __forceinline__ long long word(long long i) const {
+        return ((((i >> l) * warps) + wid) << l) + (i & ((1 << l) - 1));
+    }
+};
 template <class S>
-__device__ __forceinline__ void prop_slice(int32_t n, long long& w0, long long& w1) {
-    const long long nw = ((long long)n + 31) / 32;
-    const long long warps = (long long)S::blocks() * (blockDim.x >> 5);
-    const long long wid = (long long)S::block() * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const long long per = (nw + warps - 1) / warps;
-    w0 = min(wid * per, nw);
-    w1 = min(w0 + per, nw);
+__device__ __forceinline__ PropSlice prop_slice(int32_t n) {
+    PropSlice P;
+    P.nw = ((long long)n + 31) / 32;
+    P.warps = (long long)S::blocks() * (blockDim.x >> 5);
+    P.wid = (long long)S::block() * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    P.l = P.nw >= 64 * P.warps ? 5 : P.nw >= 16 * P.warps ? 3 : 0;
+    const long long runs = (P.nw + (1 << P.l) - 1) >> P.l;
+    P.cnt = ((runs + P.warps - 1 - P.wid) / P.warps) << P.l;
+    return P;
 }
 
 // A warp's queue of vertices (| direction << 31) in shared memory.
@@ -134,47 +231,71 @@ __device__ __forceinline__ void prop_drain(PropQueue& Q, F&& f) {
     Q.cnt = 0;
     __syncwarp();
 }
-// Queues the set bits of the lanes' words x (direction 0) and y (direction 1),
-// word0 + lane each; f is called when the queue is full.
-template <class F>
-__device__ __forceinline__ void prop_queue_bits(PropQueue& Q, uint32_t x, uint32_t y, long long word0, F&& f) {
-    const uint32_t v0 = (uint32_t)(word0 + lane_id()) * 32u;
-    while (__any_sync(kFull, (x | y) != 0)) {
-        int nx = __popc(x), ny = __popc(y);
-        int incl = warp_incl_scan(nx + ny);
-        int total = __shfl_sync(kFull, incl, 31);
-        if (Q.cnt + total > kPropQueue) {  // warp-uniform
-            if (Q.cnt) prop_drain(Q, f);
-            if (total > kPropQueue) {
-                nx = min(nx, kPropQueue / 64);
-                ny = min(ny, kPropQueue / 64);
-                incl = warp_incl_scan(nx + ny);
-                total = __shfl_sync(kFull, incl, 31);
-            }
+// Moves set bits of the lanes' words x (direction 0) and y (direction 1) into
+// the queue, a lane's both at the same word: all of them if they fit, else some.
+__device__ __forceinline__ void prop_queue_bits(PropQueue& Q, uint32_t& x, uint32_t& y, long long word) {
+    const uint32_t v0 = (uint32_t)word * 32u;
+    int nx = __popc(x), ny = __popc(y);
+    int incl = warp_incl_scan(nx + ny);
+    int total = __shfl_sync(kFull, incl, 31);
+    if (Q.cnt + total > kPropQueue) {  // warp-uniform
+        if (Q.cnt) return;             // after the next drain
+        nx = min(nx, kPropQueue / 64);
+        ny = min(ny, kPropQueue / 64);
+        incl = warp_incl_scan(nx + ny);
+        total = __shfl_sync(kFull, incl, 31);
+    }
+    int k = Q.cnt + incl - nx - ny;
+    for (int i = 0; i < nx; ++i) {
+        Q.buf[k++] = v0 + (uint32_t)(__ffs(x) - 1);
+        x &= x - 1;
+    }
+    for (int i = 0; i < ny; ++i) {
+        Q.buf[k++] = (v0 + (uint32_t)(__ffs(y) - 1)) | 0x80000000u;
+        y &= y - 1;
+    }
+    Q.cnt += total;
+}
+// Gathers vertices from the warp's words, take(w, x, y) giving each lane's two
+// bitmap words, and calls f for them: the words are all looked at before any
+// work where the queue holds what they hold (a wave touches a few vertices in
+// each, which then share one step). Returns whether there was any. One place
+// calls f: its code is long, and copies of it cost more than they save.
+template <class T, class F>
+__device__ __forceinline__ bool prop_gather(const PropSlice& P, PropQueue& Q, T&& take, F&& f) {
+    bool did = false;
+    uint32_t x = 0, y = 0;
+    long long w = 0;
+    for (long long b = 0;;) {
+        bool left = __any_sync(kFull, (x | y) != 0);
+        while (!left && b < P.cnt) {
+            const long long i = b + lane_id();
+            w = P.word(i);
+            x = y = 0;
+            left = take(i < P.cnt && w < P.nw, w, x, y);
+            b += 32;
         }
-        int k = Q.cnt + incl - nx - ny;
-        for (int i = 0; i < nx; ++i) {
-            Q.buf[k++] = v0 + (uint32_t)(__ffs(x) - 1);
-            x &= x - 1;
+        if (left) {
+            did = true;
+            prop_queue_bits(Q, x, y, w);
+            left = __any_sync(kFull, (x | y) != 0);
         }
-        for (int i = 0; i < ny; ++i) {
-            Q.buf[k++] = (v0 + (uint32_t)(__ffs(y) - 1)) | 0x80000000u;
-            y &= y - 1;
-        }
-        Q.cnt += total;
+        if (!left && b < P.cnt) continue;
+        if (Q.cnt == 0) return did;
+        prop_drain(Q, f);
     }
 }
-// f(has, v) for the active vertices of the warp's words [w0, w1).
-template <class F>
-__device__ __forceinline__ void prop_for_active(const uint32_t* act, long long w0, long long w1, uint32_t* q, F&& f) {
+// f(has, v) for the active vertices of the warp's words.
+template <class Op, class F>
+__device__ __forceinline__ void prop_for_active(const PropGraph<Op>& G, const PropSlice& P, uint32_t* q, F&& f) {
     PropQueue Q{q, 0};
-    auto g = [&](bool has, int v, int) { f(has, v); };
-    for (long long b = w0; b < w1; b += 32) {
-        const long long w = b + lane_id();
-        const uint32_t x = w < w1 ? act[w] : 0u;
-        prop_queue_bits(Q, x, 0u, b, g);
-    }
-    prop_drain(Q, g);
+    prop_gather(
+        P, Q,
+        [&](bool in, long long w, uint32_t& x, uint32_t&) {
+            x = in ? G.active(w) : 0u;
+            return __any_sync(kFull, x != 0) != 0;
+        },
+        [&](bool has, int v, int) { f(has, v); });
 }
 
 // The marks of a warp's raises, kept in shared memory until one fence covers
@@ -183,54 +304,55 @@ struct PropMarks {
     uint32_t* buf;  // kPropMarks entries of the warp: vertex | direction << 31
     int cnt;        // warp-uniform
 };
-template <class S>
-__device__ __forceinline__ void prop_flush(const PropGraph& G, PropMarks& M) {
+template <class S, class Op>
+__device__ __forceinline__ void prop_flush(const PropGraph<Op>& G, PropMarks& M) {
     if (M.cnt == 0) return;
     __syncwarp();
     S::fence();
     for (int i = lane_id(); i < M.cnt; i += 32) {
         const uint32_t c = M.buf[i], w = c & 0x7fffffffu;
-        atomicOr(&(c >> 31 ? G.db : G.df)[w >> 5], 1u << (w & 31));
+        atomicOr(&(Op::kDirs > 1 && (c >> 31) ? G.d[Op::kDirs - 1] : G.d[0])[w >> 5], 1u << (w & 31));
     }
     M.cnt = 0;
     __syncwarp();
 }
 
-// Relax the arcs of v in direction dir (0: G with sf, 1: G^T with sb); all
-// lanes of the warp call.
-template <class S>
-__device__ __forceinline__ void prop_relax(const PropGraph& G, bool has, int v, int dir, PropMarks& M,
+// Spread v's value along its arcs in direction dir; all lanes of the warp call.
+template <class S, class Op>
+__device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op, bool has, int v, int dir, PropMarks& M,
                                            unsigned long long& arcs) {
+    using Val = typename Op::Val;
+    constexpr int D = Op::kDirs - 1;
     const int lane = lane_id();
-    const int32_t* off = dir ? G.toff : G.off;
-    const int32_t* adj = dir ? G.tadj : G.adj;
-    unsigned long long* s = dir ? G.sb : G.sf;
+    if constexpr (D == 0) dir = 0;
+    const int32_t* off = dir ? G.off[1] : G.off[0];
+    const int32_t* adj = dir ? G.adj[1] : G.adj[0];
+    Val* s = dir ? G.s[D] : G.s[0];
     int o0 = 0, o1 = 0;
-    unsigned long long st = 0;
+    Val st = Op::none();
     if (has) {
-        st = ld_volatile(&s[v]);
+        st = Op::load(s, v);
         o0 = S::ld(&off[v]);
         o1 = S::ld(&off[v + 1]);
     }
-    const uint32_t lab = (uint32_t)(st >> 32);
-    // the source named by the value may itself have been reached by a larger one
-    if (has) {
-        const uint32_t r = G.vertex((uint32_t)st);
-        if (r != (uint32_t)v && r < (uint32_t)G.n) {
-            const unsigned long long t = ld_volatile(&s[r]);
-            if ((uint32_t)(t >> 32) == lab && t > st) {
-                st = t;
-                atomicMax(&s[v], t);
+    if constexpr (Op::kNamed) {
+        if (has) {
+            const uint32_t r = op.named(st);
+            if (r != (uint32_t)v && r < (uint32_t)G.n) {
+                const Val t = Op::load(s, r);
+                if (Op::gains(t, st)) {
+                    st = t;
+                    Op::raise(s, v, t);
+                }
             }
         }
     }
     constexpr int U = kPropUnroll;
-    auto raise = [&](const int (&w)[U], const unsigned long long (&t)[U], unsigned long long to, unsigned long long* ts,
-                     int tdir) {
+    auto raise = [&](const int (&w)[U], const Val (&t)[U], const Val& to, Val* ts, int tdir) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const bool up = w[u] >= 0 && (uint32_t)(t[u] >> 32) == (uint32_t)(to >> 32) && t[u] < to;
-            if (up) atomicMax(&ts[w[u]], to);
+            const bool up = w[u] >= 0 && Op::gains(to, t[u]);
+            if (up) Op::raise(ts, w[u], to);
             const uint32_t m = __ballot_sync(kFull, up);
             if (up) M.buf[M.cnt + __popc(m & lanemask_lt())] = (uint32_t)w[u] | ((uint32_t)tdir << 31);
             M.cnt += __popc(m);
@@ -243,114 +365,110 @@ __device__ __forceinline__ void prop_relax(const PropGraph& G, bool has, int v, 
     const int most = __reduce_max_sync(kFull, len);
     for (int k = 0; k < most; k += U) {
         int w[U];
-        unsigned long long t[U];
+        Val t[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) w[u] = k + u < len ? S::ld(&adj[o0 + k + u]) : -1;
 #pragma unroll
-        for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? ld_volatile(&s[w[u]]) : 0ull;
+        for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(s, w[u]) : Op::none();
         raise(w, t, st, s, dir);
     }
     uint32_t bm = __ballot_sync(kFull, big);
     while (bm) {  // long rows by the whole warp
         const int l = __ffs(bm) - 1;
         bm &= bm - 1;
-        const unsigned long long bst = __shfl_sync(kFull, st, l);
+        const Val bst = prop_shfl(st, l);
         const int b0 = __shfl_sync(kFull, o0, l), b1 = __shfl_sync(kFull, o1, l);
-        const int bdir = __shfl_sync(kFull, dir, l);
-        const int32_t* ba = bdir ? G.tadj : G.adj;
-        unsigned long long* bs = bdir ? G.sb : G.sf;
+        const int bdir = D ? __shfl_sync(kFull, dir, l) : 0;
+        const int32_t* ba = bdir ? G.adj[1] : G.adj[0];
+        Val* bs = bdir ? G.s[D] : G.s[0];
         for (int e = b0; e < b1; e += 32 * U) {
             int w[U];
-            unsigned long long t[U];
+            Val t[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) w[u] = e + 32 * u + lane < b1 ? S::ld(&ba[e + 32 * u + lane]) : -1;
 #pragma unroll
-            for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? ld_volatile(&bs[w[u]]) : 0ull;
+            for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(bs, w[u]) : Op::none();
             raise(w, t, bst, bs, bdir);
         }
         if (lane == 0) arcs += (unsigned long long)(b1 - b0);
     }
 }
 
-// One pull of v: both values become the largest of the in-class neighbours'
-// (and, with jump, of the source each names). v's words are written by its
-// owner alone, so there is no atomic. Returns bit d set when direction d grew.
-template <class S>
-__device__ __forceinline__ int prop_pull(const PropGraph& G, bool has, int v, bool jump) {
-    unsigned long long s0[2] = {0, 0}, st[2] = {0, 0};
-    int e0[2] = {0, 0}, e1[2] = {0, 0};
-    const int32_t* const adj[2] = {G.tadj, G.adj};  // the forward value comes from in-neighbours
-    unsigned long long* const s[2] = {G.sf, G.sb};
-    if (has) {
-        e0[0] = S::ld(&G.toff[v]);
-        e1[0] = S::ld(&G.toff[v + 1]);
-        e0[1] = S::ld(&G.off[v]);
-        e1[1] = S::ld(&G.off[v + 1]);
-        s0[0] = ld_volatile(&G.sf[v]);
-        s0[1] = ld_volatile(&G.sb[v]);
+// One pull of v: its values take what its in-class neighbours (and, with jump,
+// the vertex each names) hold. v's words are written by its owner
+// alone, so there is no atomic. Returns bit d set when direction d grew.
+template <class S, class Op>
+__device__ __forceinline__ int prop_pull(const PropGraph<Op>& G, const Op& op, bool has, int v, bool jump) {
+    using Val = typename Op::Val;
+    constexpr int D = Op::kDirs, U = kPropUnroll;
+    using Part = typename Op::Part;
+    Val s0[D];
+    Part st[D];
+    int e0[D], len[D];
+    bool big = false;
+    int most = 0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {  // a value that travels along a graph comes in along the other
+        const int32_t* off = G.off[1 - d];
+        e0[d] = has ? S::ld(&off[v]) : 0;
+        len[d] = has ? S::ld(&off[v + 1]) - e0[d] : 0;
+        s0[d] = has ? Op::load(G.s[d], v) : Op::none();
     }
-    const uint32_t lab = (uint32_t)(s0[0] >> 32);
-    st[0] = s0[0];
-    st[1] = s0[1];
-    if (jump && has) {
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            const uint32_t r = G.vertex((uint32_t)s0[d]);
-            const unsigned long long t = r != (uint32_t)v && r < (uint32_t)G.n ? ld_volatile(&s[d][r]) : 0ull;
-            if ((uint32_t)(t >> 32) == lab) st[d] = max(st[d], t);
+    for (int d = 0; d < D; ++d) {
+        st[d] = Part{};
+        if (Op::kNamed && jump && has) {
+            const uint32_t r = op.named(s0[d]);
+            if (r != (uint32_t)v && r < (uint32_t)G.n) st[d] = Op::part(s0[d], Op::load(G.s[d], r));
         }
+        big |= len[d] > kPropBigRow;
+        most = max(most, len[d]);
     }
-    constexpr int U = kPropUnroll;
-    const bool big = has && max(e1[0] - e0[0], e1[1] - e0[1]) > kPropBigRow;
-    int n0 = big ? 0 : e1[0] - e0[0], n1 = big ? 0 : e1[1] - e0[1];
-    for (int k = 0; k < max(n0, n1); k += U) {
-        int w[2][U];
-        unsigned long long t[2][U];
+    if (big) most = 0;
+    for (int k = 0; k < most; k += U) {
+        int w[D][U];
+        Val t[D][U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            w[0][u] = k + u < n0 ? S::ld(&adj[0][e0[0] + k + u]) : -1;
-            w[1][u] = k + u < n1 ? S::ld(&adj[1][e0[1] + k + u]) : -1;
-        }
+        for (int d = 0; d < D; ++d)
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            t[0][u] = w[0][u] >= 0 ? ld_volatile(&s[0][w[0][u]]) : 0ull;
-            t[1][u] = w[1][u] >= 0 ? ld_volatile(&s[1][w[1][u]]) : 0ull;
-        }
+            for (int u = 0; u < U; ++u) w[d][u] = k + u < len[d] ? S::ld(&G.adj[1 - d][e0[d] + k + u]) : -1;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (w[0][u] >= 0 && (uint32_t)(t[0][u] >> 32) == lab) st[0] = max(st[0], t[0][u]);
-            if (w[1][u] >= 0 && (uint32_t)(t[1][u] >> 32) == lab) st[1] = max(st[1], t[1][u]);
-        }
+        for (int d = 0; d < D; ++d)
+#pragma unroll
+            for (int u = 0; u < U; ++u) t[d][u] = w[d][u] >= 0 ? Op::load(G.s[d], w[d][u]) : Op::none();
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+#pragma unroll
+            for (int u = 0; u < U; ++u) st[d] = Op::fold(st[d], Op::part(s0[d], t[d][u]));
     }
     uint32_t bm = __ballot_sync(kFull, big);
     while (bm) {  // long rows by the whole warp
         const int l = __ffs(bm) - 1;
         bm &= bm - 1;
-        const uint32_t blab = __shfl_sync(kFull, lab, l);
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            const int b0 = __shfl_sync(kFull, e0[d], l), b1 = __shfl_sync(kFull, e1[d], l);
-            unsigned long long m = 0;
+        for (int d = 0; d < D; ++d) {
+            const int b0 = __shfl_sync(kFull, e0[d], l), b1 = b0 + __shfl_sync(kFull, len[d], l);
+            const Val own = prop_shfl(s0[d], l);
+            Part m = Part{};
             for (int e = b0 + lane_id(); e < b1; e += 32 * U) {
                 int w[U];
-                unsigned long long t[U];
+                Val t[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) w[u] = e + 32 * u < b1 ? S::ld(&adj[d][e + 32 * u]) : -1;
+                for (int u = 0; u < U; ++u) w[u] = e + 32 * u < b1 ? S::ld(&G.adj[1 - d][e + 32 * u]) : -1;
 #pragma unroll
-                for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? ld_volatile(&s[d][w[u]]) : 0ull;
+                for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(G.s[d], w[u]) : Op::none();
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (w[u] >= 0 && (uint32_t)(t[u] >> 32) == blab) m = max(m, t[u]);
+                for (int u = 0; u < U; ++u) m = Op::fold(m, Op::part(own, t[u]));
             }
-            for (int dd = 16; dd >= 1; dd >>= 1) m = max(m, __shfl_xor_sync(kFull, m, dd));
-            if (lane_id() == l) st[d] = max(st[d], m);
+            for (int x = 16; x >= 1; x >>= 1) m = Op::fold(m, prop_shfl_xor(m, x));
+            if (lane_id() == l) st[d] = Op::fold(st[d], m);
         }
     }
     int up = 0;
 #pragma unroll
-    for (int d = 0; d < 2; ++d)
-        if (has && st[d] > s0[d]) {
-            *(volatile unsigned long long*)&s[d][v] = st[d];
+    for (int d = 0; d < D; ++d)
+        if (has && Op::more(st[d], s0[d])) {
+            Op::store(G.s[d], v, Op::with(s0[d], st[d]));
             up |= 1 << d;
         }
     return up;
@@ -410,182 +528,161 @@ __device__ __forceinline__ bool prop_checked(PropCtl* ctl, PropShared& sh, unsig
 }
 
 // A search by pulling alone. With one word per warp a lane keeps its vertex's
-// two values and the first arcs of both its rows in registers, so a pass, and
-// with it a hop, costs one round of loads; the value's own source is looked at
-// in the same round.
-template <class S>
-__device__ bool prop_search_pull(const PropGraph& G, PropCtl* ctl, PropShared& sh, unsigned int& check,
+// values and the first arcs of its rows in registers, so a pass, and with it a
+// hop, costs one round of loads; the vertex a value names is looked at in the
+// same round.
+template <class S, class Op>
+__device__ bool prop_search_pull(const PropGraph<Op>& G, const Op op, PropCtl* ctl, PropShared& sh, unsigned int& check,
                                  unsigned long long& items) {
-    long long w0, w1;
-    prop_slice<S>(G.n, w0, w1);
+    using Val = typename Op::Val;
+    constexpr int D = Op::kDirs, U = kPropUnroll;
+    const PropSlice P = prop_slice<S>(G.n);
+    const int lane = lane_id();
     if (threadIdx.x == 0) sh.idle = sh.exit = 0;
     __syncthreads();
-    auto pass = [&](bool jump) {
-        bool up = false;
-        for (long long w = w0; w < w1; ++w) {
-            const uint32_t x = G.act[w];
-            if (x == 0) continue;  // warp-uniform
-            const bool has = (x >> lane_id()) & 1u;
-            const int c = prop_pull<S>(G, has, (int)(w * 32) + lane_id(), jump);
-            up |= c != 0;
-            if (c) ++items;
-        }
-        return __any_sync(kFull, up) != 0;
-    };
-    constexpr int U = kPropUnroll;
-    const bool one = w1 - w0 == 1;
-    const int v = (int)(w0 * 32) + lane_id();
-    const bool has = one && ((G.act[w0] >> lane_id()) & 1u);
-    unsigned long long st[2] = {0, 0};
-    int w[2][U], len[2] = {0, 0};
+    const bool one = P.cnt == 1 && P.word(0) < P.nw;
+    const int v = (int)(P.word(0) * 32) + lane;
+    const bool has = one && ((G.active(P.word(0)) >> lane) & 1u);
+    Val st[D];
+    int w[D][U], most = 0;
 #pragma unroll
-    for (int u = 0; u < U; ++u) w[0][u] = w[1][u] = -1;
-    if (has) {
-        st[0] = ld_volatile(&G.sf[v]);
-        st[1] = ld_volatile(&G.sb[v]);
+    for (int d = 0; d < D; ++d) {
+        st[d] = has ? Op::load(G.s[d], v) : Op::none();
+        const int32_t* off = G.off[1 - d];
+        const int e0 = has ? S::ld(&off[v]) : 0;
+        const int len = has ? S::ld(&off[v + 1]) - e0 : 0;
+        most = max(most, len);
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            const int32_t* off = d ? G.off : G.toff;
-            const int32_t* adj = d ? G.adj : G.tadj;
-            const int e0 = S::ld(&off[v]);
-            len[d] = S::ld(&off[v + 1]) - e0;
-#pragma unroll
-            for (int u = 0; u < U; ++u) w[d][u] = u < len[d] ? S::ld(&adj[e0 + u]) : -1;
-        }
+        for (int u = 0; u < U; ++u) w[d][u] = u < len ? S::ld(&G.adj[1 - d][e0 + u]) : -1;
     }
-    const uint32_t lab = (uint32_t)(st[0] >> 32);
-    const bool fits = __all_sync(kFull, max(len[0], len[1]) <= U) != 0;
+    const bool fits = one && __all_sync(kFull, most <= U);
     auto pass_one = [&]() {
-        unsigned long long t[2][U], j[2];
+        Val t[D][U], j[D];
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            const unsigned long long* s = d ? G.sb : G.sf;
-            const uint32_t r = G.vertex((uint32_t)st[d]);
-            j[d] = has && r < (uint32_t)G.n ? ld_volatile(&s[r]) : 0ull;
+        for (int d = 0; d < D; ++d) {
+            j[d] = Op::none();
+            if constexpr (Op::kNamed) {
+                const uint32_t r = op.named(st[d]);
+                if (has && r < (uint32_t)G.n) j[d] = Op::load(G.s[d], r);
+            }
 #pragma unroll
-            for (int u = 0; u < U; ++u) t[d][u] = w[d][u] >= 0 ? ld_volatile(&s[w[d][u]]) : 0ull;
+            for (int u = 0; u < U; ++u) t[d][u] = w[d][u] >= 0 ? Op::load(G.s[d], w[d][u]) : Op::none();
         }
         bool up = false;
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            unsigned long long m = st[d];
-            if ((uint32_t)(j[d] >> 32) == lab) m = max(m, j[d]);
+        for (int d = 0; d < D; ++d) {
+            typename Op::Part m = Op::part(st[d], j[d]);
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (w[d][u] >= 0 && (uint32_t)(t[d][u] >> 32) == lab) m = max(m, t[d][u]);
-            if (has && m > st[d]) {
-                st[d] = m;
-                *(volatile unsigned long long*)&(d ? G.sb : G.sf)[v] = m;
+            for (int u = 0; u < U; ++u) m = Op::fold(m, Op::part(st[d], t[d][u]));
+            if (has && Op::more(m, st[d])) {
+                st[d] = Op::with(st[d], m);
+                Op::store(G.s[d], v, st[d]);
                 up = true;
                 ++items;
             }
         }
         return __any_sync(kFull, up) != 0;
     };
+    auto pass_all = [&](bool jump) {
+        bool up = false;
+        for (long long i = 0; i < P.cnt; ++i) {
+            const long long wd = P.word(i);
+            const uint32_t x = wd < P.nw ? G.active(wd) : 0u;
+            if (x == 0) continue;  // warp-uniform
+            const int c = prop_pull<S>(G, op, (x >> lane) & 1u, (int)(wd * 32) + lane, jump);
+            up |= c != 0;
+            items += (unsigned long long)__popc(c);
+        }
+        return __any_sync(kFull, up) != 0;
+    };
     for (;;) {
         PropIdle<S> id(ctl, sh);
         for (;;) {
-            if (one && fits ? pass_one() : pass(true)) id.wake();
+            if (fits ? pass_one() : pass_all(true)) id.wake();
             else if (id.rest()) break;
         }
         if (!S::sync(&ctl->bar, &ctl->err)) return false;
         ++check;
-        const bool left = one && fits ? pass_one() : pass(false);
+        const bool left = fits ? pass_one() : pass_all(false);
         bool more = false;
         if (!prop_checked<S>(ctl, sh, check, left, &more)) return false;
         if (!more) return true;
     }
 }
 
-// One search: relax until no vertex is dirty. Every thread of the scope calls
+// One search: spread until no vertex is dirty. Every thread of the scope calls
 // it; `check` numbers the checks of the launch (the same in every block). With
 // a deadline (globaltimer ns; 0: none) it may end early, vertices still dirty.
 // Returns false when a wait ran out (the caller returns at once).
-template <class S>
-__device__ bool prop_search(const PropGraph& G, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
+template <class S, class Op>
+__device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
                             unsigned int& check, uint64_t deadline, unsigned long long& items,
                             unsigned long long& arcs) {
+    using Val = typename Op::Val;
+    constexpr int D = Op::kDirs;
     const int lane = lane_id();
-    long long w0, w1;
-    prop_slice<S>(G.n, w0, w1);
+    const PropSlice P = prop_slice<S>(G.n);
     if (threadIdx.x == 0) sh.idle = sh.exit = 0;
     __syncthreads();
     PropMarks M{mk, 0};
     PropQueue Q{q, 0};
-    long long turn = 0;  // the word whose sources are looked at next
-    auto relax = [&](bool has, int v, int dir) { prop_relax<S>(G, has, v, dir, M, arcs); };
+    long long turn = 0;  // the word whose named vertices are looked at next
     for (;;) {
         PropIdle<S> id(ctl, sh);
         for (;;) {
-            // the words of the whole run are polled before any work: a wave
-            // touches a few vertices in each, which then share one step
-            bool did = false;
-            for (long long b = w0; b < w1; b += 32 * kPropPoll) {
-                uint32_t x[kPropPoll], y[kPropPoll];
-#pragma unroll
-                for (int j = 0; j < kPropPoll; ++j) {
-                    const long long w = b + 32 * j + lane;
-                    x[j] = w < w1 ? ld_volatile(&G.df[w]) : 0u;
-                    y[j] = w < w1 ? ld_volatile(&G.db[w]) : 0u;
-                }
-                uint32_t any = 0;
-#pragma unroll
-                for (int j = 0; j < kPropPoll; ++j) any |= x[j] | y[j];
-                if (!__any_sync(kFull, any != 0)) continue;
-                if (!did) {
-                    did = true;
+            bool did = prop_gather(
+                P, Q,
+                [&](bool in, long long w, uint32_t& x, uint32_t& y) {
+                    x = in ? ld_volatile(&G.d[0][w]) : 0u;
+                    y = D > 1 && in ? ld_volatile(&G.d[D - 1][w]) : 0u;
+                    if (!__any_sync(kFull, (x | y) != 0)) return false;
                     id.wake();
-                }
-#pragma unroll
-                for (int j = 0; j < kPropPoll; ++j) {
-                    const long long w = b + 32 * j + lane;
-                    if (x[j]) x[j] = atomicExch(&G.df[w], 0u);
-                    if (y[j]) y[j] = atomicExch(&G.db[w], 0u);
-                }
-                S::fence();
-#pragma unroll
-                for (int j = 0; j < kPropPoll; ++j) {
-                    items += (unsigned long long)(__popc(x[j]) + __popc(y[j]));
-                    prop_queue_bits(Q, x[j], y[j], b + 32 * j, relax);
-                }
-            }
-            if (did) {
-                prop_drain(Q, relax);
-                prop_flush<S>(G, M);
-            }
-            // nothing dirty: look whether the source that a vertex of the next
-            // word names was itself reached by a larger one (paths are walked
-            // hop by hop; this takes the rest of one in a step)
-            if (!did && w1 > w0) {
-                if (++turn >= w1 - w0) turn = 0;
-                const long long w = w0 + turn;
-                const uint32_t x = G.act[w];
-                uint32_t up[2] = {0, 0};
-                if (x != 0) {  // warp-uniform
-                    const bool has = (x >> lane) & 1u;
-                    const long long v = w * 32 + lane;
-                    unsigned long long st[2], t[2];
-                    st[0] = has ? ld_volatile(&G.sf[v]) : 0ull;
-                    st[1] = has ? ld_volatile(&G.sb[v]) : 0ull;
-#pragma unroll
-                    for (int d = 0; d < 2; ++d) {
-                        const uint32_t r = G.vertex((uint32_t)st[d]);
-                        t[d] = has && r != (uint32_t)v && r < (uint32_t)G.n ? ld_volatile(&(d ? G.sb : G.sf)[r]) : 0ull;
-                    }
-#pragma unroll
-                    for (int d = 0; d < 2; ++d) {
-                        const bool u = t[d] > st[d] && (t[d] >> 32) == (st[d] >> 32);
-                        if (u) atomicMax(&(d ? G.sb : G.sf)[v], t[d]);
-                        up[d] = __ballot_sync(kFull, u);
-                    }
-                }
-                if (up[0] | up[1]) {
-                    did = true;
-                    id.wake();
+                    if (x) x = atomicExch(&G.d[0][w], 0u);
+                    if (y) y = atomicExch(&G.d[D - 1][w], 0u);
                     S::fence();
-                    __syncwarp();
-                    if (lane == 0 && up[0]) atomicOr(&G.df[w], up[0]);
-                    if (lane == 0 && up[1]) atomicOr(&G.db[w], up[1]);
+                    items += (unsigned long long)(__popc(x) + __popc(y));
+                    return __any_sync(kFull, (x | y) != 0) != 0;
+                },
+                [&](bool has, int v, int dir) { prop_relax<S>(G, op, has, v, dir, M, arcs); });
+            if (did) prop_flush<S>(G, M);
+            // nothing dirty: look whether the vertex that a value of the next
+            // word names holds a larger one itself (paths are walked hop by
+            // hop; this takes the rest of one in a step)
+            if constexpr (Op::kNamed) {
+                if (!did && P.cnt > 0 && !deadline) {
+                    if (++turn >= P.cnt) turn = 0;
+                    const long long w = P.word(turn);
+                    const uint32_t a = w < P.nw ? G.active(w) : 0u;
+                    uint32_t up[D];
+                    uint32_t any = 0;
+                    if (a != 0) {  // warp-uniform
+                        const bool has = (a >> lane) & 1u;
+                        const long long v = w * 32 + lane;
+                        Val st[D], t[D];
+#pragma unroll
+                        for (int d = 0; d < D; ++d) st[d] = has ? Op::load(G.s[d], v) : Op::none();
+#pragma unroll
+                        for (int d = 0; d < D; ++d) {
+                            const uint32_t r = op.named(st[d]);
+                            t[d] = has && r != (uint32_t)v && r < (uint32_t)G.n ? Op::load(G.s[d], r) : Op::none();
+                        }
+#pragma unroll
+                        for (int d = 0; d < D; ++d) {
+                            const bool u = has && Op::gains(t[d], st[d]);
+                            if (u) Op::raise(G.s[d], v, t[d]);
+                            up[d] = __ballot_sync(kFull, u);
+                            any |= up[d];
+                        }
+                    }
+                    if (any) {
+                        did = true;
+                        id.wake();
+                        S::fence();
+                        __syncwarp();
+#pragma unroll
+                        for (int d = 0; d < D; ++d)
+                            if (lane == 0 && up[d]) atomicOr(&G.d[d][w], up[d]);
+                    }
                 }
             }
             if (!did && id.rest()) break;
@@ -599,7 +696,12 @@ __device__ bool prop_search(const PropGraph& G, PropCtl* ctl, PropShared& sh, ui
         ++check;
         bool left = false;
         if (!deadline)
-            for (long long w = w0 + lane; w < w1; w += 32) left |= (ld_volatile(&G.df[w]) | ld_volatile(&G.db[w])) != 0;
+            for (long long i = lane; i < P.cnt; i += 32) {
+                const long long w = P.word(i);
+                if (w >= P.nw) continue;
+#pragma unroll
+                for (int d = 0; d < D; ++d) left |= ld_volatile(&G.d[d][w]) != 0;
+            }
         bool more = false;
         if (!prop_checked<S>(ctl, sh, check, left, &more)) return false;
         if (!more) return true;
@@ -637,14 +739,14 @@ __device__ __forceinline__ bool prop_count(PropCtl* ctl, unsigned int& step, uns
 // The batches from the state in sf/sb/act until every active vertex is
 // finished (`active` of them): trimming inside the classes, the two searches,
 // the labelling. Self-loops must not be in the graph. The ring of counters
-// starts zero. pull: the searches only pull. head_ns: time limit of the first batch's head start (0: none);
+// starts zero. kPull: the searches only pull. head_ns: time limit of the first batch's head start (0: none);
 // with it the state's keys start zero, and the first batch sets them.
-template <class S>
-__device__ bool prop_batches(const PropGraph& G, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
-                             unsigned long long active, bool pull, uint64_t head_ns) {
+template <class S, bool kPull>
+__device__ bool prop_batches(const PropGraph<PropMax>& G, const PropMax op, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
+                             unsigned long long active, uint64_t head_ns) {
     const int lane = lane_id();
-    long long w0, w1;
-    prop_slice<S>(G.n, w0, w1);
+    const PropSlice P = prop_slice<S>(G.n);
+    unsigned long long *const sf = G.s[0], *const sb = G.s[1];
     unsigned int check = 0;
     unsigned long long items = 0, arcs = 0, done = 0;
     int batches = 0;
@@ -653,16 +755,16 @@ __device__ bool prop_batches(const PropGraph& G, PropCtl* ctl, PropShared& sh, u
         // ---- vertices with no arc from, or no arc to, a vertex of their class
         for (int pass = 0; pass < kPropTrimPasses; ++pass) {
             unsigned long long cnt = 0;
-            prop_for_active(G.act, w0, w1, q, [&](bool has, int v) {
+            prop_for_active(G, P, q, [&](bool has, int v) {
                 if (!has) return;
-                const uint32_t lab = (uint32_t)(ld_volatile(&G.sf[v]) >> 32);
-                const int o0 = S::ld(&G.off[v]), o1 = S::ld(&G.off[v + 1]);
-                const int i0 = S::ld(&G.toff[v]), i1 = S::ld(&G.toff[v + 1]);
-                if (prop_any_in_class<S>(G.adj, o0, o1, G.sf, lab) &&
-                    prop_any_in_class<S>(G.tadj, i0, i1, G.sf, lab))
+                const uint32_t lab = (uint32_t)(ld_volatile(&sf[v]) >> 32);
+                const int o0 = S::ld(&G.off[0][v]), o1 = S::ld(&G.off[0][v + 1]);
+                const int i0 = S::ld(&G.off[1][v]), i1 = S::ld(&G.off[1][v + 1]);
+                if (prop_any_in_class<S>(G.adj[0], o0, o1, sf, lab) &&
+                    prop_any_in_class<S>(G.adj[1], i0, i1, sf, lab))
                     return;
-                *(volatile unsigned long long*)&G.sf[v] = prop_pack(kPropDone, 0);
-                *(volatile unsigned long long*)&G.sb[v] = prop_pack(kPropDone, 0);
+                *(volatile unsigned long long*)&sf[v] = prop_pack(kPropDone, 0);
+                *(volatile unsigned long long*)&sb[v] = prop_pack(kPropDone, 0);
                 G.rep[v] = v;
                 atomicAnd(&G.act[v >> 5], ~(1u << (v & 31)));
                 ++cnt;
@@ -673,52 +775,54 @@ __device__ bool prop_batches(const PropGraph& G, PropCtl* ctl, PropShared& sh, u
             if (got * 8 < active - done) break;
         }
         if (done >= active) break;
-        if (pull) {
-            if (!prop_search_pull<S>(G, ctl, sh, check, items)) return false;
+        if constexpr (kPull) {
+            if (!prop_search_pull<S>(G, op, ctl, sh, check, items)) return false;
         } else {
             // ---- every active vertex is a source. A head start: the largest
             // source alone, so that a giant SCC is flooded once before the
             // others' values wander through it
             unsigned long long grew = 2 * (active - done);
             if (batches == 0 && head_ns) {
-                const uint32_t b = G.vertex(0xffffffffu);
+                const uint32_t b = op.vertex(0xffffffffu);
                 if (S::block() == 0 && threadIdx.x == 0) {
-                    const unsigned long long st = G.sf[b];
+                    const unsigned long long st = sf[b];
                     if ((uint32_t)(st >> 32) != kPropDone) {
-                        G.sf[b] = G.sb[b] = st | 0xffffffffull;
-                        G.df[b >> 5] = G.db[b >> 5] = 1u << (b & 31);
+                        sf[b] = sb[b] = st | 0xffffffffull;
+                        G.d[0][b >> 5] = G.d[1][b >> 5] = 1u << (b & 31);
                     }
                 }
                 if (!S::sync(&ctl->bar, &ctl->err)) return false;
-                if (!prop_search<S>(G, ctl, sh, q, mk, check, globaltimer_ns() + head_ns, items, arcs)) return false;
+                if (!prop_search<S>(G, op, ctl, sh, q, mk, check, globaltimer_ns() + head_ns, items, arcs)) return false;
                 unsigned long long cnt = 0;
-                for (long long w = w0; w < w1; ++w) {
-                    const uint32_t x = G.act[w];
+                for (long long i = 0; i < P.cnt; ++i) {
+                    const long long w = P.word(i);
+                    const uint32_t x = w < P.nw ? G.act[w] : 0u;
                     if (x == 0) continue;  // warp-uniform
                     const long long v = w * 32 + lane;
                     bool f = false, r = false;
                     if ((x >> lane) & 1u) {
-                        const unsigned long long sf = G.sf[v], sb = G.sb[v];
-                        const uint32_t key = G.key((uint32_t)v);
-                        f = (uint32_t)sf < key;
-                        r = (uint32_t)sb < key;
-                        if (f) G.sf[v] = prop_pack((uint32_t)(sf >> 32), key);
-                        if (r) G.sb[v] = prop_pack((uint32_t)(sb >> 32), key);
+                        const unsigned long long a = sf[v], b2 = sb[v];
+                        const uint32_t key = op.key((uint32_t)v);
+                        f = (uint32_t)a < key;
+                        r = (uint32_t)b2 < key;
+                        if (f) sf[v] = prop_pack((uint32_t)(a >> 32), key);
+                        if (r) sb[v] = prop_pack((uint32_t)(b2 >> 32), key);
                     }
                     const uint32_t mf = __ballot_sync(kFull, f), mr = __ballot_sync(kFull, r);
                     if (lane == 0) {
-                        G.df[w] |= mf;
-                        G.db[w] |= mr;
+                        G.d[0][w] |= mf;
+                        G.d[1][w] |= mr;
                         cnt += __popc(mf) + __popc(mr);
                     }
                 }
                 if (!prop_count<S>(ctl, step, cnt, grew)) return false;
             } else {
-                for (long long w = w0 + lane; w < w1; w += 32) {
-                    const uint32_t x = G.act[w];
+                for (long long i = lane; i < P.cnt; i += 32) {
+                    const long long w = P.word(i);
+                    const uint32_t x = w < P.nw ? G.act[w] : 0u;
                     if (x) {
-                        G.df[w] = x;
-                        G.db[w] = x;
+                        G.d[0][w] = x;
+                        G.d[1][w] = x;
                     }
                 }
                 if (!S::sync(&ctl->bar, &ctl->err)) return false;
@@ -728,39 +832,40 @@ __device__ bool prop_batches(const PropGraph& G, PropCtl* ctl, PropShared& sh, u
             // the vertices it raised dirty
             while (grew * kPropSweepMin >= (unsigned long long)G.n) {
                 unsigned long long cnt = 0;
-                for (long long w = w0; w < w1; ++w) {
-                    const uint32_t x = G.act[w];
+                for (long long i = 0; i < P.cnt; ++i) {
+                    const long long w = P.word(i);
+                    const uint32_t x = w < P.nw ? G.act[w] : 0u;
                     if (x == 0) continue;  // warp-uniform
                     const bool has = (x >> lane) & 1u;
-                    const int c = prop_pull<S>(G, has, (int)(w * 32) + lane, false);
+                    const int c = prop_pull<S>(G, op, has, (int)(w * 32) + lane, false);
                     const uint32_t cf = __ballot_sync(kFull, c & 1), cb = __ballot_sync(kFull, c & 2);
                     if (lane == 0) {
-                        G.df[w] = cf;
-                        G.db[w] = cb;
+                        G.d[0][w] = cf;
+                        G.d[1][w] = cb;
                         cnt += __popc(cf) + __popc(cb);
                     }
                 }
                 items += cnt;
                 if (!prop_count<S>(ctl, step, cnt, grew)) return false;
             }
-            if (!prop_search<S>(G, ctl, sh, q, mk, check, 0, items, arcs)) return false;
+            if (!prop_search<S>(G, op, ctl, sh, q, mk, check, 0, items, arcs)) return false;
         }
         // ---- labelling (Alg. 1): equal maxima finish a vertex, the others'
         // class becomes the hash of the old one and the two maxima
         unsigned long long cnt = 0;
-        prop_for_active(G.act, w0, w1, q, [&](bool has, int v) {
+        prop_for_active(G, P, q, [&](bool has, int v) {
             if (!has) return;
-            const unsigned long long f = ld_volatile(&G.sf[v]), r = ld_volatile(&G.sb[v]);
+            const unsigned long long f = ld_volatile(&sf[v]), r = ld_volatile(&sb[v]);
             if (f == r) {
-                G.sf[v] = G.sb[v] = prop_pack(kPropDone, 0);
-                const uint32_t r = G.vertex((uint32_t)f);
+                sf[v] = sb[v] = prop_pack(kPropDone, 0);
+                const uint32_t r = op.vertex((uint32_t)f);
                 if (r >= (uint32_t)G.n) atomicCAS(&ctl->err, 0, SCC_ERR_INTERNAL);  // never: a value names a vertex
                 G.rep[v] = r < (uint32_t)G.n ? (int32_t)r : v;
                 atomicAnd(&G.act[v >> 5], ~(1u << (v & 31)));
                 ++cnt;
             } else {
                 const int32_t lab = class_hash((int32_t)(uint32_t)(f >> 32), (int32_t)(uint32_t)f, (int32_t)(uint32_t)r);
-                G.sf[v] = G.sb[v] = prop_pack((uint32_t)lab, G.key((uint32_t)v));
+                sf[v] = sb[v] = prop_pack((uint32_t)lab, op.key((uint32_t)v));
             }
         });
         unsigned long long got = 0;
