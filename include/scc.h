@@ -10,7 +10,8 @@
  * every active vertex as a source and keeps, per vertex, the largest source
  * reaching it and the largest it reaches: all that Alg. 1's labels use. A graph
  * of fewer than 8 arcs a vertex without hubs (no row of more than 64 arcs and
- * 16 times the mean) runs such batches from the start. The single- and
+ * 16 times the mean) runs such batches from the start, on the graph contracted
+ * along mutual arcs when those join much of it. The single- and
  * multi-source searches use vertical granularity control (bounded multi-hop
  * local searches, Sec. 3.1-3.2) and a hash-bag frontier (Sec. 3.3). All of it
  * runs in hand-written CUDA kernels on one GPU.

@@ -23,11 +23,16 @@
  * dense rounds of Sec. 4.2; on the others both directions share each round.
  * The labels never depend on these choices.
  *
- * Execution: one persistent kernel; each thread block takes the next graph from
- * a device work queue (largest graphs first) and runs its whole SCC alone, with
+ * Execution: where a group of consecutive graphs (up to 2^24 vertices) holds at
+ * least 2^17 vertices in graphs without hubs, those run together as one graph
+ * over the whole grid, by signature propagation (scc.h). The others go through
+ * one persistent kernel; each thread block takes the next graph from a device
+ * work queue (largest graphs first) and runs its whole SCC alone, with
  * block-level synchronisation between rounds, then takes the next graph. The
  * host is not involved until every graph is done, so a run is one CUDA graph
- * (captured once per configuration and output buffer, then replayed).
+ * (captured once per configuration and output buffer, then replayed). The
+ * tunables below are the persistent kernel's; the autotuner samples the graphs
+ * it takes.
  *
  * Packed input (one int32 CSR for all graphs, per-graph int64 bases):
  *   vbase[g], g = 0..G: first vertex of graph g in the packed vertex space;

@@ -696,7 +696,9 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
         EvTimer tp(s);
         tp.start();
         PropArgs a = prop_args(h);
-        a.pull = prop_pulls(h->mt, h->di.num_sms);
+        Scratch tmp(s);
+        SCC_TRY(tmp.alloc(&a.con_n, prop_con_words(n)));
+        SCC_TRY(tmp.alloc(&a.con_m, 2 * (size_t)h->mt));
         a.out = dst;
         PropResult r;
         SCC_TRY(run_prop(a, &r, s));
@@ -780,7 +782,7 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
 
         // ---- the remaining pivots (Alg. 1): signature propagation
         if ((int64_t)hc[1] < N) {
-            PropArgs a = prop_args(h);  // marking, not pulling: a hub's row would be read in every pass
+            PropArgs a = prop_args(h);
             a.label = h->label;
             a.N = N - (int64_t)hc[1];
             t.start();

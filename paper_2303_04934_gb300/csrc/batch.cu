@@ -223,6 +223,8 @@ __device__ void bind_ws(const BatchArgs& A, Ws& W) {
          at<uint64_t>(b, L.hub_item1));
 }
 
+__device__ __forceinline__ bool graph_has_hubs(long long n, long long m, long long maxdeg);
+
 // ------------------------------------------------------------- block helpers --
 struct BlockShared {
     int graph;
@@ -525,7 +527,7 @@ __device__ bool scc_one_graph(const BatchArgs& A, Ws& W, int g, BlockShared& sh,
     // or more (hubs: a round lasts as long as its longest local search, which
     // grows fastest where degrees are high or skewed), 2048 otherwise
     maxdeg = block_max(maxdeg, sh);
-    const bool hubby = m >= 8ll * n || (long long)maxdeg * n >= 16ll * max(m, 1ll);
+    const bool hubby = graph_has_hubs(n, m, (long long)maxdeg);
     const int tau_g = A.tau > 0 ? A.tau : (hubby ? 128 : 2048);
     if (na > 0) {
         block_exclusive_scan(W.cnt, n, sh);
@@ -885,7 +887,16 @@ constexpr long long kGroupArcs = 1ll << 27;   // bounds the groups' scratch
 struct GroupPlan {
     int g0, g1;
     long long v0, v1, e0, e1;
+    long long mesh_arcs = 0;  // arcs of the graphs taken by signature propagation (-1: none is)
+    bool blocks = true;       // some graph of the group is left to a block
 };
+
+// Vertices without hubs' worth of graphs from which a group runs them by
+// signature propagation over the whole grid (prop.cu) and not a block each: a
+// block takes a 1 M-vertex torus in 159 ms, all 128 tori of 1 k to 1 M vertices
+// together take the grid 25 ms. Below, the group's launches and 33 bytes a vertex
+// of working memory would buy little: the blocks' graphs are small.
+constexpr long long kGroupMesh = 1ll << 17;
 
 // Groups of consecutive graphs (host only): greedily, as many consecutive
 // graphs as fit in max_v vertices and max_a arcs; a graph larger than either
@@ -917,6 +928,32 @@ void plan_groups(int G, const long long* vb, const long long* eb, long long max_
         ok[g] = 1;
     }
     flush(G);
+}
+
+// Which graphs each group takes by signature propagation: mesh[g] = 1 for those
+// without hubs (hub[g] == 0) of the groups that hold enough of them.
+void plan_mesh(const long long* vb, const long long* eb, const unsigned char* hub, int G,
+               std::vector<GroupPlan>& groups, std::vector<unsigned char>& mesh) {
+    mesh.assign((size_t)G + 1, 0);
+    for (GroupPlan& gr : groups) {
+        long long v = 0, a = 0;
+        for (int g = gr.g0; g < gr.g1; ++g)
+            if (!hub[g]) {
+                v += vb[g + 1] - vb[g];
+                a += eb[g + 1] - eb[g];
+            }
+        gr.mesh_arcs = v >= kGroupMesh ? a : -1;
+        gr.blocks = gr.mesh_arcs < 0;
+        for (int g = gr.g0; g < gr.g1 && gr.mesh_arcs >= 0; ++g) {
+            mesh[g] = hub[g] == 0;
+            gr.blocks = gr.blocks || hub[g];
+        }
+    }
+}
+
+// A graph of at least 8 arcs a vertex or with a row of at least 16 times the mean.
+__device__ __forceinline__ bool graph_has_hubs(long long n, long long m, long long maxdeg) {
+    return m >= 8 * n || maxdeg * n >= 16 * max(m, 1ll);
 }
 
 // last g in [lo, hi) with a[g] <= x (a non-decreasing, a[lo] <= x)
@@ -1006,16 +1043,37 @@ __global__ void k_group_localize(const long long* __restrict__ vbase, const long
 }  // namespace
 }  // namespace scc
 
+namespace scc {
+// Device buffers of the groups' passes (enqueue_groups).
+struct GroupBufs {
+    int32_t* gt_off = nullptr;       // G^T, packed like offsets
+    int32_t* gt_adj = nullptr;       // packed like targets
+    unsigned char* gt_ok = nullptr;  // graph is in a group
+    unsigned char* mesh = nullptr;   // graph is taken by signature propagation
+    int32_t *grp_off = nullptr, *grp_adj = nullptr, *grp_toff = nullptr;  // one group's CSR and G^T offsets
+    unsigned char* grp_scratch = nullptr;
+    TransposeScratch ts{};
+    // signature propagation of one group
+    unsigned long long* state = nullptr;  // 2 n
+    uint32_t* bits = nullptr;             // 3 words per 32 vertices
+    int32_t *rep = nullptr, *minid = nullptr;
+    int32_t *con_n = nullptr, *con_m = nullptr;
+    void* dev = nullptr;
+};
+}  // namespace scc
+
 struct scc_batch {
     DeviceInfo di;
     int32_t G = 0;
     long long nv = 0, na = 0;
     long long n_max = 0, m_max = 0;
+    long long blk_n_max = 0, blk_m_max = 0;  // of the graphs left to the blocks
+    int32_t nblk = 0;                        // their number
     long long* vbase = nullptr;
     long long* ebase = nullptr;
     int32_t* offsets = nullptr;
     int32_t* targets = nullptr;
-    int32_t* order = nullptr;       // all graphs, largest first
+    int32_t* order = nullptr;       // the graphs left to the blocks, largest first
     std::vector<int32_t> order_h;
     std::vector<long long> vb_h, eb_h;
     int* flags = nullptr;           // [0] work-queue head, [1] error
@@ -1024,12 +1082,7 @@ struct scc_batch {
     // G^T computed before the persistent launch, for groups of consecutive
     // graphs (one grid-wide transpose each)
     std::vector<scc::GroupPlan> groups;
-    int32_t* gt_off = nullptr;       // packed like offsets
-    int32_t* gt_adj = nullptr;       // packed like targets
-    unsigned char* gt_ok = nullptr;  // graph is in a group
-    int32_t *grp_off = nullptr, *grp_adj = nullptr, *grp_toff = nullptr;  // one group's CSR and G^T offsets
-    unsigned char* grp_scratch = nullptr;
-    TransposeScratch ts{};
+    scc::GroupBufs gb;
     scc_batch_config cfg;
     // working memory for the current configuration
     unsigned char* ws = nullptr;
@@ -1123,7 +1176,7 @@ int prepare(scc_batch* h, cudaStream_t s) {
     WsLayout L;
     BatchDims d;
     int blocks = 0;
-    SCC_TRY(plan_workspace(h->di, h->cfg, h->n_max, h->m_max, h->G, default_budget(), &L, &d, &blocks));
+    SCC_TRY(plan_workspace(h->di, h->cfg, h->blk_n_max, h->blk_m_max, h->nblk, default_budget(), &L, &d, &blocks));
     const size_t need = L.bytes * (size_t)blocks;
     if (h->ws && (h->ws_bytes < need)) {
         dfree(h->ws, s);
@@ -1180,40 +1233,140 @@ BatchArgs args_for(const scc_batch_config& cfg, unsigned char* ws, const WsLayou
 
 BatchArgs make_args(scc_batch* h, const int32_t* order, int norder, int32_t* out) {
     return args_for(h->cfg, h->ws, h->L, h->D, h->flags, h->times, h->G, h->vbase, h->ebase, h->offsets, h->targets,
-                    order, norder, out, h->gt_off, h->gt_adj, h->gt_ok);
+                    order, norder, out, h->gb.gt_off, h->gb.gt_adj, h->gb.gt_ok);
 }
 
-// G^T of every group (after the reset kernel, before the persistent launch);
-// the passes' self-check errors go to the batch's error flag.
-int enqueue_groups(scc_batch* h, cudaStream_t s) {
-    TransposeScratch ts = h->ts;
-    ts.err = h->flags + 1;
-    for (const auto& gr : h->groups) {
+// G^T of every group, and with `prop` the labels of the graphs its plan gives to
+// signature propagation (after the reset kernel, before the persistent
+// launch); the passes' errors go to *err.
+int enqueue_groups(const std::vector<GroupPlan>& groups, const GroupBufs& B, const long long* vbase,
+                   const long long* ebase, const int32_t* offsets, const int32_t* targets, int32_t* out, bool prop,
+                   uint64_t seed, unsigned long long* times, int* err, int num_sms, cudaStream_t s) {
+    TransposeScratch ts = B.ts;
+    ts.err = err;
+    for (const auto& gr : groups) {
         const long long ng = gr.v1 - gr.v0, mg = gr.e1 - gr.e0;
-        const int grid = h->di.num_sms * 4;
-        k_group_csr<<<grid, 256, 0, s>>>(h->vbase, h->ebase, h->offsets, h->targets, gr.g0, gr.g1, gr.v0, gr.e0, ng,
-                                         mg, h->grp_off, h->grp_adj);
+        const int grid = num_sms * 4;
+        k_group_csr<<<grid, 256, 0, s>>>(vbase, ebase, offsets, targets, gr.g0, gr.g1, gr.v0, gr.e0, ng, mg,
+                                         B.grp_off, B.grp_adj);
         SCC_LAUNCH();
-        SCC_TRY(launch_transpose_keep_self(h->grp_off, h->grp_adj, (int32_t)ng, mg, ts, h->grp_toff,
-                                           h->gt_adj + gr.e0, h->di.num_sms, s));
-        k_group_localize<<<grid, 256, 0, s>>>(h->vbase, h->ebase, gr.g0, gr.g1, gr.v0, gr.e0, ng, mg, h->grp_toff,
-                                              h->gt_off, h->gt_adj);
+        SCC_TRY(launch_transpose_keep_self(B.grp_off, B.grp_adj, (int32_t)ng, mg, ts, B.grp_toff, B.gt_adj + gr.e0,
+                                           num_sms, s));
+        if (prop && gr.mesh_arcs >= 0) {
+            const size_t nw = (size_t)(ng + 31) / 32;
+            PropArgs a;
+            a.off = B.grp_off;
+            a.adj = B.grp_adj;
+            a.toff = B.grp_toff;
+            a.tadj = B.gt_adj + gr.e0;
+            a.n = (int32_t)ng;
+            a.m = mg;
+            a.seed = seed;
+            a.sf = B.state;
+            a.sb = B.state + ng;
+            a.act = B.bits;
+            a.df = B.bits + nw;
+            a.db = B.bits + 2 * nw;
+            a.mesh_arcs = gr.mesh_arcs;
+            a.con_n = B.con_n;
+            a.con_m = B.con_m;
+            a.rep = B.rep;
+            a.minid = B.minid;
+            a.out = out + gr.v0;
+            a.dev = B.dev;
+            a.num_sms = num_sms;
+            a.vbase = vbase;
+            a.mesh = B.mesh;
+            a.g0 = gr.g0;
+            a.g1 = gr.g1;
+            a.times = times;
+            a.time_words = kTimeWords;
+            SCC_TRY(enqueue_prop(a, err, s));
+        }
+        if (!gr.blocks && prop) continue;
+        k_group_localize<<<grid, 256, 0, s>>>(vbase, ebase, gr.g0, gr.g1, gr.v0, gr.e0, ng, mg, B.grp_toff, B.gt_off,
+                                              B.gt_adj);
         SCC_LAUNCH();
     }
     return SCC_OK;
 }
 
-int enqueue(scc_batch* h, const int32_t* order, int norder, int32_t* out, cudaStream_t s) {
-    BatchArgs A = make_args(h, order, norder, out);
-    k_batch_reset<<<1, 1, 0, s>>>(h->flags, h->flags + 1);
-    SCC_LAUNCH();
-    SCC_TRY(enqueue_groups(h, s));
-    batch_kernel_for(h->cfg)<<<h->blocks, h->cfg.block, batch_smem_bytes(h->cfg.block), s>>>(A);
-    SCC_LAUNCH();
+void free_groups(GroupBufs* B, cudaStream_t s) {
+    dfree(B->gt_off, s);
+    dfree(B->gt_adj, s);
+    dfree(B->gt_ok, s);
+    dfree(B->mesh, s);
+    dfree(B->grp_off, s);
+    dfree(B->grp_adj, s);
+    dfree(B->grp_toff, s);
+    dfree(B->grp_scratch, s);
+    dfree(B->state, s);
+    dfree(B->bits, s);
+    dfree(B->rep, s);
+    dfree(B->minid, s);
+    dfree(B->con_n, s);
+    dfree(B->con_m, s);
+    dfree(B->dev, s);
+    *B = GroupBufs();
+}
+
+// Buffers for the plan of a batch of nv vertices and na arcs in G graphs.
+int alloc_groups(const std::vector<GroupPlan>& groups, const std::vector<unsigned char>& ok,
+                 const std::vector<unsigned char>& mesh, int G, long long nv, long long na, GroupBufs* B,
+                 cudaStream_t s) {
+    if (groups.empty()) return SCC_OK;
+    long long ng_max = 0, mg_max = 0, np_max = 0, mp_max = 0;
+    for (const auto& gr : groups) {
+        ng_max = std::max(ng_max, gr.v1 - gr.v0);
+        mg_max = std::max(mg_max, gr.e1 - gr.e0);
+        if (gr.mesh_arcs >= 0) {
+            np_max = std::max(np_max, gr.v1 - gr.v0);
+            mp_max = std::max(mp_max, gr.e1 - gr.e0);
+        }
+    }
+    SCC_TRY(dalloc_t(&B->gt_off, (size_t)(nv + G) + 1, s));
+    SCC_TRY(dalloc_t(&B->gt_adj, (size_t)na + 1, s));
+    SCC_TRY(dalloc_t(&B->gt_ok, (size_t)G + 1, s));
+    SCC_CUDA(cudaMemcpyAsync(B->gt_ok, ok.data(), (size_t)G, cudaMemcpyHostToDevice, s));
+    SCC_TRY(dalloc_t(&B->grp_off, (size_t)ng_max + 1, s));
+    SCC_TRY(dalloc_t(&B->grp_toff, (size_t)ng_max + 1, s));
+    SCC_TRY(dalloc_t(&B->grp_adj, (size_t)mg_max + 8, s));
+    SCC_TRY(dalloc_t(&B->grp_scratch, transpose_scratch_bytes(mg_max), s));
+    transpose_scratch_carve(B->grp_scratch, mg_max, &B->ts);
+    SCC_TRY(transpose_set_attributes());  // before any capture
+    if (np_max > 0) {
+        int per_sm = 0;
+        SCC_TRY(prop_blocks_per_sm(&per_sm));  // before any capture
+        SCC_TRY(dalloc_t(&B->mesh, (size_t)G + 1, s));
+        SCC_CUDA(cudaMemcpyAsync(B->mesh, mesh.data(), (size_t)G, cudaMemcpyHostToDevice, s));
+        SCC_TRY(dalloc_t(&B->state, 2 * (size_t)np_max, s));
+        SCC_TRY(dalloc_t(&B->bits, 3 * (((size_t)np_max + 31) / 32), s));
+        SCC_TRY(dalloc_t(&B->rep, (size_t)np_max, s));
+        SCC_TRY(dalloc_t(&B->minid, (size_t)np_max, s));
+        SCC_TRY(dalloc_t(&B->con_n, prop_con_words(np_max), s));
+        SCC_TRY(dalloc_t(&B->con_m, 2 * (size_t)mp_max, s));
+        SCC_TRY(dalloc(&B->dev, prop_dev_bytes(), s));
+    }
     return SCC_OK;
 }
 
-// Capture the reset and the persistent kernel as one CUDA graph.
+// The launches of one run over the graphs `order` (those left to the blocks);
+// the handle's own order is a run of the whole batch, signature propagation
+// included.
+int enqueue_run(scc_batch* h, const int32_t* order, int norder, int32_t* out, cudaStream_t s) {
+    k_batch_reset<<<1, 1, 0, s>>>(h->flags, h->flags + 1);
+    SCC_LAUNCH();
+    SCC_TRY(enqueue_groups(h->groups, h->gb, h->vbase, h->ebase, h->offsets, h->targets, out, order == h->order,
+                           h->cfg.seed, h->times, h->flags + 1, h->di.num_sms, s));
+    if (norder > 0) {
+        BatchArgs A = make_args(h, order, norder, out);
+        batch_kernel_for(h->cfg)<<<h->blocks, h->cfg.block, batch_smem_bytes(h->cfg.block), s>>>(A);
+        SCC_LAUNCH();
+    }
+    return SCC_OK;
+}
+
+// Capture a run's launches as one CUDA graph.
 int capture(scc_batch* h, const int32_t* order, int norder, int32_t* out) {
     drop_exec(h);
     cudaStream_t cs;
@@ -1221,13 +1374,7 @@ int capture(scc_batch* h, const int32_t* order, int norder, int32_t* out) {
     cudaGraph_t graph = nullptr;
     int rc = cuda_err(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     if (rc == SCC_OK) {
-        BatchArgs A = make_args(h, order, norder, out);
-        k_batch_reset<<<1, 1, 0, cs>>>(h->flags, h->flags + 1);
-        rc = enqueue_groups(h, cs);
-        if (rc == SCC_OK) {
-            batch_kernel_for(h->cfg)<<<h->blocks, h->cfg.block, batch_smem_bytes(h->cfg.block), cs>>>(A);
-            rc = cuda_err(cudaGetLastError());
-        }
+        rc = enqueue_run(h, order, norder, out, cs);
         const int rc2 = cuda_err(cudaStreamEndCapture(cs, &graph));
         if (rc == SCC_OK) rc = rc2;
     }
@@ -1256,12 +1403,12 @@ int capture(scc_batch* h, const int32_t* order, int norder, int32_t* out) {
 
 // One run over `order` into `out` (device), timed with CUDA events.
 int run_order(scc_batch* h, const int32_t* order, int norder, int32_t* out, cudaStream_t s, double* ms) {
-    if (!h->ws) SCC_TRY(prepare(h, s));
+    if (!h->ws && norder > 0) SCC_TRY(prepare(h, s));
     cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
     SCC_CUDA(cudaStreamIsCapturing(s, &cst));
     if (cst != cudaStreamCaptureStatusNone) {
         // the caller is capturing: add the launches to the caller's graph
-        return enqueue(h, order, norder, out, s);
+        return enqueue_run(h, order, norder, out, s);
     }
     if (!h->exec_valid || h->exec_out != out || h->exec_order != order || h->exec_norder != norder)
         SCC_TRY(capture(h, order, norder, out));
@@ -1291,13 +1438,7 @@ int run_order(scc_batch* h, const int32_t* order, int norder, int32_t* out, cuda
 void batch_free(scc_batch* h, cudaStream_t s) {
     drop_exec(h);
     dfree(h->ws, s);
-    dfree(h->gt_off, s);
-    dfree(h->gt_adj, s);
-    dfree(h->gt_ok, s);
-    dfree(h->grp_off, s);
-    dfree(h->grp_adj, s);
-    dfree(h->grp_toff, s);
-    dfree(h->grp_scratch, s);
+    free_groups(&h->gb, s);
     dfree(h->vbase, s);
     dfree(h->ebase, s);
     dfree(h->offsets, s);
@@ -1310,16 +1451,28 @@ void batch_free(scc_batch* h, cudaStream_t s) {
 
 // One block per graph: its CSR is well formed (offsets start at 0, do not
 // decrease and end at its arc count; targets in [0, n_g)); *bad set otherwise.
+// hub[g]: graph_has_hubs.
 __global__ void k_batch_validate(int32_t G, const long long* vbase, const long long* ebase, const int32_t* off,
-                                 const int32_t* adj, int* bad) {
+                                 const int32_t* adj, int* bad, unsigned char* hub) {
+    __shared__ int s_most;
     for (int g = blockIdx.x; g < G; g += gridDim.x) {
         const long long n = vbase[g + 1] - vbase[g];
         const long long m = ebase[g + 1] - ebase[g];
         const int32_t* o = off + vbase[g] + g;
         const int32_t* a = adj + ebase[g];
+        if (threadIdx.x == 0) s_most = 0;
+        __syncthreads();
         if (threadIdx.x == 0 && (o[0] != 0 || (long long)o[n] != m)) atomicExch(bad, 1);
-        for (long long v = threadIdx.x; v < n; v += blockDim.x)
+        int most = 0;
+        for (long long v = threadIdx.x; v < n; v += blockDim.x) {
             if (o[v] > o[v + 1]) atomicExch(bad, 1);
+            else most = max(most, o[v + 1] - o[v]);
+        }
+        most = __reduce_max_sync(kFull, most);
+        if (lane_id() == 0) atomicMax(&s_most, most);
+        __syncthreads();
+        if (threadIdx.x == 0) hub[g] = graph_has_hubs(n, m, s_most);
+        __syncthreads();
         for (long long e = threadIdx.x; e < m; e += blockDim.x)
             if (a[e] < 0 || (long long)a[e] >= n) atomicExch(bad, 1);
     }
@@ -1359,51 +1512,45 @@ int batch_create_impl(scc_batch* h, int32_t G, const int64_t* vbase, const int64
         SCC_CUDA(cudaMemcpyAsync(h->targets, targets, sizeof(int32_t) * (size_t)h->na, cudaMemcpyDefault, s));
     Scratch tmp(s);
     int* bad = nullptr;
+    unsigned char* hub_d = nullptr;
+    std::vector<unsigned char> hub((size_t)G + 1, 0);
     SCC_TRY(tmp.alloc(&bad, 1));
+    SCC_TRY(tmp.alloc(&hub_d, (size_t)G + 1));
     SCC_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
     if (G > 0) {
         k_batch_validate<<<std::min<int32_t>(G, 65535), 256, 0, s>>>(G, h->vbase, h->ebase, h->offsets, h->targets,
-                                                                     bad);
+                                                                     bad, hub_d);
         SCC_LAUNCH();
+        SCC_CUDA(cudaMemcpyAsync(hub.data(), hub_d, (size_t)G, cudaMemcpyDeviceToHost, s));
     }
     int hbad = 0;
     SCC_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     SCC_CUDA(cudaStreamSynchronize(s));
     tmp.release(bad);
     if (hbad) return SCC_ERR_INVALID_ARG;
-    // processing order: decreasing work (arcs + vertices), so long graphs start first
-    h->order_h.resize((size_t)G);
-    for (int32_t g = 0; g < G; ++g) h->order_h[g] = g;
+    // groups of consecutive graphs for the G^T computed before each launch: up
+    // to kGroupVerts vertices and kGroupArcs arcs each; a larger graph is left
+    // to its block
+    std::vector<unsigned char> ok, mesh;
+    plan_groups(G, h->vb_h.data(), h->eb_h.data(), kGroupVerts, kGroupArcs, h->groups, ok);
+    plan_mesh(h->vb_h.data(), h->eb_h.data(), hub.data(), G, h->groups, mesh);
+    SCC_TRY(alloc_groups(h->groups, ok, mesh, G, h->nv, h->na, &h->gb, s));
+    // the blocks' order: decreasing work (arcs + vertices), so long graphs start first
+    for (int32_t g = 0; g < G; ++g)
+        if (!mesh[g]) {
+            h->order_h.push_back(g);
+            h->blk_n_max = std::max(h->blk_n_max, h->vb_h[g + 1] - h->vb_h[g]);
+            h->blk_m_max = std::max(h->blk_m_max, h->eb_h[g + 1] - h->eb_h[g]);
+        }
+    h->nblk = (int32_t)h->order_h.size();
     std::stable_sort(h->order_h.begin(), h->order_h.end(), [&](int32_t a, int32_t b) {
         const long long wa = (h->eb_h[a + 1] - h->eb_h[a]) + (h->vb_h[a + 1] - h->vb_h[a]);
         const long long wb = (h->eb_h[b + 1] - h->eb_h[b]) + (h->vb_h[b + 1] - h->vb_h[b]);
         return wa > wb;
     });
     SCC_TRY(dalloc_t(&h->order, (size_t)G + 1, s));
-    if (G > 0)
-        SCC_CUDA(cudaMemcpyAsync(h->order, h->order_h.data(), sizeof(int32_t) * (size_t)G, cudaMemcpyHostToDevice, s));
-    // groups of consecutive graphs for the G^T computed before each launch: up
-    // to kGroupVerts vertices and kGroupArcs arcs each; a larger graph is left
-    // to its block
-    std::vector<unsigned char> ok;
-    plan_groups(G, h->vb_h.data(), h->eb_h.data(), kGroupVerts, kGroupArcs, h->groups, ok);
-    long long ng_max = 0, mg_max = 0;
-    for (const auto& gr : h->groups) {
-        ng_max = std::max(ng_max, gr.v1 - gr.v0);
-        mg_max = std::max(mg_max, gr.e1 - gr.e0);
-    }
-    if (!h->groups.empty()) {
-        SCC_TRY(dalloc_t(&h->gt_off, (size_t)(h->nv + G) + 1, s));
-        SCC_TRY(dalloc_t(&h->gt_adj, (size_t)h->na + 1, s));
-        SCC_TRY(dalloc_t(&h->gt_ok, (size_t)G + 1, s));
-        SCC_CUDA(cudaMemcpyAsync(h->gt_ok, ok.data(), (size_t)G, cudaMemcpyHostToDevice, s));
-        SCC_TRY(dalloc_t(&h->grp_off, (size_t)ng_max + 1, s));
-        SCC_TRY(dalloc_t(&h->grp_toff, (size_t)ng_max + 1, s));
-        SCC_TRY(dalloc_t(&h->grp_adj, (size_t)mg_max + 8, s));
-        SCC_TRY(dalloc_t(&h->grp_scratch, transpose_scratch_bytes(mg_max), s));
-        transpose_scratch_carve(h->grp_scratch, mg_max, &h->ts);
-        SCC_TRY(transpose_set_attributes());  // before any capture
-    }
+    if (h->nblk > 0)
+        SCC_CUDA(cudaMemcpyAsync(h->order, h->order_h.data(), sizeof(int32_t) * (size_t)h->nblk, cudaMemcpyHostToDevice, s));
     SCC_CUDA(cudaStreamSynchronize(s));
     memset(&h->st, 0, sizeof(h->st));
     h->st.graphs = G;
@@ -1468,7 +1615,8 @@ void batch_runner_destroy(BatchRunner* r, cudaStream_t s) {
 }
 
 // bad[g] = 1 when graph g of a packed batch is malformed (offsets not starting
-// at 0, decreasing or not ending at m_g; a target outside [0, n_g)), else 0.
+// at 0, decreasing or not ending at m_g; a target outside [0, n_g)), else 0, or
+// 2 if it has hubs.
 __global__ void k_batch_validate_each(int32_t G, const long long* vbase, const long long* ebase, const int32_t* off,
                                       const int32_t* adj, int* bad) {
     for (int g = blockIdx.x; g < G; g += gridDim.x) {
@@ -1476,15 +1624,24 @@ __global__ void k_batch_validate_each(int32_t G, const long long* vbase, const l
         const long long m = ebase[g + 1] - ebase[g];
         const int32_t* o = off + vbase[g] + g;
         const int32_t* a = adj + ebase[g];
-        __shared__ int s_bad;
-        if (threadIdx.x == 0) s_bad = (o[0] != 0 || (long long)o[n] != m);
+        __shared__ int s_bad, s_most;
+        if (threadIdx.x == 0) {
+            s_bad = (o[0] != 0 || (long long)o[n] != m);
+            s_most = 0;
+        }
         __syncthreads();
         bool b = false;
-        for (long long v = threadIdx.x; v < n; v += blockDim.x) b |= o[v] > o[v + 1];
+        int most = 0;
+        for (long long v = threadIdx.x; v < n; v += blockDim.x) {
+            b |= o[v] > o[v + 1];
+            most = max(most, o[v + 1] - o[v]);
+        }
         for (long long e = threadIdx.x; e < m; e += blockDim.x) b |= a[e] < 0 || (long long)a[e] >= n;
         if (b) s_bad = 1;
+        most = __reduce_max_sync(kFull, most);
+        if (lane_id() == 0) atomicMax(&s_most, most);
         __syncthreads();
-        if (threadIdx.x == 0) bad[g] = s_bad;
+        if (threadIdx.x == 0) bad[g] = s_bad ? 1 : graph_has_hubs(n, m, s_most) ? 2 : 0;
         __syncthreads();
     }
 }
@@ -1501,17 +1658,48 @@ bool batch_runner_fits(const BatchRunner* r, long long n, long long m) { return 
 size_t batch_runner_bytes(const BatchRunner* r) { return r->bytes; }
 const int* batch_runner_err(const BatchRunner* r) { return r->flags + 1; }
 
-int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vbase, const long long* ebase,
-                         const int32_t* offsets, const int32_t* targets, const int32_t* order, int32_t norder,
-                         int32_t* out, cudaStream_t s) {
-    if (norder > r->gcap) return SCC_ERR_INVALID_ARG;
-    BatchArgs A = args_for(r->cfg, r->ws, r->L, r->D, r->flags, r->times, G, vbase, ebase, offsets, targets, order,
-                           norder, out);
+int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const long long* eb_h,
+                         const unsigned char* hub, const long long* vbase, const long long* ebase,
+                         const int32_t* offsets, const int32_t* targets, std::vector<int32_t>& order,
+                         int32_t* order_d, int32_t* out, cudaStream_t s) {
+    if ((long long)order.size() > r->gcap) return SCC_ERR_INVALID_ARG;
     k_batch_reset<<<1, 1, 0, s>>>(r->flags, r->flags + 1);
     SCC_LAUNCH();
-    batch_kernel_for(r->cfg)<<<r->blocks, r->cfg.block, batch_smem_bytes(r->cfg.block), s>>>(A);
-    SCC_LAUNCH();
-    return SCC_OK;
+    GroupBufs B;  // freed, stream-ordered, when the launches are enqueued
+    int rc = SCC_OK;
+    if (hub) {
+        std::vector<GroupPlan> groups;
+        std::vector<unsigned char> ok, mesh;
+        plan_groups(G, vb_h, eb_h, kGroupVerts, kGroupArcs, groups, ok);
+        plan_mesh(vb_h, eb_h, hub, G, groups, mesh);
+        bool any = false;
+        for (const GroupPlan& gr : groups) any = any || gr.mesh_arcs >= 0;
+        if (any) {
+            rc = alloc_groups(groups, ok, mesh, G, vb_h[G], eb_h[G], &B, s);
+            if (rc == SCC_ERR_OOM) {  // a block for every graph, as without groups
+                free_groups(&B, s);
+                mesh.assign((size_t)G + 1, 0);
+                rc = SCC_OK;
+            } else if (rc == SCC_OK)
+                rc = enqueue_groups(groups, B, vbase, ebase, offsets, targets, out, true, r->cfg.seed, nullptr,
+                                    r->flags + 1, r->di.num_sms, s);
+            order.erase(std::remove_if(order.begin(), order.end(), [&](int32_t g) { return mesh[g] != 0; }),
+                        order.end());
+        }
+    }
+    const int32_t norder = (int32_t)order.size();
+    if (rc == SCC_OK && norder > 0) {
+        rc = cuda_err(cudaMemcpyAsync(order_d, order.data(), sizeof(int32_t) * (size_t)norder, cudaMemcpyHostToDevice, s));
+        if (rc == SCC_OK) {
+            BatchArgs A = args_for(r->cfg, r->ws, r->L, r->D, r->flags, r->times, G, vbase, ebase, offsets, targets,
+                                   order_d, norder, out, B.gt_off, B.gt_adj, B.gt_ok);
+            batch_kernel_for(r->cfg)<<<r->blocks, r->cfg.block, batch_smem_bytes(r->cfg.block), s>>>(A);
+            count_launch();
+            rc = cuda_err(cudaGetLastError());
+        }
+    }
+    free_groups(&B, s);
+    return rc;
 }
 
 }  // namespace scc
@@ -1591,7 +1779,7 @@ SCC_API int scc_batch_run(scc_batch_handle h, int32_t* labels_out, void* stream_
     if (h->G == 0 || h->nv == 0) return SCC_OK;
     const bool dev_out = is_device_ptr(labels_out);
     int32_t* dst = dev_out ? labels_out : h->labels;
-    SCC_TRY(run_order(h, h->order, h->G, dst, stream, nullptr));
+    SCC_TRY(run_order(h, h->order, h->nblk, dst, stream, nullptr));
     if (!dev_out) {
         SCC_CUDA(cudaMemcpyAsync(labels_out, h->labels, sizeof(int32_t) * (size_t)h->nv, cudaMemcpyDeviceToHost, stream));
         SCC_CUDA(cudaStreamSynchronize(stream));
@@ -1604,16 +1792,16 @@ SCC_API int scc_batch_autotune(scc_batch_handle h, int32_t sample, void* stream_
     cudaStream_t stream = (cudaStream_t)stream_;
     if (!h) return SCC_ERR_INVALID_ARG;
     const scc_batch_config base = h->cfg;
-    if (h->G == 0) {
+    if (h->nblk == 0) {  // nothing that the blocks' configuration could change
         if (best) *best = base;
         if (best_ms) *best_ms = 0;
         return SCC_OK;
     }
     // the sample: every k-th graph of the size order, so it spans the size range
     std::vector<int32_t> sub;
-    const int32_t want = (sample <= 0 || sample >= h->G) ? h->G : sample;
-    const double step = (double)h->G / (double)want;
-    for (int32_t i = 0; i < want; ++i) sub.push_back(h->order_h[(size_t)std::min<double>(h->G - 1, i * step)]);
+    const int32_t want = (sample <= 0 || sample >= h->nblk) ? h->nblk : sample;
+    const double step = (double)h->nblk / (double)want;
+    for (int32_t i = 0; i < want; ++i) sub.push_back(h->order_h[(size_t)std::min<double>(h->nblk - 1, i * step)]);
     Scratch tmp(stream);
     int32_t* dsub = nullptr;
     SCC_TRY(tmp.alloc(&dsub, sub.size()));

@@ -1,6 +1,7 @@
 // Host-side declarations shared by the library's translation units.
 #pragma once
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 
 #include "../../include/scc.h"
@@ -313,15 +314,26 @@ struct PropArgs {
     uint64_t seed;
     unsigned long long *sf, *sb;   // n words each
     uint32_t *act, *df, *db;       // ceil(n / 32) words each
-    bool pull = false;             // the searches only pull (prop_pulls)
     int32_t* rep;                  // n
     const int32_t* label = nullptr;
     long long N = 0;
     int32_t* minid = nullptr;      // n (label == nullptr)
     int32_t* out = nullptr;        // n (label == nullptr)
+    int32_t* con_n = nullptr;      // prop_con_words(n) (label == nullptr)
+    int32_t* con_m = nullptr;      // 2 m (label == nullptr)
     void* dev = nullptr;           // prop_dev_bytes()
     int num_sms = 0;
+    // A group [g0, g1) of a batch's graphs as one graph (label == nullptr): the
+    // labels of the graphs with mesh[g] != 0, counted from their own first
+    // vertex, into out (the group's first vertex); times: their records.
+    const long long* vbase = nullptr;
+    const unsigned char* mesh = nullptr;
+    int g0 = 0, g1 = 0;
+    long long mesh_arcs = 0;       // arcs of those graphs
+    unsigned long long* times = nullptr;
+    int time_words = 0;
 };
+inline size_t prop_con_words(int64_t n) { return (size_t)(8 * n + (n + 31) / 32); }
 struct PropResult {
     int status = 0;
     int64_t active = 0;   // untrimmed vertices
@@ -340,6 +352,10 @@ __host__ __device__ inline bool prop_skewed(unsigned long long max_deg, unsigned
     return max_deg > 64 && max_deg * n > 16 * m;
 }
 int run_prop(const PropArgs& a, PropResult* res, cudaStream_t st);
+// The launches alone (they can be captured once prop_blocks_per_sm was called);
+// an error goes to *err (device) if that is 0.
+int enqueue_prop(const PropArgs& a, int* err, cudaStream_t st);
+int prop_blocks_per_sm(int* out);
 
 // Multi-source reachability (reach.cu): mask word(s) of v get bit j iff src[j]
 // reaches v along (off, adj), whose transpose is (toff, tadj); words = 1 (k <=
@@ -376,12 +392,19 @@ void batch_runner_destroy(BatchRunner* r, cudaStream_t s);
 bool batch_runner_fits(const BatchRunner* r, long long n, long long m);
 size_t batch_runner_bytes(const BatchRunner* r);
 const int* batch_runner_err(const BatchRunner* r);  // device error flag of the last launch
-// bad[g] (device int[G]) = 1 when graph g of a packed batch is malformed
+// bad[g] (device int[G]) = 1 when graph g of a packed batch is malformed, else 2
+// when it has hubs (or 8 arcs a vertex), else 0
 int batch_validate_each(int32_t G, const long long* vbase, const long long* ebase, const int32_t* offsets,
                         const int32_t* targets, int* bad, cudaStream_t s);
-int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vbase, const long long* ebase,
-                         const int32_t* offsets, const int32_t* targets, const int32_t* order, int32_t norder,
-                         int32_t* out, cudaStream_t s);
+// Enqueues the SCCs of the packed graphs `order` (host, largest first; order_d:
+// device, G entries). hub (host, per graph; null: a graph is malformed and every
+// other one gets a block): graphs without hubs may run together over the
+// whole grid, with temporaries of up to batch_group_bytes.
+int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const long long* eb_h,
+                         const unsigned char* hub, const long long* vbase, const long long* ebase,
+                         const int32_t* offsets, const int32_t* targets, std::vector<int32_t>& order,
+                         int32_t* order_d, int32_t* out, cudaStream_t s);
+inline size_t batch_group_bytes(int64_t n, int64_t m) { return (size_t)(70 * n + 29 * m); }
 
 // Mask reachability on fixed buffers (no allocation, no events).
 // Low-diameter decomposition (Sec. 5.1, Alg. 4) on the symmetric CSR: batch i

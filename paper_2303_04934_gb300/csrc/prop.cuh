@@ -45,7 +45,6 @@ constexpr int kPropQueue = 256;    // vertices a warp gathers before it works on
 constexpr int kPropMarks = 384;    // marks a warp gathers before it publishes them
 constexpr int kPropBigRow = 64;    // rows longer than this are relaxed by the whole warp
 constexpr int kPropUnroll = 4;     // arcs of a row in flight per lane
-constexpr unsigned kPropSweepMin = 1;  // a sweep follows while the last one raised n values or more
 constexpr int kPropTrimPasses = 3; // trimming passes at the start of a batch, at most
 constexpr uint64_t kPropIdleTimeoutNs = 20000000000ull;  // an idle block gives up after 20 s (others may work that long)
 
@@ -79,6 +78,10 @@ struct PropCtl {
     unsigned long long best;  // smaller degree << 32 | key of the vertex that becomes the largest source
     int batches, searches;
     int pivot;
+    unsigned int merged[2];    // vertices merged by mutual arcs: in the sample, in the rest
+    unsigned int hooked[3];    // ... and by a round, a ring over the rounds
+    unsigned int nodes;        // vertices of the contracted graph
+    unsigned int arcs2[2];     // arcs of the contracted graph and of its transpose
     int status;  // 0 finished, 1 a skewed graph (nothing done but the first trim)
     unsigned int first;  // vertices in the first pivot's SCC
 };
@@ -175,7 +178,8 @@ __device__ __forceinline__ V prop_shfl_xor(const V& x, int d) {
 template <class Op>
 struct PropGraph {
     using Val = typename Op::Val;
-    const int32_t* off[2];  // the graph, its transpose
+    const int32_t* off[2];  // the graph, its transpose: row v of [k] is adj[k][off[k][v] .. end[k][v])
+    const int32_t* end[2];
     const int32_t* adj[2];
     int32_t n;
     Val* s[Op::kDirs];            // values; direction 1 travels along the transpose
@@ -326,6 +330,7 @@ __device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op,
     const int lane = lane_id();
     if constexpr (D == 0) dir = 0;
     const int32_t* off = dir ? G.off[1] : G.off[0];
+    const int32_t* end = dir ? G.end[1] : G.end[0];
     const int32_t* adj = dir ? G.adj[1] : G.adj[0];
     Val* s = dir ? G.s[D] : G.s[0];
     int o0 = 0, o1 = 0;
@@ -333,7 +338,7 @@ __device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op,
     if (has) {
         st = Op::load(s, v);
         o0 = S::ld(&off[v]);
-        o1 = S::ld(&off[v + 1]);
+        o1 = S::ld(&end[v]);
     }
     if constexpr (Op::kNamed) {
         if (has) {
@@ -411,7 +416,7 @@ __device__ __forceinline__ int prop_pull(const PropGraph<Op>& G, const Op& op, b
     for (int d = 0; d < D; ++d) {  // a value that travels along a graph comes in along the other
         const int32_t* off = G.off[1 - d];
         e0[d] = has ? S::ld(&off[v]) : 0;
-        len[d] = has ? S::ld(&off[v + 1]) - e0[d] : 0;
+        len[d] = has ? S::ld(&G.end[1 - d][v]) - e0[d] : 0;
         s0[d] = has ? Op::load(G.s[d], v) : Op::none();
     }
 #pragma unroll
@@ -529,12 +534,13 @@ __device__ __forceinline__ bool prop_checked(PropCtl* ctl, PropShared& sh, unsig
 
 // A search by pulling alone. With one word per warp a lane keeps its vertex's
 // values and the first arcs of its rows in registers, so a pass, and with it a
-// hop, costs one round of loads; the vertex a value names is looked at in the
-// same round.
+// hop, costs one round of loads (a longer row one more for every kPropUnroll
+// arcs); the vertex a value names is looked at in the same round.
 template <class S, class Op>
 __device__ bool prop_search_pull(const PropGraph<Op>& G, const Op op, PropCtl* ctl, PropShared& sh, unsigned int& check,
                                  unsigned long long& items) {
     using Val = typename Op::Val;
+    using Part = typename Op::Part;
     constexpr int D = Op::kDirs, U = kPropUnroll;
     const PropSlice P = prop_slice<S>(G.n);
     const int lane = lane_id();
@@ -544,20 +550,21 @@ __device__ bool prop_search_pull(const PropGraph<Op>& G, const Op op, PropCtl* c
     const int v = (int)(P.word(0) * 32) + lane;
     const bool has = one && ((G.active(P.word(0)) >> lane) & 1u);
     Val st[D];
-    int w[D][U], most = 0;
+    int w[D][U], e0[D], len[D], most = 0;
 #pragma unroll
     for (int d = 0; d < D; ++d) {
         st[d] = has ? Op::load(G.s[d], v) : Op::none();
-        const int32_t* off = G.off[1 - d];
-        const int e0 = has ? S::ld(&off[v]) : 0;
-        const int len = has ? S::ld(&off[v + 1]) - e0 : 0;
-        most = max(most, len);
+        e0[d] = has ? S::ld(&G.off[1 - d][v]) : 0;
+        len[d] = has ? S::ld(&G.end[1 - d][v]) - e0[d] : 0;
+        most = max(most, len[d]);
 #pragma unroll
-        for (int u = 0; u < U; ++u) w[d][u] = u < len ? S::ld(&G.adj[1 - d][e0 + u]) : -1;
+        for (int u = 0; u < U; ++u) w[d][u] = u < len[d] ? S::ld(&G.adj[1 - d][e0[d] + u]) : -1;
     }
-    const bool fits = one && __all_sync(kFull, most <= U);
+    most = __reduce_max_sync(kFull, most);
+    const bool fits = one && most <= 4 * U;
     auto pass_one = [&]() {
         Val t[D][U], j[D];
+        Part m[D];
 #pragma unroll
         for (int d = 0; d < D; ++d) {
             j[d] = Op::none();
@@ -568,19 +575,36 @@ __device__ bool prop_search_pull(const PropGraph<Op>& G, const Op op, PropCtl* c
 #pragma unroll
             for (int u = 0; u < U; ++u) t[d][u] = w[d][u] >= 0 ? Op::load(G.s[d], w[d][u]) : Op::none();
         }
-        bool up = false;
 #pragma unroll
         for (int d = 0; d < D; ++d) {
-            typename Op::Part m = Op::part(st[d], j[d]);
+            m[d] = Op::part(st[d], j[d]);
 #pragma unroll
-            for (int u = 0; u < U; ++u) m = Op::fold(m, Op::part(st[d], t[d][u]));
-            if (has && Op::more(m, st[d])) {
-                st[d] = Op::with(st[d], m);
+            for (int u = 0; u < U; ++u) m[d] = Op::fold(m[d], Op::part(st[d], t[d][u]));
+        }
+        for (int k = U; k < most; k += U) {  // warp-uniform
+            int x[D][U];
+#pragma unroll
+            for (int d = 0; d < D; ++d)
+#pragma unroll
+                for (int u = 0; u < U; ++u) x[d][u] = k + u < len[d] ? S::ld(&G.adj[1 - d][e0[d] + k + u]) : -1;
+#pragma unroll
+            for (int d = 0; d < D; ++d)
+#pragma unroll
+                for (int u = 0; u < U; ++u) t[d][u] = x[d][u] >= 0 ? Op::load(G.s[d], x[d][u]) : Op::none();
+#pragma unroll
+            for (int d = 0; d < D; ++d)
+#pragma unroll
+                for (int u = 0; u < U; ++u) m[d] = Op::fold(m[d], Op::part(st[d], t[d][u]));
+        }
+        bool up = false;
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+            if (has && Op::more(m[d], st[d])) {
+                st[d] = Op::with(st[d], m[d]);
                 Op::store(G.s[d], v, st[d]);
                 up = true;
                 ++items;
             }
-        }
         return __any_sync(kFull, up) != 0;
     };
     auto pass_all = [&](bool jump) {
@@ -708,15 +732,15 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
     }
 }
 
-// Whether a vertex w != v of v's class is in the row.
+// Whether a vertex w != v of v's class is in v's row.
 template <class S>
 __device__ __forceinline__ bool prop_any_in_class(const int32_t* adj, int o0, int o1, const unsigned long long* s,
-                                                  uint32_t lab) {
+                                                  uint32_t lab, int v) {
     for (int e = o0; e < o1; e += 2) {
         const int w0 = S::ld(&adj[e]);
         const int w1 = e + 1 < o1 ? S::ld(&adj[e + 1]) : w0;
         const uint32_t l0 = (uint32_t)(ld_volatile(&s[w0]) >> 32), l1 = (uint32_t)(ld_volatile(&s[w1]) >> 32);
-        if (l0 == lab || l1 == lab) return true;
+        if ((l0 == lab && w0 != v) || (l1 == lab && w1 != v)) return true;
     }
     return false;
 }
@@ -738,11 +762,10 @@ __device__ __forceinline__ bool prop_count(PropCtl* ctl, unsigned int& step, uns
 
 // The batches from the state in sf/sb/act until every active vertex is
 // finished (`active` of them): trimming inside the classes, the two searches,
-// the labelling. Self-loops must not be in the graph. The ring of counters
-// starts zero. kPull: the searches only pull. head_ns: time limit of the first batch's head start (0: none);
+// the labelling. The ring of counters starts zero. kPull: the searches only pull. head_ns: time limit of the first batch's head start (0: none);
 // with it the state's keys start zero, and the first batch sets them.
 template <class S, bool kPull>
-__device__ bool prop_batches(const PropGraph<PropMax>& G, const PropMax op, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
+__device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const PropMax op, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
                              unsigned long long active, uint64_t head_ns) {
     const int lane = lane_id();
     const PropSlice P = prop_slice<S>(G.n);
@@ -758,10 +781,10 @@ __device__ bool prop_batches(const PropGraph<PropMax>& G, const PropMax op, Prop
             prop_for_active(G, P, q, [&](bool has, int v) {
                 if (!has) return;
                 const uint32_t lab = (uint32_t)(ld_volatile(&sf[v]) >> 32);
-                const int o0 = S::ld(&G.off[0][v]), o1 = S::ld(&G.off[0][v + 1]);
-                const int i0 = S::ld(&G.off[1][v]), i1 = S::ld(&G.off[1][v + 1]);
-                if (prop_any_in_class<S>(G.adj[0], o0, o1, sf, lab) &&
-                    prop_any_in_class<S>(G.adj[1], i0, i1, sf, lab))
+                const int o0 = S::ld(&G.off[0][v]), o1 = S::ld(&G.end[0][v]);
+                const int i0 = S::ld(&G.off[1][v]), i1 = S::ld(&G.end[1][v]);
+                if (prop_any_in_class<S>(G.adj[0], o0, o1, sf, lab, v) &&
+                    prop_any_in_class<S>(G.adj[1], i0, i1, sf, lab, v))
                     return;
                 *(volatile unsigned long long*)&sf[v] = prop_pack(kPropDone, 0);
                 *(volatile unsigned long long*)&sb[v] = prop_pack(kPropDone, 0);
@@ -828,9 +851,10 @@ __device__ bool prop_batches(const PropGraph<PropMax>& G, const PropMax op, Prop
                 if (!S::sync(&ctl->bar, &ctl->err)) return false;
             }
             // ---- sweeps that pull every active vertex (no atomics, coalesced
-            // rows) while a sweep raises much of the graph; the last one leaves
-            // the vertices it raised dirty
-            while (grew * kPropSweepMin >= (unsigned long long)G.n) {
+            // rows) while the last one raised as many values as vertices were
+            // active at first: a sweep costs 12-25 ps a value, marking 42 ps a
+            // raise. The last one leaves the vertices it raised dirty
+            while (grew >= active) {
                 unsigned long long cnt = 0;
                 for (long long i = 0; i < P.cnt; ++i) {
                     const long long w = P.word(i);

@@ -116,6 +116,8 @@ int launch_reach(const ReachArgs& a, cudaStream_t st) {
     memset(&P, 0, sizeof(P));
     P.G.off[0] = a.off;
     P.G.off[1] = a.toff;
+    P.G.end[0] = a.off + 1;
+    P.G.end[1] = a.toff + 1;
     P.G.adj[0] = a.adj;
     P.G.adj[1] = a.tadj;
     P.G.n = a.n;

@@ -155,7 +155,9 @@ struct Resident {
 // SCC holds its copy of the input, G^T and the transpose's staging, the run
 // state (labels, maxima, bitmaps), the pair tables and the hash bags.
 size_t plain_bytes(int64_t n, int64_t m) { return (size_t)(18 * m + 360 * n) + ((size_t)64 << 20); }
-size_t batched_bytes(int64_t n, int64_t m) { return (size_t)(8 * (n + 1) + 4 * m + 4 * n) + 4096; }
+size_t batched_bytes(int64_t n, int64_t m) {
+    return (size_t)(8 * (n + 1) + 4 * m + 4 * n) + 4096 + batch_group_bytes(n, m);
+}
 size_t reach_bytes(int64_t n) { return (size_t)(16 * n) + 4096; }
 
 double ms_between(Clock::time_point a, Clock::time_point b) {
@@ -432,16 +434,19 @@ void run_batched(scc_server* S, std::vector<ReqPtr>& u) {
     if (rc == SCC_OK) rc = cuda_err(cudaMemcpyAsync(bad.data(), bad_d, sizeof(int) * G, cudaMemcpyDeviceToHost, S->cs));
     if (rc == SCC_OK) rc = cuda_err(cudaStreamSynchronize(S->cs));
     std::vector<int32_t> order;
-    for (int32_t g = 0; g < G; ++g)
+    std::vector<unsigned char> hub(G, 0);
+    for (int32_t g = 0; g < G; ++g) {
+        hub[g] = bad[g] == 2;
+        bad[g] &= 1;
         if (!bad[g]) order.push_back(g);
+    }
     std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
         return (u[a]->m + u[a]->n) > (u[b]->m + u[b]->n);
     });
     const int32_t nvalid = (int32_t)order.size();
     if (rc == SCC_OK && nvalid > 0)
-        rc = cuda_err(cudaMemcpyAsync(ord_d, order.data(), 4 * (size_t)nvalid, cudaMemcpyHostToDevice, S->cs));
-    if (rc == SCC_OK && nvalid > 0)
-        rc = batch_runner_enqueue(S->runner, G, vb_d, eb_d, off_d, adj_d, ord_d, nvalid, lab_d, S->cs);
+        rc = batch_runner_enqueue(S->runner, G, vb.data(), eb.data(), nvalid == G ? hub.data() : nullptr, vb_d, eb_d,
+                                  off_d, adj_d, order, ord_d, lab_d, S->cs);
     if (rc == SCC_OK && nvalid == 0) *err_h = SCC_OK;
     else if (rc == SCC_OK)
         rc = cuda_err(cudaMemcpyAsync(err_h, batch_runner_err(S->runner), sizeof(int), cudaMemcpyDeviceToHost, S->cs));

@@ -106,3 +106,33 @@ def test_hub_and_the_batches_after_its_scc(into):
     a, b = (leaf, hub) if into else (hub, leaf)
     ring = np.array([g.n, g.n + 1, g.n + 2]), np.array([g.n + 1, g.n + 2, g.n])
     _check(_csr(g.n + 3, np.concatenate([src, a, ring[0]]), np.concatenate([g.targets, b, ring[1]]), "hub"))
+
+
+def _mutual(n, extra, share, seed):
+    """A ring of random blocks of mutual arcs (chains and cliques of ids far apart
+    and close by) with one-way arcs between them."""
+    rng = np.random.default_rng(seed)
+    a = rng.integers(0, n, int(share * n))
+    b = np.where(rng.random(len(a)) < 0.5, (a + 1) % n, rng.integers(0, n, len(a)))
+    x, y = rng.integers(0, n, extra), rng.integers(0, n, extra)
+    keep, keep2 = a != b, x != y
+    a, b, x, y = a[keep], b[keep], x[keep2], y[keep2]
+    return _csr(n, np.concatenate([a, b, x]), np.concatenate([b, a, y]), f"mutual{n}_{share}")
+
+
+@pytest.mark.parametrize("n", [65535, 65536, 65537, 70001, 400_000, 1_300_000])
+@pytest.mark.parametrize("share", [0.3, 0.6, 1.0])
+def test_contraction_along_mutual_arcs(n, share):
+    """Graphs around the size from which mutual arcs are contracted, with too few
+    of them, enough, and so many that a giant node remains."""
+    _check(_mutual(n, n, share, seed=n + int(10 * share)))
+
+
+def test_contraction_extremes():
+    n = 100_000
+    i = np.arange(n)
+    _check(_csr(n, np.concatenate([i, (i + 1) % n]), np.concatenate([(i + 1) % n, i]), "two_way_ring"))  # one node
+    star = np.arange(1, 60)  # many small stars: every node's rows meet in its centre
+    c = np.repeat(np.arange(0, n, 60)[:-1], 59)
+    leaf = c + np.tile(star, len(c) // 59)
+    _check(_csr(n, np.concatenate([c, leaf, c[:-60]]), np.concatenate([leaf, c, c[60:]]), "stars"))
