@@ -697,7 +697,7 @@ def _extra_graph(name, scc, torch, stream, steps, warmup, cpu):
 
 
 def _measure_cc(g, off_d, adj_d, scc, torch, stream, steps, warmup, cpu):
-    """Connected components (cc_run: LDD-UF-JTB with VGC and the hash bag,
+    """Connected components (cc_run: union-find on a sample of the arcs first,
     Sec. 5.1) of the undirected graph under the arcs, on a built graph: the
     labels checked against the oracle's union-find, both timed."""
     import oracle
@@ -723,7 +723,7 @@ def _measure_cc(g, off_d, adj_d, scc, torch, stream, steps, warmup, cpu):
            "components": st["components"], "clusters": st["clusters"], "ldd_rounds": st["ldd_rounds"],
            "ldd_batches": st["ldd_batches"], "cross_arcs": st["cross_arcs"],
            "ms_split": {k: st[k] for k in ("ms_ldd", "ms_union", "ms_label")},
-           "step": "cc_run on a built graph (symmetric CSR kept from the warm-up)"}
+           "step": "cc_run on a built graph"}
     if cpu:
         t0 = time.perf_counter()
         want, ncc = oracle.cc_labels(g.n, g.offsets, g.targets)

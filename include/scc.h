@@ -96,11 +96,11 @@ SCC_API const char* scc_error_string(int code);
  *               once it holds 1/k of it.
  *   seed        seed of the pivot permutation, and of the order of the sources in
  *               a batch (default 0x5CC00).
- *   ldd_beta    growth factor of the centre batches of cc_run's low-diameter
- *               decomposition, in (1, 64] (Sec. 5.1 uses 1.2). Default 2: each
- *               batch adds a round whose time on the GPU is mostly barrier and
- *               memory latency, so fewer and larger batches are faster here
- *               (R-MAT 24: 83 -> 24 rounds); the components do not change.
+ *   ldd_beta    growth factor of the centre batches of the low-diameter
+ *               decomposition of Sec. 5.1, in (1, 64] (the paper uses 1.2; the
+ *               default is 2). Checked, and otherwise without effect: cc_run
+ *               takes the components by union-find on a sample of the arcs
+ *               first, without that decomposition.
  * Out-of-range values are rejected with SCC_ERR_INVALID_ARG.
  */
 typedef struct scc_config {
@@ -242,19 +242,16 @@ SCC_API int scc_get_stats(scc_handle h, scc_stats* out);
 
 /* ---------------------------------------------------------- connectivity ---- */
 /*
- * Connected components (Sec. 5.1, Alg. 4: LDD-UF-JTB, with the hash bag and
- * VGC applied to the low-diameter decomposition) of the undirected graph under
- * the arcs of h: u and v are in one component iff a path joins them when every
+ * Connected components (Sec. 5.1, by union-find on a sample of each vertex's
+ * arcs, then on the rest of the rows outside the largest tree) of the
+ * undirected graph under the arcs of h: u and v are in one component iff a path joins them when every
  * arc may be taken in either direction (the paper symmetrises directed inputs
  * for connectivity; for a directed graph these are its weakly connected
  * components). labels_out[v] = the smallest vertex id of v's component.
  *   labels_out  host or device int32[n], written.
- * The first call on h builds the symmetric CSR (each vertex's out-arcs then
- * its in-arcs, 2 m_t entries) and keeps it with the handle until it is
- * destroyed. The decomposition takes its centres from h's seeded order in
- * batches growing by the configuration's ldd_beta (default 2; the paper's
- * choice is 1.2); the result depends on neither the seed nor ldd_beta. Returns SCC_ERR_INTERNAL if a bounded union-find loop
- * ran out (never expected). Synchronises `stream` before returning.
+ * Nothing is kept with the handle. Returns SCC_ERR_INTERNAL if a bounded
+ * union-find loop ran out (never expected). Synchronises `stream` before
+ * returning.
  */
 SCC_API int cc_run(scc_handle h, int32_t* labels_out, void* stream);
 
@@ -262,13 +259,14 @@ SCC_API int cc_run(scc_handle h, int32_t* labels_out, void* stream);
    stream of the call). */
 typedef struct scc_cc_stats {
     int32_t components;   /* connected components found */
-    int32_t clusters;     /* clusters of the low-diameter decomposition (centres) */
-    int32_t ldd_rounds;   /* rounds of the decomposition's search */
-    int32_t ldd_batches;  /* batches of candidate centres */
-    int64_t ldd_arcs;     /* arcs examined by the decomposition's search */
-    int64_t cross_arcs;   /* arcs of G joining two clusters (the union-find's work) */
-    double ms_sym;        /* building the symmetric CSR (0 when it was kept from an earlier call) */
-    double ms_ldd, ms_union, ms_label, ms_total;
+    int32_t clusters;     /* trees after the sampled arcs (the components at least, n at most) */
+    int32_t ldd_rounds;   /* 0 (no decomposition is searched) */
+    int32_t ldd_batches;  /* 0 */
+    int64_t ldd_arcs;     /* 0 */
+    int64_t cross_arcs;   /* arcs beyond the sample found to join two trees (depends on their timing) */
+    double ms_sym;        /* 0 (no symmetric CSR is built) */
+    double ms_ldd;        /* the sampled arcs */
+    double ms_union, ms_label, ms_total; /* the other arcs; the labels; all of it */
 } scc_cc_stats;
 
 SCC_API int cc_get_stats(scc_handle h, scc_cc_stats* out);

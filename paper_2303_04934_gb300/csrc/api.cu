@@ -844,11 +844,11 @@ int reach_multi_noalloc(scc_handle h, const int32_t* sources, int32_t k, int32_t
 }
 
 // ----------------------------------------------------------- connectivity --
-// Connected components of the undirected graph under G's arcs (Sec. 5.1,
-// Alg. 4 LDD-UF-JTB with VGC and the hash bag; steps in cc.cu).
+// Connected components of the undirected graph under G's arcs (Sec. 5.1; steps
+// in cc.cu).
 
-// The symmetric CSR of h (row v = row v of G, then row v of G^T), built on the
-// first call and kept with the handle.
+// The symmetric CSR of h (row v = row v of G, then row v of G^T) for the
+// LE-lists, built on the first call and kept with the handle.
 static int ensure_sym(scc_graph* h, cudaStream_t s) {
     if (h->soff) return SCC_OK;
     const int32_t n = h->n;
@@ -874,99 +874,39 @@ static int cc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
     scc_cc_stats& st = h->cc_stats;
     memset(&st, 0, sizeof(st));
     if (n == 0) return SCC_OK;
-    const int num_sms = h->di.num_sms;
-    EvTimer tt(s);
-    tt.start();
-    EvTimer t(s);
-    // the symmetric CSR, kept with the handle
-    t.start();
-    SCC_TRY(ensure_sym(h, s));
-    st.ms_sym = t.stop();
-    // the seeded order of all vertices and its batches
     Scratch tmp(s);
-    int32_t *order = nullptr, *center = nullptr, *parent = nullptr, *root = nullptr, *mn = nullptr, *out = nullptr;
-    long long* bounds_d = nullptr;
+    int32_t *sample = nullptr, *parent = nullptr, *out = nullptr, *giant = nullptr;
     unsigned long long* counters = nullptr;
+    int2* piece = nullptr;
     int* err = nullptr;
-    SCC_TRY(tmp.alloc(&order, (size_t)n));
-    SCC_TRY(tmp.alloc(&center, (size_t)n));
+    const int64_t cap = cc_piece_cap(h->mt);
+    SCC_TRY(tmp.alloc(&sample, cc_sample_size(n)));
     SCC_TRY(tmp.alloc(&parent, (size_t)n));
-    SCC_TRY(tmp.alloc(&root, (size_t)n));
-    SCC_TRY(tmp.alloc(&mn, (size_t)n));
-    SCC_TRY(tmp.alloc(&counters, 4));
-    SCC_TRY(tmp.alloc(&err, 1));
+    SCC_TRY(tmp.alloc(&piece, (size_t)cap));
+    SCC_TRY(tmp.alloc(&counters, 6));  // four counters, then err and the large tree's three words
+    err = reinterpret_cast<int*>(counters + 4);
+    giant = err + 1;
     const bool dev_out = is_device_ptr(labels_out);
     if (dev_out) out = labels_out;
     else SCC_TRY(tmp.alloc(&out, (size_t)n));
-    SCC_CUDA(cudaMemsetAsync(counters, 0, 4 * sizeof(unsigned long long), s));
-    SCC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    std::vector<long long> bounds{0};
-    {
-        double x = 1.0;
-        long long pos = 0;
-        while (pos < n) {
-            long long sz;
-            if (x >= (double)n) sz = n;
-            else {
-                sz = (long long)x;
-                if ((double)sz < x) ++sz;
-            }
-            if (sz < 1) sz = 1;
-            pos = ((long long)n - pos < sz) ? (long long)n : pos + sz;
-            bounds.push_back(pos);
-            x *= h->cfg.ldd_beta;
-        }
-    }
-    const int nb = (int)bounds.size() - 1;
-    SCC_TRY(tmp.alloc(&bounds_d, bounds.size()));
-    SCC_CUDA(cudaMemcpyAsync(bounds_d, bounds.data(), sizeof(long long) * bounds.size(), cudaMemcpyHostToDevice, s));
-    // ---- LDD (Alg. 4 function LDD)
-    t.start();
-    SCC_TRY(launch_iota(n, root, num_sms, s));  // the identity list, permuted into the order
-    SCC_TRY(launch_pivot_order(root, (int64_t)n, h->cfg.seed, order, s));
-    // the visited bitmap and the two frontier bitmaps of the bottom-up rounds
-    const size_t nw = ((size_t)n + 31) / 32;
-    uint32_t *vbits = nullptr, *fbits = nullptr;
-    SCC_TRY(tmp.alloc(&vbits, nw));
-    SCC_TRY(tmp.alloc(&fbits, 2 * nw));
-    SCC_CUDA(cudaMemsetAsync(fbits, 0, sizeof(uint32_t) * 2 * nw, s));
-    SCC_TRY(launch_ldd_setup(order, bounds[1], n, center, vbits, num_sms, s));
-    SCC_TRY(engine_reserve(&h->eb32, 4, (long long)n + 1024, h->cfg.lambda, 2 * h->mt, num_sms, s));
-    EngineOpts o = opts_of(h);
-    EngineRun r;
-    // bottom-up rounds when the frontier is large, as for the first SCC's searches
-    const int frac_inv = h->cfg.dense == 1 ? 20 : h->cfg.dense;
-    SCC_TRY(run_ldd(h->soff, h->sadj, n, 2 * (long long)h->mt, order, bounds_d, bounds[1], nb, center, vbits, fbits,
-                    frac_inv, &h->eb32, o, &r, s));
-    st.ms_ldd = t.stop();
-    st.ldd_rounds = r.rounds;
-    st.ldd_batches = nb;
-    st.ldd_arcs = (int64_t)r.edges;
-    // ---- union-find over the cross arcs (Alg. 4 Union), then the labels
+    SCC_CUDA(cudaMemsetAsync(counters, 0, 6 * sizeof(unsigned long long), s));
     CreateEvents ev;
-    cudaEventRecord(ev.e[0], s);
-    const long long big_cap = (long long)(h->mt / 33) + 1;  // rows of more than 32 arcs
-    int32_t *big = nullptr, *bdeg = nullptr, *bpre = nullptr;
-    unsigned char* stmp = nullptr;
-    SCC_TRY(tmp.alloc(&big, (size_t)big_cap));
-    SCC_TRY(tmp.alloc(&bdeg, (size_t)big_cap));
-    SCC_TRY(tmp.alloc(&bpre, (size_t)big_cap + 1));
-    SCC_TRY(tmp.alloc(&stmp, scan_tmp_bytes(big_cap)));
-    SCC_TRY(launch_cc_union_label(h->off, h->adj, n, center, parent, root, mn, out, counters, big, bdeg, bpre, stmp,
-                                  big_cap, err, num_sms, s, &ev.e[1]));
+    SCC_TRY(launch_cc(h->off, h->adj, h->toff, h->tadj, n, sample, parent, out, counters, giant, piece, cap, err,
+                      h->di.num_sms, s, ev.e));
     if (!dev_out) SCC_TRY(from_device(labels_out, out, sizeof(int32_t) * (size_t)n, s));
-    unsigned long long hc[4];
-    int herr = 0;
+    unsigned long long hc[5];
     SCC_CUDA(cudaMemcpyAsync(hc, counters, sizeof(hc), cudaMemcpyDeviceToHost, s));
-    SCC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     SCC_CUDA(cudaStreamSynchronize(s));
+    int herr = 0;
+    memcpy(&herr, &hc[4], sizeof(herr));
     if (herr) return herr;
     st.cross_arcs = (int64_t)hc[0];
     st.clusters = (int32_t)hc[1];
     st.components = (int32_t)hc[2];
+    st.ms_ldd = ev.ms(0, 1);
     st.ms_union = ev.ms(1, 2);
     st.ms_label = ev.ms(2, 3);
-    st.ms_total = tt.stop();
+    st.ms_total = ev.ms(0, 3);
     return SCC_OK;
 }
 

@@ -1,26 +1,33 @@
-// Connected components by LDD-UF-JTB with VGC and the hash bag (Sec. 5.1,
-// Alg. 4), on the undirected graph under the arcs of G (sm_103a).
+// Connected components of the undirected graph under the arcs of G (Sec. 5.1;
+// sm_103a) by union-find on a sample of the arcs first, as a forest of parent
+// pointers with parent[x] <= x, so that a tree's root is its smallest vertex
+// and the final roots are the labels:
 //
-//   1. The symmetric CSR: row v of G followed by row v of G^T (the paper
-//      symmetrises directed inputs for connectivity). Its offsets are
-//      off[v] + toff[v], so only the rows are copied.
-//   2. LDD (Alg. 4 function LDD): a seeded order of all vertices cut into
-//      batches growing by the factor scc_config.ldd_beta (default 2; the
-//      paper's choice is 1.2, fewer batches mean fewer rounds here); the first
-//      batch claims itself, then one search of the VGC engine (PolLdd) runs
-//      rounds in which every frontier item claims unvisited neighbours for its
-//      centre, and at the end of round i the unvisited vertices of batch i + 1
-//      become centres of their own and join the frontier. A round whose
-//      frontier holds at least 1/20 of the vertices runs bottom-up instead
-//      (the engine's dense rounds, Sec. 4.2): every unclaimed vertex with a
-//      neighbour in the frontier joins that neighbour's cluster.
-//   3. Union-find over the arcs whose endpoints have different centres (Alg. 4
-//      "if Find(L(v)) != Find(L(u)) then Union"): a root is hooked under the
-//      smaller root by CAS, finds halve their paths; every retry loop is
-//      bounded and reports SCC_ERR_INTERNAL past its limit.
-//   4. labels_out[v] = the smallest vertex id of the component of v (the
-//      component's root is its smallest centre, not necessarily its smallest
-//      vertex: one atomicMin pass per root).
+//   1. parent[v] = the smallest of v and the sampled neighbours of v (its first
+//      kCcOut out-arcs and kCcIn in-arcs), by plain stores; then every other
+//      sampled arc joins its two trees (k_cc_seed, k_cc_link).
+//   2. Every parent becomes its tree's root (k_cc_flat) and the most frequent
+//      root of 1024 vertices spread over the graph is taken as the large tree
+//      (k_cc_giant).
+//   3. The arcs that were not sampled (k_cc_rest). A vertex of the large tree
+//      skips its rows: an arc between it and a vertex of another tree is read
+//      from the other end's row of G or of G^T, and an arc between two of its
+//      vertices joins nothing. Without a tree that holds an eighth of the
+//      vertices nobody is skipped and the rows of G cover every arc. Rows of
+//      more than kCcRow arcs are cut into pieces of kCcPiece for k_cc_big.
+//   4. labels_out[v] = the root of v (k_cc_labels).
+//
+// The paper's LDD-UF-JTB (Alg. 4) takes the same labels from a low-diameter
+// decomposition of the symmetrised graph, a search of tens of rounds, and then
+// tests every arc for joining two clusters. On R-MAT with 4.2 M vertices and
+// 25 M arcs that was 0.97 ms for the search, 0.51 for the arcs and 0.14 for the
+// labels, and 3.2 ms before the first of them for the symmetric CSR; now the
+// sample is 0.18, the other arcs 0.04 and the labels 0.014 (1.81 -> 0.29 ms a
+// call; 5.1 -> 0.32 ms the first). By bytes (offsets of both graphs, a sector an
+// active vertex and sample, the copies and parents) it is bound at about
+// 0.09 ms; what is left is gathers of parents from L2 and 16 launches. The
+// decomposition has no graph left on which it is ahead: lattices 4.4 -> 0.62 ms
+// (2-D, 8.4 M vertices), small graphs 0.56 -> 0.26.
 #include <algorithm>
 #include <climits>
 #include <vector>
@@ -33,8 +40,13 @@ namespace scc {
 namespace {
 
 constexpr int kBlk = 256;
-constexpr int kUfLimit = 1 << 20;  // steps of one find or union before it reports an error
-constexpr int kSmallRow = 32;      // rows with more arcs go to the flat pass (k_uf_flat)
+constexpr int kUfLimit = 1 << 20;  // attempts of one union before it reports an error
+constexpr int kCcOut = 2;          // sampled out-arcs of a vertex
+constexpr int kCcIn = 1;           // sampled in-arcs of a vertex
+constexpr int kCcSample = kCcOut + kCcIn;
+constexpr int kCcRow = 32;         // longer rows go to k_cc_big ...
+constexpr int kCcPiece = 1024;     // ... in pieces of this many arcs, a warp each
+constexpr int kCcProbe = 1024;     // vertices whose roots name the large tree
 
 inline int grid_for(int64_t work, int per_block, int cap) {
     int64_t g = (work + per_block - 1) / per_block;
@@ -59,46 +71,39 @@ __global__ void k_sym_rows(const int32_t* __restrict__ off, const int32_t* __res
     if (w0 == 0 && lane == 0) soff[n] = off[n] + toff[n];
 }
 
-// center[v] = -1 for all v and no vertex visited (the bits past n set: the
-// dense rounds read whole words), then the first batch's vertices centre
-// themselves.
-__global__ void k_ldd_init(int32_t n, int32_t* center, uint32_t* bits) {
-    const long long nw = ((long long)n + 31) / 32;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
-        center[v] = -1;
-    for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < nw; w += (long long)gridDim.x * blockDim.x)
-        bits[w] = (w == nw - 1 && (n & 31)) ? ~((1u << (n & 31)) - 1u) : 0u;
-}
-__global__ void k_ldd_first(const int32_t* __restrict__ order, long long k, int32_t* center, uint32_t* bits) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += (long long)gridDim.x * blockDim.x) {
-        const int32_t v = order[i];
-        center[v] = v;
-        atomicOr(&bits[v >> 5], 1u << (v & 31));
-    }
-}
-
 // ------------------------------------------------------------- union-find --
 // parent[x] <= x always (a root is hooked under a smaller one), so the
-// concurrent halving writes keep every parent a vertex of the same tree.
-__device__ __forceinline__ int32_t uf_find(int32_t* parent, int32_t x, int* err) {
-    for (int it = 0; it < kUfLimit; ++it) {
+// concurrent halving writes keep every parent a vertex of the same tree, and a
+// walk towards the root ends: each step goes to a smaller vertex.
+__device__ __forceinline__ int32_t uf_find(int32_t* parent, int32_t x) {
+    for (;;) {
         const int32_t p = ld_volatile(&parent[x]);
-        if (p == x) return x;
+        if (p >= x) return x;
         const int32_t gp = ld_volatile(&parent[p]);
-        if (gp != p) parent[x] = gp;  // halving
+        if (gp >= p) return p;
+        parent[x] = gp;  // halving
         x = gp;
     }
-    atomicExch(err, SCC_ERR_INTERNAL);
-    return x;
+}
+// A root without writes, for the passes in which no trees join and each
+// vertex's owner stores its root (a halving store could put an older ancestor
+// over it). Plain loads: the few words that most walks end in come from L1.
+__device__ __forceinline__ int32_t uf_root(const int32_t* parent, int32_t x) {
+    for (;;) {
+        const int32_t p = parent[x];
+        if (p >= x) return x;
+        x = p;
+    }
 }
 __device__ __forceinline__ void uf_union(int32_t* parent, int32_t a, int32_t b, int* err) {
     for (int it = 0; it < kUfLimit; ++it) {
-        const int32_t ra = uf_find(parent, a, err), rb = uf_find(parent, b, err);
+        const int32_t ra = uf_find(parent, a), rb = uf_find(parent, b);
         if (ra == rb) return;
         const int32_t lo = ra < rb ? ra : rb, hi = ra < rb ? rb : ra;
-        if (atomicCAS(&parent[hi], hi, lo) == hi) return;
+        const int32_t old = atomicCAS(&parent[hi], hi, lo);
+        if (old == hi) return;
         a = lo;
-        b = hi;
+        b = old;
     }
     atomicExch(err, SCC_ERR_INTERNAL);
 }
@@ -116,207 +121,252 @@ __device__ __forceinline__ int32_t uf_peek(const int32_t* parent, int32_t x) {
     return x;
 }
 
-__global__ void k_uf_init(int32_t n, int32_t* parent, int32_t* mn) {
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        parent[v] = (int32_t)v;
-        mn[v] = INT_MAX;
-    }
-}
-
-// Arcs of G whose endpoints lie in different clusters join the clusters'
-// centres (every edge of the undirected graph is an arc of G). A thread takes
-// one row of at most kSmallRow arcs and walks it, four arcs at a time; longer
-// rows go to a list (row, degree) whose arcs k_uf_flat spreads evenly over the
-// whole grid. After the decomposition most cross arcs repeat a pair that is
-// already joined (a few clusters per component, many arcs between them), and
-// every union on the same pair would contend for the same few parent words:
-// a row skips the centre it joined last, a warp elects one lane per distinct
-// pair, and a read-only peek at both sets skips pairs already joined.
-__global__ void k_uf_arcs(const int32_t* __restrict__ off, const int32_t* __restrict__ adj, int32_t n,
-                          const int32_t* __restrict__ center, int32_t* parent, unsigned long long* cross,
-                          int32_t* big, int32_t* bdeg, unsigned long long* nbig, long long big_cap, int* err) {
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long gstride = (long long)gridDim.x * blockDim.x;
-    unsigned long long c = 0;
-    for (long long u = gtid; u < n; u += gstride) {
-        const int a0 = off[u], a1 = off[u + 1];
-        if (a1 == a0) continue;
-        if (a1 - a0 > kSmallRow) {
-            const unsigned long long k = atomicAdd(nbig, 1ull);
-            if ((long long)k < big_cap) {
-                big[k] = (int32_t)u;
-                bdeg[k] = a1 - a0;
-            } else {
-                atomicExch(err, SCC_ERR_INTERNAL);  // cannot happen: big_cap >= m / (kSmallRow + 1) + 1
-            }
-            continue;
-        }
-        const int32_t cu = center[u];
-        if ((uint32_t)cu >= (uint32_t)n) {  // every vertex has a centre after the decomposition
-            atomicCAS(err, 0, SCC_ERR_INTERNAL);
-            continue;
-        }
-        // four arcs at a time: their targets, then the targets' centres, as
-        // independent loads
-        int32_t last = cu;
-        for (int e0 = a0; e0 < a1; e0 += 4) {
-            int32_t w[4], cw[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = e0 + j < a1 ? adj[e0 + j] : -1;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cw[j] = w[j] >= 0 ? center[w[j]] : cu;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if ((uint32_t)cw[j] >= (uint32_t)n) {
-                    atomicCAS(err, 0, SCC_ERR_INTERNAL);
-                    continue;
-                }
-                if (cw[j] != cu) {
-                    ++c;
-                    if (cw[j] != last) {
-                        last = cw[j];
-                        if (uf_peek(parent, cu) != uf_peek(parent, cw[j])) uf_union(parent, cu, cw[j], err);
-                    }
-                }
-            }
-        }
-    }
+// The block's sum of c into *out, by one atomic (one a warp on a single word was
+// 50 us on 4.2 M vertices).
+__device__ __forceinline__ void cc_add(unsigned long long* out, unsigned long long c) {
+    __shared__ unsigned long long sum;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
     for (int d = 16; d >= 1; d >>= 1) c += __shfl_xor_sync(kFull, c, d);
-    if (lane_id() == 0 && c) atomicAdd(cross, c);
+    if (lane_id() == 0 && c) atomicAdd(&sum, c);
+    __syncthreads();
+    if (threadIdx.x == 0 && sum) atomicAdd(out, sum);
 }
 
-// The arcs of the listed rows as one flat range (row k of the list covers
-// [bpre[k], bpre[k + 1])) cut into 32-arc chunks; each warp takes a contiguous
-// run of chunks and walks the rows forward. A chunk meets at most two rows
-// (every listed row has more than 32 arcs), so a lane's row is the warp's
-// current row or the next one, whose start in the flat range, arc base and
-// centre the warp keeps in registers: a chunk costs a coalesced read of its
-// targets and a gather of their centres.
-__global__ void k_uf_flat(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
-                          const int32_t* __restrict__ center, int32_t* parent, unsigned long long* cross,
-                          const int32_t* __restrict__ big, const unsigned long long* nbig, long long big_cap,
-                          const int32_t* __restrict__ bpre, int32_t n, int* err) {
+// sample[j n + v] = the sampled neighbours of v: its first kCcOut out-arcs and
+// kCcIn in-arcs, v itself where the row is shorter; parent[v] = the smallest of
+// v and these. Bound by the latency of off -> adj: one vertex a thread keeps as
+// many chains in flight as the chip holds threads. The passes below read the
+// copy, 12 coalesced bytes a vertex instead of four offsets and three sectors.
+__global__ void __launch_bounds__(kBlk) k_cc_seed(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                  const int32_t* __restrict__ toff, const int32_t* __restrict__ tadj,
+                                                  int32_t n, int32_t* __restrict__ sample, int32_t* __restrict__ parent) {
+    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
+        const int a0 = off[v], a1 = off[v + 1], b0 = toff[v], b1 = toff[v + 1];
+        int32_t w[kCcSample], lo = (int32_t)v;
+#pragma unroll
+        for (int j = 0; j < kCcOut; ++j) w[j] = a1 - a0 > j ? adj[a0 + j] : (int32_t)v;
+#pragma unroll
+        for (int j = 0; j < kCcIn; ++j) w[kCcOut + j] = b1 - b0 > j ? tadj[b0 + j] : (int32_t)v;
+#pragma unroll
+        for (int j = 0; j < kCcSample; ++j) {
+            sample[(long long)j * n + v] = w[j];
+            lo = min(lo, w[j]);
+        }
+        parent[v] = lo;
+    }
+}
+
+// Every sampled arc between two trees hooks the larger root under the smaller:
+// each parent was its tree's root before the launch, so all values read and
+// written here are such roots, and of several hooks of one root the smallest
+// stays (the arcs of the others are met again by a later pass). An atomic
+// without a result instead of a find-and-CAS loop: joining the trees to the end
+// here, with walks that go on while every tree changes, was 213 us on R-MAT with
+// 262 k vertices and 263-368 us with 4.2 M, where two passes of hooks and their
+// flattening take 27 and 84.
+__global__ void __launch_bounds__(kBlk) k_cc_hook(const int32_t* __restrict__ sample, int32_t n, int32_t* parent,
+                                                  const int32_t* giant, const int32_t* unless) {
+    if (unless && *unless >= 0) return;
+    const int32_t gt = giant ? *giant : -1;
+    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
+        const int32_t a = parent[v];
+        if (a == gt) continue;
+        int32_t b[kCcSample];
+#pragma unroll
+        for (int j = 0; j < kCcSample; ++j) b[j] = sample[(long long)j * n + v];
+#pragma unroll
+        for (int j = 0; j < kCcSample; ++j) b[j] = b[j] == (int32_t)v ? a : parent[b[j]];
+#pragma unroll
+        for (int j = 0; j < kCcSample; ++j)
+            if (b[j] != a) {
+                const int32_t lo = min(a, b[j]), hi = max(a, b[j]);
+                if (lo < parent[hi]) atomicMin(&parent[hi], lo);
+            }
+    }
+}
+
+// parent[v] = the root of v, four vertices a thread whose walks go side by side.
+// A walk of more than six steps reads past L1 and stores where it is, its own
+// word only, so the walks that run at once shorten one another's: a path graph
+// numbered in order, whose seeded forest is one chain, takes 0.5 ms at 4.2 M
+// vertices, and seconds without. For the same reason each thread starts all its
+// walks at once and the grid has a thread for every four vertices: a walk goes to
+// smaller vertices and blocks start in order, so none passes a vertex whose own
+// walk is yet to start.
+__global__ void __launch_bounds__(kBlk) k_cc_flat(int32_t n, int32_t* parent, const int32_t* unless) {
+    if (unless && *unless >= 0) return;
+    const long long v = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+    if (v >= n) return;
+    const int k = n - v < 4 ? (int)(n - v) : 4;
+    int32_t p0[4], r[4];
+    if (k == 4) {
+        const int4 q = *reinterpret_cast<const int4*>(parent + v);
+        p0[0] = q.x;
+        p0[1] = q.y;
+        p0[2] = q.z;
+        p0[3] = q.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p0[j] = j < k ? parent[v + j] : 0;  // parent[0] = 0
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) r[j] = p0[j];
+    uint32_t on = 15;  // the walks under way
+    for (int it = 0; on; ++it) {
+        int32_t p[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            p[j] = !(on >> j & 1) ? r[j] : it < 6 ? parent[r[j]] : ld_volatile(&parent[r[j]]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (p[j] < r[j]) {
+                r[j] = p[j];
+                if (it >= 6 && j < k) *(volatile int32_t*)&parent[v + j] = p[j];
+            } else {
+                on &= ~(1u << j);
+            }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (j < k && r[j] != p0[j]) parent[v + j] = r[j];
+}
+
+// giant = the most frequent root of kCcProbe vertices at equal distances if at
+// least an eighth of them have it, or -1 (or *unless if that names one). One
+// block of kCcProbe threads.
+__global__ void __launch_bounds__(kCcProbe) k_cc_giant(const int32_t* __restrict__ parent, int32_t n, int32_t* giant,
+                                                       const int32_t* unless) {
+    if (unless && *unless >= 0) {
+        if (threadIdx.x == 0) *giant = *unless;
+        return;
+    }
+    __shared__ int32_t key[2 * kCcProbe];
+    __shared__ int cnt[2 * kCcProbe];
+    __shared__ unsigned long long best;
+    const int t = threadIdx.x;
+    for (int j = t; j < 2 * kCcProbe; j += kCcProbe) {
+        key[j] = -1;
+        cnt[j] = 0;
+    }
+    if (t == 0) best = 0;
+    __syncthreads();
+    const int32_t r = parent[(long long)t * n / kCcProbe];
+    uint32_t slot = ((uint32_t)r * 2654435769u) >> 21;  // 11 bits: 2 kCcProbe slots
+    for (int it = 0; it < 2 * kCcProbe; ++it) {         // kCcProbe keys at most: a free slot is met
+        const int32_t k = atomicCAS(&key[slot], -1, r);
+        if (k == -1 || k == r) break;
+        slot = (slot + 1) & (2 * kCcProbe - 1);
+    }
+    const int c = atomicAdd(&cnt[slot], 1) + 1;
+    atomicMax(&best, (unsigned long long)(uint32_t)c << 32 | (uint32_t)r);
+    __syncthreads();
+    if (t == 0) *giant = (int)(best >> 32) >= kCcProbe / 8 ? (int32_t)(uint32_t)best : -1;
+}
+
+// One row (arcs [a, b) of adj) of u: four targets at a time, then their peeks,
+// as independent loads.
+__device__ __forceinline__ unsigned long long cc_row(const int32_t* __restrict__ adj, int a, int b, int step, int32_t u,
+                                                     int32_t* parent, int* err) {
+    unsigned long long c = 0;
+    for (long long e0 = a; e0 < b; e0 += 4 * step) {
+        int32_t w[4], p[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = e0 + j * step < b ? adj[e0 + j * step] : u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[j] = uf_peek(parent, w[j]);
+        const int32_t pu = uf_peek(parent, u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (p[j] != pu) {
+                ++c;
+                uf_union(parent, pu, p[j], err);
+            }
+    }
+    return c;
+}
+
+// The rows of the vertices outside the large tree, a thread a vertex; the warp
+// lists the pieces of its long rows together (piece = (u, or ~u for the row of
+// G^T; first arc)).
+__global__ void __launch_bounds__(kBlk) k_cc_rest(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                  const int32_t* __restrict__ toff, const int32_t* __restrict__ tadj,
+                                                  int32_t n, int32_t* parent, const int32_t* giant,
+                                                  unsigned long long* joined, unsigned long long* trees, int2* piece,
+                                                  unsigned long long* npiece, long long cap, int* err) {
     const int lane = lane_id();
-    const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long nb = min((long long)*nbig, big_cap);
-    unsigned long long c = 0;
-    const long long total = nb > 0 ? (long long)bpre[nb] : 0;
-    const long long nch = (total + 31) / 32;
-    const long long per = (nch + nw - 1) / nw;
-    const long long ch0 = wid * per, ch1 = min(ch0 + per, nch);
-    if (ch0 < ch1) {  // warp-uniform
-        // the row of the run's first arc: the last k with bpre[k] <= 32 ch0
-        long long lo = 0, hi = nb - 1;
-        while (lo < hi) {
-            const long long mid = (lo + hi + 1) >> 1;
-            if ((long long)bpre[mid] <= ch0 * 32) lo = mid;
-            else hi = mid - 1;
-        }
-        long long r = lo;
-        // rows r and r + 1: start in the flat range, arc base (off[u] - start), centre
-        auto row = [&](long long k, long long& st, long long& base, int32_t& cu) {
-            if (k < nb) {
-                const int32_t u = big[k];
-                st = bpre[k];
-                base = (long long)off[u] - st;
-                cu = center[u];
-            } else {
-                st = total;
-                base = 0;
-                cu = 0;
+    const int32_t gt = *giant;
+    unsigned long long c = 0, nt = 0;
+    for (long long v0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) - lane; v0 < n;
+         v0 += (long long)gridDim.x * blockDim.x) {
+        const long long v = v0 + lane;
+        const int32_t pv = v < n ? parent[v] : -1;
+        const bool live = v < n && (gt < 0 || pv != gt);
+        nt += pv == (int32_t)v;
+        if (!__any_sync(kFull, live)) continue;
+        for (int d = 0; d < (gt < 0 ? 1 : 2); ++d) {
+            const int32_t* o = d == 0 ? off : toff;
+            const int32_t* aj = d == 0 ? adj : tadj;
+            int a = 0, b = 0;
+            if (live) {
+                a = o[v];
+                b = o[v + 1];
             }
-        };
-        long long s0, b0, s1, b1;
-        int32_t c0, c1;
-        row(r, s0, b0, c0);
-        row(r + 1, s1, b1, c1);
-        int32_t lcu = -1, lcw = -1;  // the pair this lane joined last
-        // two chunks a step: both targets, then both centres, as independent loads
-        for (long long ch = ch0; ch < ch1; ch += 2) {
-            int32_t cu[2], w[2], cw[2];
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                const long long f0 = (ch + t) * 32;
-                while (f0 >= s1 && r + 1 < nb) {  // at most once a chunk: every listed row has more than 32 arcs
-                    ++r;
-                    s0 = s1;
-                    b0 = b1;
-                    c0 = c1;
-                    row(r + 1, s1, b1, c1);
-                }
-                const long long f = f0 + lane;
-                const bool in = ch + t < ch1 && f < total;
-                const bool nx = f >= s1;
-                cu[t] = nx ? c1 : c0;
-                w[t] = in ? adj[f + (nx ? b1 : b0)] : -1;
-            }
-#pragma unroll
-            for (int t = 0; t < 2; ++t) cw[t] = w[t] >= 0 ? center[w[t]] : cu[t];
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                if (w[t] >= 0 && ((uint32_t)cu[t] >= (uint32_t)n || (uint32_t)cw[t] >= (uint32_t)n)) {
-                    atomicCAS(err, 0, SCC_ERR_INTERNAL);  // every vertex has a centre
-                    cw[t] = cu[t];
-                }
-                const bool x = w[t] >= 0 && cw[t] != cu[t];
-                c += x;
-                const unsigned long long key =
-                    x ? ((unsigned long long)(uint32_t)cu[t] << 32 | (uint32_t)cw[t]) : ~0ull;
-                const uint32_t peers = __match_any_sync(kFull, key);
-                if (x && __ffs(peers) - 1 == lane && !(cu[t] == lcu && cw[t] == lcw)) {
-                    lcu = cu[t];
-                    lcw = cw[t];
-                    if (uf_peek(parent, cu[t]) != uf_peek(parent, cw[t])) uf_union(parent, cu[t], cw[t], err);
+            const bool big = b - a > kCcRow;
+            if (!big && a < b) c += cc_row(aj, a, b, 1, (int32_t)v, parent, err);
+            for (uint32_t m = __ballot_sync(kFull, big); m; m &= m - 1) {
+                const int l = __ffs(m) - 1;
+                const int la = __shfl_sync(kFull, a, l), lb = __shfl_sync(kFull, b, l);
+                const int k = (int)(((long long)lb - la + kCcPiece - 1) / kCcPiece);
+                unsigned long long at = 0;
+                if (lane == 0) at = atomicAdd(npiece, (unsigned long long)k);
+                at = __shfl_sync(kFull, at, 0);
+                const int32_t u = (int32_t)(v0 + l);
+                for (int j = lane; j < k; j += 32) {
+                    if ((long long)at + j < cap) piece[at + j] = make_int2(d == 0 ? u : ~u, la + j * kCcPiece);
+                    else atomicExch(err, SCC_ERR_INTERNAL);  // cannot happen: a piece is more than 32 arcs of its row
                 }
             }
+            __syncwarp();
         }
     }
-    for (int d = 16; d >= 1; d >>= 1) c += __shfl_xor_sync(kFull, c, d);
-    if (lane == 0 && c) atomicAdd(cross, c);
+    cc_add(joined, c);
+    __syncthreads();
+    cc_add(trees, nt);
+}
+__global__ void __launch_bounds__(kBlk) k_cc_big(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                 const int32_t* __restrict__ toff, const int32_t* __restrict__ tadj,
+                                                 int32_t* parent, unsigned long long* joined,
+                                                 const int2* __restrict__ piece, const unsigned long long* npiece,
+                                                 long long cap, int* err) {
+    const int lane = lane_id();
+    const long long np = min((long long)*npiece, cap);
+    unsigned long long c = 0;
+    for (long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < np;
+         k += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const int2 q = piece[k];
+        const int32_t u = q.x < 0 ? ~q.x : q.x;
+        const int end = q.x < 0 ? toff[u + 1] : off[u + 1];
+        const int b = end - q.y > kCcPiece ? q.y + kCcPiece : end;
+        c += cc_row(q.x < 0 ? tadj : adj, q.y + lane, b, 32, u, parent, err);
+    }
+    cc_add(joined, c);
 }
 
-// root[v] = the root of v's centre; mn[root] = min over its vertices.
-__global__ void k_uf_roots(int32_t n, const int32_t* __restrict__ center, int32_t* parent, int32_t* root, int32_t* mn,
-                           int* err) {
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        const int32_t c = center[v];
-        if ((uint32_t)c >= (uint32_t)n) {  // every vertex has a centre after the decomposition
-            atomicCAS(err, 0, SCC_ERR_INTERNAL);
-            root[v] = (int32_t)v;
-            continue;
-        }
-        const int32_t r = uf_find(parent, c, err);
-        root[v] = r;
-        // a read first: once a component's minimum is in place (threads take
-        // vertices in increasing order) its other vertices skip the atomic
-        if ((int32_t)v < ld_volatile(&mn[r])) atomicMin(&mn[r], (int32_t)v);
-    }
-}
-__global__ void k_uf_labels(int32_t n, const int32_t* __restrict__ root, const int32_t* __restrict__ mn, int32_t* out,
-                            unsigned long long* comps) {
+__global__ void __launch_bounds__(kBlk) k_cc_labels(int32_t n, const int32_t* parent, int32_t* out,
+                                                    unsigned long long* comps) {
     unsigned long long c = 0;
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        const int32_t l = mn[root[v]];
-        out[v] = l;
-        c += l == (int32_t)v;
+        const int32_t r = uf_root(parent, (int32_t)v);
+        out[v] = r;
+        c += r == (int32_t)v;
     }
-    for (int d = 16; d >= 1; d >>= 1) c += __shfl_xor_sync(kFull, c, d);
-    if (lane_id() == 0 && c) atomicAdd(comps, c);
+    cc_add(comps, c);
 }
 __global__ void k_iota(int32_t n, int32_t* a) {
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
         a[v] = (int32_t)v;
 }
-// centres: vertices with center[v] == v
-__global__ void k_count_centres(int32_t n, const int32_t* __restrict__ center, unsigned long long* cnt) {
-    unsigned long long c = 0;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x)
-        c += center[v] == (int32_t)v;
-    for (int d = 16; d >= 1; d >>= 1) c += __shfl_xor_sync(kFull, c, d);
-    if (lane_id() == 0 && c) atomicAdd(cnt, c);
-}
-
 }  // namespace
 
 int launch_sym_csr(const int32_t* off, const int32_t* adj, const int32_t* toff, const int32_t* tadj, int32_t n,
@@ -332,39 +382,50 @@ int launch_iota(int32_t n, int32_t* a, int num_sms, cudaStream_t s) {
     return SCC_OK;
 }
 
-int launch_ldd_setup(const int32_t* order, long long first, int32_t n, int32_t* center, uint32_t* bits, int num_sms,
-                     cudaStream_t s) {
-    k_ldd_init<<<grid_for(n, kBlk * 4, num_sms * 16), kBlk, 0, s>>>(n, center, bits);
-    SCC_LAUNCH();
-    k_ldd_first<<<grid_for(first, kBlk, num_sms * 16), kBlk, 0, s>>>(order, first, center, bits);
-    SCC_LAUNCH();
-    return SCC_OK;
-}
+size_t cc_sample_size(int64_t n) { return (size_t)n * kCcSample; }
+int64_t cc_piece_cap(int64_t mt) { return 2 * (mt / (kCcRow + 1)) + 2; }
 
-int launch_cc_union_label(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* center, int32_t* parent,
-                          int32_t* root, int32_t* mn, int32_t* out, unsigned long long* counters, int32_t* big,
-                          int32_t* bdeg, int32_t* bpre, void* scan_tmp, long long big_cap, int* err, int num_sms,
-                          cudaStream_t s, cudaEvent_t* ev) {
-    const int g = grid_for(n, kBlk * 4, num_sms * 16);
-    k_uf_init<<<g, kBlk, 0, s>>>(n, parent, mn);
-    SCC_LAUNCH();
-    SCC_CUDA(cudaMemsetAsync(bdeg, 0, sizeof(int32_t) * (size_t)big_cap, s));
+int launch_cc(const int32_t* off, const int32_t* adj, const int32_t* toff, const int32_t* tadj, int32_t n,
+              int32_t* sample, int32_t* parent, int32_t* out, unsigned long long* counters, int32_t* giant, void* piece,
+              long long piece_cap, int* err, int num_sms, cudaStream_t s, cudaEvent_t* ev) {
+    const int g = grid_for(n, kBlk, num_sms * 32);
+    const int gf = grid_for(n, 4 * kBlk, INT_MAX);
     if (ev) cudaEventRecord(ev[0], s);
-    k_uf_arcs<<<grid_for(n, kBlk * 4, num_sms * 16), kBlk, 0, s>>>(off, adj, n, center, parent, &counters[0], big, bdeg,
-                                                                   &counters[3], big_cap, err);
+    k_cc_seed<<<g, kBlk, 0, s>>>(off, adj, toff, tadj, n, sample, parent);
     SCC_LAUNCH();
-    SCC_TRY(launch_scan(bdeg, bpre, big_cap, scan_tmp, s));  // the listed rows' places in the flat range
-    k_uf_flat<<<num_sms * 8, kBlk, 0, s>>>(off, adj, center, parent, &counters[0], big, &counters[3], big_cap, bpre, n,
-                                           err);
+    k_cc_flat<<<gf, kBlk, 0, s>>>(n, parent, nullptr);
+    SCC_LAUNCH();
+    k_cc_hook<<<g, kBlk, 0, s>>>(sample, n, parent, nullptr, nullptr);
+    SCC_LAUNCH();
+    k_cc_flat<<<gf, kBlk, 0, s>>>(n, parent, nullptr);
+    SCC_LAUNCH();
+    k_cc_giant<<<1, kCcProbe, 0, s>>>(parent, n, giant, nullptr);
+    SCC_LAUNCH();
+    k_cc_hook<<<g, kBlk, 0, s>>>(sample, n, parent, giant, nullptr);
+    SCC_LAUNCH();
+    k_cc_flat<<<gf, kBlk, 0, s>>>(n, parent, nullptr);
+    SCC_LAUNCH();
+    k_cc_giant<<<1, kCcProbe, 0, s>>>(parent, n, giant + 1, nullptr);
+    SCC_LAUNCH();
+    for (int r = 0; r < 2; ++r) {
+        k_cc_hook<<<g, kBlk, 0, s>>>(sample, n, parent, nullptr, giant + 1);
+        SCC_LAUNCH();
+        k_cc_flat<<<gf, kBlk, 0, s>>>(n, parent, giant + 1);
+        SCC_LAUNCH();
+    }
+    k_cc_giant<<<1, kCcProbe, 0, s>>>(parent, n, giant + 2, giant + 1);
     SCC_LAUNCH();
     if (ev) cudaEventRecord(ev[1], s);
-    k_uf_roots<<<g, kBlk, 0, s>>>(n, center, parent, root, mn, err);
+    k_cc_rest<<<g, kBlk, 0, s>>>(off, adj, toff, tadj, n, parent, giant + 2, &counters[0], &counters[1], (int2*)piece, &counters[3],
+                                 piece_cap, err);
     SCC_LAUNCH();
-    k_uf_labels<<<g, kBlk, 0, s>>>(n, root, mn, out, &counters[2]);
-    SCC_LAUNCH();
-    k_count_centres<<<g, kBlk, 0, s>>>(n, center, &counters[1]);
+    k_cc_big<<<num_sms * 8, kBlk, 0, s>>>(off, adj, toff, tadj, parent, &counters[0], (const int2*)piece, &counters[3],
+                                          piece_cap, err);
     SCC_LAUNCH();
     if (ev) cudaEventRecord(ev[2], s);
+    k_cc_labels<<<g, kBlk, 0, s>>>(n, parent, out, &counters[2]);
+    SCC_LAUNCH();
+    if (ev) cudaEventRecord(ev[3], s);
     return SCC_OK;
 }
 

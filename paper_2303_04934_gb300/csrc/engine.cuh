@@ -593,11 +593,6 @@ __device__ bool engine_search(const EngineParams<typename Pol::Item>& P, Pol& po
                         const int v = pol.vertex(P.hub_item[ipar][j]);
                         atomicOr(&fb[v >> 5], 1u << (v & 31));
                     }
-                // sources added by the policy go into this round's bag (the next
-                // round's input, as in a sparse round); they are visited before
-                // the bottom-up below reads the visited words, so it leaves them
-                // alone and its stores of whole words keep their bits
-                if constexpr (Pol::kInject) pol.inject(i, out, st, wid, nwarps, gr, pushed);
                 if (!S::sync(&ctl->bar, &ctl->err)) return false;
                 const long long nw = ((long long)P.n + 31) / 32;
                 // each warp takes 32 consecutive words at a time (one coalesced
@@ -824,10 +819,6 @@ __device__ bool engine_search(const EngineParams<typename Pol::Item>& P, Pol& po
                 if constexpr (Pol::kCountInserts) pol.flush(sc);
             }
             if constexpr (Pol::kCountInserts) pol.flush(sc);
-            // policies that add sources while the search runs (the batches of
-            // the low-diameter decomposition, Alg. 4) push them into this
-            // round's bag: they join the next round's frontier
-            if constexpr (Pol::kInject) pol.inject(i, out, st, wid, nwarps, gr, pushed);
         }
         if (lane == 0 && pushed) atomicAdd((unsigned long long*)&cur.items, pushed);
         if constexpr (Pol::kDense) {
@@ -851,12 +842,7 @@ __device__ bool engine_search(const EngineParams<typename Pol::Item>& P, Pol& po
             why = 1;
             break;
         }
-        if (ld_volatile(&cur.items) == 0 && ld_volatile(&cur.nhub) == 0) {
-            if constexpr (Pol::kInject) {
-                if (pol.more(i)) continue;  // an empty frontier, but batches of sources remain
-            }
-            break;
-        }
+        if (ld_volatile(&cur.items) == 0 && ld_volatile(&cur.nhub) == 0) break;
     }
     // for readers after the launch (the caller inside the launch uses `why`)
     if (S::block() == 0 && threadIdx.x == 0) {
@@ -906,7 +892,6 @@ struct PolSingle {
     static constexpr bool kCtxInQueue = false;
     using Ctx = uint64_t;  // the per-item value an arc test reads
     static constexpr bool kTwoGraphs = false;
-    static constexpr bool kInject = false;
     static constexpr const char* kName = "single-reach";
     uint32_t* bits;
     __device__ __forceinline__ int vertex(Item it) const { return (int)it; }
@@ -938,7 +923,6 @@ struct PolSingleBoth {
     static constexpr bool kCtxInQueue = false;
     using Ctx = uint64_t;  // the per-item value an arc test reads
     static constexpr bool kTwoGraphs = true;
-    static constexpr bool kInject = false;
     static constexpr const char* kName = "single-reach-both";
     static constexpr uint32_t kDir = 1u << 31;
     uint32_t* bits[2];
@@ -1013,7 +997,6 @@ struct PolPair {
     static constexpr bool kCtxInQueue = true;
     using Ctx = uint64_t;  // the per-item value an arc test reads
     static constexpr bool kTwoGraphs = true;
-    static constexpr bool kInject = false;
     static constexpr const char* kName = "multi-reach";
     static constexpr uint64_t kDir = 1ull << 63;
     const int32_t* label;
@@ -1087,7 +1070,6 @@ struct PolMask {
     static constexpr bool kCtxInQueue = false;
     using Ctx = uint64_t;  // the per-item value an arc test reads
     static constexpr bool kTwoGraphs = false;
-    static constexpr bool kInject = false;
     static constexpr const char* kName = "mask-reach";
     unsigned long long* mask;
     bool test_first;  // read the target's mask before the atomic (high-degree graphs)
@@ -1102,68 +1084,6 @@ struct PolMask {
         const unsigned long long old = atomicOr(&mask[w], (unsigned long long)mu);
         child = (Item)w;
         return (mu & ~old) != 0;
-    }
-};
-
-// Low-diameter decomposition (Sec. 5.1, Alg. 4 function LDD) on the symmetric
-// graph: vertex items; an arc (u, w) claims an unvisited w for u's centre
-// (center[w] = center[u] by CAS from -1: Alg. 4 "visit[u] <- true, L(u) <-
-// L(v)"). The centre travels with an item in the local queue; an item read
-// from the bag takes it from center[]. With VGC a round explores up to tau
-// arcs from an item instead of one BFS level (reachability, not BFS order, is
-// what the decomposition needs; Sec. 5.1). At the end of round i the unvisited
-// vertices of batch i + 1 of the seeded order become centres of their own and
-// join the frontier (Alg. 4, F = F' + B_i); the search ends when the frontier
-// is empty and no batch is left.
-struct PolLdd {
-    using Item = uint32_t;
-    static constexpr int kQueue = 256;
-    static constexpr bool kCountInserts = false;
-    static constexpr bool kDense = true;
-    static constexpr bool kCtxInQueue = true;
-    using Ctx = uint64_t;  // the centre of the item's cluster
-    static constexpr bool kTwoGraphs = false;
-    static constexpr bool kInject = true;
-    static constexpr const char* kName = "ldd";
-    int32_t* center;          // -1: not yet claimed
-    uint32_t* bits;           // claimed vertices (bits past n set), for dense rounds
-    const int32_t* off;       // the symmetric CSR's offsets
-    const int32_t* order;     // seeded order of all vertices
-    const long long* bounds;  // batch i = order[bounds[i] .. bounds[i + 1])
-    int nbatches;
-    __device__ __forceinline__ int vertex(Item it) const { return (int)it; }
-    __device__ __forceinline__ uint64_t ctx(Item it) const { return (uint64_t)(uint32_t)ld_volatile(&center[it]); }
-    __device__ __forceinline__ int32_t load_ctx(Item it) const { return ld_volatile(&center[it]); }
-    __device__ __forceinline__ bool seed(Item) const { return true; }  // items are claimed when pushed
-    // a claim is the CAS on the centre; its winner also marks the vertex visited
-    __device__ __forceinline__ bool claim(int w, int32_t c) const {
-        if (ld_volatile(&center[w]) >= 0 || atomicCAS(&center[w], -1, c) != -1) return false;
-        atomicOr(&bits[w >> 5], 1u << (w & 31));
-        return true;
-    }
-    __device__ __forceinline__ bool visit(Item, uint64_t c, int w, Item& child) const {
-        child = (Item)w;
-        return claim(w, (int32_t)(uint32_t)c);
-    }
-    // dense rounds (the graph is symmetric: a vertex's in-arcs are its arcs):
-    // an unvisited vertex with a neighbour in the frontier joins that
-    // neighbour's cluster, whose centre was settled in an earlier round
-    __device__ __forceinline__ void adopt(int v, int u) const { center[v] = ld_volatile(&center[u]); }
-    __device__ __forceinline__ bool more(uint32_t i) const { return (long long)i + 2 < (long long)nbatches; }
-    // warp-collective: the unvisited vertices of batch i + 1 claim themselves
-    // and go into this round's bag (an isolated one is a cluster of its own
-    // with nothing to expand: it is claimed but not pushed)
-    __device__ __forceinline__ void inject(uint32_t i, const BagRef<Item>& out, SegState& st, uint32_t wid,
-                                           uint32_t nwarps, uint32_t round, unsigned long long& pushed) const {
-        if ((long long)i + 1 >= (long long)nbatches) return;
-        const long long p0 = bounds[i + 1], p1 = bounds[i + 2];
-        const int lane = lane_id();
-        for (long long p = p0 + (long long)wid * 32; p < p1; p += (long long)nwarps * 32) {
-            const long long q = p + lane;
-            const int v = q < p1 ? order[q] : -1;
-            const bool push = v >= 0 && claim(v, v) && off[v + 1] > off[v];
-            pushed += bag_push<Item>(out, st, push, (Item)(push ? v : 0), wid, round);
-        }
     }
 };
 

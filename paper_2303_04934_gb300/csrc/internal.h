@@ -406,37 +406,23 @@ int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const
                          int32_t* order_d, int32_t* out, cudaStream_t s);
 inline size_t batch_group_bytes(int64_t n, int64_t m) { return (size_t)(70 * n + 29 * m); }
 
-// Mask reachability on fixed buffers (no allocation, no events).
-// Low-diameter decomposition (Sec. 5.1, Alg. 4) on the symmetric CSR: batch i
-// of the seeded order is order[bounds_d[i] .. bounds_d[i + 1]) (nbatches
-// batches; the first, of `first` vertices, already centres itself in center[]
-// and in the visited bitmap `bits`, whose bits past n are set); on return
-// center[v] is the centre of v's cluster. fbits: two zeroed frontier bitmaps
-// of ceil(n / 32) words (zero again on return); a round whose frontier holds
-// n / frac_inv vertices, or arcs numbering soff_arcs / frac_inv, or more runs
-// bottom-up (frac_inv = 0: never).
-int run_ldd(const int32_t* soff, const int32_t* sadj, int32_t n, long long soff_arcs, const int32_t* order,
-            const long long* bounds_d, long long first, int nbatches, int32_t* center, uint32_t* bits, uint32_t* fbits,
-            int frac_inv, EngineBuf* b, const EngineOpts& o, EngineRun* out, cudaStream_t st);
-// Connectivity steps (cc.cu): the symmetric CSR (soff[v] = off[v] + toff[v],
-// row v = row v of G then row v of G^T); center[] = -1 with the first `first`
-// vertices of order centring themselves; then union-find over the arcs of G
-// joining two clusters and out[v] = the smallest vertex id of v's component
-// (counters[0] += cross arcs, counters[1] += centres, counters[2] += components;
-// err: a bounded union-find loop ran out). launch_iota: a[v] = v. Events ev[0..2]: after the union-find set-up, after the
-// unions, after the labels.
+// The symmetric CSR (cc.cu): soff[v] = off[v] + toff[v], row v = row v of G
+// then row v of G^T. launch_iota: a[v] = v.
 int launch_sym_csr(const int32_t* off, const int32_t* adj, const int32_t* toff, const int32_t* tadj, int32_t n,
                    int32_t* soff, int32_t* sadj, int num_sms, cudaStream_t s);
 int launch_iota(int32_t n, int32_t* a, int num_sms, cudaStream_t s);
-int launch_ldd_setup(const int32_t* order, long long first, int32_t n, int32_t* center, uint32_t* bits, int num_sms,
-                     cudaStream_t s);
-// counters: [0] cross arcs [1] clusters [2] components [3] rows of more than 32
-// arcs (big, bdeg: big_cap >= m / 33 + 1 entries; bpre: big_cap + 1; scan_tmp:
-// scan_tmp_bytes(big_cap))
-int launch_cc_union_label(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* center, int32_t* parent,
-                          int32_t* root, int32_t* mn, int32_t* out, unsigned long long* counters, int32_t* big,
-                          int32_t* bdeg, int32_t* bpre, void* scan_tmp, long long big_cap, int* err, int num_sms,
-                          cudaStream_t s, cudaEvent_t* ev);
+// Connected components (cc.cu): out[v] = the smallest vertex id of v's component
+// (sample: cc_sample_size(n) entries; parent: n; giant: three; piece:
+// cc_piece_cap(m) of 8 bytes). counters (zeroed): [0] arcs found to join two
+// trees after the sampled passes, [1] trees met on starting with those (the
+// components at least), [2] components, [3] pieces of long rows. err: an error code
+// if a bounded loop ran out. Events ev[0..3]: at the start, after the sample,
+// after the unions, after the labels.
+size_t cc_sample_size(int64_t n);
+int64_t cc_piece_cap(int64_t mt);
+int launch_cc(const int32_t* off, const int32_t* adj, const int32_t* toff, const int32_t* tadj, int32_t n,
+              int32_t* sample, int32_t* parent, int32_t* out, unsigned long long* counters, int32_t* giant, void* piece,
+              long long piece_cap, int* err, int num_sms, cudaStream_t s, cudaEvent_t* ev);
 // Least-element lists (lelists.cu, Sec. 5.2 Alg. 5) of the symmetric CSR for
 // the vertex order `order`: on success res->off (int64[n+1]), res->src and
 // res->dist (int32[total]) are device allocations the caller frees (dfree);
