@@ -323,6 +323,7 @@ static int reach_masks(scc_graph* h, const int32_t* dsrc, int32_t k, int32_t dir
 int reach_multi_wide(scc_graph* h, const int32_t* sources_d, int32_t k, int32_t dir,
                           unsigned long long* mask2, cudaStream_t s) {
     if (!h || !sources_d || !mask2 || k < 1 || k > 128 || (dir != 0 && dir != 1)) return SCC_ERR_INVALID_ARG;
+    if ((uintptr_t)mask2 & 15) return SCC_ERR_INVALID_ARG;  // a vertex's two words are one access
     h->last = s;
     return reach_masks(h, sources_d, k, dir, mask2, 2, s);
 }
@@ -1104,7 +1105,7 @@ int scc_debug_reach_multi_wide(scc_handle h, const int32_t* sources, int32_t k, 
     }
     SCC_TRY(reserve_run_state(h, s));
     SCC_TRY(to_device(h->sources, sources, sizeof(int32_t) * (size_t)k, s));
-    const bool dev_out = is_device_ptr(out);
+    const bool dev_out = is_device_ptr(out) && ((uintptr_t)out & 15) == 0;
     unsigned long long* mask2 = reinterpret_cast<unsigned long long*>(out);
     if (!dev_out) SCC_TRY(dalloc_t(&mask2, 2 * (size_t)std::max(n, 1), s));
     int rc = reach_multi_wide(h, h->sources, k, dir, mask2, s);

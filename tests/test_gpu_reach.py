@@ -83,3 +83,21 @@ def test_hub_first():
     with make_graph(g) as G:
         _check(G, g, src)
         _check(G, g, np.array([n0 + 4], np.int32))
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2])
+def test_wide_masks_at_any_word(shift):
+    """Two-word masks into a device buffer that starts `shift` words after a 16-byte boundary."""
+    import torch
+    g = gg.torus(2, 60, 0.5, seed=9)
+    src = np.random.default_rng(3).integers(0, g.n, 100).astype(np.int32)
+    want = np.zeros(2 * g.n, np.uint64)
+    want[0::2] = oracle.reach_mask(g.n, g.offsets, g.targets, src[:64])
+    want[1::2] = oracle.reach_mask(g.n, g.offsets, g.targets, src[64:])
+    buf = torch.full((2 * g.n + 4,), -1, dtype=torch.int64, device="cuda")
+    with make_graph(g) as G:
+        scc.scc_debug_reach_multi_wide(G.h, src, 100, 0, buf[shift:shift + 2 * g.n])
+        torch.cuda.synchronize()
+    got = buf.cpu().numpy().view(np.uint64)
+    assert np.array_equal(got[shift:shift + 2 * g.n], want)
+    assert (got[:shift] == ~np.uint64(0)).all() and (got[shift + 2 * g.n:] == ~np.uint64(0)).all()
