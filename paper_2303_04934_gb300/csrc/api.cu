@@ -394,9 +394,56 @@ struct ChunkStreams {
     }
 };
 
+// A small graph, in one launch: intake and transposition by one block. *done:
+// false if the graph has self-loops (the general path drops them).
+static int create_small(scc_graph* h, int32_t n, int64_t m, const int32_t* offsets, const int32_t* targets,
+                        cudaStream_t s, bool* done) {
+    EvTimer t(s);
+    t.start();
+    Scratch tmp(s);
+    int* out = nullptr;
+    SCC_TRY(tmp.alloc(&out, 3));
+    SCC_TRY(dalloc_t(&h->off, (size_t)n + 1, s));
+    SCC_TRY(dalloc_t(&h->adj, (size_t)m, s));
+    SCC_TRY(dalloc_t(&h->toff, (size_t)n + 1, s));
+    SCC_TRY(dalloc_t(&h->tadj, (size_t)m, s));
+    const int32_t *off_src = offsets, *adj_src = targets;
+    if (!is_device_ptr(offsets)) {
+        SCC_TRY(to_device(h->off, offsets, sizeof(int32_t) * ((size_t)n + 1), s));
+        off_src = h->off;
+    }
+    if (m > 0 && !is_device_ptr(targets)) {
+        SCC_TRY(to_device(h->adj, targets, sizeof(int32_t) * (size_t)m, s));
+        adj_src = h->adj;
+    }
+    SCC_TRY(launch_small_graph(off_src, adj_src, n, m, h->off, h->adj, h->toff, h->tadj, out, s));
+    int res[3] = {0, 0, 0};
+    SCC_CUDA(cudaMemcpyAsync(res, out, sizeof(res), cudaMemcpyDeviceToHost, s));
+    h->create_ms[0] = t.stop();
+    SCC_CUDA(cudaStreamSynchronize(s));
+    if (res[0]) return SCC_ERR_INVALID_ARG;
+    h->max_out = res[1];
+    h->mt = m;
+    *done = res[2] == 0;
+    if (!*done) {
+        for (int32_t** p : {&h->off, &h->adj, &h->toff, &h->tadj}) {
+            dfree(*p, s);
+            *p = nullptr;
+        }
+    }
+    return SCC_OK;
+}
+
 static int graph_create_impl(scc_graph* h, int32_t n, int64_t m, const int32_t* offsets, const int32_t* targets,
                              cudaStream_t s) {
     SCC_TRY(device_info(&h->di));
+    if (small_graph(n, m)) {
+        h->n = n;
+        h->m_in = m;
+        bool done = false;
+        SCC_TRY(create_small(h, n, m, offsets, targets, s, &done));
+        if (done) return SCC_OK;
+    }
     CreateEvents ce;
     cudaEventRecord(ce.e[0], s);
     h->n = n;
