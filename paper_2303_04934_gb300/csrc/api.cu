@@ -30,7 +30,8 @@ struct scc_graph {
     int32_t* tadj = nullptr;
     scc_config cfg;
     cudaStream_t last = nullptr;
-    // run state (allocated on first use, reused)
+    // run state (parts of one allocation made on first use)
+    void* run_state = nullptr;
     int32_t* label = nullptr;
     int32_t* rep = nullptr;
     int32_t* act = nullptr;
@@ -199,23 +200,36 @@ int reserve_run_state(scc_graph* h, cudaStream_t s) {
     if (h->label) return SCC_OK;
     const int64_t n = h->n;
     const int64_t nw = (n + 31) / 32;
-    SCC_TRY(dalloc_t(&h->label, n, s));
-    SCC_TRY(dalloc_t(&h->rep, n, s));
-    SCC_TRY(dalloc_t(&h->act, n, s));
-    SCC_TRY(dalloc_t(&h->tmp_a, n + 1, s));
-    SCC_TRY(dalloc_t(&h->tmp_b, n + 1, s));
-    SCC_TRY(dalloc(&h->scan_tmp, scan_tmp_bytes(n), s));
-    SCC_TRY(dalloc_t(&h->sources, std::max<int64_t>(n, 128), s));
-    SCC_TRY(dalloc_t(&h->fmax, n, s));
-    SCC_TRY(dalloc_t(&h->bmax, n, s));
-    SCC_TRY(dalloc_t(&h->bits_f, nw, s));
-    SCC_TRY(dalloc_t(&h->bits_b, nw, s));
-    SCC_TRY(dalloc_t(&h->counters, 4, s));
-    SCC_TRY(dalloc_t(&h->flags, 4, s));
-    SCC_TRY(dalloc_t(&h->fbits, 2 * nw, s));
+    // one allocation, cut at 256-byte boundaries: seventeen were 40 us of the
+    // first call on a small graph
+    struct Part {
+        void** p;
+        size_t bytes;
+    } const part[] = {{(void**)&h->label, sizeof(int32_t) * (size_t)n},
+                      {(void**)&h->rep, sizeof(int32_t) * (size_t)n},
+                      {(void**)&h->act, sizeof(int32_t) * (size_t)n},
+                      {(void**)&h->tmp_a, sizeof(int32_t) * ((size_t)n + 1)},
+                      {(void**)&h->tmp_b, sizeof(int32_t) * ((size_t)n + 1)},
+                      {(void**)&h->scan_tmp, scan_tmp_bytes(n)},
+                      {(void**)&h->sources, sizeof(int32_t) * (size_t)std::max<int64_t>(n, 128)},
+                      {(void**)&h->fmax, sizeof(unsigned long long) * (size_t)n},
+                      {(void**)&h->bmax, sizeof(unsigned long long) * (size_t)n},
+                      {(void**)&h->bits_f, sizeof(uint32_t) * (size_t)nw},
+                      {(void**)&h->bits_b, sizeof(uint32_t) * (size_t)nw},
+                      {(void**)&h->counters, 4 * sizeof(unsigned long long)},
+                      {(void**)&h->flags, 4 * sizeof(int)},
+                      {(void**)&h->fbits, 2 * sizeof(uint32_t) * (size_t)nw},
+                      {(void**)&h->prop_dev, prop_dev_bytes()},
+                      {(void**)&h->act_bits, sizeof(uint32_t) * (size_t)nw}};
+    size_t total = 0;
+    for (const Part& x : part) total += (x.bytes + 255) & ~(size_t)255;
+    SCC_TRY(dalloc(&h->run_state, total, s));
+    unsigned char* at = static_cast<unsigned char*>(h->run_state);
+    for (const Part& x : part) {
+        *x.p = at;
+        at += (x.bytes + 255) & ~(size_t)255;
+    }
     SCC_CUDA(cudaMemsetAsync(h->fbits, 0, sizeof(uint32_t) * (size_t)std::max<int64_t>(2 * nw, 1), s));
-    SCC_TRY(dalloc(&h->prop_dev, prop_dev_bytes(), s));
-    SCC_TRY(dalloc_t(&h->act_bits, nw, s));
     return SCC_OK;
 }
 
@@ -611,24 +625,9 @@ static void graph_free(scc_graph* h, cudaStream_t s) {
     dfree(h->adj, s);
     dfree(h->toff, s);
     dfree(h->tadj, s);
-    dfree(h->label, s);
-    dfree(h->rep, s);
-    dfree(h->act, s);
-    dfree(h->tmp_a, s);
-    dfree(h->tmp_b, s);
-    dfree(h->scan_tmp, s);
-    dfree(h->sources, s);
-    dfree(h->fmax, s);
-    dfree(h->bmax, s);
-    dfree(h->bits_f, s);
-    dfree(h->bits_b, s);
-    dfree(h->counters, s);
-    dfree(h->flags, s);
+    dfree(h->run_state, s);
     dfree(h->tab[0], s);
     dfree(h->tab[1], s);
-    dfree(h->fbits, s);
-    dfree(h->prop_dev, s);
-    dfree(h->act_bits, s);
     engine_release(&h->eb32, s);
     engine_release(&h->eb64, s);
     dfree(h->soff, s);
