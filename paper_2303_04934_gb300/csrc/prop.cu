@@ -126,7 +126,7 @@ __device__ int prop_select(const uint32_t* act, long long nw, const unsigned int
 }
 
 // A cooperative grid that also reads graph arrays it wrote itself.
-struct PropScope : GridScope {
+struct PropScope : PropGrid {
     __device__ __forceinline__ static int32_t ld(const int32_t* p) { return *p; }
 };
 
@@ -234,8 +234,9 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
         __syncwarp();
         got = __reduce_add_sync(kFull, got);
         if (lane == 0 && got) atomicAdd(&ctl->merged[part], got);
-        if (!S::sync(&ctl->bar, &ctl->err)) return false;
-        const unsigned long long m = ld_volatile(&ctl->merged[part]);
+        unsigned long long m;
+        if (!S::sync_then(&ctl->bar, &ctl->err, m, [&] { return (unsigned long long)ld_volatile(&ctl->merged[part]); }))
+            return false;
         if (part == 0 && m * kConSample * 5 < active * 2) return true;
         if (part == 1 && !sample && m * 5 < active * 2) return true;
         merged += m;
@@ -275,8 +276,9 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
         got = __reduce_add_sync(kFull, got);
         if (S::block() == 0 && threadIdx.x == 0) ctl->hooked[(r + 1) % 3] = 0;
         if (lane == 0 && got) atomicAdd(&ctl->hooked[r], got);
-        if (!S::sync(&ctl->bar, &ctl->err)) return false;
-        merged = ld_volatile(&ctl->hooked[r]);
+        if (!S::sync_then(&ctl->bar, &ctl->err, merged,
+                          [&] { return (unsigned long long)ld_volatile(&ctl->hooked[r]); }))
+            return false;
         flatten();
         if (!S::sync(&ctl->bar, &ctl->err)) return false;
     }

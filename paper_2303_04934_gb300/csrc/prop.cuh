@@ -483,6 +483,49 @@ __device__ __forceinline__ int prop_pull(const PropGraph<Op>& G, const Op& op, b
     return up;
 }
 
+// The grid, with a barrier that takes one round trip less than grid_sync: the
+// arrivals are tickets of a count that only grows (zero at the launch), so a
+// block need not read a generation before it arrives, and no last arrival has to
+// release the others. What all threads read behind it is read by one thread of
+// each block (f) and handed round, instead of by every warp from one word. Create,
+// run and destroy of a 2D torus 33^2 264 -> 240 us, 256^2 1216 -> 1133, k-NN of 1 M
+// points 1541 -> 1482.
+struct PropGrid : GridScope {
+    template <class F>
+    __device__ __forceinline__ static bool sync_then(GridBarrier* b, int* err, unsigned long long& val, F&& f) {
+        __shared__ unsigned long long s_val;
+        __shared__ int s_ok;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int ok = 1;
+            __threadfence();
+            if (gridDim.x > 1) {
+                unsigned long long* at = reinterpret_cast<unsigned long long*>(b);
+                const unsigned long long end = (atomicAdd(at, 1ull) / gridDim.x + 1) * gridDim.x;
+                const uint64_t t0 = globaltimer_ns();
+                for (int it = 0; ld_volatile(at) < end; ++it) {
+                    if (gridDim.x > 128) __nanosleep(32);  // so many polls get in the way of the arrivals
+                    if ((it & 63) == 63 && globaltimer_ns() - t0 > kBarrierTimeoutNs) {
+                        atomicCAS(err, 0, SCC_ERR_TIMEOUT);
+                        ok = 0;
+                        break;
+                    }
+                }
+                __threadfence();
+            }
+            s_val = f();
+            s_ok = ok;
+        }
+        __syncthreads();
+        val = s_val;
+        return s_ok != 0;
+    }
+    __device__ __forceinline__ static bool sync(GridBarrier* b, int* err) {
+        unsigned long long x;
+        return sync_then(b, err, x, [] { return 0ull; });
+    }
+};
+
 // A warp's idle state within its block, and the block's within the grid.
 template <class S>
 struct PropIdle {
@@ -529,11 +572,14 @@ template <class S>
 __device__ __forceinline__ bool prop_checked(PropCtl* ctl, PropShared& sh, unsigned int check, bool left, bool* more) {
     if (__any_sync(kFull, left) && lane_id() == 0) atomicMax(&ctl->found, check);
     if (S::block() == 0 && threadIdx.x == 0) *(volatile int*)&ctl->idle = 0;  // no block counts itself in between the two barriers
-    if (!S::sync(&ctl->bar, &ctl->err)) return false;
-    *more = ld_volatile(&ctl->found) == check;
-    if (threadIdx.x == 0) sh.idle = sh.exit = 0;
-    __syncthreads();
-    return ld_volatile(&ctl->err) == 0;
+    unsigned long long x;
+    if (!S::sync_then(&ctl->bar, &ctl->err, x, [&] {
+            sh.idle = sh.exit = 0;
+            return (unsigned long long)(uint32_t)ld_volatile(&ctl->err) << 32 | ld_volatile(&ctl->found);
+        }))
+        return false;
+    *more = (uint32_t)x == check;
+    return (x >> 32) == 0;
 }
 
 // A search by pulling alone. With one word per warp a lane keeps its vertex's
@@ -758,10 +804,8 @@ __device__ __forceinline__ bool prop_count(PropCtl* ctl, unsigned int& step, uns
     for (int d = 16; d >= 1; d >>= 1) mine += __shfl_xor_sync(kFull, mine, d);
     if (S::block() == 0 && threadIdx.x == 0) ctl->count[(step + 1) & 3] = 0;
     if (lane_id() == 0 && mine) atomicAdd(&ctl->count[step & 3], mine);
-    if (!S::sync(&ctl->bar, &ctl->err)) return false;
-    sum = ld_volatile(&ctl->count[step & 3]);
-    ++step;
-    return true;
+    const unsigned int at = step++ & 3;
+    return S::sync_then(&ctl->bar, &ctl->err, sum, [&] { return ld_volatile(&ctl->count[at]); });
 }
 
 // The batches from the state in sf/sb/act until every active vertex is

@@ -30,6 +30,20 @@ namespace {
 constexpr int kReachBlock = 256;
 constexpr int kReachWarps = kReachBlock / kWarp;
 
+// The grid with the common barrier: there are four in a call, and with PropGrid's
+// the pulling loop came out 5% slower (2D torus 504^2, 64 sources 3.1 -> 3.3 ms).
+struct ReachScope : GridScope {
+    template <class F>
+    __device__ __forceinline__ static bool sync_then(GridBarrier* b, int* err, unsigned long long& val, F&& f) {
+        __shared__ unsigned long long s_val;
+        if (!grid_sync(b, err)) return false;
+        if (threadIdx.x == 0) s_val = f();
+        __syncthreads();
+        val = s_val;
+        return true;
+    }
+};
+
 template <class Op>
 struct ReachParams {
     PropGraph<Op> G;  // off[0], adj[0]: the direction of the search
@@ -47,7 +61,7 @@ __device__ __forceinline__ PropOr2::Val bit_of(const PropOr2::Val&, int j) {
 
 template <class Op, bool kPull>
 __global__ void __launch_bounds__(kReachBlock, 4) k_reach(const __grid_constant__ ReachParams<Op> P) {
-    using S = GridScope;
+    using S = ReachScope;
     using Val = typename Op::Val;
     __shared__ uint32_t s_q[kReachWarps][kPropQueue];
     __shared__ uint32_t s_mk[kReachWarps][kPropMarks];
