@@ -905,7 +905,11 @@ static int ensure_sym(scc_graph* h, cudaStream_t s) {
         dfree(so, s);
         return SCC_ERR_OOM;
     }
-    const int rc = launch_sym_csr(h->off, h->adj, h->toff, h->tadj, n, so, sa, h->di.num_sms, s);
+    Scratch tmp(s);
+    int2* piece = nullptr;
+    const int64_t cap = sym_piece_cap(h->mt);
+    int rc = tmp.alloc(&piece, (size_t)cap + 1);
+    if (rc == SCC_OK) rc = launch_sym_csr(h->off, h->adj, h->toff, h->tadj, n, so, sa, piece, cap, h->di.num_sms, s);
     if (rc != SCC_OK) {
         dfree(so, s);
         dfree(sa, s);

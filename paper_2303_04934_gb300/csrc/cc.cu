@@ -53,10 +53,25 @@ inline int grid_for(int64_t work, int per_block, int cap) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, cap));
 }
 
-// Row v of the symmetric CSR: G's row, then G^T's (one warp per vertex).
-__global__ void k_sym_rows(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
-                           const int32_t* __restrict__ toff, const int32_t* __restrict__ tadj, int32_t n,
-                           int32_t* __restrict__ soff, int32_t* __restrict__ sadj) {
+// Row v of the symmetric CSR: G's row, then G^T's (one warp per vertex). Rows of
+// more than kSymRow arcs are listed in pieces of so many (v, or ~v for the row of
+// G^T; first arc) and copied by k_sym_big: a hub's row by one warp held the pass
+// up (R-MAT of 262 k vertices, 8 M entries, first LE-lists 1.84 -> 1.63 ms).
+constexpr int kSymRow = 1024;
+__device__ __forceinline__ void sym_copy(const int32_t* __restrict__ src, int32_t* __restrict__ dst, int cnt) {
+    for (int e = lane_id(); e < cnt; e += 128) {
+        int32_t x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = e + 32 * j < cnt ? src[e + 32 * j] : 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (e + 32 * j < cnt) dst[e + 32 * j] = x[j];
+    }
+}
+__global__ void __launch_bounds__(kBlk) k_sym_rows(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                   const int32_t* __restrict__ toff, const int32_t* __restrict__ tadj,
+                                                   int32_t n, int32_t* __restrict__ soff, int32_t* __restrict__ sadj,
+                                                   int2* __restrict__ piece, unsigned int* npiece, unsigned int cap) {
     const int lane = lane_id();
     const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -64,11 +79,36 @@ __global__ void k_sym_rows(const int32_t* __restrict__ off, const int32_t* __res
         const int a0 = off[v], a1 = off[v + 1], b0 = toff[v], b1 = toff[v + 1];
         const long long s0 = (long long)a0 + b0;
         if (lane == 0) soff[v] = (int32_t)s0;
-        for (int e = a0 + lane; e < a1; e += 32) sadj[s0 + (e - a0)] = adj[e];
-        const long long s1 = s0 + (a1 - a0);
-        for (int e = b0 + lane; e < b1; e += 32) sadj[s1 + (e - b0)] = tadj[e];
+        for (int d = 0; d < 2; ++d) {
+            const int lo = d == 0 ? a0 : b0, hi = d == 0 ? a1 : b1;
+            if (hi - lo <= kSymRow) {
+                sym_copy((d == 0 ? adj : tadj) + lo, sadj + (d == 0 ? s0 : s0 + (a1 - a0)), hi - lo);
+                continue;
+            }
+            const int k = (int)(((long long)hi - lo + kSymRow - 1) / kSymRow);
+            unsigned int at = 0;
+            if (lane == 0) at = atomicAdd(npiece, (unsigned int)k);
+            at = __shfl_sync(kFull, at, 0);
+            for (int j = lane; j < k; j += 32)
+                if (at + j < cap) piece[at + j] = make_int2(d == 0 ? (int)v : ~(int)v, lo + j * kSymRow);
+        }
     }
     if (w0 == 0 && lane == 0) soff[n] = off[n] + toff[n];
+}
+__global__ void __launch_bounds__(kBlk) k_sym_big(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                  const int32_t* __restrict__ toff, const int32_t* __restrict__ tadj,
+                                                  int32_t* __restrict__ sadj, const int2* __restrict__ piece,
+                                                  const unsigned int* npiece, unsigned int cap) {
+    const unsigned int np = min(*npiece, cap);
+    const unsigned int nw = (gridDim.x * blockDim.x) >> 5;
+    for (unsigned int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < np; k += nw) {
+        const int2 q = piece[k];
+        const bool t = q.x < 0;
+        const int v = t ? ~q.x : q.x;
+        const int end = t ? toff[v + 1] : off[v + 1];
+        // entry e of a row of G is e + toff[v] in the symmetric CSR, of G^T e + off[v + 1]
+        sym_copy((t ? tadj : adj) + q.y, sadj + ((long long)q.y + (t ? off[v + 1] : toff[v])), min(end - q.y, kSymRow));
+    }
 }
 
 // ------------------------------------------------------------- union-find --
@@ -369,9 +409,16 @@ __global__ void k_iota(int32_t n, int32_t* a) {
 }
 }  // namespace
 
+int64_t sym_piece_cap(int64_t mt) { return 4 * (mt / (kSymRow + 1)) + 2; }
+
 int launch_sym_csr(const int32_t* off, const int32_t* adj, const int32_t* toff, const int32_t* tadj, int32_t n,
-                   int32_t* soff, int32_t* sadj, int num_sms, cudaStream_t s) {
-    k_sym_rows<<<num_sms * 8, kBlk, 0, s>>>(off, adj, toff, tadj, n, soff, sadj);
+                   int32_t* soff, int32_t* sadj, void* piece, int64_t cap, int num_sms, cudaStream_t s) {
+    unsigned int* npiece = reinterpret_cast<unsigned int*>(piece);  // the first entry holds their number
+    int2* const list = reinterpret_cast<int2*>(piece) + 1;
+    SCC_CUDA(cudaMemsetAsync(npiece, 0, sizeof(int2), s));
+    k_sym_rows<<<num_sms * 8, kBlk, 0, s>>>(off, adj, toff, tadj, n, soff, sadj, list, npiece, (unsigned int)cap);
+    SCC_LAUNCH();
+    k_sym_big<<<num_sms * 8, kBlk, 0, s>>>(off, adj, toff, tadj, sadj, list, npiece, (unsigned int)cap);
     SCC_LAUNCH();
     return SCC_OK;
 }

@@ -412,8 +412,9 @@ inline size_t batch_group_bytes(int64_t n, int64_t m) { return (size_t)(70 * n +
 
 // The symmetric CSR (cc.cu): soff[v] = off[v] + toff[v], row v = row v of G
 // then row v of G^T. launch_iota: a[v] = v.
+int64_t sym_piece_cap(int64_t mt);  // piece: this and one entry more, of 8 bytes
 int launch_sym_csr(const int32_t* off, const int32_t* adj, const int32_t* toff, const int32_t* tadj, int32_t n,
-                   int32_t* soff, int32_t* sadj, int num_sms, cudaStream_t s);
+                   int32_t* soff, int32_t* sadj, void* piece, int64_t cap, int num_sms, cudaStream_t s);
 int launch_iota(int32_t n, int32_t* a, int num_sms, cudaStream_t s);
 // Connected components (cc.cu): out[v] = the smallest vertex id of v's component
 // (sample: cc_sample_size(n) entries; parent: n; giant: three; piece:
