@@ -642,18 +642,17 @@ def _extra_graph(name, scc, torch, stream, steps, warmup, cpu):
     if spec["kind"] == "torus" and spec["dims"] == 2:
         out["note"] = "L2-resident (about 1.3 MB of CSR): a bandwidth fraction is not meaningful"
     # the run's algorithmic bytes, counted as for the benchmark graph (8 B per
-    # arc examined, 8 B per item expanded, 16 B per pair inserted, 20 B per
+    # arc examined, 8 B per item expanded or value raised, 20 B per
     # active vertex per labelling), over the run's mean time (create excluded)
     last = sts[-1]
     E = last["engine_arcs"] + last["multi_arcs"]
     P = last["engine_items"] + last["multi_items"]
-    I = last["pairs"]
     act = (g.n - last["n_trimmed"]) + last["multi_active_sum"]
-    run_bytes = 8 * E + 8 * P + 16 * I + 20 * act
+    run_bytes = 8 * E + 8 * P + 20 * act
     run_ms = sum(out["run_ms"].values())
     peak = float(_read_peaks().get("hbm_gbs", 6800.0))
-    out["run_roofline"] = {"bound": "hbm", "bytes_formula": "8 E + 8 P + 16 I + 20 sum(active per labelling)",
-                           "E_arcs": E, "P_items": P, "I_pairs": I, "active_labelled": act,
+    out["run_roofline"] = {"bound": "hbm", "bytes_formula": "8 E + 8 P + 20 sum(active per labelling)",
+                           "E_arcs": E, "P_items": P, "active_labelled": act,
                            "algorithmic_bytes": run_bytes, "run_ms": run_ms,
                            "achieved_gbs": run_bytes / (run_ms / 1e3) / 1e9 if run_ms > 0 else None,
                            "frac": run_bytes / (run_ms / 1e3) / 1e9 / peak if run_ms > 0 else None, "peak": peak,
@@ -1063,9 +1062,8 @@ def main():
     #     arc + 4 B per vertex (row offsets of the tiles);
     #   intake pass (copy + range check + bucket histogram of the targets):
     #     read and write 4 B per arc;
-    #   multi-reachability batch loop: 8 B per arc examined (target + label),
-    #     8 B row offsets per item expanded, 16 B per pair inserted (table
-    #     slot + bag slot).
+    #   signature propagation: 8 B per arc followed (the head's value), 8 B per
+    #     value raised.
     peaks = _read_peaks()
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     peak_src = "measured" if "hbm_gbs" in peaks else "fallback"
@@ -1082,9 +1080,9 @@ def main():
             sum(s["ms_transpose_part"] for s in stats), len(stats), len(stats) * (10 * m + 4 * n)),
         "k_copy_check_hist (intake: copy, range check, bucket histogram)": (
             sum(s["ms_transpose_hist"] for s in stats), len(stats), len(stats) * (8 * m)),
-        "bgss_kernel (multi-reachability batch loop)": (
+        "k_prop (signature propagation)": (
             sum(s["ms_multi_search"] for s in stats), sum(s["multi_launches"] for s in stats),
-            sum(8 * s["multi_arcs"] + 8 * s["multi_items"] + 16 * s["pairs"] for s in stats)),
+            sum(8 * s["multi_arcs"] + 8 * s["multi_items"] for s in stats)),
     }
     kname, (kms, klaunch, kbytes) = max(cands.items(), key=lambda kv: kv[1][0])
     achieved = kbytes / (kms / 1e3) / 1e9 if kms > 0 else 0.0
@@ -1183,18 +1181,16 @@ def main():
     line["split_ms"] = {"create": evs[0].elapsed_time(evs[1]), "run": t_run, "destroy": evs[2].elapsed_time(evs[3])}
     # the whole run's algorithmic bytes (counted from the run's own counters):
     # 4 B target + 4 B label or visited word per arc examined, 8 B row offsets
-    # per item expanded, 16 B per pair inserted (table slot + bag slot), 20 B per
-    # active vertex per labelling (the first SCC's over the untrimmed vertices,
-    # then one per multi-reachability batch); the step adds the transpose
+    # per item expanded or value raised, 20 B per active vertex per labelling
+    # (the first SCC's, over the untrimmed vertices); the step adds the transpose
     # build's 12m + 12n
     E = last["engine_arcs"] + last["multi_arcs"]
     P = last["engine_items"] + last["multi_items"]
-    I = last["pairs"]
     act = (n - last["n_trimmed"]) + last["multi_active_sum"]
-    run_bytes = 8 * E + 8 * P + 16 * I + 20 * act
+    run_bytes = 8 * E + 8 * P + 20 * act
     line["run_roofline"] = {
-        "bound": "hbm", "bytes_formula": "8 E + 8 P + 16 I + 20 sum(active per labelling)",
-        "E_arcs": E, "P_items": P, "I_pairs": I, "active_labelled": act, "algorithmic_bytes": run_bytes,
+        "bound": "hbm", "bytes_formula": "8 E + 8 P + 20 sum(active per labelling)",
+        "E_arcs": E, "P_items": P, "active_labelled": act, "algorithmic_bytes": run_bytes,
         "scc_run_ms": t_run, "achieved_gbs": run_bytes / (t_run / 1e3) / 1e9 if t_run > 0 else None,
         "frac": run_bytes / (t_run / 1e3) / 1e9 / hbm_peak if t_run > 0 else None, "peak": hbm_peak,
         "step_bytes": run_bytes + a1_bytes, "step_ms": ms / args.steps,

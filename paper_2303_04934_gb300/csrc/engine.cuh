@@ -1008,7 +1008,7 @@ struct PolPair {
     __device__ __forceinline__ int vertex(Item it) const { return (int)((it >> 32) & 0x7fffffffu); }
     __device__ __forceinline__ int graph(Item it) const { return (int)(it >> 63); }
     // labels change between the batches of one launch (the labelling passes of
-    // the device-side batch loop), so they are read with coherent loads, never
+    // the batched kernel), so they are read with coherent loads, never
     // through the read-only data path
     __device__ __forceinline__ uint64_t ctx(Item it) const { return (uint64_t)(uint32_t)label[vertex(it)]; }
     __device__ __forceinline__ int32_t load_ctx(Item it) const { return label[vertex(it)]; }

@@ -209,7 +209,6 @@ int launch_class_trim(const int32_t* act, int64_t N, const int32_t* off, const i
 int launch_label_first(const uint32_t* bf, const uint32_t* bb, int32_t n, int32_t s, int32_t* label, int32_t* rep,
                        unsigned long long* ndone, cudaStream_t s_);
 
-// Labelling after a multi-reachability round (Alg. 1; Sec. 4.4).
 // labels_out[v] = min{u : rep[u] == rep[v]} (canonical minimum).
 int launch_canonicalize(const int32_t* rep, int32_t n, int32_t* minid, int32_t* labels_out, int* bad,
                         cudaStream_t s);

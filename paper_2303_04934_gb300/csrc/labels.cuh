@@ -1,6 +1,6 @@
 // Labelling after a forward and a backward multi-reachability search
 // (Alg. 1 label step; Sec. 4.4), as grid-stride device functions of the
-// device-side batch loop.
+// batched kernel.
 //
 // T_out holds pairs (v, s) with s ~> v, T_in pairs (v, s) with v ~> s, both as
 // keys v << 32 | s in open-addressed tables. For every touched vertex v:

@@ -29,9 +29,9 @@
 // before it), or resumes the search.
 //
 // Measured against batches of doubling size whose searches kept every pair (the
-// whole create + run + destroy, GB300): 2D torus 33^2 2.59 -> 0.42 ms, 256^2
-// 11.7 -> 1.31, k-NN of 1 M points 13.9 -> 2.05, 3D torus 256^3 12.8 -> 9.2
-// (41 -> 9.1 when the first pivot misses the giant SCC). Of 9.2 ms the head
+// whole create + run + destroy, GB300): 2D torus 33^2 1.37 -> 0.24 ms, 256^2
+// 11.8 -> 1.15, k-NN of 1 M points 12.2 -> 1.5, 3D torus 256^3 12.8 -> 8.5
+// (41 -> 8.5 when the first pivot misses the giant SCC). Of 8.5 ms the head
 // start takes 4.2: its wave is a few vertices per warp wide, so it is bound by
 // the time of a hop (about 20 us there), not by traffic.
 #pragma once
