@@ -25,7 +25,9 @@
  *
  * Execution: where a group of consecutive graphs (up to 2^24 vertices) holds at
  * least 2^17 vertices in graphs without hubs, those run together as one graph
- * over the whole grid, by signature propagation (scc.h). The others go through
+ * over the whole grid, by signature propagation (scc.h), unless the graphs
+ * without hubs hold more than 2^24 vertices in all and more than 128 times the
+ * largest of them: so many keep the blocks evenly busy. The others go through
  * one persistent kernel; each thread block takes the next graph from a device
  * work queue (largest graphs first) and runs its whole SCC alone, with
  * block-level synchronisation between rounds, then takes the next graph. The

@@ -898,6 +898,17 @@ struct GroupPlan {
 // of working memory would buy little: the blocks' graphs are small.
 constexpr long long kGroupMesh = 1ll << 17;
 
+// The grid takes the groups one after another at 2.4-3.8 ns a vertex; the blocks
+// take all graphs at once at about 1.2, but their span is at least the largest
+// graph's time alone, 0.19 us a vertex. So a batch whose graphs without hubs hold
+// more than kMeshMany times the vertices of the largest of them, and more than a
+// group, goes to the blocks (ms, grid against blocks; graphs, half of them tori,
+// log-uniform from 1 k to the size given): 256 to 1 M (ratio 21) 79 / 193, 1024 to
+// 1 M (74) 224 / 256, 2048 to 300 k (173) 135 / 116, 4096 to 1 M (304) 950 / 550.
+// Within a group's vertices the grid is ahead at any ratio: 1024 to 10 k (2 M
+// vertices) 5.3 / 14, to 100 k (11 M) 26 / 45.
+constexpr long long kMeshMany = 128;
+
 // Groups of consecutive graphs (host only): greedily, as many consecutive
 // graphs as fit in max_v vertices and max_a arcs; a graph larger than either
 // limit ends the current group and belongs to none (its block builds its
@@ -935,6 +946,14 @@ void plan_groups(int G, const long long* vb, const long long* eb, long long max_
 void plan_mesh(const long long* vb, const long long* eb, const unsigned char* hub, int G,
                std::vector<GroupPlan>& groups, std::vector<unsigned char>& mesh) {
     mesh.assign((size_t)G + 1, 0);
+    long long all = 0, most = 0;
+    for (const GroupPlan& gr : groups)
+        for (int g = gr.g0; g < gr.g1; ++g)
+            if (!hub[g]) {
+                all += vb[g + 1] - vb[g];
+                most = std::max(most, vb[g + 1] - vb[g]);
+            }
+    const bool many = all > kGroupVerts && all > kMeshMany * most;
     for (GroupPlan& gr : groups) {
         long long v = 0, a = 0;
         for (int g = gr.g0; g < gr.g1; ++g)
@@ -942,7 +961,7 @@ void plan_mesh(const long long* vb, const long long* eb, const unsigned char* hu
                 v += vb[g + 1] - vb[g];
                 a += eb[g + 1] - eb[g];
             }
-        gr.mesh_arcs = v >= kGroupMesh ? a : -1;
+        gr.mesh_arcs = v >= kGroupMesh && !many ? a : -1;
         gr.blocks = gr.mesh_arcs < 0;
         for (int g = gr.g0; g < gr.g1 && gr.mesh_arcs >= 0; ++g) {
             mesh[g] = hub[g] == 0;

@@ -77,3 +77,15 @@ def test_served_unit(malformed):
             assert np.array_equal(out[:g.n], oracle.scc_labels(g.n, g.offsets, g.targets)[0]), g.name
         if bad is not None:
             assert srv.wait(bad)[0] == scc.SCC_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("copies", [1000, 1040])
+def test_many_equal_graphs(copies):
+    """Tori of 128^2 on either side of 2^24 vertices together, where the blocks take them over from the grid."""
+    import torch
+    g = gg.torus(2, 128, 0.5, seed=2300)
+    p = gg.pack([g] * copies)
+    with scc.SccBatch(p) as B:
+        lab = B.labels().reshape(copies, g.n)
+        assert torch.equal(lab, lab[:1].expand(copies, -1))
+        assert np.array_equal(lab[0].cpu().numpy(), oracle.scc_labels(g.n, g.offsets, g.targets)[0])
