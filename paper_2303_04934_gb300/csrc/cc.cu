@@ -344,14 +344,21 @@ __global__ void __launch_bounds__(kBlk) k_cc_rest(const int32_t* __restrict__ of
         const bool live = v < n && (gt < 0 || pv != gt);
         nt += pv == (int32_t)v;
         if (!__any_sync(kFull, live)) continue;
-        for (int d = 0; d < (gt < 0 ? 1 : 2); ++d) {
-            const int32_t* o = d == 0 ? off : toff;
-            const int32_t* aj = d == 0 ? adj : tadj;
-            int a = 0, b = 0;
-            if (live) {
-                a = o[v];
-                b = o[v + 1];
+        // both rows' ends at once: most of these vertices have no arcs
+        int lo[2] = {0, 0}, hi[2] = {0, 0};
+        if (live) {
+            lo[0] = off[v];
+            hi[0] = off[v + 1];
+            if (gt >= 0) {
+                lo[1] = toff[v];
+                hi[1] = toff[v + 1];
             }
+        }
+        if (!__any_sync(kFull, lo[0] < hi[0] || lo[1] < hi[1])) continue;
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            const int32_t* aj = d == 0 ? adj : tadj;
+            const int a = lo[d], b = hi[d];
             const bool big = b - a > kCcRow;
             if (!big && a < b) c += cc_row(aj, a, b, 1, (int32_t)v, parent, err);
             for (uint32_t m = __ballot_sync(kFull, big); m; m &= m - 1) {
