@@ -107,6 +107,15 @@ SCC_API int scc_debug_pair_table(const uint64_t* keys, int64_t count, int64_t in
 SCC_API int64_t scc_debug_launch_count(void);
 
 /*
+ * The loop by which a warp (or a thread: lanes = 1) walks the arcs [beg, end) of
+ * a row, four a lane and step (host only, no device work): what lane `lane` of
+ * `lanes` (1 to 32) visits. *steps receives the steps taken, *places the arcs
+ * visited, *first and *last the first and the last of them (-1: none).
+ */
+SCC_API int scc_debug_row_steps(int32_t beg, int32_t end, int32_t lane, int32_t lanes, int64_t* steps,
+                                int64_t* places, int64_t* first, int64_t* last);
+
+/*
  * The failure path of the grid barrier that separates the rounds of every
  * cooperative search (the bounded device wait behind SCC_ERR_TIMEOUT; the paper
  * has no counterpart). One cooperative launch of two blocks per SM meets at one

@@ -1235,6 +1235,25 @@ int scc_debug_multi_reach(scc_handle h, const int32_t* labels, const int32_t* so
 
 int64_t scc_debug_launch_count(void) { return launch_count(); }
 
+int scc_debug_row_steps(int32_t beg, int32_t end, int32_t lane, int32_t lanes, int64_t* steps, int64_t* places,
+                        int64_t* first, int64_t* last) {
+    if (beg < 0 || end < beg || lanes < 1 || lanes > 32 || lane < 0 || lane >= lanes || !steps || !places || !first ||
+        !last)
+        return SCC_ERR_INVALID_ARG;
+    *steps = *places = 0;
+    *first = *last = -1;
+    row_steps<4>(beg, end, (uint32_t)lane, (uint32_t)lanes, [&](const uint32_t (&x)[4]) {
+        ++*steps;
+        for (uint32_t at : x)
+            if (at != kNoArc) {
+                if (*first < 0) *first = at;
+                *last = at;
+                ++*places;
+            }
+    });
+    return SCC_OK;
+}
+
 int scc_debug_barrier_timeout(int32_t absent_block, int64_t limit_ns, int32_t* n_arrived, void* stream) {
     if (!n_arrived || limit_ns < 1000 || limit_ns > 1000000000ll || absent_block < -1) return SCC_ERR_INVALID_ARG;
     int c = 0;

@@ -147,6 +147,26 @@ struct Feistel {
     }
 };
 
+// ------------------------------------------------------------------ rows --
+// The arcs [beg, end) of a row, U of each of `lanes` lanes at a time: f(x) gets
+// the lane's U places of a step, kNoArc past the end; every lane takes the same
+// steps. Places are unsigned: a row may end at 2^31 - 1 (the largest arc count a
+// graph may have), and as an int the place after its last step would wrap to a
+// negative one below the end.
+constexpr uint32_t kNoArc = 0xffffffffu;
+template <int U, class F>
+__host__ __device__ __forceinline__ void row_steps(int32_t beg, int32_t end, uint32_t lane, uint32_t lanes, F&& f) {
+    for (uint32_t e = (uint32_t)beg; e < (uint32_t)end; e += lanes * U) {
+        uint32_t x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t at = e + lanes * u + lane;
+            x[u] = at < (uint32_t)end ? at : kNoArc;
+        }
+        f(x);
+    }
+}
+
 // ------------------------------------------------------------ misc helpers --
 __host__ __device__ __forceinline__ int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 

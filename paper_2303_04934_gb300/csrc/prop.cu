@@ -201,8 +201,8 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
     *done = false;
     // f(v, u) for the mutual arcs of v to smaller vertices
     auto mutual = [&](int v, auto&& f) {
-        const int o0 = G.off[0][v], o1 = min(G.end[0][v], o0 + kConRow);
-        const int i0 = G.off[1][v], i1 = min(G.end[1][v], i0 + kConRow);
+        const int o0 = G.off[0][v], o1 = o0 + min(G.end[0][v] - o0, kConRow);
+        const int i0 = G.off[1][v], i1 = i0 + min(G.end[1][v] - i0, kConRow);
         for (int e = o0; e < o1; ++e) {
             const int u = G.adj[0][e];
             if (u >= v) continue;
@@ -337,10 +337,10 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
         if (r != v) *(volatile int32_t*)&C.cid[v] = a;
         const int o0 = G.off[0][v], o1 = G.end[0][v];
         int cnt = 0;
-        for (int e = o0; e < o1; e += 4) {
+        row_steps<4>(o0, o1, 0, 1, [&](const uint32_t (&x)[4]) {
             int u[4], b[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) u[k] = e + k < o1 ? G.adj[0][e + k] : -1;
+            for (int k = 0; k < 4; ++k) u[k] = x[k] != kNoArc ? G.adj[0][x[k]] : -1;
 #pragma unroll
             for (int k = 0; k < 4; ++k) b[k] = u[k] >= 0 ? parent[u[k]] : -1;
 #pragma unroll
@@ -351,7 +351,7 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
                     ++cnt;
                     atomicAdd(&C.end[1][b[k]], 1);
                 }
-        }
+        });
         if (cnt) atomicAdd(&C.end[0][a], cnt);
     }
     __syncwarp();
@@ -392,10 +392,10 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
         const int a = ld_volatile(&C.cid[v]);
         if ((unsigned int)a >= n2) continue;
         const int o0 = G.off[0][v], o1 = G.end[0][v];
-        for (int e = o0; e < o1; e += 4) {
+        row_steps<4>(o0, o1, 0, 1, [&](const uint32_t (&x)[4]) {
             int b[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) b[k] = e + k < o1 ? G.adj[0][e + k] : -1;
+            for (int k = 0; k < 4; ++k) b[k] = x[k] != kNoArc ? G.adj[0][x[k]] : -1;
 #pragma unroll
             for (int k = 0; k < 4; ++k) b[k] = b[k] >= 0 ? ld_volatile(&C.cid[b[k]]) : -1;
             int p[4], t[4];
@@ -411,7 +411,7 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
                     C.adj[0][p[k]] = b[k];
                     C.adj[1][t[k]] = a;
                 }
-        }
+        });
     }
     __syncwarp();
     if (!S::sync(&ctl->bar, &ctl->err)) return false;

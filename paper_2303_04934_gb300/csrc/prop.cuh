@@ -390,15 +390,15 @@ __device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op,
         const int bdir = D ? __shfl_sync(kFull, dir, l) : 0;
         const int32_t* ba = bdir ? G.adj[1] : G.adj[0];
         Val* bs = bdir ? G.s[D] : G.s[0];
-        for (int e = b0; e < b1; e += 32 * U) {
+        row_steps<U>(b0, b1, lane, 32, [&](const uint32_t (&x)[U]) {
             int w[U];
             Val t[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) w[u] = e + 32 * u + lane < b1 ? S::ld(&ba[e + 32 * u + lane]) : -1;
+            for (int u = 0; u < U; ++u) w[u] = x[u] != kNoArc ? S::ld(&ba[x[u]]) : -1;
 #pragma unroll
             for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(bs, w[u]) : Op::none();
             raise(w, t, bst, bs, bdir);
-        }
+        });
         if (lane == 0) arcs += (unsigned long long)(b1 - b0);
     }
 }
@@ -459,16 +459,16 @@ __device__ __forceinline__ int prop_pull(const PropGraph<Op>& G, const Op& op, b
             const int b0 = __shfl_sync(kFull, e0[d], l), b1 = b0 + __shfl_sync(kFull, len[d], l);
             const Val own = prop_shfl(s0[d], l);
             Part m = Part{};
-            for (int e = b0 + lane_id(); e < b1; e += 32 * U) {
+            row_steps<U>(b0, b1, lane_id(), 32, [&](const uint32_t (&x)[U]) {
                 int w[U];
                 Val t[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) w[u] = e + 32 * u < b1 ? S::ld(&G.adj[1 - d][e + 32 * u]) : -1;
+                for (int u = 0; u < U; ++u) w[u] = x[u] != kNoArc ? S::ld(&G.adj[1 - d][x[u]]) : -1;
 #pragma unroll
                 for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(G.s[d], w[u]) : Op::none();
 #pragma unroll
                 for (int u = 0; u < U; ++u) m = Op::fold(m, Op::part(own, t[u]));
-            }
+            });
             for (int x = 16; x >= 1; x >>= 1) m = Op::fold(m, prop_shfl_xor(m, x));
             if (lane_id() == l) st[d] = Op::fold(st[d], m);
         }
@@ -786,9 +786,9 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
 template <class S>
 __device__ __forceinline__ bool prop_any_in_class(const int32_t* adj, int o0, int o1, const unsigned long long* s,
                                                   uint32_t lab, int v) {
-    for (int e = o0; e < o1; e += 2) {
+    for (uint32_t e = (uint32_t)o0; e < (uint32_t)o1; e += 2) {  // unsigned as in row_steps
         const int w0 = S::ld(&adj[e]);
-        const int w1 = e + 1 < o1 ? S::ld(&adj[e + 1]) : w0;
+        const int w1 = e + 1 < (uint32_t)o1 ? S::ld(&adj[e + 1]) : w0;
         const uint32_t l0 = (uint32_t)(ld_volatile(&s[w0]) >> 32), l1 = (uint32_t)(ld_volatile(&s[w1]) >> 32);
         if ((l0 == lab && w0 != v) || (l1 == lab && w1 != v)) return true;
     }

@@ -319,8 +319,8 @@ __global__ void k_bits_to_bytes(const uint32_t* __restrict__ bits, const int32_t
 // list, four arcs in flight, early exit at the first arc inside the class.
 __device__ __forceinline__ bool has_class_arc(const int32_t* __restrict__ off, const int32_t* __restrict__ adj,
                                               const int32_t* label, int32_t v, int32_t L) {
-    const int e1 = off[v + 1];
-    for (int e = off[v]; e < e1; e += 4) {
+    const uint32_t e1 = (uint32_t)off[v + 1];
+    for (uint32_t e = (uint32_t)off[v]; e < e1; e += 4) {  // unsigned as in row_steps
         int w[4], lw[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) w[k] = e + k < e1 ? adj[e + k] : -1;

@@ -33,7 +33,7 @@ EXPORTED = [
     "le_lists_run", "le_lists_get", "le_get_stats",
     "scc_graph_info", "scc_debug_csr", "scc_debug_trim", "scc_debug_pivot_order", "scc_debug_single_reach",
     "scc_debug_multi_reach", "scc_debug_reach_multi_wide", "scc_debug_hashbag", "scc_debug_pair_table", "scc_debug_launch_count",
-    "scc_debug_barrier_timeout", "scc_debug_le_lists",
+    "scc_debug_row_steps", "scc_debug_barrier_timeout", "scc_debug_le_lists",
     "scc_batch_config_default", "scc_batch_create", "scc_batch_destroy", "scc_batch_set_config",
     "scc_batch_get_config", "scc_batch_run", "scc_batch_autotune", "scc_batch_get_stats",
     "scc_debug_batch_times", "scc_debug_batch_groups", "scc_debug_serve_admission", "scc_debug_serve_unit",
@@ -172,6 +172,7 @@ def load() -> ctypes.CDLL:
         "scc_debug_hashbag": ([vp, i64, i32, i32, vp, P(i64), P(i32), vp], ctypes.c_int),
         "scc_debug_pair_table": ([vp, i64, i64, vp, P(i64), P(i32), vp], ctypes.c_int),
         "scc_debug_launch_count": ([], ctypes.c_int64),
+        "scc_debug_row_steps": ([i32, i32, i32, i32, P(i64), P(i64), P(i64), P(i64)], ctypes.c_int),
         "scc_debug_barrier_timeout": ([i32, i64, P(i32), vp], ctypes.c_int),
         "scc_debug_le_lists": ([vp, i64, i64, P(i64), vp], ctypes.c_int),
         "scc_batch_config_default": ([P(scc_batch_config)], ctypes.c_int),
@@ -649,6 +650,13 @@ def scc_debug_pair_table(keys, count: int, init_cap: int, out, stream=None):
 
 def scc_debug_launch_count() -> int:
     return int(load().scc_debug_launch_count())
+
+
+def scc_debug_row_steps(beg: int, end: int, lane: int, lanes: int) -> tuple:
+    """(steps, arcs, first, last) of a lane's walk of the arcs [beg, end) of a row (host only)."""
+    out = [ctypes.c_int64() for _ in range(4)]
+    _check(load().scc_debug_row_steps(beg, end, lane, lanes, *[ctypes.byref(x) for x in out]), "scc_debug_row_steps")
+    return tuple(x.value for x in out)
 
 
 def scc_debug_barrier_timeout(absent_block: int, limit_ns: int, stream=None) -> tuple[int, int]:
