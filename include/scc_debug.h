@@ -107,6 +107,15 @@ SCC_API int scc_debug_pair_table(const uint64_t* keys, int64_t count, int64_t in
 SCC_API int64_t scc_debug_launch_count(void);
 
 /*
+ * Which forms of the searches the last scc_run (*run_form) and the last
+ * reach_multi (*reach_form) on h took, as bits (0: marking searches alone, or
+ * none yet): 1 the searches only pulled, 2 the graph was contracted along
+ * mutual arcs, 4 the first batch had a head start, 8 a hub's own two sets came
+ * first. A run whose first SCC is found by a search of its own reports 0.
+ */
+SCC_API int scc_debug_forms(scc_handle h, int32_t* run_form, int32_t* reach_form);
+
+/*
  * The loop by which a warp (or a thread: lanes = 1) walks the arcs [beg, end) of
  * a row, four a lane and step (host only, no device work): what lane `lane` of
  * `lanes` (1 to 32) visits. *steps receives the steps taken, *places the arcs

@@ -23,6 +23,7 @@ struct scc_graph {
     int64_t m_in = 0;      // arcs of the input
     int64_t mt = 0;        // arcs without self-loops (= arcs of G^T)
     int32_t max_out = 0;   // the longest row of the input
+    int32_t max_in = -1;   // the longest row of G^T (found on first use)
     int32_t hub = -1;      // a vertex of large degree both ways (found on first use)
     int32_t* off = nullptr;
     int32_t* adj = nullptr;
@@ -52,6 +53,7 @@ struct scc_graph {
     int64_t tab_alloc[2] = {0, 0};
     EngineBuf eb32, eb64;
     scc_stats stats;
+    int32_t run_form = 0, reach_form = 0;  // kForm* of the last scc_run and reach_multi
     double create_ms[5] = {0, 0, 0, 0, 0};  // total, histogram, partition, rows, split
     // connectivity: the symmetric CSR (built on the first cc_run) and its stats
     int32_t* soff = nullptr;
@@ -315,9 +317,16 @@ static int reach_masks(scc_graph* h, const int32_t* dsrc, int32_t k, int32_t dir
     a.dev = h->prop_dev;
     a.num_sms = h->di.num_sms;
     EngineOpts o = opts_of(h);
-    const bool skewed = prop_skewed((unsigned long long)h->max_out, (unsigned long long)n, (unsigned long long)h->mt);
+    // hubs of either direction: a search reads the rows of both graphs (pulling
+    // those of the one, marking those of the other)
+    bool skewed = prop_skewed((unsigned long long)h->max_out, (unsigned long long)n, (unsigned long long)h->mt);
+    if (!skewed) {
+        if (h->max_in < 0) SCC_TRY(longest_row(h->toff, n, h->counters + 3, h->di.num_sms, &h->max_in, s));
+        skewed = prop_skewed((unsigned long long)h->max_in, (unsigned long long)n, (unsigned long long)h->mt);
+    }
     const bool hubs = o.high_degree && skewed && h->mt >= kHubArcs;
     a.pull = !skewed && prop_pulls(h->mt, h->di.num_sms);
+    h->reach_form = (a.pull ? kFormPull : 0) | (hubs ? kFormHubFirst : 0);
     if (hubs) {
         if (h->hub < 0) SCC_TRY(find_hub(h->off, h->toff, n, h->counters + 3, h->di.num_sms, &h->hub, s));
         SCC_TRY(engine_reserve(&h->eb32, 4, (long long)n + 1024, h->cfg.lambda, h->mt, h->di.num_sms, s));
@@ -731,6 +740,7 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
     scc_stats& st = h->stats;
     memset(&st, 0, sizeof(st));
     st.tau = opts_of(h).tau;
+    h->run_form = 0;
     if (n == 0) return SCC_OK;
     SCC_TRY(reserve_run_state(h, s));
     EngineOpts o = opts_of(h);
@@ -749,6 +759,7 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
         a.out = dst;
         PropResult r;
         SCC_TRY(run_prop(a, &r, s));
+        h->run_form = r.form;
         if (r.status == 0) {
             if (host_out) SCC_CUDA(cudaMemcpyAsync(labels_out, dst, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost, s));
             st.n_trimmed = (int32_t)(n - r.active);
@@ -1234,6 +1245,13 @@ int scc_debug_multi_reach(scc_handle h, const int32_t* labels, const int32_t* so
 }
 
 int64_t scc_debug_launch_count(void) { return launch_count(); }
+
+int scc_debug_forms(scc_handle h, int32_t* run_form, int32_t* reach_form) {
+    if (!h || !run_form || !reach_form) return SCC_ERR_INVALID_ARG;
+    *run_form = h->run_form;
+    *reach_form = h->reach_form;
+    return SCC_OK;
+}
 
 int scc_debug_row_steps(int32_t beg, int32_t end, int32_t lane, int32_t lanes, int64_t* steps, int64_t* places,
                         int64_t* first, int64_t* last) {

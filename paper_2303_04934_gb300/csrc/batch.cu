@@ -970,7 +970,9 @@ void plan_mesh(const long long* vb, const long long* eb, const unsigned char* hu
     }
 }
 
-// A graph of at least 8 arcs a vertex or with a row of at least 16 times the mean.
+// A graph of at least 8 arcs a vertex or with a row (of G, and where the grid is
+// to take it also of G^T: an in-hub's row is read as often) of at least 16 times
+// the mean.
 __device__ __forceinline__ bool graph_has_hubs(long long n, long long m, long long maxdeg) {
     return m >= 8 * n || maxdeg * n >= 16 * max(m, 1ll);
 }
@@ -1468,32 +1470,62 @@ void batch_free(scc_batch* h, cudaStream_t s) {
     dfree(h->labels, s);
 }
 
-// One block per graph: its CSR is well formed (offsets start at 0, do not
-// decrease and end at its arc count; targets in [0, n_g)); *bad set otherwise.
-// hub[g]: graph_has_hubs.
-__global__ void k_batch_validate(int32_t G, const long long* vbase, const long long* ebase, const int32_t* off,
-                                 const int32_t* adj, int* bad, unsigned char* hub) {
-    __shared__ int s_most;
-    for (int g = blockIdx.x; g < G; g += gridDim.x) {
-        const long long n = vbase[g + 1] - vbase[g];
-        const long long m = ebase[g + 1] - ebase[g];
-        const int32_t* o = off + vbase[g] + g;
-        const int32_t* a = adj + ebase[g];
-        if (threadIdx.x == 0) s_most = 0;
-        __syncthreads();
-        if (threadIdx.x == 0 && (o[0] != 0 || (long long)o[n] != m)) atomicExch(bad, 1);
-        int most = 0;
-        for (long long v = threadIdx.x; v < n; v += blockDim.x) {
-            if (o[v] > o[v + 1]) atomicExch(bad, 1);
-            else most = max(most, o[v + 1] - o[v]);
+// The block's graph (n vertices, m arcs): *bad when its CSR is malformed
+// (offsets not starting at 0, decreasing or not ending at m; a target outside
+// [0, n)), *hub: graph_has_hubs, by the longest row of G or, where G has none
+// that long, of G^T (indeg: n zeroed counters). The targets are eight a thread at
+// a time, so that their loads, and the additions that count them, overlap.
+__device__ void block_validate(const int32_t* __restrict__ o, const int32_t* __restrict__ a, long long n, long long m,
+                               int32_t* indeg, bool* bad, bool* hub) {
+    __shared__ int s_bad, s_out, s_in;
+    if (threadIdx.x == 0) {
+        s_bad = (o[0] != 0 || (long long)o[n] != m);
+        s_out = s_in = 0;
+    }
+    __syncthreads();
+    bool b = false;
+    int most = 0;
+    for (long long v = threadIdx.x; v < n; v += blockDim.x) {
+        if (o[v] > o[v + 1]) b = true;
+        else most = max(most, o[v + 1] - o[v]);
+    }
+    most = __reduce_max_sync(kFull, most);
+    if (lane_id() == 0) atomicMax(&s_out, most);
+    __syncthreads();
+    const bool out_hub = graph_has_hubs(n, m, s_out);
+    most = 0;
+    constexpr int U = 8;
+    for (long long e0 = threadIdx.x; e0 < m; e0 += (long long)U * blockDim.x) {
+        int32_t w[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) w[k] = e0 + (long long)k * blockDim.x < m ? a[e0 + (long long)k * blockDim.x] : 0;
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            if (e0 + (long long)k * blockDim.x >= m) continue;
+            if (w[k] < 0 || (long long)w[k] >= n) b = true;
+            else if (!out_hub) most = max(most, atomicAdd(&indeg[w[k]], 1) + 1);
         }
-        most = __reduce_max_sync(kFull, most);
-        if (lane_id() == 0) atomicMax(&s_most, most);
-        __syncthreads();
-        if (threadIdx.x == 0) hub[g] = graph_has_hubs(n, m, s_most);
-        __syncthreads();
-        for (long long e = threadIdx.x; e < m; e += blockDim.x)
-            if (a[e] < 0 || (long long)a[e] >= n) atomicExch(bad, 1);
+    }
+    most = __reduce_max_sync(kFull, most);
+    if (lane_id() == 0 && most) atomicMax(&s_in, most);
+    if (b) s_bad = 1;
+    __syncthreads();
+    *bad = s_bad != 0;
+    *hub = out_hub || graph_has_hubs(n, m, s_in);
+    __syncthreads();
+}
+
+// One block per graph: *bad set if its CSR is malformed; hub[g]: it has hubs.
+__global__ void k_batch_validate(int32_t G, const long long* vbase, const long long* ebase, const int32_t* off,
+                                 const int32_t* adj, int32_t* indeg, int* bad, unsigned char* hub) {
+    for (int g = blockIdx.x; g < G; g += gridDim.x) {
+        bool b, h;
+        block_validate(off + vbase[g] + g, adj + ebase[g], vbase[g + 1] - vbase[g], ebase[g + 1] - ebase[g],
+                       indeg + vbase[g], &b, &h);
+        if (threadIdx.x == 0) {
+            if (b) atomicExch(bad, 1);
+            hub[g] = h;
+        }
     }
 }
 
@@ -1537,8 +1569,10 @@ int batch_create_impl(scc_batch* h, int32_t G, const int64_t* vbase, const int64
     SCC_TRY(tmp.alloc(&hub_d, (size_t)G + 1));
     SCC_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
     if (G > 0) {
+        // the labels' buffer counts the in-arcs for now
+        SCC_CUDA(cudaMemsetAsync(h->labels, 0, sizeof(int32_t) * (size_t)h->nv, s));
         k_batch_validate<<<std::min<int32_t>(G, 65535), 256, 0, s>>>(G, h->vbase, h->ebase, h->offsets, h->targets,
-                                                                     bad, hub_d);
+                                                                     h->labels, bad, hub_d);
         SCC_LAUNCH();
         SCC_CUDA(cudaMemcpyAsync(hub.data(), hub_d, (size_t)G, cudaMemcpyDeviceToHost, s));
     }
@@ -1633,42 +1667,22 @@ void batch_runner_destroy(BatchRunner* r, cudaStream_t s) {
     delete r;
 }
 
-// bad[g] = 1 when graph g of a packed batch is malformed (offsets not starting
-// at 0, decreasing or not ending at m_g; a target outside [0, n_g)), else 0, or
-// 2 if it has hubs.
+// bad[g] = 1 when graph g of a packed batch is malformed, else 2 if it has hubs, else 0.
 __global__ void k_batch_validate_each(int32_t G, const long long* vbase, const long long* ebase, const int32_t* off,
-                                      const int32_t* adj, int* bad) {
+                                      const int32_t* adj, int32_t* indeg, int* bad) {
     for (int g = blockIdx.x; g < G; g += gridDim.x) {
-        const long long n = vbase[g + 1] - vbase[g];
-        const long long m = ebase[g + 1] - ebase[g];
-        const int32_t* o = off + vbase[g] + g;
-        const int32_t* a = adj + ebase[g];
-        __shared__ int s_bad, s_most;
-        if (threadIdx.x == 0) {
-            s_bad = (o[0] != 0 || (long long)o[n] != m);
-            s_most = 0;
-        }
-        __syncthreads();
-        bool b = false;
-        int most = 0;
-        for (long long v = threadIdx.x; v < n; v += blockDim.x) {
-            b |= o[v] > o[v + 1];
-            most = max(most, o[v + 1] - o[v]);
-        }
-        for (long long e = threadIdx.x; e < m; e += blockDim.x) b |= a[e] < 0 || (long long)a[e] >= n;
-        if (b) s_bad = 1;
-        most = __reduce_max_sync(kFull, most);
-        if (lane_id() == 0) atomicMax(&s_most, most);
-        __syncthreads();
-        if (threadIdx.x == 0) bad[g] = s_bad ? 1 : graph_has_hubs(n, m, s_most) ? 2 : 0;
-        __syncthreads();
+        bool b, h;
+        block_validate(off + vbase[g] + g, adj + ebase[g], vbase[g + 1] - vbase[g], ebase[g + 1] - ebase[g],
+                       indeg + vbase[g], &b, &h);
+        if (threadIdx.x == 0) bad[g] = b ? 1 : h ? 2 : 0;
     }
 }
 
-int batch_validate_each(int32_t G, const long long* vbase, const long long* ebase, const int32_t* offsets,
-                        const int32_t* targets, int* bad, cudaStream_t s) {
+int batch_validate_each(int32_t G, long long nv, const long long* vbase, const long long* ebase,
+                        const int32_t* offsets, const int32_t* targets, int32_t* indeg, int* bad, cudaStream_t s) {
     if (G <= 0) return SCC_OK;
-    k_batch_validate_each<<<std::min<int32_t>(G, 65535), 256, 0, s>>>(G, vbase, ebase, offsets, targets, bad);
+    SCC_CUDA(cudaMemsetAsync(indeg, 0, sizeof(int32_t) * (size_t)nv, s));
+    k_batch_validate_each<<<std::min<int32_t>(G, 65535), 256, 0, s>>>(G, vbase, ebase, offsets, targets, indeg, bad);
     SCC_LAUNCH();
     return SCC_OK;
 }

@@ -337,8 +337,11 @@ struct PropArgs {
     int time_words = 0;
 };
 inline size_t prop_con_words(int64_t n) { return (size_t)(8 * n + (n + 31) / 32); }
+// Forms of the searches of a run or of a reach_multi call (scc_debug_forms).
+enum { kFormPull = 1, kFormContracted = 2, kFormHeadStart = 4, kFormHubFirst = 8 };
 struct PropResult {
     int status = 0;
+    int form = 0;         // kFormPull, kFormContracted, kFormHeadStart
     int64_t active = 0;   // untrimmed vertices
     int32_t first = 0;    // vertices in the SCC of the first pivot
     int batches = 0;      // batches that ran searches
@@ -381,6 +384,8 @@ struct ReachArgs {
     int num_sms;
 };
 int run_reach(const ReachArgs& a, cudaStream_t st);
+// The longest row of a CSR (n > 0); tmp: one device word.
+int longest_row(const int32_t* off, int32_t n, unsigned long long* tmp, int num_sms, int32_t* most, cudaStream_t st);
 // A vertex whose smaller degree is the largest (n > 0); tmp: one device word.
 int find_hub(const int32_t* off, const int32_t* toff, int32_t n, unsigned long long* tmp, int num_sms, int32_t* hub,
              cudaStream_t st);
@@ -396,9 +401,10 @@ bool batch_runner_fits(const BatchRunner* r, long long n, long long m);
 size_t batch_runner_bytes(const BatchRunner* r);
 const int* batch_runner_err(const BatchRunner* r);  // device error flag of the last launch
 // bad[g] (device int[G]) = 1 when graph g of a packed batch is malformed, else 2
-// when it has hubs (or 8 arcs a vertex), else 0
-int batch_validate_each(int32_t G, const long long* vbase, const long long* ebase, const int32_t* offsets,
-                        const int32_t* targets, int* bad, cudaStream_t s);
+// when it has hubs in either direction (or 8 arcs a vertex), else 0. indeg: nv
+// words of scratch (nv: the batch's vertices).
+int batch_validate_each(int32_t G, long long nv, const long long* vbase, const long long* ebase,
+                        const int32_t* offsets, const int32_t* targets, int32_t* indeg, int* bad, cudaStream_t s);
 // Enqueues the SCCs of the packed graphs `order` (host, largest first; order_d:
 // device, G entries). hub (host, per graph; null: a graph is malformed and every
 // other one gets a block): graphs without hubs may run together over the

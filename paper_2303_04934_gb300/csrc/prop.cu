@@ -555,9 +555,10 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
         op.k0 = P.k0;
         prop_node_state<S>(N, op, C);
         if (!S::sync(&ctl->bar, &ctl->err)) return;
-        if (!(arcs2 <= kPropPullArcs * threads && arcs2 <= kConPullRow * (unsigned long long)N.n
-                  ? prop_batches<S, true>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)
-                  : prop_batches<S, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)))
+        const bool pull2 = arcs2 <= kPropPullArcs * threads && arcs2 <= kConPullRow * (unsigned long long)N.n;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = kFormContracted | (pull2 ? kFormPull : 0);
+        if (!(pull2 ? prop_batches<S, true>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)
+                    : prop_batches<S, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)))
             return;
         const PropSlice Q = prop_slice<S>(N.n);
         for (long long i = 0; i < Q.cnt; ++i) {
@@ -596,6 +597,7 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
         prop_times(P, t0);
         return;
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = pull ? kFormPull : head_ns ? kFormHeadStart : 0;
     if (!(pull ? prop_batches<S, true>(G, op, ctl, sh, q, mk, active, 0)
                : prop_batches<S, false>(G, op, ctl, sh, q, mk, active, head_ns)))
         return;
@@ -720,6 +722,7 @@ int run_prop(const PropArgs& a, PropResult* res, cudaStream_t st) {
     SCC_CUDA(cudaStreamSynchronize(st));
     if (c.err) return c.err;
     res->status = c.status;
+    res->form = c.form;
     res->active = (int64_t)c.active0;
     res->first = (int32_t)c.first;
     res->batches = c.batches;

@@ -84,6 +84,7 @@ struct PropCtl {
     unsigned int arcs2[2];     // arcs of the contracted graph and of its transpose
     int status;  // 0 finished, 1 a skewed graph (nothing done but the first trim)
     unsigned int first;  // vertices in the first pivot's SCC
+    int form;            // kForm* taken
 };
 
 struct PropShared {

@@ -124,6 +124,14 @@ __global__ void k_hub(const int32_t* __restrict__ off, const int32_t* __restrict
     if (lane_id() == 0 && b > ld_volatile(best)) atomicMax(best, b);
 }
 
+__global__ void k_longest_row(const int32_t* __restrict__ off, int32_t n, unsigned long long* best) {
+    unsigned long long b = 0;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+        b = max(b, (unsigned long long)(off[v + 1] - off[v]));
+    for (int d = 16; d >= 1; d >>= 1) b = max(b, __shfl_xor_sync(kFull, b, d));
+    if (lane_id() == 0 && b > ld_volatile(best)) atomicMax(best, b);
+}
+
 template <class Op>
 int launch_reach(const ReachArgs& a, cudaStream_t st) {
     ReachParams<Op> P;
@@ -171,16 +179,26 @@ int run_reach(const ReachArgs& a, cudaStream_t st) {
     return a.words == 1 ? launch_reach<PropOr>(a, st) : launch_reach<PropOr2>(a, st);
 }
 
-int find_hub(const int32_t* off, const int32_t* toff, int32_t n, unsigned long long* tmp, int num_sms, int32_t* hub,
-             cudaStream_t st) {
+// One device word, cleared, filled by `launch` and read back.
+template <class F>
+static int word_of(unsigned long long* tmp, int32_t* out, cudaStream_t st, F&& launch) {
     SCC_CUDA(cudaMemsetAsync(tmp, 0, sizeof(unsigned long long), st));
-    k_hub<<<num_sms * 4, 256, 0, st>>>(off, toff, n, tmp);
+    launch();
     SCC_LAUNCH();
     unsigned long long b = 0;
     SCC_CUDA(cudaMemcpyAsync(&b, tmp, sizeof(b), cudaMemcpyDeviceToHost, st));
     SCC_CUDA(cudaStreamSynchronize(st));
-    *hub = (int32_t)(uint32_t)b;
+    *out = (int32_t)(uint32_t)b;
     return SCC_OK;
+}
+
+int longest_row(const int32_t* off, int32_t n, unsigned long long* tmp, int num_sms, int32_t* most, cudaStream_t st) {
+    return word_of(tmp, most, st, [&] { k_longest_row<<<num_sms * 4, 256, 0, st>>>(off, n, tmp); });
+}
+
+int find_hub(const int32_t* off, const int32_t* toff, int32_t n, unsigned long long* tmp, int num_sms, int32_t* hub,
+             cudaStream_t st) {
+    return word_of(tmp, hub, st, [&] { k_hub<<<num_sms * 4, 256, 0, st>>>(off, toff, n, tmp); });
 }
 
 }  // namespace scc

@@ -430,7 +430,7 @@ void run_batched(scc_server* S, std::vector<ReqPtr>& u) {
             rc = cuda_err(cudaMemcpyAsync(adj_d + eb[g], sa, 4 * (size_t)r.m, cudaMemcpyDefault, S->cs));
     }
     // malformed graphs are left out of the launch (and fail on their own)
-    if (rc == SCC_OK) rc = batch_validate_each(G, vb_d, eb_d, off_d, adj_d, bad_d, S->cs);
+    if (rc == SCC_OK) rc = batch_validate_each(G, vb[G], vb_d, eb_d, off_d, adj_d, lab_d, bad_d, S->cs);
     if (rc == SCC_OK) rc = cuda_err(cudaMemcpyAsync(bad.data(), bad_d, sizeof(int) * G, cudaMemcpyDeviceToHost, S->cs));
     if (rc == SCC_OK) rc = cuda_err(cudaStreamSynchronize(S->cs));
     std::vector<int32_t> order;
