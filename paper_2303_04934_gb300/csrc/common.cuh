@@ -150,7 +150,7 @@ struct Feistel {
 // ------------------------------------------------------------------ rows --
 // The arcs [beg, end) of a row, U of each of `lanes` lanes at a time: f(x) gets
 // the lane's U places of a step, kNoArc past the end; every lane takes the same
-// steps. Places are unsigned: a row may end at 2^31 - 1 (the largest arc count a
+// steps, until f returns false if it returns a bool. Places are unsigned: a row may end at 2^31 - 1 (the largest arc count a
 // graph may have), and as an int the place after its last step would wrap to a
 // negative one below the end.
 constexpr uint32_t kNoArc = 0xffffffffu;
@@ -163,7 +163,11 @@ __host__ __device__ __forceinline__ void row_steps(int32_t beg, int32_t end, uin
             const uint32_t at = e + lanes * u + lane;
             x[u] = at < (uint32_t)end ? at : kNoArc;
         }
-        f(x);
+        if constexpr (std::is_same_v<decltype(f(x)), bool>) {
+            if (!f(x)) return;
+        } else {
+            f(x);
+        }
     }
 }
 

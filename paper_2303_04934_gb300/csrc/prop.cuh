@@ -783,17 +783,26 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
     }
 }
 
-// Whether a vertex w != v of v's class is in v's row.
-template <class S>
+// Whether a vertex w != v of v's class (lab) is in v's row [o0, o1): by one thread
+// (lanes = 1), or by the warp, all of whose lanes call.
+template <class S, int kLanes>
 __device__ __forceinline__ bool prop_any_in_class(const int32_t* adj, int o0, int o1, const unsigned long long* s,
                                                   uint32_t lab, int v) {
-    for (uint32_t e = (uint32_t)o0; e < (uint32_t)o1; e += 2) {  // unsigned as in row_steps
-        const int w0 = S::ld(&adj[e]);
-        const int w1 = e + 1 < (uint32_t)o1 ? S::ld(&adj[e + 1]) : w0;
-        const uint32_t l0 = (uint32_t)(ld_volatile(&s[w0]) >> 32), l1 = (uint32_t)(ld_volatile(&s[w1]) >> 32);
-        if ((l0 == lab && w0 != v) || (l1 == lab && w1 != v)) return true;
-    }
-    return false;
+    constexpr int U = kLanes == 1 ? 2 : kPropUnroll;
+    bool found = false;
+    row_steps<U>(o0, o1, kLanes == 1 ? 0 : lane_id(), kLanes, [&](const uint32_t (&x)[U]) {
+        int w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) w[u] = x[u] != kNoArc ? S::ld(&adj[x[u]]) : v;
+        uint32_t l[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) l[u] = (uint32_t)(ld_volatile(&s[w[u]]) >> 32);
+#pragma unroll
+        for (int u = 0; u < U; ++u) found |= l[u] == lab && w[u] != v;
+        if constexpr (kLanes > 1) found = __any_sync(kFull, found) != 0;
+        return !found;
+    });
+    return found;
 }
 
 // The vertices finished by a counting step, summed over the scope. The counters
@@ -828,13 +837,30 @@ __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const Prop
         for (int pass = 0; pass < kPropTrimPasses; ++pass) {
             unsigned long long cnt = 0;
             prop_for_active(G, P, q, [&](bool has, int v) {
-                if (!has) return;
-                const uint32_t lab = (uint32_t)(ld_volatile(&sf[v]) >> 32);
-                const int o0 = S::ld(&G.off[0][v]), o1 = S::ld(&G.end[0][v]);
-                const int i0 = S::ld(&G.off[1][v]), i1 = S::ld(&G.end[1][v]);
-                if (prop_any_in_class<S>(G.adj[0], o0, o1, sf, lab, v) &&
-                    prop_any_in_class<S>(G.adj[1], i0, i1, sf, lab, v))
-                    return;
+                uint32_t lab = 0;
+                int o0 = 0, o1 = 0, i0 = 0, i1 = 0;
+                if (has) {
+                    lab = (uint32_t)(ld_volatile(&sf[v]) >> 32);
+                    o0 = S::ld(&G.off[0][v]);
+                    o1 = S::ld(&G.end[0][v]);
+                    i0 = S::ld(&G.off[1][v]);
+                    i1 = S::ld(&G.end[1][v]);
+                }
+                const bool big = o1 - o0 > kPropBigRow || i1 - i0 > kPropBigRow;
+                bool stays = has && !big && prop_any_in_class<S, 1>(G.adj[0], o0, o1, sf, lab, v) &&
+                             prop_any_in_class<S, 1>(G.adj[1], i0, i1, sf, lab, v);
+                // long rows by the whole warp: a hub whose neighbours have all
+                // left its class is read to its end
+                for (uint32_t bm = __ballot_sync(kFull, big); bm; bm &= bm - 1) {
+                    const int l = __ffs(bm) - 1, hv = __shfl_sync(kFull, v, l);
+                    const uint32_t hl = __shfl_sync(kFull, lab, l);
+                    const bool in = prop_any_in_class<S, 32>(G.adj[0], __shfl_sync(kFull, o0, l),
+                                                             __shfl_sync(kFull, o1, l), sf, hl, hv) &&
+                                    prop_any_in_class<S, 32>(G.adj[1], __shfl_sync(kFull, i0, l),
+                                                             __shfl_sync(kFull, i1, l), sf, hl, hv);
+                    if (lane == l) stays = in;
+                }
+                if (!has || stays) return;
                 *(volatile unsigned long long*)&sf[v] = prop_pack(kPropDone, 0);
                 *(volatile unsigned long long*)&sb[v] = prop_pack(kPropDone, 0);
                 G.rep[v] = v;
