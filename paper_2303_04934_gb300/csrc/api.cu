@@ -319,11 +319,10 @@ static int reach_masks(scc_graph* h, const int32_t* dsrc, int32_t k, int32_t dir
     EngineOpts o = opts_of(h);
     // hubs of either direction: a search reads the rows of both graphs (pulling
     // those of the one, marking those of the other)
-    bool skewed = prop_skewed((unsigned long long)h->max_out, (unsigned long long)n, (unsigned long long)h->mt);
-    if (!skewed) {
-        if (h->max_in < 0) SCC_TRY(longest_row(h->toff, n, h->counters + 3, h->di.num_sms, &h->max_in, s));
-        skewed = prop_skewed((unsigned long long)h->max_in, (unsigned long long)n, (unsigned long long)h->mt);
-    }
+    if (h->max_in < 0) SCC_TRY(longest_row(h->toff, n, h->counters + 3, h->di.num_sms, &h->max_in, s));
+    const bool skewed = prop_skewed((unsigned long long)std::max(h->max_out, h->max_in), (unsigned long long)n,
+                                    (unsigned long long)h->mt);
+    a.row = dir ? h->max_in : h->max_out;
     const bool hubs = o.high_degree && skewed && h->mt >= kHubArcs;
     a.pull = !skewed && prop_pulls(h->mt, h->di.num_sms);
     h->reach_form = (a.pull ? kFormPull : 0) | (hubs ? kFormHubFirst : 0);

@@ -378,6 +378,7 @@ struct ReachArgs {
     unsigned long long* mask;  // n * words
     uint32_t* dirty;           // ceil(n / 32)
     bool pull = false;         // the search only pulls (prop_pulls)
+    int32_t row = 0;           // the longest row of off (pull: not read)
     const uint32_t* from_hub = nullptr;
     const uint32_t* to_hub = nullptr;
     void* dev;  // prop_dev_bytes()

@@ -360,12 +360,16 @@ __device__ bool prop_contract(const PropGraph<PropMax>& G, const PropCon& C, Pro
     const PropSlice Q = prop_slice<S>((int32_t)n2);
 #pragma unroll 1
     for (int d = 0; d < 2; ++d) {
-        unsigned int sum = 0;
+        unsigned int sum = 0, most = 0;
         for (long long i = 0; i < Q.cnt; ++i) {
             const long long c = Q.word(i) * 32 + lane;
-            if (c < n2) sum += (unsigned int)ld_volatile(&C.end[d][c]);
+            const unsigned int k = c < n2 ? (unsigned int)ld_volatile(&C.end[d][c]) : 0u;
+            sum += k;
+            most = max(most, k);
         }
         sum = __reduce_add_sync(kFull, sum);
+        most = __reduce_max_sync(kFull, most);
+        if (lane == 0 && most > (unsigned int)kPropHub) atomicMax(&ctl->max_row2, most);
         unsigned int at = 0;
         if (lane == 0 && sum) at = atomicAdd(&ctl->arcs2[d], sum);
         at = __shfl_sync(kFull, at, 0);
@@ -487,6 +491,7 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
                     const int32_t l = P.label[v];
                     a = l >= 0;
                     lab = (uint32_t)l;
+                    if (a) mx = max(mx, (unsigned int)max(G.end[0][v] - G.off[0][v], G.end[1][v] - G.off[1][v]));
                 }
                 const unsigned long long st =
                     a ? prop_pack(lab, head_ns ? 0u : op.key((uint32_t)v)) : PropMax::none();
@@ -514,6 +519,10 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
             }
             __syncthreads();
             if (threadIdx.x == 0 && s_n) atomicAdd(&ctl->active0, (unsigned long long)s_n);
+        }
+        if (!P.fresh) {
+            mx = __reduce_max_sync(kFull, mx);
+            if (lane == 0 && mx > (unsigned int)kPropHub) atomicMax(&ctl->max_deg, mx);
         }
         if (!S::sync(&ctl->bar, &ctl->err)) return;
     }
@@ -555,10 +564,16 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
         op.k0 = P.k0;
         prop_node_state<S>(N, op, C);
         if (!S::sync(&ctl->bar, &ctl->err)) return;
-        const bool pull2 = arcs2 <= kPropPullArcs * threads && arcs2 <= kConPullRow * (unsigned long long)N.n;
+        // a node's row is as long as its vertices' rows together
+        const bool hubs = ld_volatile(&ctl->max_row2) > (unsigned int)kPropHub;
+        if (hubs && !prop_list_hubs<S>(N, ctl, P.minid)) return;
+        const unsigned int nhub = hubs ? ld_volatile(&ctl->nhub) : 0u;
+        const bool pull2 =
+            !hubs && arcs2 <= kPropPullArcs * threads && arcs2 <= kConPullRow * (unsigned long long)N.n;
         if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = kFormContracted | (pull2 ? kFormPull : 0);
-        if (!(pull2 ? prop_batches<S, true>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)
-                    : prop_batches<S, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)))
+        if (!(pull2  ? prop_batches<S, true, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0, nullptr, 0)
+              : hubs ? prop_batches<S, false, true>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0, P.minid, nhub)
+                     : prop_batches<S, false, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0, nullptr, 0)))
             return;
         const PropSlice Q = prop_slice<S>(N.n);
         for (long long i = 0; i < Q.cnt; ++i) {
@@ -597,9 +612,14 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
         prop_times(P, t0);
         return;
     }
+    // the rest of a graph with hubs (a fresh one has none: its rows are short)
+    const bool hubs = !P.fresh && ld_volatile(&ctl->max_deg) > (unsigned int)kPropHub;
+    if (hubs && !prop_list_hubs<S>(G, ctl, P.minid)) return;
+    const unsigned int nhub = hubs ? ld_volatile(&ctl->nhub) : 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = pull ? kFormPull : head_ns ? kFormHeadStart : 0;
-    if (!(pull ? prop_batches<S, true>(G, op, ctl, sh, q, mk, active, 0)
-               : prop_batches<S, false>(G, op, ctl, sh, q, mk, active, head_ns)))
+    if (!(pull   ? prop_batches<S, true, false>(G, op, ctl, sh, q, mk, active, 0, nullptr, 0)
+          : hubs ? prop_batches<S, false, true>(G, op, ctl, sh, q, mk, active, 0, P.minid, nhub)
+                 : prop_batches<S, false, false>(G, op, ctl, sh, q, mk, active, head_ns, nullptr, 0)))
         return;
     if (!P.fresh) return;
     // ---- canonical labels: the smallest vertex of each SCC

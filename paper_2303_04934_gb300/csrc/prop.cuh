@@ -45,6 +45,9 @@ constexpr int kPropQueue = 256;    // vertices a warp gathers before it works on
 constexpr int kPropMarks = 384;    // marks a warp gathers before it publishes them
 constexpr int kPropBigRow = 64;    // rows longer than this are relaxed by the whole warp
 constexpr int kPropUnroll = 4;     // arcs of a row in flight per lane
+constexpr int kPropHub = 2048;     // rows longer than this are shared by the idle warps of the grid ...
+constexpr int kPropPiece = 512;    // ... in pieces of this many arcs
+constexpr int kPropTasks = 24;     // rows shared at a time
 constexpr int kPropTrimPasses = 3; // trimming passes at the start of a batch, at most
 constexpr uint64_t kPropIdleTimeoutNs = 20000000000ull;  // an idle block gives up after 20 s (others may work that long)
 
@@ -66,15 +69,29 @@ __host__ __device__ __forceinline__ uint32_t prop_unmix(uint32_t x) {
     return x;
 }
 
+// A long row that the warps share: a warp takes the next piece by one addition
+// to `next`, which holds the number of pieces beside it, so a claim on a slot that
+// has ended, or holds another row by now, is judged by that row's own count.
+struct PropTask {
+    unsigned long long next;  // pieces << 32 | next piece; 0: free
+    unsigned int read;        // claimed pieces whose claimers have read v
+    uint32_t v;               // vertex | direction << 31
+};
+
 struct PropCtl {
     GridBarrier bar;
+    // idle blocks, and the slots of rows with pieces to take: read as one word
+    alignas(8) int idle;
+    unsigned int open;
+    unsigned int taken;       // slots in use
     int err;
-    int idle;                 // idle blocks
+    PropTask task[kPropTasks];
+    unsigned int nhub;        // vertices with a row of more than kPropHub arcs
     unsigned int found;       // last check that found work left
     unsigned long long count[4];  // vertices finished by a counting step, a ring over the steps
     unsigned long long items, arcs;
     unsigned long long active0;  // active vertices after the first trim
-    unsigned int max_deg;
+    unsigned int max_deg, max_row2;  // the longest row: of an active vertex, of the contracted graph
     unsigned long long best;  // smaller degree << 32 | key of the vertex that becomes the largest source
     int batches, searches;
     int pivot;
@@ -90,6 +107,7 @@ struct PropCtl {
 struct PropShared {
     int idle;  // idle warps of the block
     int exit;  // the search is over (or failed)
+    unsigned int open;  // rows that have pieces to take
 };
 
 __device__ __forceinline__ unsigned long long prop_pack(uint32_t lab, uint32_t key) {
@@ -326,10 +344,144 @@ __device__ __forceinline__ void prop_flush(const PropGraph<Op>& G, PropMarks& M)
     __syncwarp();
 }
 
-// Spread v's value along its arcs in direction dir; all lanes of the warp call.
+// Puts the row of c (vertex | direction << 31) up for the warps to share: the
+// slot, or -1 when all are in use. One thread calls.
+template <class S>
+__device__ __forceinline__ int prop_post(PropCtl* ctl, uint32_t c, int len) {
+    constexpr unsigned int kAll = (1u << kPropTasks) - 1;
+    unsigned int t = ld_volatile(&ctl->taken);
+    for (int i = 0; i < kPropTasks && (t & kAll) != kAll; ++i) {
+        const int j = __ffs(~t) - 1;
+        t = atomicOr(&ctl->taken, 1u << j);
+        if ((t >> j) & 1u) continue;
+        PropTask& T = ctl->task[j];
+        // open before there is a piece to claim: whoever takes the last one then
+        // closes the slot for certain (a claim may come from an earlier look)
+        *(volatile uint32_t*)&T.v = c;
+        atomicOr(&ctl->open, 1u << j);
+        S::fence();
+        atomicExch(&T.next, (unsigned long long)((len - 1) / kPropPiece + 1) << 32);
+        return j;
+    }
+    return -1;
+}
+// The next piece of the row in slot j, if any is left: its vertex | direction
+// << 31 in *c. One thread calls. The slot is free once every claimer has read v.
+template <class S>
+__device__ __forceinline__ bool prop_claim(PropCtl* ctl, int j, uint32_t* c, unsigned int* piece) {
+    PropTask& T = ctl->task[j];
+    const unsigned long long x = atomicAdd(&T.next, 1ull);
+    const unsigned int p = (unsigned int)x, pieces = (unsigned int)(x >> 32);
+    if (p >= pieces) return false;
+    S::fence();
+    *c = ld_volatile(&T.v);
+    *piece = p;
+    if (p + 1 == pieces) atomicAnd(&ctl->open, ~(1u << j));
+    S::fence();
+    if (atomicAdd(&T.read, 1u) + 1 == pieces) {
+        *(volatile unsigned int*)&T.read = 0;
+        atomicExch(&T.next, 0ull);
+        S::fence();
+        atomicAnd(&ctl->taken, ~(1u << j));
+    }
+    return true;
+}
+
+// The warp marks the heads it raised among t, whose vertices are w (< 0: none).
 template <class S, class Op>
-__device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op, bool has, int v, int dir, PropMarks& M,
-                                           unsigned long long& arcs) {
+__device__ __forceinline__ void prop_raise(const PropGraph<Op>& G, const int (&w)[kPropUnroll],
+                                           const typename Op::Val (&t)[kPropUnroll], const typename Op::Val& to,
+                                           typename Op::Val* ts, int tdir, PropMarks& M) {
+#pragma unroll
+    for (int u = 0; u < kPropUnroll; ++u) {
+        const bool up = w[u] >= 0 && Op::gains(to, t[u]);
+        if (up) Op::raise(ts, w[u], to);
+        const uint32_t m = __ballot_sync(kFull, up);
+        if (up) M.buf[M.cnt + __popc(m & lanemask_lt())] = (uint32_t)w[u] | ((uint32_t)tdir << 31);
+        M.cnt += __popc(m);
+    }
+    if (M.cnt > kPropMarks - 32 * kPropUnroll) prop_flush<S>(G, M);
+}
+// Arcs [b0, b1) of a row of direction dir, whose vertex holds st, by the warp.
+template <class S, class Op>
+__device__ __forceinline__ void prop_relax_row(const PropGraph<Op>& G, const typename Op::Val& st, int b0, int b1, int dir,
+                                               PropMarks& M) {
+    using Val = typename Op::Val;
+    constexpr int U = kPropUnroll;
+    const int32_t* adj = dir ? G.adj[1] : G.adj[0];
+    Val* s = dir ? G.s[Op::kDirs - 1] : G.s[0];
+    row_steps<U>(b0, b1, lane_id(), 32, [&](const uint32_t (&x)[U]) {
+        int w[U];
+        Val t[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) w[u] = x[u] != kNoArc ? S::ld(&adj[x[u]]) : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(s, w[u]) : Op::none();
+        prop_raise<S>(G, w, t, st, s, dir, M);
+    });
+}
+
+// A hub's row is long: by one warp it takes 9 ns an arc, with all others waiting
+// for what lies behind it. So it is put up in pieces, and idle warps take some: the
+// row of `put` (vertex | direction << 31; kFull: none) first, then those in
+// `slots`. Returns the number of marks in mk. Only searches of graphs that have
+// such rows are compiled with it (kHubs): lattices lost 4-6% to its registers.
+// One call, 64 sources, GB300, by one warp against shared: a star of 1 M two-way
+// arcs 24.3 -> 0.13 ms, 16 stars of 65 k 13.5 -> 0.30; SCC of the 16 stars 49.7 ->
+// 2.0 ms. Bound and piece (there, SCC): 8192 and 2048 2.65 ms, 2048 and 1024 2.17,
+// 2048 and 256 2.02; rows of 1 k are as fast by a warp of their own.
+template <class S, class Op>
+__device__ __noinline__ int prop_share(const PropGraph<Op> G, PropCtl* ctl, uint32_t put, uint32_t slots, uint32_t* mk,
+                                       int cnt) {
+    constexpr int D = Op::kDirs - 1;
+    PropMarks M{mk, cnt};
+    unsigned long long arcs = 0;
+    auto row = [&](uint32_t c, int& b0, int& b1) {
+        const int v = (int)(c & 0x7fffffffu), d = (int)(c >> 31);
+        b0 = S::ld(&(d ? G.off[1] : G.off[0])[v]);
+        b1 = S::ld(&(d ? G.end[1] : G.end[0])[v]);
+    };
+    int whole = 0;  // no slot was free: one piece, the row
+    if (put != kFull) {
+        int b0, b1, j = -1;
+        row(put, b0, b1);
+        if (lane_id() == 0) j = prop_post<S>(ctl, put, b1 - b0);
+        j = __shfl_sync(kFull, j, 0);
+        if (j >= 0) slots = 1u << j;
+        else whole = 1;
+    }
+    for (; slots | whole; slots &= slots - 1) {
+        for (;;) {
+            uint32_t c = put;
+            int b0, b1;
+            if (!whole) {
+                unsigned int piece = 0;
+                bool got = false;
+                if (lane_id() == 0) got = prop_claim<S>(ctl, __ffs(slots) - 1, &c, &piece);
+                if (!__shfl_sync(kFull, (int)got, 0)) break;
+                c = __shfl_sync(kFull, c, 0);
+                piece = __shfl_sync(kFull, piece, 0);
+                row(c, b0, b1);
+                b0 += (int)piece * kPropPiece;
+                if (b1 - b0 > kPropPiece) b1 = b0 + kPropPiece;
+            } else {
+                row(c, b0, b1);
+            }
+            const int d = D ? (int)(c >> 31) : 0;
+            prop_relax_row<S>(G, Op::load(d ? G.s[D] : G.s[0], c & 0x7fffffffu), b0, b1, d, M);
+            arcs += (unsigned long long)(b1 - b0);
+            if (whole) break;
+        }
+        whole = 0;
+    }
+    if (lane_id() == 0 && arcs) atomicAdd(&ctl->arcs, arcs);
+    return M.cnt;
+}
+
+// Spread v's value along its arcs in direction dir; all lanes of the warp call.
+template <class S, bool kHubs, class Op>
+__device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op, PropCtl* ctl, bool has, int v, int dir,
+                                           PropMarks& M, unsigned long long& arcs) {
     using Val = typename Op::Val;
     constexpr int D = Op::kDirs - 1;
     const int lane = lane_id();
@@ -358,17 +510,6 @@ __device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op,
         }
     }
     constexpr int U = kPropUnroll;
-    auto raise = [&](const int (&w)[U], const Val (&t)[U], const Val& to, Val* ts, int tdir) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool up = w[u] >= 0 && Op::gains(to, t[u]);
-            if (up) Op::raise(ts, w[u], to);
-            const uint32_t m = __ballot_sync(kFull, up);
-            if (up) M.buf[M.cnt + __popc(m & lanemask_lt())] = (uint32_t)w[u] | ((uint32_t)tdir << 31);
-            M.cnt += __popc(m);
-        }
-        if (M.cnt > kPropMarks - 32 * U) prop_flush<S>(G, M);
-    };
     const bool big = o1 - o0 > kPropBigRow;
     const int len = big ? 0 : o1 - o0;
     arcs += (unsigned long long)len;
@@ -380,35 +521,30 @@ __device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op,
         for (int u = 0; u < U; ++u) w[u] = k + u < len ? S::ld(&adj[o0 + k + u]) : -1;
 #pragma unroll
         for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(s, w[u]) : Op::none();
-        raise(w, t, st, s, dir);
+        prop_raise<S>(G, w, t, st, s, dir, M);
     }
-    uint32_t bm = __ballot_sync(kFull, big);
-    while (bm) {  // long rows by the whole warp
+    for (uint32_t bm = __ballot_sync(kFull, big); bm; bm &= bm - 1) {  // long rows by the whole warp
         const int l = __ffs(bm) - 1;
-        bm &= bm - 1;
         const Val bst = prop_shfl(st, l);
         const int b0 = __shfl_sync(kFull, o0, l), b1 = __shfl_sync(kFull, o1, l);
         const int bdir = D ? __shfl_sync(kFull, dir, l) : 0;
-        const int32_t* ba = bdir ? G.adj[1] : G.adj[0];
-        Val* bs = bdir ? G.s[D] : G.s[0];
-        row_steps<U>(b0, b1, lane, 32, [&](const uint32_t (&x)[U]) {
-            int w[U];
-            Val t[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) w[u] = x[u] != kNoArc ? S::ld(&ba[x[u]]) : -1;
-#pragma unroll
-            for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? Op::load(bs, w[u]) : Op::none();
-            raise(w, t, bst, bs, bdir);
-        });
+        if constexpr (kHubs)
+            if (b1 - b0 > kPropHub && S::blocks() > 1) {
+                M.cnt = prop_share<S, Op>(G, ctl, (uint32_t)__shfl_sync(kFull, v, l) | ((uint32_t)bdir << 31), 0, M.buf, M.cnt);
+                continue;
+            }
+        prop_relax_row<S>(G, bst, b0, b1, bdir, M);
         if (lane == 0) arcs += (unsigned long long)(b1 - b0);
     }
 }
 
 // One pull of v: its values take what its in-class neighbours (and, with jump,
 // the vertex each names) hold. v's words are written by its owner
-// alone, so there is no atomic. Returns bit d set when direction d grew.
+// alone, so there is no atomic. Returns bit d set when direction d grew. Rows of
+// more than `most_row` arcs are left out.
 template <class S, class Op>
-__device__ __forceinline__ int prop_pull(const PropGraph<Op>& G, const Op& op, bool has, int v, bool jump) {
+__device__ __forceinline__ int prop_pull(const PropGraph<Op>& G, const Op& op, bool has, int v, bool jump,
+                                         int most_row = INT32_MAX) {
     using Val = typename Op::Val;
     constexpr int D = Op::kDirs, U = kPropUnroll;
     using Part = typename Op::Part;
@@ -422,6 +558,7 @@ __device__ __forceinline__ int prop_pull(const PropGraph<Op>& G, const Op& op, b
         const int32_t* off = G.off[1 - d];
         e0[d] = has ? S::ld(&off[v]) : 0;
         len[d] = has ? S::ld(&G.end[1 - d][v]) - e0[d] : 0;
+        if (len[d] > most_row) len[d] = 0;
         s0[d] = has ? Op::load(G.s[d], v) : Op::none();
     }
 #pragma unroll
@@ -528,7 +665,7 @@ struct PropGrid : GridScope {
 };
 
 // A warp's idle state within its block, and the block's within the grid.
-template <class S>
+template <class S, bool kHubs>
 struct PropIdle {
     PropCtl* ctl;
     PropShared& sh;
@@ -542,8 +679,8 @@ struct PropIdle {
             atomicSub(&ctl->idle, 1);
     }
     // after a pass over the warp's words that found nothing: true when the
-    // search is over (or a wait ran out)
-    __device__ __forceinline__ bool rest() {
+    // search is over (or a wait ran out); open: the rows to help with
+    __device__ __forceinline__ bool rest(uint32_t& open) {
         if (!idle) {
             idle = true;
             if (lane_id() == 0) {
@@ -556,7 +693,9 @@ struct PropIdle {
             __syncwarp();
             t0 = globaltimer_ns();
         } else if (threadIdx.x == 0 && S::blocks() > 1) {
-            if (ld_volatile(&ctl->idle) >= S::blocks()) {
+            const unsigned long long x = ld_volatile(reinterpret_cast<unsigned long long*>(&ctl->idle));
+            if (kHubs) *(volatile unsigned int*)&sh.open = (unsigned int)(x >> 32);
+            if ((int)(unsigned int)x >= S::blocks()) {
                 atomicExch(&sh.exit, 1);
             } else if (globaltimer_ns() - t0 > kPropIdleTimeoutNs) {
                 atomicCAS(&ctl->err, 0, SCC_ERR_TIMEOUT);
@@ -564,6 +703,7 @@ struct PropIdle {
             }
         }
         const int ex = lane_id() == 0 ? ld_volatile(&sh.exit) : 0;
+        if (kHubs) open = __shfl_sync(kFull, lane_id() == 0 ? ld_volatile(&sh.open) : 0u, 0);
         return __shfl_sync(kFull, ex, 0) != 0;
     }
 };
@@ -576,6 +716,7 @@ __device__ __forceinline__ bool prop_checked(PropCtl* ctl, PropShared& sh, unsig
     unsigned long long x;
     if (!S::sync_then(&ctl->bar, &ctl->err, x, [&] {
             sh.idle = sh.exit = 0;
+            sh.open = 0;
             return (unsigned long long)(uint32_t)ld_volatile(&ctl->err) << 32 | ld_volatile(&ctl->found);
         }))
         return false;
@@ -595,7 +736,10 @@ __device__ bool prop_search_pull(const PropGraph<Op>& G, const Op op, PropCtl* c
     constexpr int D = Op::kDirs, U = kPropUnroll;
     const PropSlice P = prop_slice<S>(G.n);
     const int lane = lane_id();
-    if (threadIdx.x == 0) sh.idle = sh.exit = 0;
+    if (threadIdx.x == 0) {
+        sh.idle = sh.exit = 0;
+        sh.open = 0;
+    }
     __syncthreads();
     const bool one = P.cnt == 1 && P.word(0) < P.nw;
     const int v = (int)(P.word(0) * 32) + lane;
@@ -671,10 +815,11 @@ __device__ bool prop_search_pull(const PropGraph<Op>& G, const Op op, PropCtl* c
         return __any_sync(kFull, up) != 0;
     };
     for (;;) {
-        PropIdle<S> id(ctl, sh);
+        PropIdle<S, false> id(ctl, sh);
+        uint32_t open;
         for (;;) {
             if (fits ? pass_one() : pass_all(true)) id.wake();
-            else if (id.rest()) break;
+            else if (id.rest(open)) break;
         }
         if (!S::sync(&ctl->bar, &ctl->err)) return false;
         ++check;
@@ -689,7 +834,7 @@ __device__ bool prop_search_pull(const PropGraph<Op>& G, const Op op, PropCtl* c
 // it; `check` numbers the checks of the launch (the same in every block). With
 // a deadline (globaltimer ns; 0: none) it may end early, vertices still dirty.
 // Returns false when a wait ran out (the caller returns at once).
-template <class S, class Op>
+template <class S, bool kHubs, class Op>
 __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
                             unsigned int& check, uint64_t deadline, unsigned long long& items,
                             unsigned long long& arcs) {
@@ -697,13 +842,17 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
     constexpr int D = Op::kDirs;
     const int lane = lane_id();
     const PropSlice P = prop_slice<S>(G.n);
-    if (threadIdx.x == 0) sh.idle = sh.exit = 0;
+    if (threadIdx.x == 0) {
+        sh.idle = sh.exit = 0;
+        sh.open = 0;
+    }
     __syncthreads();
     PropMarks M{mk, 0};
     PropQueue Q{q, 0};
     long long turn = 0;  // the word whose named vertices are looked at next
     for (;;) {
-        PropIdle<S> id(ctl, sh);
+        PropIdle<S, kHubs> id(ctl, sh);
+        uint32_t help = 0;  // rows of others to help with
         for (;;) {
             bool did = prop_gather(
                 P, Q,
@@ -718,7 +867,15 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
                     items += (unsigned long long)(__popc(x) + __popc(y));
                     return __any_sync(kFull, (x | y) != 0) != 0;
                 },
-                [&](bool has, int v, int dir) { prop_relax<S>(G, op, has, v, dir, M, arcs); });
+                [&](bool has, int v, int dir) { prop_relax<S, kHubs>(G, op, ctl, has, v, dir, M, arcs); });
+            if constexpr (kHubs)
+                if (help) {
+                    id.wake();
+                    M.cnt = prop_share<S, Op>(G, ctl, kFull, help, M.buf, M.cnt);
+                    if (lane == 0) atomicAnd(&sh.open, ~help);  // no pieces left there
+                    help = 0;
+                    did = true;
+                }
             if (did) prop_flush<S>(G, M);
             // nothing dirty: look whether the vertex that a value of the next
             // word names holds a larger one itself (paths are walked hop by
@@ -760,7 +917,7 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
                     }
                 }
             }
-            if (!did && id.rest()) break;
+            if (!did && id.rest(help)) break;
             if (deadline) {
                 const uint64_t now = lane == 0 ? globaltimer_ns() : 0;
                 if (__shfl_sync(kFull, now, 0) > deadline) break;
@@ -818,13 +975,83 @@ __device__ __forceinline__ bool prop_count(PropCtl* ctl, unsigned int& step, uns
     return S::sync_then(&ctl->bar, &ctl->err, sum, [&] { return ld_volatile(&ctl->count[at]); });
 }
 
+// The active vertices with a row of more than kPropHub arcs, into hub (a word a
+// vertex), their number ctl->nhub. Ends at a barrier.
+template <class S>
+__device__ __forceinline__ bool prop_list_hubs(const PropGraph<PropMax>& G, PropCtl* ctl, int32_t* hub) {
+    const PropSlice P = prop_slice<S>(G.n);
+    for (long long i = 0; i < P.cnt; ++i) {
+        const long long w = P.word(i);
+        if (w >= P.nw) break;
+        if (!((G.act[w] >> lane_id()) & 1u)) continue;
+        const int v = (int)(w * 32) + lane_id();
+        if (max(S::ld(&G.end[0][v]) - S::ld(&G.off[0][v]), S::ld(&G.end[1][v]) - S::ld(&G.off[1][v])) > kPropHub)
+            hub[atomicAdd(&ctl->nhub, 1u)] = v;
+    }
+    __syncwarp();
+    return S::sync(&ctl->bar, &ctl->err);
+}
+
+// The long rows that a sweep left out, in pieces dealt out to all warps, 32 hubs
+// at a time: a piece's vertex is raised by an atomic, and is dirty if it was.
+// Returns the raises.
+template <class S>
+__device__ __forceinline__ unsigned long long prop_pull_hubs(const PropGraph<PropMax>& G, const PropSlice& P,
+                                                             const int32_t* hub, unsigned int nhub) {
+    constexpr int U = kPropUnroll;
+    const int lane = lane_id();
+    unsigned long long cnt = 0;
+    long long first = 0;  // the warp that takes the next piece
+    for (unsigned int j0 = 0; j0 < nhub; j0 += 32) {
+        const int v = j0 + lane < nhub ? hub[j0 + lane] : -1;
+        const bool on = v >= 0 && ((G.act[v >> 5] >> (v & 31)) & 1u);
+        for (int d = 0; d < 2; ++d) {
+            const int b0 = on ? S::ld(&G.off[1 - d][v]) : 0, len = on ? S::ld(&G.end[1 - d][v]) - b0 : 0;
+            const int mine = len > kPropHub ? (len - 1) / kPropPiece + 1 : 0;
+            const int incl = warp_incl_scan(mine);  // 2^31 / kPropPiece and 32 in all at most
+            const int all = __shfl_sync(kFull, incl, 31);
+            long long p = P.wid - first;
+            if (p < 0) p += P.warps;
+            first = (first + all) % P.warps;
+            for (; p < all; p += P.warps) {
+                const int l = __popc(__ballot_sync(kFull, incl <= (int)p));  // the first lane with incl > p
+                const int hv = __shfl_sync(kFull, v, l), hlen = __shfl_sync(kFull, len, l);
+                const int at = ((int)p - __shfl_sync(kFull, incl - mine, l)) * kPropPiece;
+                const int lo = __shfl_sync(kFull, b0, l) + at;
+                const unsigned long long own = PropMax::load(G.s[d], hv);
+                uint32_t m = 0;
+                row_steps<U>(lo, lo + min(hlen - at, kPropPiece), lane, 32, [&](const uint32_t (&x)[U]) {
+                    int w[U];
+                    unsigned long long t[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) w[u] = x[u] != kNoArc ? S::ld(&G.adj[1 - d][x[u]]) : -1;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) t[u] = w[u] >= 0 ? PropMax::load(G.s[d], w[u]) : PropMax::none();
+#pragma unroll
+                    for (int u = 0; u < U; ++u) m = max(m, PropMax::part(own, t[u]));
+                });
+                m = __reduce_max_sync(kFull, m);
+                if (lane == 0 && PropMax::more(m, own)) {
+                    PropMax::raise(G.s[d], hv, PropMax::with(own, m));
+                    atomicOr(&G.d[d][hv >> 5], 1u << (hv & 31));
+                    ++cnt;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    return cnt;
+}
+
 // The batches from the state in sf/sb/act until every active vertex is
 // finished (`active` of them): trimming inside the classes, the two searches,
 // the labelling. The ring of counters starts zero. kPull: the searches only pull. head_ns: time limit of the first batch's head start (0: none);
-// with it the state's keys start zero, and the first batch sets them.
-template <class S, bool kPull>
+// with it the state's keys start zero, and the first batch sets them. kHubs: there
+// are rows of more than kPropHub arcs, those of the vertices hub[0 .. nhub)
+// (prop_list_hubs).
+template <class S, bool kPull, bool kHubs>
 __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const PropMax op, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
-                             unsigned long long active, uint64_t head_ns) {
+                             unsigned long long active, uint64_t head_ns, const int32_t* hub, unsigned int nhub) {
     const int lane = lane_id();
     const PropSlice P = prop_slice<S>(G.n);
     unsigned long long *const sf = G.s[0], *const sb = G.s[1];
@@ -847,11 +1074,13 @@ __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const Prop
                     i1 = S::ld(&G.end[1][v]);
                 }
                 const bool big = o1 - o0 > kPropBigRow || i1 - i0 > kPropBigRow;
-                bool stays = has && !big && prop_any_in_class<S, 1>(G.adj[0], o0, o1, sf, lab, v) &&
+                // a hub is left to the searches, which share its row
+                const bool is_hub = kHubs && max(o1 - o0, i1 - i0) > kPropHub;
+                bool stays = is_hub || has && !big && prop_any_in_class<S, 1>(G.adj[0], o0, o1, sf, lab, v) &&
                              prop_any_in_class<S, 1>(G.adj[1], i0, i1, sf, lab, v);
-                // long rows by the whole warp: a hub whose neighbours have all
-                // left its class is read to its end
-                for (uint32_t bm = __ballot_sync(kFull, big); bm; bm &= bm - 1) {
+                // long rows by the whole warp: if the neighbours have all left
+                // the class, a row is read to its end
+                for (uint32_t bm = __ballot_sync(kFull, big && !is_hub); bm; bm &= bm - 1) {
                     const int l = __ffs(bm) - 1, hv = __shfl_sync(kFull, v, l);
                     const uint32_t hl = __shfl_sync(kFull, lab, l);
                     const bool in = prop_any_in_class<S, 32>(G.adj[0], __shfl_sync(kFull, o0, l),
@@ -890,7 +1119,7 @@ __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const Prop
                     }
                 }
                 if (!S::sync(&ctl->bar, &ctl->err)) return false;
-                if (!prop_search<S>(G, op, ctl, sh, q, mk, check, globaltimer_ns() + head_ns, items, arcs)) return false;
+                if (!prop_search<S, kHubs>(G, op, ctl, sh, q, mk, check, globaltimer_ns() + head_ns, items, arcs)) return false;
                 unsigned long long cnt = 0;
                 for (long long i = 0; i < P.cnt; ++i) {
                     const long long w = P.word(i);
@@ -936,7 +1165,7 @@ __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const Prop
                     const uint32_t x = w < P.nw ? G.act[w] : 0u;
                     if (x == 0) continue;  // warp-uniform
                     const bool has = (x >> lane) & 1u;
-                    const int c = prop_pull<S>(G, op, has, (int)(w * 32) + lane, false);
+                    const int c = prop_pull<S>(G, op, has, (int)(w * 32) + lane, false, kHubs ? kPropHub : INT32_MAX);
                     const uint32_t cf = __ballot_sync(kFull, c & 1), cb = __ballot_sync(kFull, c & 2);
                     if (lane == 0) {
                         G.d[0][w] = cf;
@@ -944,10 +1173,15 @@ __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const Prop
                         cnt += __popc(cf) + __popc(cb);
                     }
                 }
+                if constexpr (kHubs) {
+                    __syncwarp();
+                    if (!S::sync(&ctl->bar, &ctl->err)) return false;
+                    cnt += prop_pull_hubs<S>(G, P, hub, nhub);
+                }
                 items += cnt;
                 if (!prop_count<S>(ctl, step, cnt, grew)) return false;
             }
-            if (!prop_search<S>(G, op, ctl, sh, q, mk, check, 0, items, arcs)) return false;
+            if (!prop_search<S, kHubs>(G, op, ctl, sh, q, mk, check, 0, items, arcs)) return false;
         }
         // ---- labelling (Alg. 1): equal maxima finish a vertex, the others'
         // class becomes the hash of the old one and the two maxima

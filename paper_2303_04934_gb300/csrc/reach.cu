@@ -17,6 +17,7 @@
 // 64-bit masks by the engine's rounds. The R-MAT time is the hub's four bitmap
 // searches; the masks' own search ends after a few hops.
 #include <algorithm>
+#include <climits>
 #include <cstring>
 
 #include "common.cuh"
@@ -59,7 +60,8 @@ __device__ __forceinline__ PropOr2::Val bit_of(const PropOr2::Val&, int j) {
     return {j < 64 ? 1ull << j : 0ull, j < 64 ? 0ull : 1ull << (j - 64)};
 }
 
-template <class Op, bool kPull>
+// kHubs: for a graph with rows of more than kPropHub arcs
+template <class Op, bool kPull, bool kHubs>
 __global__ void __launch_bounds__(kReachBlock, 4) k_reach(const __grid_constant__ ReachParams<Op> P) {
     using S = ReachScope;
     using Val = typename Op::Val;
@@ -109,7 +111,7 @@ __global__ void __launch_bounds__(kReachBlock, 4) k_reach(const __grid_constant_
     unsigned int check = 0;
     unsigned long long items = 0, arcs = 0;
     if constexpr (kPull) prop_search_pull<S>(G, Op{}, ctl, sh, check, items);
-    else prop_search<S>(G, Op{}, ctl, sh, q, mk, check, 0, items, arcs);
+    else prop_search<S, kHubs>(G, Op{}, ctl, sh, q, mk, check, 0, items, arcs);
 }
 
 // The vertex of the largest smaller degree, degree << 32 | vertex.
@@ -152,19 +154,25 @@ int launch_reach(const ReachArgs& a, cudaStream_t st) {
     P.to_hub = a.to_hub;
     static int per_sm = -1;
     if (per_sm < 0) {
-        int x = 0, y = 0;
-        SCC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_reach<Op, false>, kReachBlock, 0));
-        SCC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_reach<Op, true>, kReachBlock, 0));
-        if (std::min(x, y) < 1) return SCC_ERR_CUDA;
-        per_sm = std::min(x, y);
+        int x = INT_MAX;
+        for (const void* k : {(const void*)k_reach<Op, true, false>, (const void*)k_reach<Op, false, false>,
+                              (const void*)k_reach<Op, false, true>}) {
+            int y = 0;
+            SCC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k, kReachBlock, 0));
+            x = std::min(x, y);
+        }
+        if (x < 1) return SCC_ERR_CUDA;
+        per_sm = x;
     }
     const long long nw = ((long long)a.n + 31) / 32;
     const int grid =
         (int)std::max<long long>(1, std::min<long long>(per_sm * a.num_sms, (nw + kReachWarps - 1) / kReachWarps));
-    const bool pull = a.pull;
+    const void* const kernel = a.pull             ? (const void*)k_reach<Op, true, false>
+                               : a.row > kPropHub ? (const void*)k_reach<Op, false, true>
+                                                  : (const void*)k_reach<Op, false, false>;
     SCC_CUDA(cudaMemsetAsync(P.ctl, 0, sizeof(PropCtl), st));
     void* args[] = {(void*)&P};
-    SCC_CUDA(cudaLaunchCooperativeKernel(pull ? (const void*)k_reach<Op, true> : (const void*)k_reach<Op, false>, dim3(grid), dim3(kReachBlock), args, 0, st));
+    SCC_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(kReachBlock), args, 0, st));
     count_launch();
     PropCtl c;
     SCC_CUDA(cudaMemcpyAsync(&c, P.ctl, sizeof(c), cudaMemcpyDeviceToHost, st));

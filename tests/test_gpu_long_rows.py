@@ -1,13 +1,16 @@
 """Rows far longer than the mean in the searches: a vertex's row is never left to
-one thread. Results against the oracle, and the time of the searches against
-what one thread needs for such a row (90 ns an arc, two dependent loads)."""
+one thread, nor a hub's to one warp. Results against the oracle, and the time of
+a hub's trimming and searches against what one thread needs for its row (90 ns
+an arc, two dependent loads)."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_2303_04934_gb300 import graphgen as gg
+from paper_2303_04934_gb300 import scc
 
 from gpu_util import ensure_lib, labels_of, make_graph
+from test_gpu_hubs import check_reach
 
 pytestmark = pytest.mark.gpu
 
@@ -46,3 +49,59 @@ def test_trimming_of_a_hub_whose_neighbours_are_finished(into):
         st = G.stats()
     assert st["n_trimmed"] == leaves and st["first_scc_size"] == 60000
     assert st["ms_multi_search"] * 1e6 < 40 * leaves
+
+
+def _stars(n, k, two_way=True, into=False):
+    """k disjoint stars on n vertices, centres 0 .. k - 1; one-way stars have a centre on a cycle of two."""
+    leaf = np.arange(2 * k, n)
+    c = leaf % k
+    ring = np.arange(k)
+    a, b = (leaf, c) if into else (c, leaf)
+    src, dst = [a, ring, k + ring], [b, k + ring, ring]
+    if two_way:
+        src.append(b)
+        dst.append(a)
+    p = np.random.default_rng(k).permutation(n)
+    return _csr(n, p[np.concatenate(src)], p[np.concatenate(dst)], f"stars{k}_{two_way}_{into}")
+
+
+# rows just below, at and above the bound from which they are shared (2048 arcs), pieces (512) and their remainders,
+# more shared rows than there are slots (32), and one row of everything
+@pytest.mark.parametrize("n, k", [(2049, 1), (2050, 1), (2051, 1), (2052, 1), (2600, 1), (5000, 2), (40000, 7),
+                                  (200_000, 64), (600_000, 200), (1_000_000, 3), (3_000_000, 1)])
+@pytest.mark.parametrize("two_way, into", [(True, False), (False, False), (False, True)])
+def test_stars(n, k, two_way, into):
+    g = _stars(n, k, two_way, into)
+    rng = np.random.default_rng(n)
+    want, _ = oracle.scc_labels(g.n, g.offsets, g.targets)
+    with make_graph(g) as G:
+        for _ in range(2):
+            assert np.array_equal(labels_of(G), want), g.name
+        for ns in (1, 64, 128):
+            check_reach(G, g, rng.integers(0, n, ns).astype(np.int32))
+
+
+def _clusters(n, k, extra, seed):
+    """k clusters joined by mutual arcs (each one node when contracted) with one-way arcs between vertices of any."""
+    rng = np.random.default_rng(seed)
+    of = np.sort(rng.integers(0, k, n) ** 2 // k)  # sizes from large to none
+    i = np.arange(n)
+    first = np.searchsorted(of, of)
+    j = first + rng.integers(0, 1 << 30, n) % np.maximum(i - first, 1)
+    m = i != first
+    x = rng.integers(0, n, extra)
+    y = x + (rng.random(extra) * (n - x)).astype(np.int64)
+    keep = x != y
+    p = rng.permutation(n)
+    src, dst = np.concatenate([i[m], j[m], x[keep]]), np.concatenate([j[m], i[m], y[keep]])
+    return _csr(n, p[src], p[dst], f"clusters{k}")
+
+
+@pytest.mark.parametrize("n, k, extra", [(70_000, 3, 60_000), (300_000, 40, 300_000), (1_500_000, 1000, 3_000_000)])
+def test_giant_nodes_of_a_contracted_graph(n, k, extra):
+    g = _clusters(n, k, extra, seed=k)
+    want, _ = oracle.scc_labels(g.n, g.offsets, g.targets)
+    with make_graph(g) as G:
+        for _ in range(2):
+            assert np.array_equal(labels_of(G), want), g.name
+        assert scc.scc_debug_forms(G.h)[0] == scc.FORM_CONTRACTED
