@@ -116,6 +116,14 @@ SCC_API int64_t scc_debug_launch_count(void);
 SCC_API int scc_debug_forms(scc_handle h, int32_t* run_form, int32_t* reach_form);
 
 /*
+ * In the searches of scc_run and reach_multi that meet no barrier, a block with
+ * nothing to do waits for the others, and gives up (SCC_ERR_TIMEOUT) when no
+ * block has found new work for 20 s. This sets that limit for h's later calls
+ * (0: 20 s again; at most that).
+ */
+SCC_API int scc_debug_idle_limit(scc_handle h, int64_t limit_ns);
+
+/*
  * The loop by which a warp (or a thread: lanes = 1) walks the arcs [beg, end) of
  * a row, four a lane and step (host only, no device work): what lane `lane` of
  * `lanes` (1 to 32) visits. *steps receives the steps taken, *places the arcs

@@ -53,6 +53,7 @@ struct scc_graph {
     int64_t tab_alloc[2] = {0, 0};
     EngineBuf eb32, eb64;
     scc_stats stats;
+    uint64_t idle_ns = 0;  // scc_debug_idle_limit (0: the library's own)
     int32_t run_form = 0, reach_form = 0;  // kForm* of the last scc_run and reach_multi
     double create_ms[5] = {0, 0, 0, 0, 0};  // total, histogram, partition, rows, split
     // connectivity: the symmetric CSR (built on the first cc_run) and its stats
@@ -316,6 +317,7 @@ static int reach_masks(scc_graph* h, const int32_t* dsrc, int32_t k, int32_t dir
     a.dirty = h->act_bits;
     a.dev = h->prop_dev;
     a.num_sms = h->di.num_sms;
+    a.idle_ns = h->idle_ns;
     EngineOpts o = opts_of(h);
     // hubs of either direction: a search reads the rows of both graphs (pulling
     // those of the one, marking those of the other)
@@ -721,6 +723,7 @@ static PropArgs prop_args(scc_graph* h) {
     a.minid = h->tmp_b;
     a.dev = h->prop_dev;
     a.num_sms = h->di.num_sms;
+    a.idle_ns = h->idle_ns;
     return a;
 }
 
@@ -1249,6 +1252,12 @@ int scc_debug_forms(scc_handle h, int32_t* run_form, int32_t* reach_form) {
     if (!h || !run_form || !reach_form) return SCC_ERR_INVALID_ARG;
     *run_form = h->run_form;
     *reach_form = h->reach_form;
+    return SCC_OK;
+}
+
+int scc_debug_idle_limit(scc_handle h, int64_t limit_ns) {
+    if (!h || limit_ns < 0 || limit_ns > 20000000000ll) return SCC_ERR_INVALID_ARG;
+    h->idle_ns = (uint64_t)limit_ns;
     return SCC_OK;
 }
 

@@ -335,6 +335,7 @@ struct PropArgs {
     long long mesh_arcs = 0;       // arcs of those graphs
     unsigned long long* times = nullptr;
     int time_words = 0;
+    uint64_t idle_ns = 0;          // an idle block's wait ends when no block woke for so long (0: 20 s)
 };
 inline size_t prop_con_words(int64_t n) { return (size_t)(8 * n + (n + 31) / 32); }
 // Forms of the searches of a run or of a reach_multi call (scc_debug_forms).
@@ -383,6 +384,7 @@ struct ReachArgs {
     const uint32_t* to_hub = nullptr;
     void* dev;  // prop_dev_bytes()
     int num_sms;
+    uint64_t idle_ns = 0;      // as in PropArgs
 };
 int run_reach(const ReachArgs& a, cudaStream_t st);
 // The longest row of a CSR (n > 0); tmp: one device word.

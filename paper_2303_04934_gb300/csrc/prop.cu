@@ -66,6 +66,7 @@ struct PropParams {
     int g0, g1;
     unsigned long long* times;
     int time_words;
+    uint64_t idle_ns;
 };
 
 // The group's graph that holds vertex v (the last one that starts at or before it).
@@ -465,7 +466,10 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
     const PropSlice sl = prop_slice<S>(G.n);
     const uint64_t t0 = globaltimer_ns();
     unsigned long long active = P.N;
-    if (threadIdx.x == 0) s_n = 0;
+    if (threadIdx.x == 0) {
+        s_n = 0;
+        sh.idle_ns = P.idle_ns;
+    }
     __syncthreads();
     // ---- state of every vertex; with fresh, vertices without in- or out-arcs
     // are finished (Sec. 4.1)
@@ -716,6 +720,7 @@ static int launch_prop(const PropArgs& a, cudaStream_t st) {
     P.g1 = a.g1;
     P.times = a.times;
     P.time_words = a.time_words;
+    P.idle_ns = a.idle_ns ? a.idle_ns : kPropIdleTimeoutNs;
     int per_sm = 0;
     SCC_TRY(prop_blocks_per_sm(&per_sm));
     const long long nw = ((long long)a.n + 31) / 32;

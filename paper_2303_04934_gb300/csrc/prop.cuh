@@ -49,7 +49,7 @@ constexpr int kPropHub = 2048;     // rows longer than this are shared by the id
 constexpr int kPropPiece = 512;    // ... in pieces of this many arcs
 constexpr int kPropTasks = 24;     // rows shared at a time
 constexpr int kPropTrimPasses = 3; // trimming passes at the start of a batch, at most
-constexpr uint64_t kPropIdleTimeoutNs = 20000000000ull;  // an idle block gives up after 20 s (others may work that long)
+constexpr uint64_t kPropIdleTimeoutNs = 20000000000ull;  // an idle block gives up when no block woke for 20 s
 
 // A bijection of the 32-bit integers (the finaliser of MurmurHash3, Appleby) and its inverse.
 __host__ __device__ __forceinline__ uint32_t prop_mix(uint32_t x) {
@@ -80,8 +80,9 @@ struct PropTask {
 
 struct PropCtl {
     GridBarrier bar;
-    // idle blocks, and the slots of rows with pieces to take: read as one word
-    alignas(8) int idle;
+    // idle blocks (low 16 bits, signed) under a count of the blocks that woke, and
+    // the slots of rows with pieces to take: read as one word
+    alignas(8) unsigned int idle;
     unsigned int open;
     unsigned int taken;       // slots in use
     int err;
@@ -105,6 +106,7 @@ struct PropCtl {
 };
 
 struct PropShared {
+    uint64_t idle_ns;  // the limit of an idle block's wait
     int idle;  // idle warps of the block
     int exit;  // the search is over (or failed)
     unsigned int open;  // rows that have pieces to take
@@ -671,12 +673,13 @@ struct PropIdle {
     PropShared& sh;
     bool idle = false;
     uint64_t t0 = 0;
+    unsigned int woken = 0;  // as last seen
     __device__ __forceinline__ PropIdle(PropCtl* c, PropShared& s) : ctl(c), sh(s) {}
     __device__ __forceinline__ void wake() {
         if (!idle) return;
         idle = false;
         if (lane_id() == 0 && atomicSub(&sh.idle, 1) == (int)(blockDim.x >> 5) && S::blocks() > 1)
-            atomicSub(&ctl->idle, 1);
+            atomicAdd(&ctl->idle, 0xffffu);  // one idle block less, one woken more
     }
     // after a pass over the warp's words that found nothing: true when the
     // search is over (or a wait ran out); open: the rows to help with
@@ -686,7 +689,7 @@ struct PropIdle {
             if (lane_id() == 0) {
                 S::fence();
                 if (atomicAdd(&sh.idle, 1) == (int)(blockDim.x >> 5) - 1) {
-                    if (S::blocks() > 1) atomicAdd(&ctl->idle, 1);
+                    if (S::blocks() > 1) atomicAdd(&ctl->idle, 1u);
                     else atomicExch(&sh.exit, 1);
                 }
             }
@@ -695,9 +698,14 @@ struct PropIdle {
         } else if (threadIdx.x == 0 && S::blocks() > 1) {
             const unsigned long long x = ld_volatile(reinterpret_cast<unsigned long long*>(&ctl->idle));
             if (kHubs) *(volatile unsigned int*)&sh.open = (unsigned int)(x >> 32);
-            if ((int)(unsigned int)x >= S::blocks()) {
+            const unsigned int seen = (unsigned int)x & 0xffff0000u;
+            if (seen != woken) {  // a chain of vertices may keep others at work for as long as it is
+                woken = seen;
+                t0 = globaltimer_ns();
+            }
+            if ((int)(int16_t)(unsigned int)x >= S::blocks()) {
                 atomicExch(&sh.exit, 1);
-            } else if (globaltimer_ns() - t0 > kPropIdleTimeoutNs) {
+            } else if (globaltimer_ns() - t0 > sh.idle_ns) {
                 atomicCAS(&ctl->err, 0, SCC_ERR_TIMEOUT);
                 atomicExch(&sh.exit, 1);
             }
@@ -712,7 +720,7 @@ struct PropIdle {
 template <class S>
 __device__ __forceinline__ bool prop_checked(PropCtl* ctl, PropShared& sh, unsigned int check, bool left, bool* more) {
     if (__any_sync(kFull, left) && lane_id() == 0) atomicMax(&ctl->found, check);
-    if (S::block() == 0 && threadIdx.x == 0) *(volatile int*)&ctl->idle = 0;  // no block counts itself in between the two barriers
+    if (S::block() == 0 && threadIdx.x == 0) *(volatile unsigned int*)&ctl->idle = 0;  // no block counts itself in between the two barriers
     unsigned long long x;
     if (!S::sync_then(&ctl->bar, &ctl->err, x, [&] {
             sh.idle = sh.exit = 0;

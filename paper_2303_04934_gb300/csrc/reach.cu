@@ -53,6 +53,7 @@ struct ReachParams {
     int k;
     const uint32_t* from_hub;  // vertices the hub reaches in the direction of the search (null: no hub)
     const uint32_t* to_hub;    // vertices that reach it
+    uint64_t idle_ns;
 };
 
 __device__ __forceinline__ unsigned long long bit_of(const unsigned long long&, int j) { return 1ull << j; }
@@ -77,6 +78,7 @@ __global__ void __launch_bounds__(kReachBlock, 4) k_reach(const __grid_constant_
     uint32_t* mk = s_mk[threadIdx.x >> 5];
     const PropSlice sl = prop_slice<S>(G.n);
     if (threadIdx.x == 0) {
+        sh.idle_ns = P.idle_ns;
         s_hub = Op::none();
         s_bad = 0;
     }
@@ -152,6 +154,7 @@ int launch_reach(const ReachArgs& a, cudaStream_t st) {
     P.k = a.k;
     P.from_hub = a.from_hub;
     P.to_hub = a.to_hub;
+    P.idle_ns = a.idle_ns ? a.idle_ns : kPropIdleTimeoutNs;
     static int per_sm = -1;
     if (per_sm < 0) {
         int x = INT_MAX;

@@ -33,7 +33,7 @@ EXPORTED = [
     "le_lists_run", "le_lists_get", "le_get_stats",
     "scc_graph_info", "scc_debug_csr", "scc_debug_trim", "scc_debug_pivot_order", "scc_debug_single_reach",
     "scc_debug_multi_reach", "scc_debug_reach_multi_wide", "scc_debug_hashbag", "scc_debug_pair_table", "scc_debug_launch_count",
-    "scc_debug_forms", "scc_debug_row_steps", "scc_debug_barrier_timeout", "scc_debug_le_lists",
+    "scc_debug_forms", "scc_debug_idle_limit", "scc_debug_row_steps", "scc_debug_barrier_timeout", "scc_debug_le_lists",
     "scc_batch_config_default", "scc_batch_create", "scc_batch_destroy", "scc_batch_set_config",
     "scc_batch_get_config", "scc_batch_run", "scc_batch_autotune", "scc_batch_get_stats",
     "scc_debug_batch_times", "scc_debug_batch_groups", "scc_debug_serve_admission", "scc_debug_serve_unit",
@@ -173,6 +173,7 @@ def load() -> ctypes.CDLL:
         "scc_debug_pair_table": ([vp, i64, i64, vp, P(i64), P(i32), vp], ctypes.c_int),
         "scc_debug_launch_count": ([], ctypes.c_int64),
         "scc_debug_forms": ([vp, P(i32), P(i32)], ctypes.c_int),
+        "scc_debug_idle_limit": ([vp, i64], ctypes.c_int),
         "scc_debug_row_steps": ([i32, i32, i32, i32, P(i64), P(i64), P(i64), P(i64)], ctypes.c_int),
         "scc_debug_barrier_timeout": ([i32, i64, P(i32), vp], ctypes.c_int),
         "scc_debug_le_lists": ([vp, i64, i64, P(i64), vp], ctypes.c_int),
@@ -662,6 +663,10 @@ def scc_debug_forms(h) -> tuple:
     a, b = ctypes.c_int32(), ctypes.c_int32()
     _check(load().scc_debug_forms(h, ctypes.byref(a), ctypes.byref(b)), "scc_debug_forms")
     return a.value, b.value
+
+
+def scc_debug_idle_limit(h, limit_ns: int) -> None:
+    _check(load().scc_debug_idle_limit(h, limit_ns), "scc_debug_idle_limit")
 
 
 def scc_debug_row_steps(beg: int, end: int, lane: int, lanes: int) -> tuple:
