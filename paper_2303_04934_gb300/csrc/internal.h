@@ -350,7 +350,7 @@ struct PropResult {
     unsigned long long items = 0, arcs = 0;
 };
 size_t prop_dev_bytes();
-bool prop_pulls(long long m, int num_sms);
+bool reach_pulls(long long m, int num_sms);
 // A graph with a row of more than 64 arcs and of more than 16 times the mean
 // degree: a hub's value grows several times, and each time costs its whole row,
 // while the first SCC's bitmap searches read it once (the batched kernel draws
@@ -378,7 +378,7 @@ struct ReachArgs {
     int words;
     unsigned long long* mask;  // n * words
     uint32_t* dirty;           // ceil(n / 32)
-    bool pull = false;         // the search only pulls (prop_pulls)
+    bool pull = false;         // the search only pulls (reach_pulls)
     int32_t row = 0;           // the longest row of off (pull: not read)
     const uint32_t* from_hub = nullptr;
     const uint32_t* to_hub = nullptr;

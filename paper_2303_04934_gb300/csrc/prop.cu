@@ -16,12 +16,12 @@ namespace {
 constexpr int kPropBlock = 256;
 constexpr int kPropRegions = 1024;
 constexpr int kPropWarps = kPropBlock / kWarp;
-// Arcs per thread up to which searches only pull (a pass over all of them is
-// then one hop of every path). Pulling against marking, run alone: 2D torus 524 k
+// Quarters of an arc per thread of the chip up to which searches only pull (a pass
+// over all of them is then one hop of every path). Pulling against marking, run alone: 2D torus 524 k
 // vertices (6.7 arcs a thread) 19.7 / 21.9 ms, 3D torus 512 k (5.9) 1.35 / 1.50,
 // k-NN 200 k x 5 (6.4) 0.88 / 1.02, k-NN 400 k x 3 (7.7) 2.8 / 2.3, 3D torus 1 M
 // (11.6) 2.4 / 1.9, 2D torus 1 M (13.5) 31 / 16.
-constexpr long long kPropPullArcs = 7;
+constexpr long long kPropPull = 28, kReachPull = 28;
 // Vertices from which the first batch has a head start (of at most n / 4 ns):
 // 3D torus 256^3 28 -> 11 ms with it. Below, a search is bound by its hops and
 // the wave of the head start would only come on top.
@@ -54,6 +54,7 @@ struct PropParams {
     const int32_t* label;
     unsigned long long N;
     long long m;
+    unsigned long long pull_arcs;  // up to so many arcs the searches only pull
     unsigned long long arcs;  // arcs of the graphs without hubs (m, but in a group)
     uint64_t seed;
     int32_t* minid;
@@ -447,6 +448,68 @@ __device__ __forceinline__ void prop_node_state(const PropGraph<PropMax>& N, con
     }
 }
 
+// The contracted graph's nodes as a graph.
+__device__ __forceinline__ PropGraph<PropMax> prop_nodes(const PropParams& P, const PropCtl* ctl) {
+    const PropCon& C = P.con;
+    PropGraph<PropMax> N;
+    for (int d = 0; d < 2; ++d) {
+        N.off[d] = C.beg[d];
+        N.end[d] = C.end[d];
+        N.adj[d] = C.adj[d];
+        N.s[d] = P.G.s[d];
+        N.d[d] = P.G.d[d];
+    }
+    N.n = (int32_t)ld_volatile(&ctl->nodes);
+    N.act = C.act;
+    N.rep = C.rep;
+    return N;
+}
+
+// The labels of all vertices from the SCCs of the nodes.
+template <class S>
+__device__ __forceinline__ bool prop_node_labels(const PropParams& P, const PropGraph<PropMax>& N, PropCtl* ctl) {
+    const int lane = lane_id();
+    const PropCon& C = P.con;
+    const PropGraph<PropMax>& G = P.G;
+    const PropSlice sl = prop_slice<S>(G.n);
+    const PropSlice Q = prop_slice<S>(N.n);
+    for (long long i = 0; i < Q.cnt; ++i) {
+        const long long w = Q.word(i), c = w * 32 + lane;
+        if (w >= Q.nw) break;
+        const int r = c < N.n ? C.rep[c] : -1;
+        const unsigned int x = c < N.n ? (unsigned int)C.lead[c] : 0u;
+        const uint32_t peers = __match_any_sync(kFull, r);
+        const unsigned int least = __reduce_min_sync(peers, x);
+        if (r >= 0 && lane == __ffs(peers) - 1 && (unsigned int)ld_volatile(&C.min[r]) > least)
+            atomicMin(&C.min[r], (int)least);
+    }
+    if (!S::sync(&ctl->bar, &ctl->err)) return false;
+    auto label = [&](int c) { return ld_volatile(&C.min[ld_volatile(&C.rep[c])]); };
+    const int pv = P.vbase == nullptr ? ld_volatile(&ctl->pivot) : -1;
+    const int pc = pv >= 0 ? ld_volatile(&C.cid[pv]) : -1;
+    const int pl = (unsigned int)pc < (unsigned int)N.n ? label(pc) : -1;
+    unsigned int first = 0;
+    for (long long i = 0; i < sl.cnt; ++i) {
+        const long long v = sl.word(i) * 32 + lane;
+        if (v >= G.n) continue;
+        int first_v = 0;
+        if (P.vbase != nullptr) {
+            const int g = prop_graph_of(P, v);
+            if (!P.mesh[g]) continue;
+            first_v = (int)(P.vbase[g] - P.vbase[P.g0]);
+        }
+        const int c = ld_volatile(&C.cid[v]);
+        const int l = (unsigned int)c < (unsigned int)N.n ? label(c) : (int)v;
+        first += l == pl;
+        P.out[v] = l - first_v;
+    }
+    __syncwarp();
+    first = __reduce_add_sync(kFull, first);
+    if (lane == 0 && first) atomicAdd(&ctl->first, first);
+    return true;
+}
+
+// The whole run on a graph without hubs.
 __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ PropParams P) {
     using S = PropScope;
     __shared__ PropShared sh;
@@ -460,19 +523,18 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
     uint32_t* q = s_q[threadIdx.x >> 5];
     uint32_t* mk = s_mk[threadIdx.x >> 5];
     // a head start pays where a search is bound by throughput, not by its hops
-    const unsigned long long threads = (unsigned long long)gridDim.x * blockDim.x;
-    const bool pull = P.fresh && P.arcs <= kPropPullArcs * threads;  // few arcs a thread: the searches only pull
-    const uint64_t head_ns = P.fresh && P.vbase == nullptr && G.n >= kPropHeadMin && !pull ? (uint64_t)(G.n / 4) : 0;
+    const bool pull = P.arcs <= P.pull_arcs;  // few arcs a thread: the searches only pull
+    const uint64_t head_ns = P.vbase == nullptr && G.n >= kPropHeadMin && !pull ? (uint64_t)(G.n / 4) : 0;
     const PropSlice sl = prop_slice<S>(G.n);
     const uint64_t t0 = globaltimer_ns();
-    unsigned long long active = P.N;
+    unsigned long long active;
     if (threadIdx.x == 0) {
         s_n = 0;
         sh.idle_ns = P.idle_ns;
     }
     __syncthreads();
-    // ---- state of every vertex; with fresh, vertices without in- or out-arcs
-    // are finished (Sec. 4.1)
+    // ---- state of every vertex; vertices without in- or out-arcs are finished
+    // (Sec. 4.1)
     {
         const long long len = (sl.nw + kPropRegions - 1) / kPropRegions;
         unsigned int cnt = 0, mx = 0;
@@ -481,24 +543,16 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
             const long long w = sl.word(i), v = w * 32 + lane;
             if (w >= sl.nw) break;
             bool a = false;
-            uint32_t lab = 0;
             if (v < G.n) {
-                if (P.fresh) {
-                    const int d0 = G.end[0][v] - G.off[0][v], d1 = G.end[1][v] - G.off[1][v];
-                    a = d0 > 0 && d1 > 0 && (P.vbase == nullptr || P.mesh[prop_graph_of(P, v)]);
-                    mx = max(mx, (unsigned int)max(d0, d1));
-                    if (head_ns && a) best = max(best, prop_pack((uint32_t)min(d0, d1), op.key((uint32_t)v)));
-                    G.rep[v] = (int)v;
-                    P.minid[v] = (int)v;
-                    if (!a) P.con.cid[v] = -1;
-                } else {
-                    const int32_t l = P.label[v];
-                    a = l >= 0;
-                    lab = (uint32_t)l;
-                    if (a) mx = max(mx, (unsigned int)max(G.end[0][v] - G.off[0][v], G.end[1][v] - G.off[1][v]));
-                }
+                const int d0 = G.end[0][v] - G.off[0][v], d1 = G.end[1][v] - G.off[1][v];
+                a = d0 > 0 && d1 > 0 && (P.vbase == nullptr || P.mesh[prop_graph_of(P, v)]);
+                mx = max(mx, (unsigned int)max(d0, d1));
+                if (head_ns && a) best = max(best, prop_pack((uint32_t)min(d0, d1), op.key((uint32_t)v)));
+                G.rep[v] = (int)v;
+                P.minid[v] = (int)v;
+                if (!a) P.con.cid[v] = -1;
                 const unsigned long long st =
-                    a ? prop_pack(lab, head_ns ? 0u : op.key((uint32_t)v)) : PropMax::none();
+                    a ? prop_pack(0, head_ns ? 0u : op.key((uint32_t)v)) : PropMax::none();
                 G.s[0][v] = st;
                 G.s[1][v] = st;
             }
@@ -508,124 +562,65 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
                 G.d[0][w] = 0;
                 G.d[1][w] = 0;
                 cnt += __popc(m);
-                if (P.fresh && m) atomicAdd(&P.dev->region[w / len], (unsigned int)__popc(m));
+                if (m) atomicAdd(&P.dev->region[w / len], (unsigned int)__popc(m));
             }
         }
-        if (P.fresh) {
-            for (int d = 16; d >= 1; d >>= 1) {
-                mx = max(mx, __shfl_xor_sync(kFull, mx, d));
-                best = max(best, __shfl_xor_sync(kFull, best, d));
-            }
-            if (lane == 0) {
-                atomicAdd(&s_n, cnt);
-                atomicMax(&ctl->max_deg, mx);
-                if (best) atomicMax(&ctl->best, best);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0 && s_n) atomicAdd(&ctl->active0, (unsigned long long)s_n);
+        for (int d = 16; d >= 1; d >>= 1) {
+            mx = max(mx, __shfl_xor_sync(kFull, mx, d));
+            best = max(best, __shfl_xor_sync(kFull, best, d));
         }
-        if (!P.fresh) {
-            mx = __reduce_max_sync(kFull, mx);
-            if (lane == 0 && mx > (unsigned int)kPropHub) atomicMax(&ctl->max_deg, mx);
+        if (lane == 0) {
+            atomicAdd(&s_n, cnt);
+            atomicMax(&ctl->max_deg, mx);
+            if (best) atomicMax(&ctl->best, best);
         }
+        __syncthreads();
+        if (threadIdx.x == 0 && s_n) atomicAdd(&ctl->active0, (unsigned long long)s_n);
         if (!S::sync(&ctl->bar, &ctl->err)) return;
     }
-    if (P.fresh) {
-        active = ld_volatile(&ctl->active0);
-        // that vertex becomes the largest source
-        if (head_ns && active > 0) op.k0 = op.vertex((uint32_t)ld_volatile(&ctl->best)) ^ prop_unmix(0xffffffffu);
-        const unsigned long long md = ld_volatile(&ctl->max_deg);
-        if (P.vbase == nullptr && prop_skewed(md, (unsigned long long)G.n, (unsigned long long)P.m)) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) ctl->status = 1;
-            return;
-        }
-        // the first pivot of the seeded order: statistics only (its SCC's
-        // size), found before any bit is cleared
-        if (P.vbase == nullptr && active > 0 && blockIdx.x == 0 && threadIdx.x < 32) {
-            Feistel f;
-            f.init(P.seed, active);
-            const int v = prop_select(G.act, sl.nw, P.dev->region, f.perm(0, active));
-            if (lane == 0) ctl->pivot = v;
-        }
-        if (!S::sync(&ctl->bar, &ctl->err)) return;
+    active = ld_volatile(&ctl->active0);
+    // that vertex becomes the largest source
+    if (head_ns && active > 0) op.k0 = op.vertex((uint32_t)ld_volatile(&ctl->best)) ^ prop_unmix(0xffffffffu);
+    const unsigned long long md = ld_volatile(&ctl->max_deg);
+    if (P.vbase == nullptr && prop_skewed(md, (unsigned long long)G.n, (unsigned long long)P.m)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->status = 1;
+        return;
     }
+    // the first pivot of the seeded order: statistics only (its SCC's
+    // size), found before any bit is cleared
+    if (P.vbase == nullptr && active > 0 && blockIdx.x == 0 && threadIdx.x < 32) {
+        Feistel f;
+        f.init(P.seed, active);
+        const int v = prop_select(G.act, sl.nw, P.dev->region, f.perm(0, active));
+        if (lane == 0) ctl->pivot = v;
+    }
+    if (!S::sync(&ctl->bar, &ctl->err)) return;
     bool contracted = false;
-    if (P.fresh && active > 0 && G.n >= kConMin && !prop_contract<S>(G, P.con, ctl, active, &contracted)) return;
+    if (active > 0 && G.n >= kConMin && !prop_contract<S>(G, P.con, ctl, active, &contracted)) return;
     if (contracted) {
-        const PropCon& C = P.con;
-        PropGraph<PropMax> N;
-        for (int d = 0; d < 2; ++d) {
-            N.off[d] = C.beg[d];
-            N.end[d] = C.end[d];
-            N.adj[d] = C.adj[d];
-            N.s[d] = G.s[d];
-            N.d[d] = G.d[d];
-        }
-        N.n = (int32_t)ld_volatile(&ctl->nodes);
-        N.act = C.act;
-        N.rep = C.rep;
+        const PropGraph<PropMax> N = prop_nodes(P, ctl);
         const unsigned long long arcs2 = ld_volatile(&ctl->arcs2[0]);
         op.k0 = P.k0;
-        prop_node_state<S>(N, op, C);
+        prop_node_state<S>(N, op, P.con);
         if (!S::sync(&ctl->bar, &ctl->err)) return;
         // a node's row is as long as its vertices' rows together
-        const bool hubs = ld_volatile(&ctl->max_row2) > (unsigned int)kPropHub;
-        if (hubs && !prop_list_hubs<S>(N, ctl, P.minid)) return;
-        const unsigned int nhub = hubs ? ld_volatile(&ctl->nhub) : 0u;
-        const bool pull2 =
-            !hubs && arcs2 <= kPropPullArcs * threads && arcs2 <= kConPullRow * (unsigned long long)N.n;
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = kFormContracted | (pull2 ? kFormPull : 0);
-        if (!(pull2  ? prop_batches<S, true, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0, nullptr, 0)
-              : hubs ? prop_batches<S, false, true>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0, P.minid, nhub)
-                     : prop_batches<S, false, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0, nullptr, 0)))
+        if (ld_volatile(&ctl->max_row2) > (unsigned int)kPropHub) {  // k_prop_hubs goes on
+            if (blockIdx.x == 0 && threadIdx.x == 0) ctl->status = 2;
             return;
-        const PropSlice Q = prop_slice<S>(N.n);
-        for (long long i = 0; i < Q.cnt; ++i) {
-            const long long w = Q.word(i), c = w * 32 + lane;
-            if (w >= Q.nw) break;
-            const int r = c < N.n ? C.rep[c] : -1;
-            const unsigned int x = c < N.n ? (unsigned int)C.lead[c] : 0u;
-            const uint32_t peers = __match_any_sync(kFull, r);
-            const unsigned int least = __reduce_min_sync(peers, x);
-            if (r >= 0 && lane == __ffs(peers) - 1 && (unsigned int)ld_volatile(&C.min[r]) > least)
-                atomicMin(&C.min[r], (int)least);
         }
-        if (!S::sync(&ctl->bar, &ctl->err)) return;
-        auto label = [&](int c) { return ld_volatile(&C.min[ld_volatile(&C.rep[c])]); };
-        const int pv = P.vbase == nullptr ? ld_volatile(&ctl->pivot) : -1;
-        const int pc = pv >= 0 ? ld_volatile(&C.cid[pv]) : -1;
-        const int pl = (unsigned int)pc < (unsigned int)N.n ? label(pc) : -1;
-        unsigned int first = 0;
-        for (long long i = 0; i < sl.cnt; ++i) {
-            const long long v = sl.word(i) * 32 + lane;
-            if (v >= G.n) continue;
-            int first_v = 0;
-            if (P.vbase != nullptr) {
-                const int g = prop_graph_of(P, v);
-                if (!P.mesh[g]) continue;
-                first_v = (int)(P.vbase[g] - P.vbase[P.g0]);
-            }
-            const int c = ld_volatile(&C.cid[v]);
-            const int l = (unsigned int)c < (unsigned int)N.n ? label(c) : (int)v;
-            first += l == pl;
-            P.out[v] = l - first_v;
-        }
-        __syncwarp();
-        first = __reduce_add_sync(kFull, first);
-        if (lane == 0 && first) atomicAdd(&ctl->first, first);
+        const bool pull2 = arcs2 <= P.pull_arcs && arcs2 <= kConPullRow * (unsigned long long)N.n;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = kFormContracted | (pull2 ? kFormPull : 0);
+        if (!(pull2 ? prop_batches<S, true, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)
+                    : prop_batches<S, false, false>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)))
+            return;
+        if (!prop_node_labels<S>(P, N, ctl)) return;
         prop_times(P, t0);
         return;
     }
-    // the rest of a graph with hubs (a fresh one has none: its rows are short)
-    const bool hubs = !P.fresh && ld_volatile(&ctl->max_deg) > (unsigned int)kPropHub;
-    if (hubs && !prop_list_hubs<S>(G, ctl, P.minid)) return;
-    const unsigned int nhub = hubs ? ld_volatile(&ctl->nhub) : 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = pull ? kFormPull : head_ns ? kFormHeadStart : 0;
-    if (!(pull   ? prop_batches<S, true, false>(G, op, ctl, sh, q, mk, active, 0, nullptr, 0)
-          : hubs ? prop_batches<S, false, true>(G, op, ctl, sh, q, mk, active, 0, P.minid, nhub)
-                 : prop_batches<S, false, false>(G, op, ctl, sh, q, mk, active, head_ns, nullptr, 0)))
+    if (!(pull ? prop_batches<S, true, false>(G, op, ctl, sh, q, mk, active, 0)
+               : prop_batches<S, false, false>(G, op, ctl, sh, q, mk, active, head_ns)))
         return;
-    if (!P.fresh) return;
     // ---- canonical labels: the smallest vertex of each SCC
     const int proot = P.vbase == nullptr && active > 0 && ld_volatile(&ctl->pivot) >= 0 ? ld_volatile(&G.rep[ld_volatile(&ctl->pivot)]) : -1;
     unsigned int first = 0;
@@ -662,6 +657,64 @@ __global__ void __launch_bounds__(kPropBlock, 4) k_prop(const __grid_constant__ 
     prop_times(P, t0);
 }
 
+// What may have long rows: the rest of a graph with hubs, whose first SCC is done
+// (classes in label), or (status 2) the contracted graph that k_prop left. A
+// kernel of its own: the same searches in k_prop, called from the same places,
+// cost the lattices of 1 k to 131 k vertices 3-6%, whether they ran or not.
+__global__ void __launch_bounds__(kPropBlock, 4) k_prop_hubs(const __grid_constant__ PropParams P) {
+    using S = PropScope;
+    __shared__ PropShared sh;
+    __shared__ uint32_t s_q[kPropWarps][kPropQueue];
+    __shared__ uint32_t s_mk[kPropWarps][kPropMarks];
+    const PropMax op{P.k0};
+    PropCtl* ctl = &P.dev->c;
+    const int lane = lane_id();
+    uint32_t* q = s_q[threadIdx.x >> 5];
+    uint32_t* mk = s_mk[threadIdx.x >> 5];
+    const uint64_t t0 = globaltimer_ns();
+    if (threadIdx.x == 0) sh.idle_ns = P.idle_ns;
+    __syncthreads();
+    if (P.fresh) {
+        if (ld_volatile(&ctl->status) != 2) return;
+        const PropGraph<PropMax> N = prop_nodes(P, ctl);
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->form = kFormContracted;
+        if (!prop_list_hubs<S>(N, ctl, P.minid)) return;
+        if (!prop_batches<S, false, true>(N, op, ctl, sh, q, mk, (unsigned long long)N.n, 0)) return;
+        if (!prop_node_labels<S>(P, N, ctl)) return;
+        prop_times(P, t0);
+        return;
+    }
+    const PropGraph<PropMax>& G = P.G;
+    const PropSlice sl = prop_slice<S>(G.n);
+    unsigned int mx = 0;
+    for (long long i = 0; i < sl.cnt; ++i) {
+        const long long w = sl.word(i), v = w * 32 + lane;
+        if (w >= sl.nw) break;
+        const int32_t lab = v < G.n ? P.label[v] : kDone;
+        if (lab >= 0) mx = max(mx, (unsigned int)max(G.end[0][v] - G.off[0][v], G.end[1][v] - G.off[1][v]));
+        if (v < G.n) {
+            const unsigned long long st = lab >= 0 ? prop_pack((uint32_t)lab, op.key((uint32_t)v)) : PropMax::none();
+            G.s[0][v] = st;
+            G.s[1][v] = st;
+        }
+        const uint32_t m = __ballot_sync(kFull, lab >= 0);
+        if (lane == 0) {
+            G.act[w] = m;
+            G.d[0][w] = 0;
+            G.d[1][w] = 0;
+        }
+    }
+    mx = __reduce_max_sync(kFull, mx);
+    if (lane == 0 && mx > (unsigned int)kPropHub) atomicMax(&ctl->max_deg, mx);
+    if (!S::sync(&ctl->bar, &ctl->err)) return;
+    if (ld_volatile(&ctl->max_deg) > (unsigned int)kPropHub) {
+        if (!prop_list_hubs<S>(G, ctl, P.minid)) return;
+        prop_batches<S, false, true>(G, op, ctl, sh, q, mk, P.N, 0);
+    } else {
+        prop_batches<S, false, false>(G, op, ctl, sh, q, mk, P.N, 0);
+    }
+}
+
 __global__ void k_prop_err(const PropCtl* c, int* err) {
     if (c->err != 0) atomicCAS(err, 0, c->err);
 }
@@ -670,23 +723,26 @@ __global__ void k_prop_err(const PropCtl* c, int* err) {
 
 size_t prop_dev_bytes() { return sizeof(PropDev); }
 
-// Whether the searches of a graph without hubs only pull.
-bool prop_pulls(long long m, int num_sms) { return m <= kPropPullArcs * 4ll * num_sms * kPropBlock; }
+// Whether a reach_multi search of a graph without hubs only pulls (k_prop's
+// rule is in launch_prop; both launch four blocks an SM).
+bool reach_pulls(long long m, int num_sms) { return 4 * m <= kReachPull * 4 * num_sms * kPropBlock; }
 
 // Resident blocks per SM (the first call is outside any stream capture).
 int prop_blocks_per_sm(int* out) {
     static int per_sm = -1;
     if (per_sm < 0) {
-        int x = 0;
+        int x = 0, y = 0;  // one grid for both: k_prop_hubs goes on at k_prop's barrier
         SCC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_prop, kPropBlock, 0));
-        if (x < 1) return SCC_ERR_CUDA;
-        per_sm = x;
+        SCC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_prop_hubs, kPropBlock, 0));
+        if (std::min(x, y) < 1) return SCC_ERR_CUDA;
+        per_sm = std::min(x, y);
     }
     *out = per_sm;
     return SCC_OK;
 }
 
-static int launch_prop(const PropArgs& a, cudaStream_t st) {
+// hubs: k_prop_hubs, on the rest of a graph or after k_prop.
+static int launch_prop(const PropArgs& a, bool hubs, cudaStream_t st) {
     PropParams P;
     memset(&P, 0, sizeof(P));
     P.G = PropGraph<PropMax>{{a.off, a.toff}, {a.off + 1, a.toff + 1}, {a.adj, a.tadj}, a.n, {a.sf, a.sb}, {a.df, a.db}, a.act, a.rep};
@@ -725,28 +781,34 @@ static int launch_prop(const PropArgs& a, cudaStream_t st) {
     SCC_TRY(prop_blocks_per_sm(&per_sm));
     const long long nw = ((long long)a.n + 31) / 32;
     const int full = per_sm * a.num_sms;
+    P.pull_arcs = (unsigned long long)(kPropPull * full * kPropBlock / 4);
     const int grid = (int)std::max<long long>(1, std::min<long long>(full, (nw + kPropWarps - 1) / kPropWarps));
-    SCC_CUDA(cudaMemsetAsync(P.dev, 0, sizeof(PropDev), st));
+    if (!hubs || !P.fresh) SCC_CUDA(cudaMemsetAsync(P.dev, 0, sizeof(PropDev), st));
     void* args[] = {(void*)&P};
-    SCC_CUDA(cudaLaunchCooperativeKernel((const void*)k_prop, dim3(grid), dim3(kPropBlock), args, 0, st));
+    SCC_CUDA(cudaLaunchCooperativeKernel(hubs ? (const void*)k_prop_hubs : (const void*)k_prop, dim3(grid),
+                                         dim3(kPropBlock), args, 0, st));
     count_launch();
     return SCC_OK;
 }
 
 int enqueue_prop(const PropArgs& a, int* err, cudaStream_t st) {
-    SCC_TRY(launch_prop(a, st));
+    SCC_TRY(launch_prop(a, false, st));
+    if (a.n >= kConMin) SCC_TRY(launch_prop(a, true, st));  // ends at once unless it is needed
     k_prop_err<<<1, 1, 0, st>>>(&reinterpret_cast<PropDev*>(a.dev)->c, err);
     SCC_LAUNCH();
     return SCC_OK;
 }
 
 int run_prop(const PropArgs& a, PropResult* res, cudaStream_t st) {
-    SCC_TRY(launch_prop(a, st));
     PropCtl c;
-    SCC_CUDA(cudaMemcpyAsync(&c, a.dev, sizeof(c), cudaMemcpyDeviceToHost, st));
-    SCC_CUDA(cudaStreamSynchronize(st));
-    if (c.err) return c.err;
-    res->status = c.status;
+    for (bool hubs = a.label != nullptr;; hubs = true) {
+        SCC_TRY(launch_prop(a, hubs, st));
+        SCC_CUDA(cudaMemcpyAsync(&c, a.dev, sizeof(c), cudaMemcpyDeviceToHost, st));
+        SCC_CUDA(cudaStreamSynchronize(st));
+        if (c.err) return c.err;
+        if (hubs || c.status != 2) break;
+    }
+    res->status = c.status == 1;
     res->form = c.form;
     res->active = (int64_t)c.active0;
     res->first = (int32_t)c.first;

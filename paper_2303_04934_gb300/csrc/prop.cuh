@@ -21,7 +21,7 @@
 // Schedule. What bounds these searches on a large-diameter graph is the chain
 // of dependent accesses along its paths, not bandwidth, so nothing in a search
 // waits for a barrier: vertices whose value grew are bits of a dirty bitmap, a
-// warp owns a contiguous run of its words, polls them, takes the set bits and
+// warp owns runs of its words, polls them, takes the set bits and
 // relaxes those vertices' arcs, marking the heads it raised in whichever warp's
 // words they lie. A search ends when every block is idle at once, which a
 // counter of idle blocks detects; a check of the whole bitmap between two grid
@@ -87,7 +87,8 @@ struct PropCtl {
     unsigned int taken;       // slots in use
     int err;
     PropTask task[kPropTasks];
-    unsigned int nhub;        // vertices with a row of more than kPropHub arcs
+    int32_t* hub;             // the vertices with a row of more than kPropHub arcs
+    unsigned int nhub;        // their number
     unsigned int found;       // last check that found work left
     unsigned long long count[4];  // vertices finished by a counting step, a ring over the steps
     unsigned long long items, arcs;
@@ -100,13 +101,15 @@ struct PropCtl {
     unsigned int hooked[3];    // ... and by a round, a ring over the rounds
     unsigned int nodes;        // vertices of the contracted graph
     unsigned int arcs2[2];     // arcs of the contracted graph and of its transpose
-    int status;  // 0 finished, 1 a skewed graph (nothing done but the first trim)
+    int status;  // 0 finished, 1 a skewed graph (nothing done but the first trim), 2 contracted, with long rows
     unsigned int first;  // vertices in the first pivot's SCC
     int form;            // kForm* taken
 };
 
 struct PropShared {
-    uint64_t idle_ns;  // the limit of an idle block's wait
+    uint64_t idle_ns;  // the limit of an idle block's wait, kept by its first thread:
+    uint64_t t0;       // since when it waits (0: to be set)
+    unsigned int woken, polls;  // the count of woken blocks last seen; looks since then
     int idle;  // idle warps of the block
     int exit;  // the search is over (or failed)
     unsigned int open;  // rows that have pieces to take
@@ -672,8 +675,6 @@ struct PropIdle {
     PropCtl* ctl;
     PropShared& sh;
     bool idle = false;
-    uint64_t t0 = 0;
-    unsigned int woken = 0;  // as last seen
     __device__ __forceinline__ PropIdle(PropCtl* c, PropShared& s) : ctl(c), sh(s) {}
     __device__ __forceinline__ void wake() {
         if (!idle) return;
@@ -693,21 +694,26 @@ struct PropIdle {
                     else atomicExch(&sh.exit, 1);
                 }
             }
+            if (threadIdx.x == 0) {
+                sh.t0 = 0;
+                sh.polls = 0;
+            }
             __syncwarp();
-            t0 = globaltimer_ns();
         } else if (threadIdx.x == 0 && S::blocks() > 1) {
             const unsigned long long x = ld_volatile(reinterpret_cast<unsigned long long*>(&ctl->idle));
             if (kHubs) *(volatile unsigned int*)&sh.open = (unsigned int)(x >> 32);
             const unsigned int seen = (unsigned int)x & 0xffff0000u;
-            if (seen != woken) {  // a chain of vertices may keep others at work for as long as it is
-                woken = seen;
-                t0 = globaltimer_ns();
-            }
             if ((int)(int16_t)(unsigned int)x >= S::blocks()) {
                 atomicExch(&sh.exit, 1);
-            } else if (globaltimer_ns() - t0 > sh.idle_ns) {
-                atomicCAS(&ctl->err, 0, SCC_ERR_TIMEOUT);
-                atomicExch(&sh.exit, 1);
+            } else if ((++sh.polls & 63) == 0) {  // the timer is slow to read
+                const uint64_t now = globaltimer_ns();
+                if (seen != sh.woken || sh.t0 == 0) {  // a chain of vertices may keep others at work for as long as it is
+                    sh.woken = seen;
+                    sh.t0 = now;
+                } else if (now - sh.t0 > sh.idle_ns) {
+                    atomicCAS(&ctl->err, 0, SCC_ERR_TIMEOUT);
+                    atomicExch(&sh.exit, 1);
+                }
             }
         }
         const int ex = lane_id() == 0 ? ld_volatile(&sh.exit) : 0;
@@ -996,6 +1002,7 @@ __device__ __forceinline__ bool prop_list_hubs(const PropGraph<PropMax>& G, Prop
         if (max(S::ld(&G.end[0][v]) - S::ld(&G.off[0][v]), S::ld(&G.end[1][v]) - S::ld(&G.off[1][v])) > kPropHub)
             hub[atomicAdd(&ctl->nhub, 1u)] = v;
     }
+    if (S::block() == 0 && threadIdx.x == 0) ctl->hub = hub;
     __syncwarp();
     return S::sync(&ctl->bar, &ctl->err);
 }
@@ -1055,11 +1062,11 @@ __device__ __forceinline__ unsigned long long prop_pull_hubs(const PropGraph<Pro
 // finished (`active` of them): trimming inside the classes, the two searches,
 // the labelling. The ring of counters starts zero. kPull: the searches only pull. head_ns: time limit of the first batch's head start (0: none);
 // with it the state's keys start zero, and the first batch sets them. kHubs: there
-// are rows of more than kPropHub arcs, those of the vertices hub[0 .. nhub)
-// (prop_list_hubs).
+// are rows of more than kPropHub arcs, those of the vertices that prop_list_hubs
+// listed.
 template <class S, bool kPull, bool kHubs>
 __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const PropMax op, PropCtl* ctl, PropShared& sh, uint32_t* q, uint32_t* mk,
-                             unsigned long long active, uint64_t head_ns, const int32_t* hub, unsigned int nhub) {
+                             unsigned long long active, uint64_t head_ns) {
     const int lane = lane_id();
     const PropSlice P = prop_slice<S>(G.n);
     unsigned long long *const sf = G.s[0], *const sb = G.s[1];
@@ -1184,7 +1191,7 @@ __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const Prop
                 if constexpr (kHubs) {
                     __syncwarp();
                     if (!S::sync(&ctl->bar, &ctl->err)) return false;
-                    cnt += prop_pull_hubs<S>(G, P, hub, nhub);
+                    cnt += prop_pull_hubs<S>(G, P, ld_volatile(&ctl->hub), ld_volatile(&ctl->nhub));
                 }
                 items += cnt;
                 if (!prop_count<S>(ctl, step, cnt, grew)) return false;
