@@ -326,7 +326,7 @@ static int reach_masks(scc_graph* h, const int32_t* dsrc, int32_t k, int32_t dir
                                     (unsigned long long)h->mt);
     a.row = dir ? h->max_in : h->max_out;
     const bool hubs = o.high_degree && skewed && h->mt >= kHubArcs;
-    a.pull = !skewed && reach_pulls(h->mt, h->di.num_sms);
+    a.pull = !skewed && reach_pulls(n, h->mt, h->di.num_sms);
     h->reach_form = (a.pull ? kFormPull : 0) | (hubs ? kFormHubFirst : 0);
     if (hubs) {
         if (h->hub < 0) SCC_TRY(find_hub(h->off, h->toff, n, h->counters + 3, h->di.num_sms, &h->hub, s));

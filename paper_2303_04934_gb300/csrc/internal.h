@@ -350,7 +350,7 @@ struct PropResult {
     unsigned long long items = 0, arcs = 0;
 };
 size_t prop_dev_bytes();
-bool reach_pulls(long long m, int num_sms);
+bool reach_pulls(long long n, long long m, int num_sms);
 // A graph with a row of more than 64 arcs and of more than 16 times the mean
 // degree: a hub's value grows several times, and each time costs its whole row,
 // while the first SCC's bitmap searches read it once (the batched kernel draws

@@ -16,12 +16,19 @@ namespace {
 constexpr int kPropBlock = 256;
 constexpr int kPropRegions = 1024;
 constexpr int kPropWarps = kPropBlock / kWarp;
-// Quarters of an arc per thread of the chip up to which searches only pull (a pass
-// over all of them is then one hop of every path). Pulling against marking, run alone: 2D torus 524 k
-// vertices (6.7 arcs a thread) 19.7 / 21.9 ms, 3D torus 512 k (5.9) 1.35 / 1.50,
-// k-NN 200 k x 5 (6.4) 0.88 / 1.02, k-NN 400 k x 3 (7.7) 2.8 / 2.3, 3D torus 1 M
-// (11.6) 2.4 / 1.9, 2D torus 1 M (13.5) 31 / 16.
-constexpr long long kPropPull = 28, kReachPull = 28;
+// Arcs per thread up to which searches only pull (a pass over all of them is then
+// one hop of every path), pulling against marking, ms. scc_run: 2D torus 63 k vertices
+// 1.38 / 2.55, 155 k 1.35 / 1.58, 262 k 1.8 / 1.7, DAG of 131 k vertices (387 k arcs, 2.5 a
+// thread) 1.02 / 1.34, k-NN 200 k x 5 (6.4) 0.83 / 0.83, but 3D torus 262 k (472 k arcs, 3)
+// 1.18 / 0.91, 2D 423 k 3.44 / 2.11. reach_multi, 64 sources: 2D torus 262 k (3.4) 2.98 /
+// 4.44, 360 k (4.6) 4.00 / 4.27, 3D 512 k (5.9) 0.56 / 0.65, but 2D 524 k (6.7) 8.02 / 6.51,
+// k-NN 200 k x 5 0.40 / 0.30. Since warps relax narrow waves themselves (kPropNarrow)
+// marking is ahead on some graphs from 3 arcs a thread on; on others pulling still is.
+constexpr long long kPropPullArcs = 7;
+// ... in reach_multi on graphs of about one arc a vertex, long paths, above all:
+// cycles of 300 k vertices, one source and 7: 764 / 526, 337 / 526, of 524 k 1559 / 917,
+// 846 / 916 (by rounds of the engine 1233, 1244).
+constexpr long long kReachPullPath = 3;
 // Vertices from which the first batch has a head start (of at most n / 4 ns):
 // 3D torus 256^3 28 -> 11 ms with it. Below, a search is bound by its hops and
 // the wave of the head start would only come on top.
@@ -723,9 +730,11 @@ __global__ void k_prop_err(const PropCtl* c, int* err) {
 
 size_t prop_dev_bytes() { return sizeof(PropDev); }
 
-// Whether a reach_multi search of a graph without hubs only pulls (k_prop's
-// rule is in launch_prop; both launch four blocks an SM).
-bool reach_pulls(long long m, int num_sms) { return 4 * m <= kReachPull * 4 * num_sms * kPropBlock; }
+// Whether a reach_multi search of a graph without hubs only pulls (four blocks an
+// SM, as k_prop).
+bool reach_pulls(long long n, long long m, int num_sms) {
+    return m <= (4 * m < 5 * n ? kReachPullPath : kPropPullArcs) * 4 * num_sms * kPropBlock;
+}
 
 // Resident blocks per SM (the first call is outside any stream capture).
 int prop_blocks_per_sm(int* out) {
@@ -781,8 +790,8 @@ static int launch_prop(const PropArgs& a, bool hubs, cudaStream_t st) {
     SCC_TRY(prop_blocks_per_sm(&per_sm));
     const long long nw = ((long long)a.n + 31) / 32;
     const int full = per_sm * a.num_sms;
-    P.pull_arcs = (unsigned long long)(kPropPull * full * kPropBlock / 4);
     const int grid = (int)std::max<long long>(1, std::min<long long>(full, (nw + kPropWarps - 1) / kPropWarps));
+    P.pull_arcs = (unsigned long long)(kPropPullArcs * grid * kPropBlock);
     if (!hubs || !P.fresh) SCC_CUDA(cudaMemsetAsync(P.dev, 0, sizeof(PropDev), st));
     void* args[] = {(void*)&P};
     SCC_CUDA(cudaLaunchCooperativeKernel(hubs ? (const void*)k_prop_hubs : (const void*)k_prop, dim3(grid),

@@ -23,7 +23,7 @@
 // waits for a barrier: vertices whose value grew are bits of a dirty bitmap, a
 // warp owns runs of its words, polls them, takes the set bits and
 // relaxes those vertices' arcs, marking the heads it raised in whichever warp's
-// words they lie. A search ends when every block is idle at once, which a
+// words they lie; a few it relaxes at once itself (kPropNarrow). A search ends when every block is idle at once, which a
 // counter of idle blocks detects; a check of the whole bitmap between two grid
 // barriers then confirms it (a mark may lie unseen in a block that went idle
 // before it), or resumes the search.
@@ -48,6 +48,13 @@ constexpr int kPropUnroll = 4;     // arcs of a row in flight per lane
 constexpr int kPropHub = 2048;     // rows longer than this are shared by the idle warps of the grid ...
 constexpr int kPropPiece = 512;    // ... in pieces of this many arcs
 constexpr int kPropTasks = 24;     // rows shared at a time
+// So few raised vertices are relaxed at once by the warp that raised them, so many
+// times in a row: a hop through a mark is a fence, the mark, a poll, its exchange
+// and a fence more (4 us against 0.9 on a two-way path). reach_multi, ms: ladder of 1 M
+// vertices 1850 -> 790, 3D torus of 1 M 2.43 -> 1.33 (4 vertices 1.79, 8 1.53; 32 and 8
+// hops 1.40); SCC of the 3D torus 256^3 8.4 -> 6.2 (4: 7.7, 8: 7.2).
+constexpr int kPropNarrow = 32;
+constexpr int kPropHops = 32;
 constexpr int kPropTrimPasses = 3; // trimming passes at the start of a batch, at most
 constexpr uint64_t kPropIdleTimeoutNs = 20000000000ull;  // an idle block gives up when no block woke for 20 s
 
@@ -292,9 +299,10 @@ __device__ __forceinline__ void prop_queue_bits(PropQueue& Q, uint32_t& x, uint3
 // bitmap words, and calls f for them: the words are all looked at before any
 // work where the queue holds what they hold (a wave touches a few vertices in
 // each, which then share one step). Returns whether there was any. One place
-// calls f: its code is long, and copies of it cost more than they save.
-template <class T, class F>
-__device__ __forceinline__ bool prop_gather(const PropSlice& P, PropQueue& Q, T&& take, F&& f) {
+// calls f: its code is long, and copies of it cost more than they save. When no
+// bits are left, more(Q) may fill the queue with what f found.
+template <class T, class F, class M>
+__device__ __forceinline__ bool prop_gather(const PropSlice& P, PropQueue& Q, T&& take, F&& f, M&& more) {
     bool did = false;
     uint32_t x = 0, y = 0;
     long long w = 0;
@@ -315,6 +323,7 @@ __device__ __forceinline__ bool prop_gather(const PropSlice& P, PropQueue& Q, T&
         if (!left && b < P.cnt) continue;
         if (Q.cnt == 0) return did;
         prop_drain(Q, f);
+        if (!left) more(Q);
     }
 }
 // f(has, v) for the active vertices of the warp's words.
@@ -327,7 +336,7 @@ __device__ __forceinline__ void prop_for_active(const PropGraph<Op>& G, const Pr
             x = in ? G.active(w) : 0u;
             return __any_sync(kFull, x != 0) != 0;
         },
-        [&](bool has, int v, int) { f(has, v); });
+        [&](bool has, int v, int) { f(has, v); }, [](PropQueue&) {});
 }
 
 // The marks of a warp's raises, kept in shared memory until one fence covers
@@ -484,9 +493,12 @@ __device__ __noinline__ int prop_share(const PropGraph<Op> G, PropCtl* ctl, uint
 }
 
 // Spread v's value along its arcs in direction dir; all lanes of the warp call.
+// again: the vertices are those the warp has just raised. A long row among them is
+// left to the owner of its mark, where the raises of many warps meet: a star of
+// 131 k two-way arcs, 64 sources, 0.98 ms without that, 0.1 with it.
 template <class S, bool kHubs, class Op>
 __device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op, PropCtl* ctl, bool has, int v, int dir,
-                                           PropMarks& M, unsigned long long& arcs) {
+                                           bool again, PropMarks& M, unsigned long long& arcs) {
     using Val = typename Op::Val;
     constexpr int D = Op::kDirs - 1;
     const int lane = lane_id();
@@ -530,6 +542,13 @@ __device__ __forceinline__ void prop_relax(const PropGraph<Op>& G, const Op& op,
     }
     for (uint32_t bm = __ballot_sync(kFull, big); bm; bm &= bm - 1) {  // long rows by the whole warp
         const int l = __ffs(bm) - 1;
+        if (again) {
+            if (lane == l) {
+                S::fence();
+                atomicOr(&(dir ? G.d[D] : G.d[0])[v >> 5], 1u << (v & 31));
+            }
+            continue;
+        }
         const Val bst = prop_shfl(st, l);
         const int b0 = __shfl_sync(kFull, o0, l), b1 = __shfl_sync(kFull, o1, l);
         const int bdir = D ? __shfl_sync(kFull, dir, l) : 0;
@@ -868,6 +887,7 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
         PropIdle<S, kHubs> id(ctl, sh);
         uint32_t help = 0;  // rows of others to help with
         for (;;) {
+            int hops = 0;
             bool did = prop_gather(
                 P, Q,
                 [&](bool in, long long w, uint32_t& x, uint32_t& y) {
@@ -881,7 +901,16 @@ __device__ bool prop_search(const PropGraph<Op>& G, const Op op, PropCtl* ctl, P
                     items += (unsigned long long)(__popc(x) + __popc(y));
                     return __any_sync(kFull, (x | y) != 0) != 0;
                 },
-                [&](bool has, int v, int dir) { prop_relax<S, kHubs>(G, op, ctl, has, v, dir, M, arcs); });
+                [&](bool has, int v, int dir) { prop_relax<S, kHubs>(G, op, ctl, has, v, dir, hops > 0, M, arcs); },
+                [&](PropQueue& Q) {
+                    if (M.cnt > kPropNarrow || hops == kPropHops) return;
+                    ++hops;
+                    __syncwarp();
+                    if (lane < M.cnt) Q.buf[lane] = M.buf[lane];
+                    Q.cnt = M.cnt;
+                    M.cnt = 0;
+                    __syncwarp();
+                });
             if constexpr (kHubs)
                 if (help) {
                     id.wake();
