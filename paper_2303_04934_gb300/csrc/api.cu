@@ -341,6 +341,8 @@ static int reach_masks(scc_graph* h, const int32_t* dsrc, int32_t k, int32_t dir
     return run_reach(a, s);
 }
 
+void graph_set_stream(scc_graph* h, cudaStream_t s) { h->last = s; }
+
 // reach_multi with 1..128 sources already on the device: mask2 (device, two
 // words per vertex) gets bit j of vertex v (word 2 v + j / 64, bit j % 64) iff
 // sources[j] reaches v (dir 0) or v reaches sources[j] (dir 1).

@@ -454,6 +454,8 @@ int le_lists_compute(const int32_t* soff, const int32_t* sadj, int32_t n, const 
 int run_mask_fixed(const int32_t* off, const int32_t* adj, int32_t n, const int32_t* sources, int32_t k,
                    unsigned long long* mask, const EngineBuf* b, const EngineOpts& o, EngineRun* out,
                    cudaStream_t st);
+// The stream on which h's memory is freed, until a call on h names another (api.cu).
+void graph_set_stream(scc_graph* h, cudaStream_t s);
 // reach_multi with 1..128 device sources into two mask words per vertex (api.cu).
 int reach_multi_wide(scc_graph* h, const int32_t* sources_d, int32_t k, int32_t dir, unsigned long long* mask2,
                      cudaStream_t s);

@@ -646,6 +646,7 @@ SCC_API int scc_server_add_graph(scc_server_handle S, int32_t n, int64_t m, cons
     scc_handle g = nullptr;
     if (rc == SCC_OK) rc = scc_graph_create(n, m, offsets, targets, s, &g);
     if (rc == SCC_OK) rc = cuda_err(cudaStreamSynchronize(s));
+    if (g) graph_set_stream(g, S->cs);  // s ends here; the graph may be freed before any query on it
     if (s) cudaStreamDestroy(s);
     std::lock_guard<std::mutex> lk(S->mu);
     if (rc != SCC_OK) {
