@@ -14,7 +14,10 @@
  *     admitted request are uploaded at once on a copy stream, overlapping the
  *     compute of earlier units.
  *   - units, oldest request first: every admitted SCC request small enough for
- *     the batched kernel (scc_batch.h: one block per graph) joins one launch;
+ *     the batched kernel (scc_batch.h: one block per graph) joins one launch; those
+ *     without hubs run together over the whole GPU when they hold 2^17 vertices
+ *     or more and the temporaries that takes (some 60 bytes a vertex and 30 an arc)
+ *     fit under the cap as well, else a block each as the others;
  *     reachability queries on the same resident graph and direction share one
  *     reachability launch (up to 128 sources: above 64 the search carries two
  *     mask words per vertex; each query's bits are split out on the device); a

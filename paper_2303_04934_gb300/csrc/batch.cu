@@ -894,8 +894,8 @@ struct GroupPlan {
 // Vertices without hubs' worth of graphs from which a group runs them by
 // signature propagation over the whole grid (prop.cu) and not a block each: a
 // block takes a 1 M-vertex torus in 159 ms, all 128 tori of 1 k to 1 M vertices
-// together take the grid 25 ms. Below, the group's launches and 33 bytes a vertex
-// of working memory would buy little: the blocks' graphs are small.
+// together take the grid 25 ms. Below, the group's launches and 56.5 bytes a vertex
+// and 8 an arc of working memory would buy little: the blocks' graphs are small.
 constexpr long long kGroupMesh = 1ll << 17;
 
 // The grid takes the groups one after another at 2.4-3.8 ns a vertex; the blocks
@@ -1331,20 +1331,42 @@ void free_groups(GroupBufs* B, cudaStream_t s) {
     *B = GroupBufs();
 }
 
+// The largest group, and the largest of those with signature propagation.
+struct GroupMax {
+    long long ng = 0, mg = 0, np = 0, mp = 0;
+};
+GroupMax group_max(const std::vector<GroupPlan>& groups) {
+    GroupMax x;
+    for (const auto& gr : groups) {
+        x.ng = std::max(x.ng, gr.v1 - gr.v0);
+        x.mg = std::max(x.mg, gr.e1 - gr.e0);
+        if (gr.mesh_arcs >= 0) {
+            x.np = std::max(x.np, gr.v1 - gr.v0);
+            x.mp = std::max(x.mp, gr.e1 - gr.e0);
+        }
+    }
+    return x;
+}
+
+// The bytes that alloc_groups allocates.
+size_t group_bytes(const std::vector<GroupPlan>& groups, int G, long long nv, long long na) {
+    if (groups.empty()) return 0;
+    const GroupMax x = group_max(groups);
+    size_t b = 4 * (size_t)(nv + G + 1) + 4 * (size_t)(na + 1) + 2 * (size_t)(G + 1) + 8 * (size_t)(x.ng + 1) +
+               4 * (size_t)(x.mg + 8) + transpose_scratch_bytes(x.mg);
+    if (x.np > 0)
+        b += 24 * (size_t)x.np + 12 * (((size_t)x.np + 31) / 32) + 4 * prop_con_words(x.np) + 8 * (size_t)x.mp +
+             prop_dev_bytes();
+    return b + 16 * 256;  // rounding of the allocations
+}
+
 // Buffers for the plan of a batch of nv vertices and na arcs in G graphs.
 int alloc_groups(const std::vector<GroupPlan>& groups, const std::vector<unsigned char>& ok,
                  const std::vector<unsigned char>& mesh, int G, long long nv, long long na, GroupBufs* B,
                  cudaStream_t s) {
     if (groups.empty()) return SCC_OK;
-    long long ng_max = 0, mg_max = 0, np_max = 0, mp_max = 0;
-    for (const auto& gr : groups) {
-        ng_max = std::max(ng_max, gr.v1 - gr.v0);
-        mg_max = std::max(mg_max, gr.e1 - gr.e0);
-        if (gr.mesh_arcs >= 0) {
-            np_max = std::max(np_max, gr.v1 - gr.v0);
-            mp_max = std::max(mp_max, gr.e1 - gr.e0);
-        }
-    }
+    const GroupMax x = group_max(groups);
+    const long long ng_max = x.ng, mg_max = x.mg, np_max = x.np, mp_max = x.mp;
     SCC_TRY(dalloc_t(&B->gt_off, (size_t)(nv + G) + 1, s));
     SCC_TRY(dalloc_t(&B->gt_adj, (size_t)na + 1, s));
     SCC_TRY(dalloc_t(&B->gt_ok, (size_t)G + 1, s));
@@ -1694,7 +1716,7 @@ const int* batch_runner_err(const BatchRunner* r) { return r->flags + 1; }
 int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const long long* eb_h,
                          const unsigned char* hub, const long long* vbase, const long long* ebase,
                          const int32_t* offsets, const int32_t* targets, std::vector<int32_t>& order,
-                         int32_t* order_d, int32_t* out, cudaStream_t s) {
+                         int32_t* order_d, int32_t* out, const std::function<bool(size_t)>& reserve, cudaStream_t s) {
     if ((long long)order.size() > r->gcap) return SCC_ERR_INVALID_ARG;
     k_batch_reset<<<1, 1, 0, s>>>(r->flags, r->flags + 1);
     SCC_LAUNCH();
@@ -1707,7 +1729,7 @@ int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const
         plan_mesh(vb_h, eb_h, hub, G, groups, mesh);
         bool any = false;
         for (const GroupPlan& gr : groups) any = any || gr.mesh_arcs >= 0;
-        if (any) {
+        if (any && reserve(group_bytes(groups, G, vb_h[G], eb_h[G]))) {
             rc = alloc_groups(groups, ok, mesh, G, vb_h[G], eb_h[G], &B, s);
             if (rc == SCC_ERR_OOM) {  // a block for every graph, as without groups
                 free_groups(&B, s);

@@ -1,6 +1,7 @@
 // Host-side declarations shared by the library's translation units.
 #pragma once
 #include <cstdint>
+#include <functional>
 #include <vector>
 #include <cuda_runtime.h>
 
@@ -411,12 +412,11 @@ int batch_validate_each(int32_t G, long long nv, const long long* vbase, const l
 // Enqueues the SCCs of the packed graphs `order` (host, largest first; order_d:
 // device, G entries). hub (host, per graph; null: a graph is malformed and every
 // other one gets a block): graphs without hubs may run together over the
-// whole grid, with temporaries of up to batch_group_bytes.
+// whole grid, if reserve(bytes of the temporaries that takes) allows it.
 int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const long long* eb_h,
                          const unsigned char* hub, const long long* vbase, const long long* ebase,
                          const int32_t* offsets, const int32_t* targets, std::vector<int32_t>& order,
-                         int32_t* order_d, int32_t* out, cudaStream_t s);
-inline size_t batch_group_bytes(int64_t n, int64_t m) { return (size_t)(70 * n + 29 * m); }
+                         int32_t* order_d, int32_t* out, const std::function<bool(size_t)>& reserve, cudaStream_t s);
 
 // The symmetric CSR (cc.cu): soff[v] = off[v] + toff[v], row v = row v of G
 // then row v of G^T. launch_iota: a[v] = v.

@@ -155,9 +155,7 @@ struct Resident {
 // SCC holds its copy of the input, G^T and the transpose's staging, the run
 // state (labels, maxima, bitmaps), the pair tables and the hash bags.
 size_t plain_bytes(int64_t n, int64_t m) { return (size_t)(18 * m + 360 * n) + ((size_t)64 << 20); }
-size_t batched_bytes(int64_t n, int64_t m) {
-    return (size_t)(8 * (n + 1) + 4 * m + 4 * n) + 4096 + batch_group_bytes(n, m);
-}
+size_t batched_bytes(int64_t n, int64_t m) { return (size_t)(8 * (n + 1) + 4 * m + 4 * n) + 4096; }
 size_t reach_bytes(int64_t n) { return (size_t)(16 * n) + 4096; }
 
 double ms_between(Clock::time_point a, Clock::time_point b) {
@@ -444,9 +442,20 @@ void run_batched(scc_server* S, std::vector<ReqPtr>& u) {
         return (u[a]->m + u[a]->n) > (u[b]->m + u[b]->n);
     });
     const int32_t nvalid = (int32_t)order.size();
+    // what running graphs together takes is not part of their admission: it is
+    // used when there is room for it under the cap
+    size_t grouped = 0;
+    const auto reserve = [&](size_t bytes) {
+        std::lock_guard<std::mutex> lk(S->mu);
+        if (S->mem_in_use + (int64_t)bytes > S->cfg.mem_cap_bytes) return false;
+        S->mem_in_use += (int64_t)bytes;
+        S->mem_peak = std::max(S->mem_peak, S->mem_in_use);
+        grouped = bytes;
+        return true;
+    };
     if (rc == SCC_OK && nvalid > 0)
         rc = batch_runner_enqueue(S->runner, G, vb.data(), eb.data(), nvalid == G ? hub.data() : nullptr, vb_d, eb_d,
-                                  off_d, adj_d, order, ord_d, lab_d, S->cs);
+                                  off_d, adj_d, order, ord_d, lab_d, reserve, S->cs);
     if (rc == SCC_OK && nvalid == 0) *err_h = SCC_OK;
     else if (rc == SCC_OK)
         rc = cuda_err(cudaMemcpyAsync(err_h, batch_runner_err(S->runner), sizeof(int), cudaMemcpyDeviceToHost, S->cs));
@@ -465,6 +474,7 @@ void run_batched(scc_server* S, std::vector<ReqPtr>& u) {
     if (err_h) cudaFreeHost(err_h);
     {
         std::lock_guard<std::mutex> lk(S->mu);
+        S->mem_in_use -= (int64_t)grouped;  // freed: the stream has been waited for
         S->st.batched_launches++;
         S->st.batched_graphs += G;
     }
