@@ -912,9 +912,10 @@ constexpr long long kMeshMany = 128;
 // Groups of consecutive graphs (host only): greedily, as many consecutive
 // graphs as fit in max_v vertices and max_a arcs; a graph larger than either
 // limit ends the current group and belongs to none (its block builds its
-// G^T). Groups without vertices are dropped. ok[g] = 1 for the grouped graphs.
-void plan_groups(int G, const long long* vb, const long long* eb, long long max_v, long long max_a,
-                 std::vector<GroupPlan>& groups, std::vector<unsigned char>& ok) {
+// G^T), and so does one that is malformed (bad: kGraphBad, or null). Groups
+// without vertices are dropped. ok[g] = 1 for the grouped graphs.
+void plan_groups(int G, const long long* vb, const long long* eb, const unsigned char* bad, long long max_v,
+                 long long max_a, std::vector<GroupPlan>& groups, std::vector<unsigned char>& ok) {
     groups.clear();
     ok.assign((size_t)G + 1, 0);
     GroupPlan cur{0, 0, vb[0], vb[0], eb[0], eb[0]};
@@ -928,7 +929,7 @@ void plan_groups(int G, const long long* vb, const long long* eb, long long max_
     };
     for (int g = 0; g < G; ++g) {
         const long long n = vb[g + 1] - vb[g], m = eb[g + 1] - eb[g];
-        if (n > max_v || m > max_a) {
+        if (n > max_v || m > max_a || (bad && bad[g] == kGraphBad)) {
             flush(g + 1);  // the current group ends before g
             continue;
         }
@@ -1607,7 +1608,7 @@ int batch_create_impl(scc_batch* h, int32_t G, const int64_t* vbase, const int64
     // to kGroupVerts vertices and kGroupArcs arcs each; a larger graph is left
     // to its block
     std::vector<unsigned char> ok, mesh;
-    plan_groups(G, h->vb_h.data(), h->eb_h.data(), kGroupVerts, kGroupArcs, h->groups, ok);
+    plan_groups(G, h->vb_h.data(), h->eb_h.data(), nullptr, kGroupVerts, kGroupArcs, h->groups, ok);
     plan_mesh(h->vb_h.data(), h->eb_h.data(), hub.data(), G, h->groups, mesh);
     SCC_TRY(alloc_groups(h->groups, ok, mesh, G, h->nv, h->na, &h->gb, s));
     // the blocks' order: decreasing work (arcs + vertices), so long graphs start first
@@ -1689,14 +1690,14 @@ void batch_runner_destroy(BatchRunner* r, cudaStream_t s) {
     delete r;
 }
 
-// bad[g] = 1 when graph g of a packed batch is malformed, else 2 if it has hubs, else 0.
+// bad[g]: kGraphBad, kGraphHubs or 0.
 __global__ void k_batch_validate_each(int32_t G, const long long* vbase, const long long* ebase, const int32_t* off,
                                       const int32_t* adj, int32_t* indeg, int* bad) {
     for (int g = blockIdx.x; g < G; g += gridDim.x) {
         bool b, h;
         block_validate(off + vbase[g] + g, adj + ebase[g], vbase[g + 1] - vbase[g], ebase[g + 1] - ebase[g],
                        indeg + vbase[g], &b, &h);
-        if (threadIdx.x == 0) bad[g] = b ? 1 : h ? 2 : 0;
+        if (threadIdx.x == 0) bad[g] = b ? kGraphBad : h ? kGraphHubs : 0;
     }
 }
 
@@ -1722,10 +1723,10 @@ int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const
     SCC_LAUNCH();
     GroupBufs B;  // freed, stream-ordered, when the launches are enqueued
     int rc = SCC_OK;
-    if (hub) {
+    {
         std::vector<GroupPlan> groups;
         std::vector<unsigned char> ok, mesh;
-        plan_groups(G, vb_h, eb_h, kGroupVerts, kGroupArcs, groups, ok);
+        plan_groups(G, vb_h, eb_h, hub, kGroupVerts, kGroupArcs, groups, ok);
         plan_mesh(vb_h, eb_h, hub, G, groups, mesh);
         bool any = false;
         for (const GroupPlan& gr : groups) any = any || gr.mesh_arcs >= 0;
@@ -1940,7 +1941,7 @@ SCC_API int scc_debug_batch_groups(int32_t G, const int64_t* vbase, const int64_
     }
     std::vector<scc::GroupPlan> plan;
     std::vector<unsigned char> ok;
-    scc::plan_groups(G, vb.data(), eb.data(), max_vertices, max_arcs, plan, ok);
+    scc::plan_groups(G, vb.data(), eb.data(), nullptr, max_vertices, max_arcs, plan, ok);
     for (size_t k = 0; k < plan.size(); ++k) {
         groups[2 * k] = plan[k].g0;
         groups[2 * k + 1] = plan[k].g1;

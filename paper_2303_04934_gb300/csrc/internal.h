@@ -404,14 +404,15 @@ void batch_runner_destroy(BatchRunner* r, cudaStream_t s);
 bool batch_runner_fits(const BatchRunner* r, long long n, long long m);
 size_t batch_runner_bytes(const BatchRunner* r);
 const int* batch_runner_err(const BatchRunner* r);  // device error flag of the last launch
-// bad[g] (device int[G]) = 1 when graph g of a packed batch is malformed, else 2
-// when it has hubs in either direction (or 8 arcs a vertex), else 0. indeg: nv
-// words of scratch (nv: the batch's vertices).
+// bad[g] (device int[G]) = kGraphBad when graph g of a packed batch is malformed,
+// else kGraphHubs when it has hubs in either direction (or 8 arcs a vertex),
+// else 0. indeg: nv words of scratch (nv: the batch's vertices).
+enum { kGraphHubs = 1, kGraphBad = 2 };
 int batch_validate_each(int32_t G, long long nv, const long long* vbase, const long long* ebase,
                         const int32_t* offsets, const int32_t* targets, int32_t* indeg, int* bad, cudaStream_t s);
 // Enqueues the SCCs of the packed graphs `order` (host, largest first; order_d:
-// device, G entries). hub (host, per graph; null: a graph is malformed and every
-// other one gets a block): graphs without hubs may run together over the
+// device, G entries), the malformed ones not among them. hub (host, per graph:
+// what batch_validate_each found): graphs without hubs may run together over the
 // whole grid, if reserve(bytes of the temporaries that takes) allows it.
 int batch_runner_enqueue(BatchRunner* r, int32_t G, const long long* vb_h, const long long* eb_h,
                          const unsigned char* hub, const long long* vbase, const long long* ebase,

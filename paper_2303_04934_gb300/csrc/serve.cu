@@ -434,8 +434,8 @@ void run_batched(scc_server* S, std::vector<ReqPtr>& u) {
     std::vector<int32_t> order;
     std::vector<unsigned char> hub(G, 0);
     for (int32_t g = 0; g < G; ++g) {
-        hub[g] = bad[g] == 2;
-        bad[g] &= 1;
+        hub[g] = (unsigned char)bad[g];
+        bad[g] = bad[g] == kGraphBad;
         if (!bad[g]) order.push_back(g);
     }
     std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
@@ -454,7 +454,7 @@ void run_batched(scc_server* S, std::vector<ReqPtr>& u) {
         return true;
     };
     if (rc == SCC_OK && nvalid > 0)
-        rc = batch_runner_enqueue(S->runner, G, vb.data(), eb.data(), nvalid == G ? hub.data() : nullptr, vb_d, eb_d,
+        rc = batch_runner_enqueue(S->runner, G, vb.data(), eb.data(), hub.data(), vb_d, eb_d,
                                   off_d, adj_d, order, ord_d, lab_d, reserve, S->cs);
     if (rc == SCC_OK && nvalid == 0) *err_h = SCC_OK;
     else if (rc == SCC_OK)
