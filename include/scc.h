@@ -283,7 +283,9 @@ SCC_API int cc_get_stats(scc_handle h, scc_cc_stats* out);
  * the last entry is v itself at distance 0.
  * le_lists_run computes the lists and keeps them with the handle (replacing
  * earlier ones); *total (host) receives the number of entries. The first call
- * on h builds the symmetric CSR that cc_run also uses. Synchronises `stream`.
+ * on h builds the symmetric CSR (each vertex's out-arcs, then its in-arcs) and
+ * keeps it with the handle; SCC_ERR_CAPACITY if that has more than 2^31 - 1
+ * entries (2 m_t). Synchronises `stream`.
  */
 SCC_API int le_lists_run(scc_handle h, int64_t* total, void* stream);
 /*

@@ -913,6 +913,7 @@ int reach_multi_noalloc(scc_handle h, const int32_t* sources, int32_t k, int32_t
 // LE-lists, built on the first call and kept with the handle.
 static int ensure_sym(scc_graph* h, cudaStream_t s) {
     if (h->soff) return SCC_OK;
+    if (2 * h->mt > (int64_t)INT32_MAX) return SCC_ERR_CAPACITY;  // its offsets are 32-bit
     const int32_t n = h->n;
     int32_t *so = nullptr, *sa = nullptr;
     SCC_TRY(dalloc_t(&so, (size_t)n + 1, s));
