@@ -642,50 +642,27 @@ def _extra_graph(name, scc, torch, stream, steps, warmup, cpu):
     if spec["kind"] == "torus" and spec["dims"] == 2:
         out["note"] = "L2-resident (about 1.3 MB of CSR): a bandwidth fraction is not meaningful"
     # the run's algorithmic bytes, counted as for the benchmark graph (8 B per
-    # arc examined, 8 B per item expanded or value raised, 20 B per
-    # active vertex per labelling), over the run's mean time (create excluded)
+    # arc examined, 8 B per item expanded or value spread, 20 B per untrimmed
+    # vertex labelled), over the run's mean time (create excluded)
     last = sts[-1]
     E = last["engine_arcs"] + last["multi_arcs"]
     P = last["engine_items"] + last["multi_items"]
-    act = (g.n - last["n_trimmed"]) + last["multi_active_sum"]
+    act = g.n - last["n_trimmed"]
     run_bytes = 8 * E + 8 * P + 20 * act
     run_ms = sum(out["run_ms"].values())
     peak = float(_read_peaks().get("hbm_gbs", 6800.0))
-    out["run_roofline"] = {"bound": "hbm", "bytes_formula": "8 E + 8 P + 20 sum(active per labelling)",
-                           "E_arcs": E, "P_items": P, "active_labelled": act,
-                           "algorithmic_bytes": run_bytes, "run_ms": run_ms,
-                           "achieved_gbs": run_bytes / (run_ms / 1e3) / 1e9 if run_ms > 0 else None,
-                           "frac": run_bytes / (run_ms / 1e3) / 1e9 / peak if run_ms > 0 else None, "peak": peak,
-                           "rounds": last["search_rounds"],
-                           "note": "latency-bound rounds: the time follows the rounds, not the bytes"}
+    if last["engine_launches"] == 0:  # one launch, whose pulling passes count no arcs
+        out["run_roofline"] = {"bound": "latency", "run_ms": run_ms,
+                               "note": "one launch of searches bound by their hops; no byte count"}
+    else:
+        out["run_roofline"] = {"bound": "hbm", "bytes_formula": "8 E + 8 P + 20 (untrimmed vertices)",
+                               "E_arcs": E, "P_items": P, "active_labelled": act,
+                               "algorithmic_bytes": run_bytes, "run_ms": run_ms,
+                               "achieved_gbs": run_bytes / (run_ms / 1e3) / 1e9 if run_ms > 0 else None,
+                               "frac": run_bytes / (run_ms / 1e3) / 1e9 / peak if run_ms > 0 else None, "peak": peak,
+                               "rounds": last["search_rounds"],
+                               "note": "latency-bound rounds: the time follows the rounds, not the bytes"}
     out["connectivity"] = _measure_cc(g, off_d, adj_d, scc, torch, stream, 5, 2, cpu)
-    if spec["kind"] == "knn":
-        # the hash bag of Sec. 3.3 (sampled, sigma = 50) against a reservation bag
-        # (sigma = 0: one counter hands out segments), on the multi-reachability
-        # heavy graph; scc_run alone on a built graph
-        abl = {}
-        h = scc.scc_graph_create(g.n, g.m, off_d, adj_d, stream)
-        try:
-            for name, sig in (("sampled_sigma50", 50), ("reservation", 0)):
-                c = scc.scc_config_default()
-                c.sigma = sig
-                scc.scc_set_config(h, c)
-                ts = []
-                for rep in range(3):
-                    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                    with torch.cuda.stream(stream):
-                        e0.record(stream)
-                        scc.scc_run(h, lab, stream)
-                        e1.record(stream)
-                    torch.cuda.synchronize()
-                    if rep:
-                        ts.append(e0.elapsed_time(e1))
-                st = scc.scc_get_stats(h)
-                abl[name] = {"scc_run_ms": sum(ts) / len(ts), "rounds": st["search_rounds"],
-                             "ms_multi_search": st["ms_multi_search"], "pairs": st["pairs"]}
-        finally:
-            scc.scc_graph_destroy(h)
-        out["bag_ablation"] = abl
     if cpu:
         tc = time_oracle(g)
         out["cpu_baseline"] = {"value": g.m / tc, "unit": UNIT, "cores": 1, "kind": "oracle",
@@ -693,6 +670,37 @@ def _extra_graph(name, scc, torch, stream, steps, warmup, cpu):
         out["gpu_over_oracle"] = (g.m / (ms / 1e3)) / (g.m / tc)
     del off_d, adj_d, lab
     return out
+
+
+def _bag_ablation(g, off_d, adj_d, scc, torch, stream):
+    """The hash bag of Sec. 3.3 (sampled, sigma = 50) against a reservation bag
+    (sigma = 0: one counter hands out segments) in the first SCC's searches, the
+    part of scc_run that has a bag frontier; on a built graph."""
+    abl = {}
+    lab = torch.empty(g.n, dtype=torch.int32, device="cuda")
+    h = scc.scc_graph_create(g.n, g.m, off_d, adj_d, stream)
+    try:
+        for name, sig in (("sampled_sigma50", 50), ("reservation", 0)):
+            c = scc.scc_config_default()
+            c.sigma = sig
+            scc.scc_set_config(h, c)
+            ts, engine = [], []
+            for rep in range(6):
+                e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                with torch.cuda.stream(stream):
+                    e0.record(stream)
+                    scc.scc_run(h, lab, stream)
+                    e1.record(stream)
+                torch.cuda.synchronize()
+                if rep:
+                    ts.append(e0.elapsed_time(e1))
+                    engine.append(scc.scc_get_stats(h)["ms_engine"])
+            st = scc.scc_get_stats(h)
+            abl[name] = {"scc_run_ms": sum(ts) / len(ts), "rounds": st["search_rounds"],
+                         "ms_engine": sum(engine) / len(engine)}
+    finally:
+        scc.scc_graph_destroy(h)
+    return abl
 
 
 def _measure_cc(g, off_d, adj_d, scc, torch, stream, steps, warmup, cpu):
@@ -1080,7 +1088,7 @@ def main():
             sum(s["ms_transpose_part"] for s in stats), len(stats), len(stats) * (10 * m + 4 * n)),
         "k_copy_check_hist (intake: copy, range check, bucket histogram)": (
             sum(s["ms_transpose_hist"] for s in stats), len(stats), len(stats) * (8 * m)),
-        "k_prop (signature propagation)": (
+        "k_prop (signature propagation; its marking searches' arcs alone are counted)": (
             sum(s["ms_multi_search"] for s in stats), sum(s["multi_launches"] for s in stats),
             sum(8 * s["multi_arcs"] + 8 * s["multi_items"] for s in stats)),
     }
@@ -1181,15 +1189,15 @@ def main():
     line["split_ms"] = {"create": evs[0].elapsed_time(evs[1]), "run": t_run, "destroy": evs[2].elapsed_time(evs[3])}
     # the whole run's algorithmic bytes (counted from the run's own counters):
     # 4 B target + 4 B label or visited word per arc examined, 8 B row offsets
-    # per item expanded or value raised, 20 B per active vertex per labelling
-    # (the first SCC's, over the untrimmed vertices); the step adds the transpose
+    # per item expanded or value spread, 20 B per untrimmed vertex (the first
+    # SCC's labelling); the step adds the transpose
     # build's 12m + 12n
     E = last["engine_arcs"] + last["multi_arcs"]
     P = last["engine_items"] + last["multi_items"]
-    act = (n - last["n_trimmed"]) + last["multi_active_sum"]
+    act = n - last["n_trimmed"]
     run_bytes = 8 * E + 8 * P + 20 * act
     line["run_roofline"] = {
-        "bound": "hbm", "bytes_formula": "8 E + 8 P + 20 sum(active per labelling)",
+        "bound": "hbm", "bytes_formula": "8 E + 8 P + 20 (untrimmed vertices)",
         "E_arcs": E, "P_items": P, "active_labelled": act, "algorithmic_bytes": run_bytes,
         "scc_run_ms": t_run, "achieved_gbs": run_bytes / (t_run / 1e3) / 1e9 if t_run > 0 else None,
         "frac": run_bytes / (t_run / 1e3) / 1e9 / hbm_peak if t_run > 0 else None, "peak": hbm_peak,
@@ -1207,6 +1215,7 @@ def main():
             and not args.rmat_ef):
         t_x = time.perf_counter()
         line["connectivity"] = _measure_cc(g, off_d, adj_d, scc, torch, stream, 5, 2, not args.no_cpu_baseline)
+        line["bag_ablation"] = _bag_ablation(g, off_d, adj_d, scc, torch, stream)
         del off_d, adj_d, labels_d
         torch.cuda.synchronize()
         cpu_x = not args.no_cpu_baseline
