@@ -208,9 +208,10 @@ SCC_API int reach_multi_noalloc(scc_handle h, const int32_t* sources, int32_t k,
 typedef struct scc_stats {
     int32_t n_trimmed;         /* vertices removed by trimming */
     int32_t first_scc_size;    /* size of the SCC of the first pivot */
-    int32_t batches;           /* batches run (including the first pivot's) */
+    int32_t batches;           /* batches run (with the first pivot's, where its SCC is searched for alone) */
     int32_t search_rounds;     /* rounds of the first SCC's searches, and searches of the later batches */
-    int64_t pairs;             /* times the later batches raised a vertex's largest source */
+    int64_t pairs;             /* work of the later batches' searches: values raised by passes that pull,
+                                  marks taken by searches that mark (depends on their timing) */
     int32_t table_resizes;     /* 0 (no pair table is kept) */
     int32_t engine_launches;   /* launches of the reachability engine kernel */
     double ms_trim, ms_first_scc, ms_multi_search, ms_resize, ms_label;
@@ -231,7 +232,7 @@ typedef struct scc_stats {
     double ms_class_trim;
     /* the launch of the later batches */
     int32_t multi_launches;
-    int64_t multi_arcs;        /* arcs followed from raised vertices */
+    int64_t multi_arcs;        /* arcs followed by searches that mark (passes that pull count none) */
     int64_t multi_items;       /* the same count as pairs */
     int32_t tau;               /* the VGC edge budget used (config tau, or the automatic one) */
     double ms_transpose_split; /* transpose: buckets cut into sub-buckets (ms_transpose_rows: their rows) */

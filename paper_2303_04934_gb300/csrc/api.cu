@@ -56,7 +56,7 @@ struct scc_graph {
     uint64_t idle_ns = 0;  // scc_debug_idle_limit (0: the library's own)
     int32_t run_form = 0, reach_form = 0;  // kForm* of the last scc_run and reach_multi
     double create_ms[5] = {0, 0, 0, 0, 0};  // total, histogram, partition, rows, split
-    // connectivity: the symmetric CSR (built on the first cc_run) and its stats
+    // the symmetric CSR (built on the first le_lists_run), the stats of cc_run
     int32_t* soff = nullptr;
     int32_t* sadj = nullptr;
     scc_cc_stats cc_stats;
@@ -768,7 +768,6 @@ static int scc_run_impl(scc_graph* h, int32_t* labels_out, cudaStream_t s) {
             if (host_out) SCC_CUDA(cudaMemcpyAsync(labels_out, dst, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost, s));
             st.n_trimmed = (int32_t)(n - r.active);
             st.first_scc_size = r.first;
-            st.batches = 1;
             st.ms_multi_search = tp.stop();
             prop_stats(r, &st);
             return SCC_OK;
