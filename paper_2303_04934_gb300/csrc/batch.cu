@@ -898,16 +898,16 @@ struct GroupPlan {
 // and 8 an arc of working memory would buy little: the blocks' graphs are small.
 constexpr long long kGroupMesh = 1ll << 17;
 
-// The grid takes the groups one after another at 2.4-3.8 ns a vertex; the blocks
-// take all graphs at once at about 1.2, but their span is at least the largest
-// graph's time alone, 0.19 us a vertex. So a batch whose graphs without hubs hold
-// more than kMeshMany times the vertices of the largest of them, and more than a
-// group, goes to the blocks (ms, grid against blocks; graphs, half of them tori,
-// log-uniform from 1 k to the size given): 256 to 1 M (ratio 21) 79 / 193, 1024 to
-// 1 M (74) 224 / 256, 2048 to 300 k (173) 135 / 116, 4096 to 1 M (304) 950 / 550.
-// Within a group's vertices the grid is ahead at any ratio: 1024 to 10 k (2 M
-// vertices) 5.3 / 14, to 100 k (11 M) 26 / 45.
-constexpr long long kMeshMany = 128;
+// The grid takes the groups one after another at 0.8-1.3 ns a vertex; the blocks
+// take all graphs at once at 0.9-2.7, the less the larger the graphs, but their
+// span is at least the largest graph's time alone, 0.19 us a vertex. So a batch
+// whose graphs without hubs hold more than kMeshMany times the vertices of the
+// largest of them, which has kMeshLarge or more, goes to the blocks (ms, grid
+// against blocks; graphs, half of them tori, log-uniform from 1 k to the size
+// given): 256 to 1 M (ratio 21) 53 / 226, 1024 to 1 M (74) 156 / 242, 2048 to 1 M (150)
+// 330 / 304, 4096 to 1 M (304) 661 / 555, but 2048 to 300 k (173) 98 / 120, 4096 to 300 k
+// (350) 204 / 239, 16384 to 10 k (3200) 55 / 170, 1024 to 100 k 19 / 38.
+constexpr long long kMeshMany = 128, kMeshLarge = 1ll << 19;
 
 // Groups of consecutive graphs (host only): greedily, as many consecutive
 // graphs as fit in max_v vertices and max_a arcs; a graph larger than either
@@ -954,7 +954,7 @@ void plan_mesh(const long long* vb, const long long* eb, const unsigned char* hu
                 all += vb[g + 1] - vb[g];
                 most = std::max(most, vb[g + 1] - vb[g]);
             }
-    const bool many = all > kGroupVerts && all > kMeshMany * most;
+    const bool many = all > kMeshMany * most && most >= kMeshLarge;
     for (GroupPlan& gr : groups) {
         long long v = 0, a = 0;
         for (int g = gr.g0; g < gr.g1; ++g)
