@@ -1,16 +1,19 @@
-// Batched SCC (sm_103a): many independent graphs in one persistent launch.
+// Batched SCC (sm_103a): many independent graphs, those without hubs together over
+// the whole grid, the others in one persistent launch, a block each.
 //
-// Each thread block takes the next graph from a device work queue (graphs in
-// decreasing size, so the longest ones start first) and runs the whole method
+// Consecutive graphs form groups of up to 2^24 vertices (plan_groups), each one
+// graph of disjoint parts for the grid-wide transpose of transpose.cu. Where
+// its graphs without hubs hold enough vertices (plan_mesh), the group's are run
+// as one graph by signature propagation (prop.cu), whose searches are bound by
+// the longest path, not by their number. Then, in the persistent launch, each
+// thread block takes the next of the other graphs from a device work queue
+// (in decreasing size, so the longest ones start first) and runs the whole method
 // on it alone, with __syncthreads between rounds (CtaScope of engine.cuh):
 //
 //   1. G^T of the graph (Sec. 2: a backward search is a forward search on
-//      G^T). A run through a batch handle computes it before the persistent
-//      launch for groups of consecutive graphs at once (each group, up to 2^24
-//      vertices, is one graph of disjoint parts for the grid-wide transpose of
-//      transpose.cu), and a block only points at its graph's part; graphs
-//      outside the groups (and the server's launches) build it in the block:
-//      in-degree counts, a block scan, placement.
+//      G^T): a block points at its graph's part of the group's; for graphs
+//      outside the groups, and the server's units without a group for the grid,
+//      it is built in the block: in-degree counts, a block scan, placement.
 //   2. Trimming (Sec. 4.1): vertices without in- or out-arcs are singletons.
 //   3. The pivot order: a seeded Feistel permutation of the active vertices.
 //   4. Single-pivot steps (Sec. 4.2): the first pivot's SCC by forward and
@@ -33,9 +36,9 @@
 //
 // The working memory of a block (transpose, labels, tables, hash bag, engine
 // control) is a fixed slice of one device allocation, sized for the largest
-// graph of the batch; nothing is allocated during a run, so the host captures
-// the launch (a reset kernel and the persistent kernel) as a CUDA graph once
-// and replays it.
+// graph left to the blocks; nothing is allocated during a run, so the host captures
+// its launches (a reset kernel, the groups', the persistent kernel) as a CUDA
+// graph once and replays it.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -894,7 +897,7 @@ struct GroupPlan {
 // Vertices without hubs' worth of graphs from which a group runs them by
 // signature propagation over the whole grid (prop.cu) and not a block each: a
 // block takes a 1 M-vertex torus in 159 ms, all 128 tori of 1 k to 1 M vertices
-// together take the grid 25 ms. Below, the group's launches and 56.5 bytes a vertex
+// together take the grid some 20 ms a group. Below, the group's launches and 56.5 bytes a vertex
 // and 8 an arc of working memory would buy little: the blocks' graphs are small.
 constexpr long long kGroupMesh = 1ll << 17;
 

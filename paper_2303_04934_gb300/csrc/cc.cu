@@ -17,6 +17,11 @@
 //      more than kCcRow arcs are cut into pieces of kCcPiece for k_cc_big.
 //   4. labels_out[v] = the root of v (k_cc_labels).
 //
+// Joining a few sampled neighbours of each vertex, taking the most frequent root
+// of 1024 probes for the large component and skipping its vertices afterwards is
+// Afforest (Sutton, Ben-Nun, Barak, IPDPS 2018); the passes by atomicMin and their
+// flattening are this file's.
+//
 // The paper's LDD-UF-JTB (Alg. 4) takes the same labels from a low-diameter
 // decomposition of the symmetrised graph, a search of tens of rounds, and then
 // tests every arc for joining two clusters. On R-MAT with 4.2 M vertices and

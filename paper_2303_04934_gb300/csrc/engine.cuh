@@ -183,7 +183,6 @@ struct CtaScope {
         return true;
     }
     __device__ __forceinline__ static int32_t ld(const int32_t* p) { return *p; }
-    __device__ __forceinline__ static void fence() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 };
 
 // adjacency arrays of an item's graph

@@ -166,11 +166,11 @@ void transpose_scratch_carve(unsigned char* base, int64_t m_max, TransposeScratc
 int launch_transpose_keep_self(const int32_t* off, const int32_t* adj, int32_t n, int64_t m, const TransposeScratch& ts,
                                int32_t* toff, int32_t* tadj, int num_sms, cudaStream_t s);
 int transpose_set_attributes();
-// Direct G^T for very large n: global atomics. indeg: n + 1.
 // A small graph's intake and transposition in one launch (out: three ints, see k_small_graph).
 bool small_graph(int32_t n, int64_t m);
 int launch_small_graph(const int32_t* off_src, const int32_t* adj_src, int32_t n, int64_t m, int32_t* off, int32_t* adj,
                        int32_t* toff, int32_t* tadj, int* out, cudaStream_t s);
+// Direct G^T for very large n: global atomics. indeg: n + 1.
 int launch_transpose_direct(const int32_t* off, const int32_t* adj, const int32_t* trow, int32_t n, int64_t m,
                             int32_t* indeg, void* scan_tmp, int32_t* toff, int32_t* tadj, int num_sms,
                             cudaStream_t s);

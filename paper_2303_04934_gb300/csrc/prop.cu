@@ -1,8 +1,6 @@
 // The whole SCC of a graph without hubs in one cooperative launch, and the
 // batches that remain after the first SCC of a graph with hubs (prop.cuh).
 #include <algorithm>
-#include <cstdio>
-#include <cstdlib>
 #include <cstring>
 
 #include "common.cuh"
@@ -197,8 +195,13 @@ constexpr unsigned kConSample = 16;  // one word in so many
 // x 5) keeps 3,845 nodes with 8 arcs each, most of them at a few large clusters,
 // whose rows a pull reads in every pass (first batch 407 against 242 us).
 constexpr unsigned kConPullRow = 4;
-// Vertices from which a graph is contracted: the passes take 50-70 us on small
-// ones (2D torus 33^2: 125 us without, 180 with; 256^2: 1.05 ms against 0.79-1.07).
+// Vertices from which a graph is contracted: the passes take 50-110 us on small
+// ones, which critical lattices get back early and others late. The run with it /
+// without, us, at 8 k, 16 k, 33 k, 50 k, 66 k and 90 k vertices: 2D torus p = 0.5 347 /
+// 326, 419 / 462, 620 / 735, 749 / 830, 766 / 1057, 1135 / 1542; p = 0.65 197 / 119, 216 /
+// 143, 245 / 173, 266 / 205, 284 / 233, 306 / 276; k-NN k = 5 212 / 177, 243 / 186, 294 /
+// 221, 331 / 310, 358 / 325, 396 / 431; k = 3 231 / 237, 288 / 313, 356 / 356, 389 / 518, 421
+// / 612, 462 / 807; graphs that are tried and not contracted +2%.
 constexpr int kConMin = 1 << 16;
 
 template <class S>

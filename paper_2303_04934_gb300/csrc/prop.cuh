@@ -23,17 +23,18 @@
 // waits for a barrier: vertices whose value grew are bits of a dirty bitmap, a
 // warp owns runs of its words, polls them, takes the set bits and
 // relaxes those vertices' arcs, marking the heads it raised in whichever warp's
-// words they lie; a few it relaxes at once itself (kPropNarrow). A search ends when every block is idle at once, which a
-// counter of idle blocks detects; a check of the whole bitmap between two grid
-// barriers then confirms it (a mark may lie unseen in a block that went idle
-// before it), or resumes the search.
+// words they lie; a few it relaxes at once itself (kPropNarrow), and a hub's row
+// is shared by the idle warps (prop_share). A search ends when every block is idle
+// at once, which a counter of idle blocks detects; a check of the whole bitmap
+// between two grid barriers then confirms it (a mark may lie unseen in a block that
+// went idle before it), or resumes the search.
 //
 // Measured against batches of doubling size whose searches kept every pair (the
 // whole create + run + destroy, GB300): 2D torus 33^2 1.37 -> 0.24 ms, 256^2
-// 11.8 -> 1.15, k-NN of 1 M points 12.2 -> 1.5, 3D torus 256^3 12.8 -> 8.5
-// (41 -> 8.5 when the first pivot misses the giant SCC). Of 8.5 ms the head
-// start takes 4.2: its wave is a few vertices per warp wide, so it is bound by
-// the time of a hop (about 20 us there), not by traffic.
+// 11.8 -> 1.15, k-NN of 1 M points 12.2 -> 1.5, 3D torus 256^3 12.8 -> 6.4
+// (41 -> 6.4 when the first pivot misses the giant SCC), about half of which is
+// the head start: its wave is a few vertices per warp wide, so it is bound by the
+// time of a hop, not by traffic.
 #pragma once
 #include "common.cuh"
 #include "engine.cuh"

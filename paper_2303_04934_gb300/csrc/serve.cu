@@ -152,8 +152,10 @@ struct Resident {
 };
 
 // Device bytes a request may hold while admitted (upper estimates). A full-GPU
-// SCC holds its copy of the input, G^T and the transpose's staging, the run
-// state (labels, maxima, bitmaps), the pair tables and the hash bags.
+// SCC holds its copy of the input and G^T (8 n + 8 m), then first the transpose's
+// staging (some 12 m), which is freed before the run state (42 n: labels, values,
+// bitmaps), the contraction's arrays (32 n + 8 m) or the hash bags of the first
+// SCC's searches; the rest covers the pool's reuse of freed blocks.
 size_t plain_bytes(int64_t n, int64_t m) { return (size_t)(18 * m + 360 * n) + ((size_t)64 << 20); }
 size_t batched_bytes(int64_t n, int64_t m) { return (size_t)(8 * (n + 1) + 4 * m + 4 * n) + 4096; }
 size_t reach_bytes(int64_t n) { return (size_t)(16 * n) + 4096; }
