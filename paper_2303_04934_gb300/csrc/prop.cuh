@@ -46,7 +46,7 @@ constexpr int kPropQueue = 256;    // vertices a warp gathers before it works on
 constexpr int kPropMarks = 384;    // marks a warp gathers before it publishes them
 constexpr int kPropBigRow = 64;    // rows longer than this are relaxed by the whole warp
 constexpr int kPropUnroll = 4;     // arcs of a row in flight per lane
-constexpr int kPropHub = 2048;     // rows longer than this are shared by the idle warps of the grid ...
+constexpr int kPropHub = 4096;     // rows longer than this are shared by the idle warps of the grid ...
 constexpr int kPropPiece = 512;    // ... in pieces of this many arcs
 constexpr int kPropTasks = 24;     // rows shared at a time
 // So few raised vertices are relaxed at once by the warp that raised them, so many
@@ -443,8 +443,9 @@ __device__ __forceinline__ void prop_relax_row(const PropGraph<Op>& G, const typ
 // such rows are compiled with it (kHubs): lattices lost 4-6% to its registers.
 // One call, 64 sources, GB300, by one warp against shared: a star of 1 M two-way
 // arcs 24.3 -> 0.13 ms, 16 stars of 65 k 13.5 -> 0.30; SCC of the 16 stars 49.7 ->
-// 2.0 ms. Bound and piece (there, SCC): 8192 and 2048 2.65 ms, 2048 and 1024 2.17,
-// 2048 and 256 2.02; rows of 1 k are as fast by a warp of their own.
+// 2.0 ms; pieces of 1024 there 2.2, of 256 2.0. The bound: a contracted k-NN graph of
+// 1 M points has rows of up to 3.3 k arcs, which cost its run 1089 -> 1146 us when
+// shared, and one of a 2D torus 700^2 with p = 0.7 rows of 8 k, 629 -> 525.
 template <class S, class Op>
 __device__ __noinline__ int prop_share(const PropGraph<Op> G, PropCtl* ctl, uint32_t put, uint32_t slots, uint32_t* mk,
                                        int cnt) {
@@ -1118,20 +1119,34 @@ __device__ __noinline__ bool prop_batches(const PropGraph<PropMax> G, const Prop
                     i0 = S::ld(&G.off[1][v]);
                     i1 = S::ld(&G.end[1][v]);
                 }
-                const bool big = o1 - o0 > kPropBigRow || i1 - i0 > kPropBigRow;
                 // a hub is left to the searches, which share its row
                 const bool is_hub = kHubs && max(o1 - o0, i1 - i0) > kPropHub;
-                bool stays = is_hub || has && !big && prop_any_in_class<S, 1>(G.adj[0], o0, o1, sf, lab, v) &&
-                             prop_any_in_class<S, 1>(G.adj[1], i0, i1, sf, lab, v);
-                // long rows by the whole warp: if the neighbours have all left
-                // the class, a row is read to its end
-                for (uint32_t bm = __ballot_sync(kFull, big && !is_hub); bm; bm &= bm - 1) {
+                // a thread looks at the first arcs of its rows, where most have a
+                // neighbour in the class; the rest of a long row without one there
+                // is read by the whole warp (rows of more than 64 arcs by the warp
+                // from the start: k-NN of 300 k points 545 -> 590 us a run)
+                const int oe = o0 + min(o1 - o0, kPropBigRow), ie = i0 + min(i1 - i0, kPropBigRow);
+                bool more0 = false, more1 = false;
+                bool stays = is_hub;
+                if (has && !is_hub) {
+                    stays = prop_any_in_class<S, 1>(G.adj[0], o0, oe, sf, lab, v);
+                    more0 = !stays && oe < o1;
+                    if (stays || more0) {
+                        stays = prop_any_in_class<S, 1>(G.adj[1], i0, ie, sf, lab, v);
+                        more1 = !stays && ie < i1;
+                        stays = stays || more1;
+                    }
+                }
+                for (uint32_t bm = __ballot_sync(kFull, stays && (more0 || more1)); bm; bm &= bm - 1) {
                     const int l = __ffs(bm) - 1, hv = __shfl_sync(kFull, v, l);
                     const uint32_t hl = __shfl_sync(kFull, lab, l);
-                    const bool in = prop_any_in_class<S, 32>(G.adj[0], __shfl_sync(kFull, o0, l),
-                                                             __shfl_sync(kFull, o1, l), sf, hl, hv) &&
-                                    prop_any_in_class<S, 32>(G.adj[1], __shfl_sync(kFull, i0, l),
-                                                             __shfl_sync(kFull, i1, l), sf, hl, hv);
+                    bool in = true;
+                    if (__shfl_sync(kFull, (int)more0, l))
+                        in = prop_any_in_class<S, 32>(G.adj[0], __shfl_sync(kFull, oe, l), __shfl_sync(kFull, o1, l), sf,
+                                                      hl, hv);
+                    if (in && __shfl_sync(kFull, (int)more1, l))
+                        in = prop_any_in_class<S, 32>(G.adj[1], __shfl_sync(kFull, ie, l), __shfl_sync(kFull, i1, l), sf,
+                                                      hl, hv);
                     if (lane == l) stays = in;
                 }
                 if (!has || stays) return;

@@ -65,10 +65,10 @@ def _stars(n, k, two_way=True, into=False):
     return _csr(n, p[np.concatenate(src)], p[np.concatenate(dst)], f"stars{k}_{two_way}_{into}")
 
 
-# rows just below, at and above the bound from which they are shared (2048 arcs), pieces (512) and their remainders,
-# more shared rows than there are slots (32), and one row of everything
-@pytest.mark.parametrize("n, k", [(2049, 1), (2050, 1), (2051, 1), (2052, 1), (2600, 1), (5000, 2), (40000, 7),
-                                  (200_000, 64), (600_000, 200), (1_000_000, 3), (3_000_000, 1)])
+# rows just below, at and above the bound from which they are shared (4096 arcs), pieces (512) and their remainders,
+# more shared rows than there are slots (24), and one row of everything
+@pytest.mark.parametrize("n, k", [(2050, 1), (4096, 1), (4097, 1), (4098, 1), (4099, 1), (4100, 1), (4700, 1), (10000, 2),
+                                  (40000, 7), (300_000, 64), (900_000, 200), (1_000_000, 3), (3_000_000, 1)])
 @pytest.mark.parametrize("two_way, into", [(True, False), (False, False), (False, True)])
 def test_stars(n, k, two_way, into):
     g = _stars(n, k, two_way, into)
@@ -105,3 +105,30 @@ def test_giant_nodes_of_a_contracted_graph(n, k, extra):
         for _ in range(2):
             assert np.array_equal(labels_of(G), want), g.name
         assert scc.scc_debug_forms(G.h)[0] == scc.FORM_CONTRACTED
+
+
+@pytest.mark.parametrize("deg", [62, 63, 64, 65, 66, 128, 300, 1000])
+@pytest.mark.parametrize("into", [False, True])
+def test_trimming_around_the_first_arcs_of_a_row(deg, into):
+    """Vertices on cycles of two whose rows (long in either direction) begin with trimmed leaves, with the other vertex
+    of the cycle before, at and past the 64 arcs that a thread looks at, and chains of two that do get trimmed; the
+    first SCC is a dense ring."""
+    ring, k = 20000, 40
+    i = np.arange(ring)
+    src, dst = [i, i], [(i + 1) % ring, (i + 7) % ring]
+    at = ring
+    for j in range(k):
+        a, b = at, at + 1
+        leaf = np.arange(at + 2, at + 2 + deg)
+        pos = (j * 7) % (deg + 1)
+        row = np.insert(leaf, pos, b)  # b among the leaves
+        src += [np.full(len(row), a), [b]] if not into else [row, [a]]
+        dst += [row, [a]] if not into else [np.full(len(row), a), [b]]
+        if j % 3 == 0:  # without the way back: a chain
+            src.pop()
+            dst.pop()
+        at += 2 + deg
+    g = _csr(at, np.concatenate([np.asarray(x) for x in src]), np.concatenate([np.asarray(x) for x in dst]), "first_arcs")
+    want, _ = oracle.scc_labels(g.n, g.offsets, g.targets)
+    with make_graph(g) as G:
+        assert np.array_equal(labels_of(G), want)
