@@ -289,12 +289,12 @@ struct EvTimer {
 namespace scc {
 
 // Arcs from which reach_multi on a graph of high degree with hubs starts with the
-// hub's own two sets: those cost 0.8-1.5 ms whatever the size (their rounds are
-// bound by latency), the masks alone about 0.04 ms a million arcs. Masks alone
-// against the hub first, R-MAT of edge factor 16, 64 sources: 1 M vertices 0.87 /
-// 0.84 ms, 2 M 1.51 / 1.01, 4 M 2.54 / 1.17, 8 M 4.35 / 1.53; without hubs or below 8
-// arcs a vertex the masks alone win (4 M x 16 uniform 1.50 / 1.64, R-MAT 4 M x 8
-// 1.52 / 1.72, k-NN 1 M x 8 0.82 / 2.09).
+// hub's own two sets: those cost 0.7-1.5 ms whatever the size (their rounds are
+// bound by latency), the masks alone 0.02-0.04 ms a million arcs. Masks alone
+// against the hub first, R-MAT of edge factor 16, 64 sources: 1 M vertices (16 M arcs)
+// 0.55 / 0.84 ms, 2 M 1.05 / 1.06, 4 M 1.70 / 1.16, 8 M 2.94 / 1.54; of edge factor 32, 1 M
+// vertices (31 M arcs) 0.98 / 0.71. Without hubs or below 8 arcs a vertex the masks
+// alone win (R-MAT 4 M x 8 1.05).
 constexpr int64_t kHubArcs = 1 << 24;
 
 // Masks of the sources dsrc (device) along direction dir: words = 1 or 2 mask

@@ -13,7 +13,7 @@
 // source of H stops at its border.
 //
 // Measured (both directions, GB300): R-MAT of 4 M vertices, 64 sources 14.6 ->
-// 2.33 ms, 3D torus of 1 M vertices, 7 sources 3.15 -> 2.30, against one search of
+// 2.30 ms, 3D torus of 1 M vertices, 7 sources 3.15 -> 1.31, against one search of
 // 64-bit masks by the engine's rounds. The R-MAT time is the hub's four bitmap
 // searches; the masks' own search ends after a few hops.
 #include <algorithm>
